@@ -50,12 +50,46 @@ __device__ __forceinline__ int find_level(const uint64_t* first, int nlev, uint6
   return lo;
 }
 
-// r-th (0-based) set bit of v
+// r-th (0-based) set bit of v, by halving (__fns steps bit by bit)
 __device__ __forceinline__ uint32_t sel64(uint64_t v, uint32_t r) {
-  const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
-  const uint32_t pl = __popc(lo);
-  if (r < pl) return __fns(lo, 0, (int)r + 1);
-  return 32 + __fns(hi, 0, (int)(r - pl) + 1);
+  uint32_t x = (uint32_t)v, at = 0;
+  const uint32_t pl = __popc(x);
+  if (r >= pl) {
+    r -= pl;
+    x = (uint32_t)(v >> 32);
+    at = 32;
+  }
+#pragma unroll
+  for (uint32_t w = 16; w > 0; w >>= 1) {
+    const uint32_t c = __popc(x & ((1u << w) - 1u));
+    if (r >= c) {
+      r -= c;
+      x >>= w;
+      at += w;
+    }
+  }
+  return at;
+}
+
+// The eight words of a 64-byte directory block, requested together: one
+// round of loads instead of one per word visited.  PADDED as the word count
+// marks a level of the library's own (16-byte aligned, padded to 2048 bits);
+// of a caller's bitvector the words at or past nw are not read.
+constexpr uint64_t PADDED = ~0ull;
+__device__ __forceinline__ void load_block(const uint64_t* lbits, uint64_t w0, uint64_t nw,
+                                           uint64_t v[8]) {
+  if (nw == PADDED) {
+    const ulonglong2* p = (const ulonglong2*)(lbits + w0);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const ulonglong2 q = p[i];
+      v[2 * i] = q.x;
+      v[2 * i + 1] = q.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = w0 + i < nw ? lbits[w0 + i] : 0ull;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -176,9 +210,9 @@ __global__ void k_dir_finish(const LevelMeta* meta, int nlev, const uint64_t* sb
 }
 
 // position (inside superblock s, relative to its start) of the r-th
-// (0-based) bit equal to bv
+// (0-based) bit equal to bv, which lies in s; nw as for load_block
 __device__ uint32_t find_in_sb(const uint64_t* lbits, const uint64_t* ldir, uint64_t s, int bv,
-                               uint32_t r) {
+                               uint32_t r, uint64_t nw) {
   const uint64_t rel = ldir[2 * s + 1];
   int b = 3;
   for (; b > 0; b--) {
@@ -188,41 +222,25 @@ __device__ uint32_t find_in_sb(const uint64_t* lbits, const uint64_t* ldir, uint
   }
   const uint32_t z = b ? (uint32_t)((rel >> (16 * b)) & 0xffffu) : 0u;
   r -= bv ? 512u * b - z : z;
-  // the target lies in this superblock, so at most 32 words are visited
-  for (uint64_t w = 32 * s + 8 * b; w < 32 * s + 32; w++) {
-    const uint64_t v = lbits[w];
-    const uint32_t c = bv ? __popcll(v) : 64 - __popcll(v);
-    if (c > r) return (uint32_t)((w - 32 * s) * 64) + sel64(bv ? v : ~v, r);
-    r -= c;
-  }
-  return 2047;
-}
-
-// The same for the sample kernel, with the target block's eight words loaded
-// together (one round of loads instead of one per word visited); words at
-// or past nw, the level's word count, are not read.
-__device__ uint32_t find_in_sb_blk(const uint64_t* lbits, const uint64_t* ldir, uint64_t s,
-                                   int bv, uint32_t r, uint64_t nw) {
-  const uint64_t rel = ldir[2 * s + 1];
-  int b = 3;
-  for (; b > 0; b--) {
-    const uint32_t z = (uint32_t)((rel >> (16 * b)) & 0xffffu);
-    const uint32_t before = bv ? 512u * b - z : z;
-    if (before <= r) break;
-  }
-  const uint32_t z = b ? (uint32_t)((rel >> (16 * b)) & 0xffffu) : 0u;
-  r -= bv ? 512u * b - z : z;
-  const uint64_t w0 = 32 * s + 8 * (uint64_t)b;
   uint64_t v[8];
-#pragma unroll
-  for (int i = 0; i < 8; i++) v[i] = w0 + i < nw ? lbits[w0 + i] : 0ull;
+  load_block(lbits, 32 * s + 8 * (uint64_t)b, nw, v);
+  uint64_t word = 0;
+  int at = -1;
 #pragma unroll
   for (int i = 0; i < 8; i++) {
-    const uint32_t c = bv ? __popcll(v[i]) : 64 - __popcll(v[i]);
-    if (c > r) return (uint32_t)((8 * b + i) * 64) + sel64(bv ? v[i] : ~v[i], r);
-    r -= c;
+    const uint64_t x = bv ? v[i] : ~v[i];
+    const uint32_t c = (uint32_t)__popcll(x);
+    if (at < 0) {
+      if (c > r) {
+        at = i;
+        word = x;
+      } else {
+        r -= c;
+      }
+    }
   }
-  return 2047;
+  if (at < 0) return 2047;
+  return (uint32_t)((8 * b + at) * 64) + sel64(word, r);
 }
 
 template <bool SMALL>
@@ -250,13 +268,16 @@ __global__ void k_select_samples(const uint64_t* bits, const LevelMeta* meta, in
   const uint64_t zs = ze - zb;
   const uint64_t nvalid = std::min<uint64_t>(2048, m.n - 2048 * s);
   const uint64_t ob = 2048 * s - zb, os = nvalid - zs;
-  const uint64_t nw = (m.n + 63) / 64;
+  // a whole superblock's words can all be read; the last one's, and those of a
+  // caller's bitvector off a 16-byte boundary, one by one up to the end
+  const bool whole = s + 1 < m.nsb && (((uintptr_t)lb) & 15) == 0;
+  const uint64_t nw = whole ? PADDED : (m.n + 63) / 64;
   const uint64_t k0 = (zb + 4095) / 4096;
   if (4096 * k0 < zb + zs)
-    samp[m.s0_off + k0] = 2048 * s + find_in_sb_blk(lb, ld, s, 0, (uint32_t)(4096 * k0 - zb), nw);
+    samp[m.s0_off + k0] = 2048 * s + find_in_sb(lb, ld, s, 0, (uint32_t)(4096 * k0 - zb), nw);
   const uint64_t k1 = (ob + 4095) / 4096;
   if (4096 * k1 < ob + os)
-    samp[m.s1_off + k1] = 2048 * s + find_in_sb_blk(lb, ld, s, 1, (uint32_t)(4096 * k1 - ob), nw);
+    samp[m.s1_off + k1] = 2048 * s + find_in_sb(lb, ld, s, 1, (uint32_t)(4096 * k1 - ob), nw);
 }
 
 // ---------------------------------------------------------------------------
@@ -401,13 +422,25 @@ __device__ uint32_t find_in_dsb(const uint64_t* lbits, const uint64_t* ldir, uin
   for (; b > 0; b--)
     if (((ldir[8 * s + 4 + b] >> (16 * d)) & 0xffffull) <= r) break;
   r -= b ? (uint32_t)((ldir[8 * s + 4 + b] >> (16 * d)) & 0xffffull) : 0u;
-  for (uint64_t w = 32 * s + 8 * b; w < 32 * s + 32; w++) {
-    const uint64_t m = digit_match(lbits[w], d);
-    const uint32_t c = __popcll(m);
-    if (c > r) return (uint32_t)((w - 32 * s) * 32 + sel64(m, r) / 2);
-    r -= c;
+  uint64_t v[8];
+  load_block(lbits, 32 * s + 8 * (uint64_t)b, PADDED, v);
+  uint64_t word = 0;
+  int at = -1;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    const uint64_t m = digit_match(v[i], d);
+    const uint32_t c = (uint32_t)__popcll(m);
+    if (at < 0) {
+      if (c > r) {
+        at = i;
+        word = m;
+      } else {
+        r -= c;
+      }
+    }
   }
-  return 1023;
+  if (at < 0) return 1023;
+  return (uint32_t)((8 * b + at) * 32) + sel64(word, r) / 2;
 }
 
 // every 4096th occurrence of each digit value: one thread per superblock
@@ -522,18 +555,30 @@ __device__ __forceinline__ uint64_t occ_before(const uint64_t* ldir, int b, uint
 }
 
 // position of occurrence q of value b, known to lie in superblocks [lo, hi]
-// of the level (q >= occurrences before lo)
+// of the level (q >= occurrences before lo); nw as for load_block.  Each step
+// reads seven evenly spaced records at once: between two samples of a dense
+// level lie four or five superblocks, found in one round of loads where a
+// binary search takes three dependent ones.
 template <bool DIG>
 __device__ uint64_t dir_select(const uint64_t* lbits, const uint64_t* ldir, int b, uint64_t q,
-                               uint64_t lo, uint64_t hi) {
+                               uint64_t lo, uint64_t hi, uint64_t nw) {
   while (lo < hi) {
-    const uint64_t mid = (lo + hi + 1) >> 1;
-    if (occ_before<DIG>(ldir, b, mid) <= q) lo = mid;
-    else hi = mid - 1;
+    const uint64_t step = (hi - lo + 7) >> 3;
+    uint64_t before[7];
+#pragma unroll
+    for (int i = 0; i < 7; i++) {
+      const uint64_t s = lo + (uint64_t)(i + 1) * step;
+      before[i] = s <= hi ? occ_before<DIG>(ldir, b, s) : ~0ull;
+    }
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < 7; i++) c += before[i] <= q ? 1u : 0u;
+    lo += c * step;
+    if (c < 7 && lo + step - 1 < hi) hi = lo + step - 1;
   }
   const uint32_t r = (uint32_t)(q - occ_before<DIG>(ldir, b, lo));
   if (DIG) return 1024 * lo + find_in_dsb(lbits, ldir, lo, (uint32_t)b, r);
-  return 2048 * lo + find_in_sb(lbits, ldir, lo, b, r);
+  return 2048 * lo + find_in_sb(lbits, ldir, lo, b, r, nw);
 }
 
 // one (level, bit or digit value) of the directory build
@@ -574,10 +619,11 @@ __global__ void k_ck_ranges(const uint64_t* bits, const uint64_t* dir, const uin
   uint64_t prev = S1;  // start of sub-range i
   constexpr int SBSH = DIG ? 10 : 11;
   const uint64_t lo_sb = S1 >> SBSH, hi_sb = (e - 1) >> SBSH;
+  const uint64_t nw = DIG ? PADDED : (sg.n + 63) / 64;
   for (int i = 0; i < 16; i++) {
     const uint64_t m = 16 * k + i;
     uint64_t start = 0;
-    if (!huge && m < M) start = i == 0 ? S1 : dir_select<DIG>(lbits, ldir, sg.b, 256 * m, lo_sb, hi_sb);
+    if (!huge && m < M) start = i == 0 ? S1 : dir_select<DIG>(lbits, ldir, sg.b, 256 * m, lo_sb, hi_sb, nw);
     sub[16 * g + i] = huge ? 0u : (m < M ? (uint32_t)(start - S1) : 0xffffffffu);
     if (!huge && i > 0 && m - 1 < M && m < M && start - prev >= CK_SPARSE_MIN) mask |= 1u << (i - 1);
     if (!huge && m < M) prev = start;
@@ -616,11 +662,12 @@ __global__ void k_ck_fill(const uint64_t* bits, const uint64_t* dir, const uint6
     const uint64_t e = (k + 1 < R) ? samp[sg.samp_off + k + 1] : sg.n;
     constexpr int SBSH = DIG ? 10 : 11;
     const uint64_t lo_sb = S1 >> SBSH, hi_sb = (e - 1) >> SBSH;
+    const uint64_t nw = DIG ? PADDED : (sg.n + 63) / 64;
     if (kd >> 63) {
       for (uint32_t j = threadIdx.x; j < 4096; j += blockDim.x) {
         const uint64_t q = 4096 * k + j;
         huge_all[4096 * gh[g] + j] =
-            q < sg.cnt ? dir_select<DIG>(lbits, ldir, sg.b, q, lo_sb, hi_sb) : ~0ull;
+            q < sg.cnt ? dir_select<DIG>(lbits, ldir, sg.b, q, lo_sb, hi_sb, nw) : ~0ull;
       }
     } else {
       uint32_t mask = (uint32_t)kd;
@@ -631,7 +678,7 @@ __global__ void k_ck_fill(const uint64_t* bits, const uint64_t* dir, const uint6
         for (uint32_t j = threadIdx.x; j < 256; j += blockDim.x) {
           const uint64_t q = 4096 * k + 256 * i + j;
           sparse_all[256 * s + j] =
-              q < sg.cnt ? (uint32_t)(dir_select<DIG>(lbits, ldir, sg.b, q, lo_sb, hi_sb) - S1)
+              q < sg.cnt ? (uint32_t)(dir_select<DIG>(lbits, ldir, sg.b, q, lo_sb, hi_sb, nw) - S1)
                          : 0xffffffffu;
         }
         s++;
@@ -908,6 +955,7 @@ struct BinLevel {
   const uint64_t* s0;
   const uint64_t* s1;
   uint64_t n, nsb, zeros;
+  uint64_t nw;  // as for load_block
   const ClarkMeta* cm;
   const uint64_t* ck64;
   const uint32_t* ck32;
@@ -923,6 +971,27 @@ __device__ __forceinline__ BinLevel bin_level(const QStruct& S, int l) {
   v.n = m.n;
   v.nsb = m.nsb;
   v.zeros = S.zeros[l];
+  v.nw = S.kind == WT_KIND_RS ? (m.n + 63) / 64 : PADDED;
+  v.cm = S.cmeta ? S.cmeta + l : nullptr;
+  v.ck64 = S.ck64;
+  v.ck32 = S.ck32;
+  return v;
+}
+
+// The same for a wavelet matrix or a balanced tree, whose levels all have n
+// bits: the offsets follow from n and l, so that no table read stands before
+// a level's first access.
+__device__ __forceinline__ BinLevel uniform_level(const QStruct& S, int l) {
+  const uint64_t nsb = (S.n + 2047) >> 11, cap = (S.n >> 12) + 1;
+  BinLevel v;
+  v.bits = S.bits + (uint64_t)l * 32 * nsb;
+  v.dir = S.dir + (uint64_t)l * 2 * (nsb + 1);
+  v.s0 = S.samp + (uint64_t)(2 * l) * cap;
+  v.s1 = v.s0 + cap;
+  v.n = S.n;
+  v.nsb = nsb;
+  v.zeros = S.zeros[l];
+  v.nw = PADDED;
   v.cm = S.cmeta ? S.cmeta + l : nullptr;
   v.ck64 = S.ck64;
   v.ck32 = S.ck32;
@@ -933,16 +1002,55 @@ __device__ __forceinline__ int get_bit(const BinLevel& v, uint64_t i) {
   return (int)((v.bits[i >> 6] >> (i & 63)) & 1ull);
 }
 
+// A level at one position x: its directory record and the words of x's
+// 512-bit block that hold bits before x.  All of it is requested at once, and
+// the lines of several positions before any of them is used: a query is
+// bound by the latency of its chain of levels (and by L2 and DRAM sectors
+// when many run), so a level costs one round of loads, where words read one
+// after another up to the position cost a round each.  With the searches of
+// dir_select and the joint walks below: 2^22 ranks on 2^30 symbols of 16
+// levels 2.85 -> 1.79 ms;
+// 2^16 mixed queries over 64 matrices of up to 2^22 symbols 270 -> 82 us.
+struct Line {
+  ulonglong2 rec;
+  uint64_t w[8];
+};
+
+__device__ __forceinline__ Line load_line(const BinLevel& v, uint64_t x) {
+  Line ln;
+  const uint32_t in = (uint32_t)(x & 511);
+  const uint64_t* p = v.bits + 8 * (x >> 9);
+  ln.rec = *(const ulonglong2*)(v.dir + 2 * (x >> 11));
+  if (v.nw == PADDED) {
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      ulonglong2 q = make_ulonglong2(0, 0);
+      if ((uint32_t)(128 * i) < in) q = ((const ulonglong2*)p)[i];
+      ln.w[2 * i] = q.x;
+      ln.w[2 * i + 1] = q.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; i++) ln.w[i] = (uint32_t)(64 * i) < in ? p[i] : 0ull;
+  }
+  return ln;
+}
+
 // zeros in [0, x), x <= n
-__device__ uint64_t rank0(const BinLevel& v, uint64_t x) {
-  const uint64_t s = x >> 11;
-  const uint32_t b = (uint32_t)((x >> 9) & 3);
-  uint64_t r = v.dir[2 * s] + ((v.dir[2 * s + 1] >> (16 * b)) & 0xffffull);
-  const uint64_t wend = x >> 6;
-  for (uint64_t w = 32 * s + 8 * b; w < wend; w++) r += 64 - __popcll(v.bits[w]);
-  const uint32_t rem = (uint32_t)(x & 63);
-  if (rem) r += rem - __popcll(v.bits[wend] & ((1ull << rem) - 1ull));
-  return r;
+__device__ __forceinline__ uint64_t zeros_before(const Line& ln, uint64_t x) {
+  const uint32_t b = (uint32_t)((x >> 9) & 3), in = (uint32_t)(x & 511), k = in >> 6;
+  const uint64_t part = (1ull << (in & 63)) - 1ull;
+  uint32_t ones = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 8; i++) {
+    const uint64_t m = i < k ? ~0ull : (i == k ? part : 0ull);
+    ones += (uint32_t)__popcll(ln.w[i] & m);
+  }
+  return ln.rec.x + ((ln.rec.y >> (16 * b)) & 0xffffull) + (in - ones);
+}
+
+__device__ __forceinline__ uint64_t rank0(const BinLevel& v, uint64_t x) {
+  return zeros_before(load_line(v, x), x);
 }
 __device__ __forceinline__ uint64_t rank1(const BinLevel& v, uint64_t x) { return x - rank0(v, x); }
 
@@ -971,119 +1079,94 @@ __device__ uint64_t select_b(const BinLevel& v, int bv, uint64_t k) {
       const uint64_t ns = ((bv ? v.n - v.zeros : v.zeros) + 4095) / 4096;
       p1 = kk + 1 < ns ? samp[kk + 1] : v.n;
     }
-    return dir_select<false>(v.bits, v.dir, bv, k, p0 >> 11, (p1 - 1) >> 11);
+    return dir_select<false>(v.bits, v.dir, bv, k, p0 >> 11, (p1 - 1) >> 11, v.nw);
   }
   const uint64_t cnt = bv ? v.n - v.zeros : v.zeros;
   const uint64_t ns = (cnt + 4095) / 4096;
   const uint64_t idx = k >> 12;
-  uint64_t lo = samp[idx] >> 11;
-  uint64_t hi = (idx + 1 < ns) ? (samp[idx + 1] >> 11) : v.nsb - 1;
-  auto before = [&](uint64_t s) -> uint64_t {
-    const uint64_t z = v.dir[2 * s];
-    return bv ? 2048 * s - z : z;
-  };
-  while (lo < hi) {
-    const uint64_t mid = (lo + hi + 1) >> 1;
-    if (before(mid) <= k) lo = mid;
-    else hi = mid - 1;
-  }
-  return 2048 * lo + find_in_sb(v.bits, v.dir, lo, bv, (uint32_t)(k - before(lo)));
+  const uint64_t lo = samp[idx] >> 11;
+  const uint64_t hi = (idx + 1 < ns) ? (samp[idx + 1] >> 11) : v.nsb - 1;
+  return dir_select<false>(v.bits, v.dir, bv, k, lo, hi, v.nw);
 }
 
-
+// Wavelet matrix.  The three operations walk down together, so that a warp
+// with a mixture of them walks once: rank and select carry the start s and
+// the end p of the symbol's class, access the position p alone.  Select then
+// walks up.
 __device__ uint64_t q_wm(const QStruct& S, int op, uint32_t c, uint64_t x) {
   const int L = S.L;
-  if (op == 0) {
-    if (x >= S.n) return NONE;
-    uint64_t pos = x, sym = 0;
-    for (int l = 0; l < L; l++) {
-      const BinLevel v = bin_level(S, l);
-      const int b = get_bit(v, pos);
-      sym = (sym << 1) | (uint64_t)b;
-      pos = b ? v.zeros + rank1(v, pos) : rank0(v, pos);
-    }
-    return sym;
-  }
-  if (c >= S.sigma) return NONE;
-  if (op == 1) {
-    if (x >= S.n) return NONE;
-    uint64_t s = 0, j = x + 1;
-    for (int l = 0; l < L; l++) {
-      const BinLevel v = bin_level(S, l);
-      const int b = (c >> (L - 1 - l)) & 1;
-      if (b) { s = v.zeros + rank1(v, s); j = v.zeros + rank1(v, j); }
-      else { s = rank0(v, s); j = rank0(v, j); }
-    }
-    return j - s;
-  }
-  if (x == 0) return NONE;
-  uint64_t s = 0, e = S.n;
+  if (op == 2 ? x == 0 : x >= S.n) return NONE;
+  if (op != 0 && c >= S.sigma) return NONE;
+  uint64_t s = 0, p = op == 0 ? x : (op == 1 ? x + 1 : S.n);
+  uint32_t sym = 0;
   for (int l = 0; l < L; l++) {
-    const BinLevel v = bin_level(S, l);
-    const int b = (c >> (L - 1 - l)) & 1;
-    if (b) { s = v.zeros + rank1(v, s); e = v.zeros + rank1(v, e); }
-    else { s = rank0(v, s); e = rank0(v, e); }
+    const BinLevel v = uniform_level(S, l);
+    const Line lp = load_line(v, p);
+    Line ls;
+    int b = (int)((c >> (L - 1 - l)) & 1u);
+    if (op == 0) b = get_bit(v, p);
+    else ls = load_line(v, s);
+    const uint64_t zp = zeros_before(lp, p);
+    p = b ? v.zeros + (p - zp) : zp;
+    if (op == 0) {
+      sym = (sym << 1) | (uint32_t)b;
+    } else {
+      const uint64_t zs = zeros_before(ls, s);
+      s = b ? v.zeros + (s - zs) : zs;
+    }
   }
-  if (x > e - s) return NONE;
+  if (op == 0) return sym;
+  if (op == 1) return p - s;
+  if (x > p - s) return NONE;
   uint64_t pos = s + x - 1;
   for (int l = L - 1; l >= 0; l--) {
-    const BinLevel v = bin_level(S, l);
-    const int b = (c >> (L - 1 - l)) & 1;
-    pos = b ? select_b(v, 1, pos - v.zeros) : select_b(v, 0, pos);
+    const BinLevel v = uniform_level(S, l);
+    const int b = (int)((c >> (L - 1 - l)) & 1u);
+    pos = select_b(v, b, b ? pos - v.zeros : pos);
   }
   return pos;
 }
 
+// Balanced tree: the node's start s and end e, and the position p in it
+// (access, rank), walked down together; select keeps every level's start and
+// the zeros before it for its way up.
 __device__ uint64_t q_wt(const QStruct& S, int op, uint32_t c, uint64_t x) {
   const int L = S.L;
-  if (op == 0) {
-    if (x >= S.n) return NONE;
-    uint64_t s = 0, e = S.n, pos = x, sym = 0;
-    for (int l = 0; l < L; l++) {
-      const BinLevel v = bin_level(S, l);
-      const uint64_t zs = rank0(v, s), zp = rank0(v, pos), ze = rank0(v, e);
-      const int b = get_bit(v, pos);
-      sym = (sym << 1) | (uint64_t)b;
-      if (!b) { pos = s + (zp - zs); e = s + (ze - zs); }
-      else { pos = s + (ze - zs) + (pos - s) - (zp - zs); s = s + (ze - zs); }
-    }
-    return sym;
-  }
-  if (c >= S.sigma) return NONE;
-  if (op == 1) {
-    if (x >= S.n) return NONE;
-    uint64_t s = 0, e = S.n, j = x + 1;
-    for (int l = 0; l < L; l++) {
-      const BinLevel v = bin_level(S, l);
-      const uint64_t zs = rank0(v, s), zj = rank0(v, j), ze = rank0(v, e);
-      const int b = (c >> (L - 1 - l)) & 1;
-      if (!b) { j = s + (zj - zs); e = s + (ze - zs); }
-      else { j = s + (ze - zs) + (j - s) - (zj - zs); s = s + (ze - zs); }
-    }
-    return j - s;
-  }
-  if (x == 0) return NONE;
-  uint64_t S0[33];
-  uint64_t s = 0, e = S.n;
+  if (op == 2 ? x == 0 : x >= S.n) return NONE;
+  if (op != 0 && c >= S.sigma) return NONE;
+  uint64_t S0[33], Z0[33];
+  uint64_t s = 0, e = S.n, p = op == 1 ? x + 1 : x;
+  uint32_t sym = 0;
   for (int l = 0; l < L; l++) {
-    S0[l] = s;
-    const BinLevel v = bin_level(S, l);
-    const uint64_t zs = rank0(v, s), ze = rank0(v, e);
-    const int b = (c >> (L - 1 - l)) & 1;
-    if (!b) e = s + (ze - zs);
-    else s = s + (ze - zs);
+    const BinLevel v = uniform_level(S, l);
+    const Line le = load_line(v, e), ls = load_line(v, s);
+    Line lp;
+    int b = (int)((c >> (L - 1 - l)) & 1u);
+    if (op != 2) lp = load_line(v, p);
+    if (op == 0) b = get_bit(v, p);
+    const uint64_t zs = zeros_before(ls, s), ze = zeros_before(le, e);
+    const uint64_t m = s + (ze - zs);  // end of the zeros' child
+    if (op == 2) {
+      S0[l] = s;
+      Z0[l] = zs;
+    } else {
+      const uint64_t zp = zeros_before(lp, p);
+      p = b ? m + (p - s) - (zp - zs) : s + (zp - zs);
+      sym = (sym << 1) | (uint32_t)b;
+    }
+    if (b) s = m;
+    else e = m;
   }
-  S0[L] = s;
+  if (op == 0) return sym;
+  if (op == 1) return p - s;
   if (x > e - s) return NONE;
-  uint64_t pos = s + x - 1;
+  uint64_t off = x - 1;
   for (int l = L - 1; l >= 0; l--) {
-    const BinLevel v = bin_level(S, l);
-    const int b = (c >> (L - 1 - l)) & 1;
-    const uint64_t off = pos - S0[l + 1];
-    const uint64_t zs = rank0(v, S0[l]);
-    pos = b ? select_b(v, 1, (S0[l] - zs) + off) : select_b(v, 0, zs + off);
+    const BinLevel v = uniform_level(S, l);
+    const int b = (int)((c >> (L - 1 - l)) & 1u);
+    off = select_b(v, b, (b ? S0[l] - Z0[l] : Z0[l]) + off) - S0[l];
   }
-  return pos;
+  return off;  // the root starts at 0
 }
 
 // Huffman-shaped tree: node (level l, prefix q) -> [start, end) on level l
@@ -1104,19 +1187,21 @@ __device__ uint64_t q_huff(const QStruct& S, int op, uint32_t c, uint64_t x) {
     uint64_t q = 0, s = 0, pos = x;
     for (int l = 0; l < S.L; l++) {
       const BinLevel v = bin_level(S, l);
+      const Line lp = load_line(v, pos), ls = load_line(v, s);
       const int b = get_bit(v, pos);
       const uint64_t child = (q << 1) | (uint64_t)b;
-      const uint64_t cnt_b = b ? (pos - s) - (rank0(v, pos) - rank0(v, s)) : rank0(v, pos) - rank0(v, s);
       uint64_t cs, ce;
-      if (!huff_node(S, l + 1, child, cs, ce)) {
+      const bool inner = huff_node(S, l + 1, child, cs, ce);
+      if (!inner) {
         // a leaf at depth l+1: canonical code -> symbol
         const int ln = l + 1;
         const uint64_t first = S.hq.len_first[ln], base = S.hq.len_base[ln];
         return S.hq.sym_by_rank[base + (child - first)];
       }
+      const uint64_t z = zeros_before(lp, pos) - zeros_before(ls, s);
       q = child;
+      pos = cs + (b ? (pos - s) - z : z);
       s = cs;
-      pos = cs + cnt_b;
     }
     return NONE;
   }
@@ -1130,44 +1215,45 @@ __device__ uint64_t q_huff(const QStruct& S, int op, uint32_t c, uint64_t x) {
     for (int l = 0; l < ln; l++) {
       const BinLevel v = bin_level(S, l);
       const int b = (int)((code >> (ln - 1 - l)) & 1u);
-      const uint64_t z = rank0(v, j) - rank0(v, s);
+      const Line lj = load_line(v, j), ls = load_line(v, s);
+      q = (q << 1) | (uint64_t)b;
+      uint64_t cs = 0, ce;
+      if (l + 1 < ln) huff_node(S, l + 1, q, cs, ce);
+      const uint64_t z = zeros_before(lj, j) - zeros_before(ls, s);
       const uint64_t cb = b ? (j - s) - z : z;
       if (l == ln - 1) return cb;
-      q = (q << 1) | (uint64_t)b;
-      uint64_t cs, ce;
-      huff_node(S, l + 1, q, cs, ce);
       s = cs;
       j = cs + cb;
     }
     return NONE;
   }
   if (x == 0 || ln == 0) return NONE;
-  uint64_t S0[33];
+  // the code's nodes and the zeros before each on the way down; only the
+  // last level's count of the code's bit decides whether there are x
+  uint64_t S0[33], Z0[33];
   uint64_t q = 0, s = 0, e = S.n;
   for (int l = 0; l < ln; l++) {
-    S0[l] = s;
     const BinLevel v = bin_level(S, l);
     const int b = (int)((code >> (ln - 1 - l)) & 1u);
-    const uint64_t z = rank0(v, e) - rank0(v, s);
-    const uint64_t cb = b ? (e - s) - z : z;
+    const uint64_t zs = rank0(v, s);
+    S0[l] = s;
+    Z0[l] = zs;
     if (l == ln - 1) {
-      if (x > cb) return NONE;
+      const uint64_t z = rank0(v, e) - zs;
+      if (x > (b ? (e - s) - z : z)) return NONE;
       break;
     }
     q = (q << 1) | (uint64_t)b;
-    uint64_t cs, ce;
-    huff_node(S, l + 1, q, cs, ce);
-    s = cs;
-    e = ce;
+    // the child [s, e) of the code's bit, from the node table
+    huff_node(S, l + 1, q, s, e);
   }
   // bottom-up: at level l the target is the off-th b-bit of node [S0[l], .)
   uint64_t off = x - 1, pos = 0;
   for (int l = ln - 1; l >= 0; l--) {
     const BinLevel v = bin_level(S, l);
     const int b = (int)((code >> (ln - 1 - l)) & 1u);
-    const uint64_t zs = rank0(v, S0[l]);
-    pos = b ? select_b(v, 1, (S0[l] - zs) + off) : select_b(v, 0, zs + off);
-    if (l > 0) off = pos - S0[l];
+    pos = select_b(v, b, (b ? S0[l] - Z0[l] : Z0[l]) + off);
+    off = pos - S0[l];
   }
   return pos;
 }
@@ -1197,16 +1283,52 @@ __device__ __forceinline__ DigLevel dig_level(const QStruct& S, int l) {
   return v;
 }
 
-// count of digit d in [0, x)
-__device__ uint64_t rank_d(const DigLevel& v, uint32_t d, uint64_t x) {
-  const uint64_t s = x >> 10;
-  const uint32_t b = (uint32_t)((x >> 8) & 3);
-  uint64_t r = v.dir[8 * s + d] + ((v.dir[8 * s + 4 + b] >> (16 * d)) & 0xffffull);
-  const uint64_t wend = x >> 5;
-  for (uint64_t w = 32 * s + 8 * b; w < wend; w++) r += __popcll(digit_match(v.bits[w], d));
-  const uint32_t rem = (uint32_t)(x & 31);
-  if (rem) r += __popcll(digit_match(v.bits[wend], d) & ((1ull << (2 * rem)) - 1ull));
-  return r;
+// A digit level at one position: the counts before its superblock and its
+// 256-digit block, and the block's words with digits before it, all
+// requested at once (see Line).
+struct DigLine {
+  ulonglong2 c01, c23;
+  uint64_t rel;
+  uint64_t w[8];
+};
+
+__device__ __forceinline__ DigLine load_dig(const DigLevel& v, uint64_t x) {
+  DigLine ln;
+  const uint32_t in = (uint32_t)(x & 255);
+  const uint64_t* r = v.dir + 8 * (x >> 10);
+  ln.c01 = *(const ulonglong2*)r;
+  ln.c23 = *(const ulonglong2*)(r + 2);
+  ln.rel = r[4 + ((x >> 8) & 3)];
+  const ulonglong2* p = (const ulonglong2*)(v.bits + 8 * (x >> 8));
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    ulonglong2 q = make_ulonglong2(0, 0);
+    if ((uint32_t)(64 * i) < in) q = p[i];
+    ln.w[2 * i] = q.x;
+    ln.w[2 * i + 1] = q.y;
+  }
+  return ln;
+}
+
+// digits equal to d (eq) and smaller than d (lt) in [0, x)
+__device__ __forceinline__ void dig_counts(const DigLine& ln, uint64_t x, uint32_t d, uint64_t& eq,
+                                           uint64_t& lt) {
+  const uint32_t in = (uint32_t)(x & 255), k = in >> 5;
+  const uint64_t part = (1ull << (2 * (in & 31))) - 1ull;
+  auto rel = [&](int v) -> uint64_t { return (ln.rel >> (16 * v)) & 0xffffull; };
+  const uint64_t c0 = ln.c01.x + rel(0), c1 = ln.c01.y + rel(1), c2 = ln.c23.x + rel(2),
+                 c3 = ln.c23.y + rel(3);
+  uint32_t e = 0, s = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 8; i++) {
+    const uint64_t m = (i < k ? ~0ull : (i == k ? part : 0ull)) & 0x5555555555555555ull;
+    const uint64_t lo = ln.w[i], hi = lo >> 1;
+    e += (uint32_t)__popcll(digit_match(lo, d) & m);
+    const uint64_t less = d == 0 ? 0ull : (d == 1 ? ~(hi | lo) : (d == 2 ? ~hi : ~(hi & lo)));
+    s += (uint32_t)__popcll(less & m);
+  }
+  eq = e + (d == 0 ? c0 : (d == 1 ? c1 : (d == 2 ? c2 : c3)));
+  lt = s + (d > 0 ? c0 : 0ull) + (d > 1 ? c1 : 0ull) + (d > 2 ? c2 : 0ull);
 }
 
 __device__ __forceinline__ uint32_t get_digit(const DigLevel& v, uint64_t i) {
@@ -1240,80 +1362,62 @@ __device__ uint64_t select_d(const DigLevel& v, uint32_t d, uint64_t k) {
       const uint64_t ns = (v.dir[8 * v.nsb + d] + 4095) / 4096;
       p1 = kk + 1 < ns ? samp[kk + 1] : v.n;
     }
-    return dir_select<true>(v.bits, v.dir, (int)d, k, p0 >> 10, (p1 - 1) >> 10);
+    return dir_select<true>(v.bits, v.dir, (int)d, k, p0 >> 10, (p1 - 1) >> 10, PADDED);
   }
   // sampled: the search starts between two samples
   const uint64_t ns = (v.dir[8 * v.nsb + d] + 4095) / 4096;
   const uint64_t lo = samp[kk] >> 10;
   const uint64_t hi = kk + 1 < ns ? samp[kk + 1] >> 10 : v.nsb - 1;
-  return dir_select<true>(v.bits, v.dir, (int)d, k, lo, hi);
+  return dir_select<true>(v.bits, v.dir, (int)d, k, lo, hi, PADDED);
 }
 
+// The node's start s and end e, and the position p in it (access, rank),
+// walked down together; select keeps for its way up every level's start and
+// the occurrences of its digit before it.
 __device__ uint64_t q_multi(const QStruct& S, int op, uint32_t c, uint64_t x) {
   const int L = S.L, D = S.levels;
+  if (op == 2 ? x == 0 : x >= S.n) return NONE;
+  if (op != 0 && c >= S.sigma) return NONE;
   auto dwidth = [&](int be) { return (2 * be + 1 < L) ? 2 : 1; };
   auto cdigit = [&](int be) -> uint32_t {
     const int w = dwidth(be);
     const int sh = L - 2 * be - w;
     return (c >> sh) & ((1u << w) - 1u);
   };
-  if (op == 0) {
-    if (x >= S.n) return NONE;
-    uint64_t s = 0, e = S.n, pos = x, sym = 0;
-    for (int be = 0; be < D; be++) {
-      const DigLevel v = dig_level(S, be);
-      const uint32_t d = get_digit(v, pos);
-      sym = (sym << dwidth(be)) | d;
-      uint64_t cs = s;
-      for (uint32_t d2 = 0; d2 < d; d2++) cs += rank_d(v, d2, e) - rank_d(v, d2, s);
-      const uint64_t rs = rank_d(v, d, s);
-      const uint64_t ne = cs + (rank_d(v, d, e) - rs);
-      pos = cs + (rank_d(v, d, pos) - rs);
-      s = cs;
-      e = ne;
-    }
-    return sym;
-  }
-  if (c >= S.sigma) return NONE;
-  if (op == 1) {
-    if (x >= S.n) return NONE;
-    uint64_t s = 0, e = S.n, j = x + 1;
-    for (int be = 0; be < D; be++) {
-      const DigLevel v = dig_level(S, be);
-      const uint32_t d = cdigit(be);
-      uint64_t cs = s;
-      for (uint32_t d2 = 0; d2 < d; d2++) cs += rank_d(v, d2, e) - rank_d(v, d2, s);
-      const uint64_t rs = rank_d(v, d, s);
-      const uint64_t ne = cs + (rank_d(v, d, e) - rs);
-      j = cs + (rank_d(v, d, j) - rs);
-      s = cs;
-      e = ne;
-    }
-    return j - s;
-  }
-  if (x == 0) return NONE;
-  uint64_t S0[17];
-  uint64_t s = 0, e = S.n;
+  uint64_t S0[17], R0[17];
+  uint64_t s = 0, e = S.n, p = op == 1 ? x + 1 : x;
+  uint32_t sym = 0;
   for (int be = 0; be < D; be++) {
-    S0[be] = s;
     const DigLevel v = dig_level(S, be);
-    const uint32_t d = cdigit(be);
-    uint64_t cs = s;
-    for (uint32_t d2 = 0; d2 < d; d2++) cs += rank_d(v, d2, e) - rank_d(v, d2, s);
-    const uint64_t ne = cs + (rank_d(v, d, e) - rank_d(v, d, s));
+    const DigLine le = load_dig(v, e), ls = load_dig(v, s);
+    DigLine lp;
+    if (op != 2) lp = load_dig(v, p);
+    const uint32_t d = op == 0 ? get_digit(v, p) : cdigit(be);
+    uint64_t qs, ts, qe, te;
+    dig_counts(ls, s, d, qs, ts);
+    dig_counts(le, e, d, qe, te);
+    const uint64_t cs = s + (te - ts);
+    if (op == 2) {
+      S0[be] = s;
+      R0[be] = qs;
+    } else {
+      uint64_t qp, tp;
+      dig_counts(lp, p, d, qp, tp);
+      p = cs + (qp - qs);
+      sym = (sym << dwidth(be)) | d;
+    }
     s = cs;
-    e = ne;
+    e = cs + (qe - qs);
   }
-  S0[D] = s;
+  if (op == 0) return sym;
+  if (op == 1) return p - s;
   if (x > e - s) return NONE;
-  uint64_t pos = s + x - 1;
+  uint64_t off = x - 1;
   for (int be = D - 1; be >= 0; be--) {
     const DigLevel v = dig_level(S, be);
-    const uint32_t d = cdigit(be);
-    const uint64_t off = pos - S0[be + 1];
-    pos = select_d(v, d, rank_d(v, d, S0[be]) + off);
+    off = select_d(v, cdigit(be), R0[be] + off) - S0[be];
   }
-  return pos;
+  return off;  // the root starts at 0
 }
 
 __device__ uint64_t q_rs(const QStruct& S, int op, uint32_t c, uint64_t x) {
@@ -1370,12 +1474,17 @@ static void fill_qstruct(const wt_struct* h, QStruct& S) {
   S.ck32 = h->d_ck32;
 }
 
+// Threads per block: single warps while they all fit on the SMs at once, so
+// that a small batch spreads over all of them.
+static unsigned query_block(uint64_t q) { return q <= (uint64_t)num_sms() * 512 ? 32u : 128u; }
+
 wt_status launch_query(wt_struct* h, int op, const uint32_t* c, const uint64_t* x, uint64_t q,
                        uint64_t* out, cudaStream_t st) {
   if (q == 0) return WT_OK;
   QStruct S;
   fill_qstruct(h, S);
-  k_query<<<(unsigned)((q + 127) / 128), 128, 0, st>>>(S, op, c, x, q, out);
+  const unsigned bt = query_block(q);
+  k_query<<<(unsigned)((q + bt - 1) / bt), bt, 0, st>>>(S, op, c, x, q, out);
   count_launch();
   CK(cudaGetLastError());
   return WT_OK;
@@ -1418,7 +1527,8 @@ wt_status launch_query_multi(wt_struct* const* hs, uint32_t nh, const uint32_t* 
   QStruct* d_tab = nullptr;
   TRY(wk.get(&d_tab, tab.size()));
   TRY(upload(d_tab, tab.data(), tab.size() * sizeof(QStruct), st));
-  k_query_multi<<<(unsigned)((q + 127) / 128), 128, 0, st>>>(d_tab, nh, sid, op, c, x, q, out);
+  const unsigned bt = query_block(q);
+  k_query_multi<<<(unsigned)((q + bt - 1) / bt), bt, 0, st>>>(d_tab, nh, sid, op, c, x, q, out);
   count_launch();
   CK(cudaGetLastError());
   return WT_OK;
