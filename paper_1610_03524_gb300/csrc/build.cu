@@ -126,20 +126,18 @@ __device__ __forceinline__ void for_each_symbol(const void* seq, uint64_t n, uin
   for (uint64_t i = nvec * PER + gtid; i < n; i += gstride) f((uint32_t)s[i]);
 }
 
-// Digit counts of the wavelet matrix's passes: pass g covers levels
-// a = g*tau .. a+t-1; its digit is the t bits below level a, its sort key the
-// digit reversed (Section 4.3: the reverse of the tau bits).
+// Digit counts of the first pass (levels 0 .. t0-1): its digit is the top t0
+// bits, its sort key the digit reversed (Section 4.3: the reverse of the tau
+// bits).
 // Validation and the first pass's digit counts, walked tile by tile (tiles
 // of `tile` symbols, as the first partition pass sees them): each tile's
-// counts of the first pass's reversed digit, and their sums, the first
-// pass's histogram, from the one read of the sequence.  The later passes
-// take their counts from their own tiles (k_tile_counts).
+// counts of the first pass's reversed digit, from one read of the sequence.
+// The later passes take their counts from their own tiles (k_tile_counts).
 template <int WB>
 __global__ void __launch_bounds__(256) k_hist_digits_tiles(const void* seq, uint64_t n,
                                                            uint32_t sigma, int L, int t0,
-                                                           uint64_t* hist, uint32_t* err,
-                                                           uint32_t* tcnt, uint32_t tcs,
-                                                           uint32_t tile, uint4* clear,
+                                                           uint32_t* err, uint32_t* tcnt,
+                                                           uint32_t tcs, uint32_t tile, uint4* clear,
                                                            uint64_t clear_units,
                                                            uint64_t clear_per) {
   using T = typename std::conditional<WB == 1, uint8_t,
@@ -148,7 +146,6 @@ __global__ void __launch_bounds__(256) k_hist_digits_tiles(const void* seq, uint
   const int tid = threadIdx.x;
   th[0][tid] = 0;
   th[1][tid] = 0;
-  uint32_t own = 0;  // this thread's reversed digit, summed over the block's tiles
   __syncthreads();
   const uint32_t rmask = (1u << t0) - 1u;
   const int rsh = 32 - L;
@@ -192,16 +189,128 @@ __global__ void __launch_bounds__(256) k_hist_digits_tiles(const void* seq, uint
     // the other buffer was written out one tile ago; this one now
     const uint32_t c = th[buf][tid];
     if (tid < (int)tcs) tcnt[ti * tcs + tid] = c;
-    own += c;
     th[buf][tid] = 0;
     buf ^= 1;
   }
   if (bad) atomicOr(err, ERR_SYMBOL);
-  // first pass: digit value = the reverse of this thread's t0-bit key
-  if (tid <= (int)rmask && own)
-    atomicAdd((unsigned long long*)&hist[__brev((uint32_t)tid) >> (32 - t0)], (unsigned long long)own);
 }
 
+// The same counts for bytes over SIG = 2 .. 8 values in a single pass
+// (DNA-like text): one warp per tile, sixteen bytes a lane and step as two
+// registers of 4-bit symbols, whose bits' three planes give each value's
+// indicators by one three-input operation; they are added in 4-bit counters,
+// and the lanes' sums by four warp reductions a tile.  No atomics, shared
+// memory or barriers: about 3 instructions per 32 symbols, so that DRAM is
+// the bound (2^32 symbols over 5 values with the zeroing of three levels:
+// 1.0 ms, 5.9 TB/s; shared-memory atomics per symbol took 1.8 ms).  A symbol >= SIG is flagged and counted as a zero (a single
+// pass scatters nothing by these counts).
+template <int SIG>
+__global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, uint64_t n,
+                                                           uint32_t* err, uint32_t* tcnt,
+                                                           uint32_t tcs, uint32_t tile,
+                                                           uint4* clear, uint64_t clear_units,
+                                                           uint64_t clear_per) {
+  constexpr int NV = SIG - 1, T0 = SIG <= 2 ? 1 : (SIG <= 4 ? 2 : 3);
+  constexpr uint32_t M = 0x11111111u;
+  const int lane = threadIdx.x & 31;
+  const uint64_t ntiles = (n + tile - 1) / tile;
+  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const bool vec = (((uintptr_t)seq) & 15) == 0;
+  uint32_t bad = 0;
+  for (uint64_t ti = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; ti < ntiles; ti += nw) {
+    if (clear) clear_share(clear, clear_units, clear_per, ti, lane, 32);
+    const uint64_t i0 = ti * tile;
+    const uint32_t len = (uint32_t)(i0 + tile < n ? tile : n - i0);
+    uint32_t cnt[NV] = {};  // of values 1 .. NV
+    if (vec && len == tile) {
+      const uint4* v = (const uint4*)(seq + i0) + lane;
+      for (uint32_t k0 = 0; k0 < tile / 16; k0 += 128) {  // 4 steps of 32 x 16 bytes
+        uint4 q[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) q[k] = __ldcs(v + k0 + 32 * k);
+        uint32_t acc[NV] = {};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+          bad |= (w[0] | w[1] | w[2] | w[3]) & 0xF8F8F8F8u;
+          const uint32_t x[2] = {(w[0] & 0x07070707u) + 16u * (w[1] & 0x07070707u),
+                                 (w[2] & 0x07070707u) + 16u * (w[3] & 0x07070707u)};
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            if (SIG < 8) bad |= (x[h] + (8u - SIG) * M) & (8u * M);
+            const uint32_t b0 = x[h] & M, b1 = (x[h] >> 1) & M, b2 = (x[h] >> 2) & M;
+#pragma unroll
+            for (int s = 1; s <= NV; s++)
+              acc[s - 1] += ((s & 1) ? b0 : ~b0) & ((s & 2) ? b1 : ~b1) & ((s & 4) ? b2 : ~b2);
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < NV; s++)  // 4-bit counters (at most 8 each) to their sum
+          cnt[s] += (((acc[s] & 0x0F0F0F0Fu) + ((acc[s] >> 4) & 0x0F0F0F0Fu)) * 0x01010101u) >> 24;
+      }
+    } else {
+      for (uint32_t i = lane; i < len; i += 32) {
+        const uint32_t x = seq[i0 + i];
+        bad |= x >= SIG ? 1u : 0u;
+#pragma unroll
+        for (int s = 1; s <= NV; s++) cnt[s - 1] += x == (uint32_t)s ? 1u : 0u;
+      }
+    }
+    // two sums per reduction (a tile has at most 8192 symbols)
+    uint32_t rest = len, mine = 0;
+#pragma unroll
+    for (int s = 0; s < NV; s += 2) {
+      const uint32_t two = __reduce_add_sync(FULL, cnt[s] | (s + 1 < NV ? cnt[s + 1] << 16 : 0u));
+      const uint32_t lo = two & 0xffffu, hi = two >> 16;
+      rest -= lo + hi;
+      if (lane == (int)rev_bits((uint32_t)(s + 1), T0)) mine = lo;
+      if (s + 1 < NV && lane == (int)rev_bits((uint32_t)(s + 2), T0)) mine = hi;
+    }
+    if (lane == 0) mine = rest;
+    tcnt[ti * tcs + lane] = mine;
+  }
+  if (__any_sync(FULL, bad != 0u) && lane == 0) atomicOr(err, ERR_SYMBOL);
+}
+
+// Launch of the first pass's tile counts (t0 levels of L, tiles of T), which
+// also zero `clear_units` 16-byte units at `clear`, a share per tile.
+static wt_status launch_first_counts(const void* seq, int w, uint64_t n, uint32_t sigma, int L,
+                                     int t0, uint32_t T, uint32_t* err, uint32_t* tcnt,
+                                     uint64_t* clear, uint64_t clear_units, cudaStream_t st) {
+  const uint64_t ntiles = (n + T - 1) / T, per = (clear_units + ntiles - 1) / ntiles;
+  const uint32_t tcs = tc_stride(t0);
+  uint4* const cl = (uint4*)clear;
+  if (w == 1 && L == t0 && sigma >= 2 && sigma <= 8) {
+    const uint8_t* sb = (const uint8_t*)seq;
+    const unsigned grid = (unsigned)std::min<uint64_t>((ntiles + 7) / 8, (uint64_t)num_sms() * 32);
+#define WT_COUNT_BYTES(S) \
+  case S: k_count_tiles_bytes<S><<<grid, 256, 0, st>>>(sb, n, err, tcnt, tcs, T, cl, clear_units, per); break
+    switch (sigma) {
+      WT_COUNT_BYTES(2);
+      WT_COUNT_BYTES(3);
+      WT_COUNT_BYTES(4);
+      WT_COUNT_BYTES(5);
+      WT_COUNT_BYTES(6);
+      WT_COUNT_BYTES(7);
+      WT_COUNT_BYTES(8);
+    }
+#undef WT_COUNT_BYTES
+  } else {
+    const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)num_sms() * 8, ntiles);
+    if (w == 1)
+      k_hist_digits_tiles<1><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
+                                                   clear_units, per);
+    else if (w == 2)
+      k_hist_digits_tiles<2><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
+                                                   clear_units, per);
+    else
+      k_hist_digits_tiles<4><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
+                                                   clear_units, per);
+  }
+  count_launch();
+  CK(cudaGetLastError());
+  return WT_OK;
+}
 
 // Histogram of a byte sequence over sigma = NV + 1 <= 8 values, four bytes
 // at a time in a 32-bit word: a byte equals v exactly when w ^ (v x
@@ -499,85 +608,94 @@ static std::vector<PassGeom> make_passes(int L, int tau, int first_w) {
   return ps;
 }
 
-// Class starts of every level of every pass of one wavelet matrix, by one
-// block (classes of level a+j are the values of the low j bits of the
-// reversed digit r: prefix sums over the histogram, read at digit rev(r),
-// folded mod 2^j), and
-// the zero count of every level (the class-0 size after its split).
-// One pass (levels a .. a+t-1): counts of the t-bit digits, given by digit
-// value (by_key = 0) or by reversed digit, the key of the splits (by_key = 1).
-__device__ void plan_wm_pass(const uint64_t* h, int by_key, int a, int t, uint64_t* cls,
-                             uint64_t* zeros) {
-  __shared__ uint64_t cnt[512];
-  __shared__ uint64_t st[512];
-  for (int j = 0; j <= t; j++) {
+// What a pass's plan gives, from the totals of its tiles' digit counts
+// (indexed by reversed digit, the key of the splits): for the wavelet matrix
+// the class starts of its levels a .. a+t (level a+j's classes are the values
+// of the key's low j bits) into cls, for a balanced tree of one pass the
+// symbol starts C[0 .. 2^t]; for both every level's zero count (the start of
+// class 2^(j-1) after split j: a level's zeros are the same in either order).
+enum PlanKind : int { PLAN_NONE = 0, PLAN_WM = 1, PLAN_WT = 2 };
+struct PassPlan {
+  int kind;
+  int a, t;
+  uint64_t* cls;    // WM
+  uint64_t* C;      // WT
+  uint64_t* zeros;  // nullptr: not wanted (digit levels)
+};
+
+// exclusive scan of n entries of v by one warp, written to out[0..n]; at
+// entry `mark` also to *at_mark
+__device__ __forceinline__ void warp_scan_to(const uint64_t* v, int n, uint64_t* out, int mark,
+                                             uint64_t* at_mark, int rev_t) {
+  const int lane = threadIdx.x & 31;
+  uint64_t carry = 0;
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int k = k0 + lane;
+    const uint64_t c = k < n ? v[rev_t ? rev_bits((uint32_t)k, rev_t) : (uint32_t)k] : 0ull;
+    uint64_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    if (k < n) {
+      if (out) out[k] = carry + x - c;
+      if (k == mark) *at_mark = carry + x - c;
+    }
+    carry += __shfl_sync(FULL, x, 31);
+  }
+  if (lane == 0 && out) out[n] = carry;
+}
+
+// One block: the plan from the totals in cnt[2^t - 1 + r] (shared memory).
+// The levels' counts are folded from the deepest up, then each level is
+// scanned by a warp of its own (one thread scanning 2^j entries for every
+// level in turn took 40-55 us, more than any other kernel of a small build).
+__device__ void plan_pass(uint64_t* cnt, const PassPlan& p) {
+  const int t = p.t, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int j = t - 1; j >= 0; j--) {
+    __syncthreads();
     const int nk = 1 << j;
-    for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-      uint64_t s = 0;
-      for (int r = k; r < (1 << t); r += nk) s += h[by_key ? r : rev_bits((uint32_t)r, t)];
-      cnt[k] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint64_t acc = 0;
-      for (int k = 0; k < nk; k++) {
-        st[k] = acc;
-        acc += cnt[k];
-      }
-      st[nk] = acc;
-    }
-    __syncthreads();
-    uint64_t* c = cls + (nk - 1 + j);
-    for (int k = threadIdx.x; k <= nk; k += blockDim.x) c[k] = st[k];
-    if (j >= 1 && threadIdx.x == 0) zeros[a + j - 1] = st[nk >> 1];
-    __syncthreads();
+    for (int k = threadIdx.x; k < nk; k += blockDim.x)
+      cnt[nk - 1 + k] = cnt[2 * nk - 1 + k] + cnt[2 * nk - 1 + k + nk];
   }
+  __syncthreads();
+  for (int j = warp; j <= t; j += nwarps) {
+    const int nk = 1 << j;
+    warp_scan_to(cnt + nk - 1, nk, p.kind == PLAN_WM ? p.cls + (nk - 1 + j) : nullptr,
+                 j && p.zeros ? nk >> 1 : -1, p.zeros + (j ? p.a + j - 1 : 0), 0);
+  }
+  if (p.kind == PLAN_WT && warp == nwarps - 1)
+    warp_scan_to(cnt + (1 << t) - 1, 1 << t, p.C, -1, nullptr, t);
 }
 
-__device__ void plan_wm_classes(const uint64_t* hist, int L, int tau, int G, uint64_t* cls,
-                                uint64_t* zeros) {
-  int hoff = 0, coff = 0;
-  for (int g = 0; g < G; g++) {
-    const int a = g * tau, t = min(tau, L - a);
-    plan_wm_pass(hist + hoff, 0, a, t, cls + coff, zeros);
-    hoff += 1 << t;
-    coff += (2 << t) + t + 1;
-  }
-}
-
-// the plan of one later pass from the totals of its tiles' digit counts
-// (indexed by reversed digit: the last row of the scanned chunk table)
-__global__ void k_plan_wm_pass(const uint64_t* totals, int a, int t, uint64_t* cls,
-                               uint64_t* zeros) {
-  plan_wm_pass(totals, 1, a, t, cls, zeros);
+// the plan of one pass from the totals of its tiles' digit counts (the last
+// row of the scanned chunk table)
+__global__ void __launch_bounds__(288) k_plan_pass(const uint64_t* totals, const PassPlan p) {
+  __shared__ uint64_t cnt[2 * TC_STRIDE];
+  for (int r = threadIdx.x; r < (1 << p.t); r += blockDim.x) cnt[(1 << p.t) - 1 + r] = totals[r];
+  plan_pass(cnt, p);
 }
 
 // Batched builds, one block per sequence of the launch: the plan of its pass
 // from the totals of its own tiles' digit counts, i.e. the difference of the
-// scanned tables' prefixes at its last and first tile (tcnt exclusive
-// within chunks of TCHUNK tiles, tchunk the chunks' exclusive prefixes with
-// the total after the last chunk).
-__global__ void k_plan_batch_pass(const SegDesc* segs, const uint32_t* tcnt,
-                                  const uint64_t* tchunk, uint32_t tcs, uint32_t ntiles) {
-  __shared__ uint64_t tot[TC_STRIDE];
+// scanned tables' prefixes at its last and first tile (tcnt exclusive within
+// chunks of 2^chsh tiles, tchunk the chunks' exclusive prefixes with the
+// total after the last chunk).
+__global__ void __launch_bounds__(288) k_plan_batch_pass(const SegDesc* segs, const uint32_t* tcnt,
+                                                         const uint64_t* tchunk, uint32_t tcs,
+                                                         uint32_t ntiles, uint32_t chsh) {
+  __shared__ uint64_t cnt[2 * TC_STRIDE];
   const SegDesc& d = segs[blockIdx.x];
   const uint32_t t0 = d.tile0, t1 = t0 + (uint32_t)((d.n + PASS_T - 1) / PASS_T);
-  const uint64_t last = (uint64_t)((ntiles + TCHUNK - 1) / TCHUNK) * tcs;
+  const uint64_t last = (uint64_t)((ntiles + (1u << chsh) - 1) >> chsh) * tcs;
   auto prefix = [&](uint32_t ti, uint32_t r) -> uint64_t {
     if (ti >= ntiles) return tchunk[last + r];
-    return tchunk[(uint64_t)(ti / TCHUNK) * tcs + r] + tcnt[(uint64_t)ti * tcs + r];
+    return tchunk[(uint64_t)(ti >> chsh) * tcs + r] + tcnt[(uint64_t)ti * tcs + r];
   };
-  for (uint32_t r = threadIdx.x; r < (1u << d.t); r += blockDim.x) tot[r] = prefix(t1, r) - prefix(t0, r);
-  __syncthreads();
-  plan_wm_pass(tot, 1, d.a, d.t, d.wm_cls, d.zeros);
-}
-
-// Wavelet-matrix plan, one block: class starts and zero counts; reset of the
-// tile tickets.
-__global__ void k_plan_wm(const uint64_t* hist, int L, int tau, int G, uint64_t* cls,
-                          uint64_t* zeros, uint32_t* tickets) {
-  plan_wm_classes(hist, L, tau, G, cls, zeros);
-  for (int g = threadIdx.x; g < 32; g += blockDim.x) tickets[g] = 0;
+  for (uint32_t r = threadIdx.x; r < (1u << d.t); r += blockDim.x)
+    cnt[(1u << d.t) - 1 + r] = prefix(t1, r) - prefix(t0, r);
+  plan_pass(cnt, PassPlan{PLAN_WM, d.a, d.t, d.wm_cls, nullptr, d.zeros});
 }
 
 // Balanced-tree helpers over C (C[v] = number of symbols < v, v in [0, 2^L]).
@@ -592,37 +710,6 @@ __global__ void k_wt_zeros(const uint64_t* C, int L, uint64_t* zeros) {
   uint64_t tot;
   block_scan_excl_u64(s, &tot);
   if (threadIdx.x == 0) zeros[l] = tot;
-}
-
-// Zero the words that hold the start of a node (not word aligned) on every
-// output level; and the padding words.  digits: only even binary levels are
-// output (digit level l/2), 2 bits per element.
-__global__ void k_wt_zero_words(const uint64_t* C, int L, uint64_t n, uint64_t* bits,
-                                const uint64_t* lvl_off, int digits) {
-  const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t total = ((uint64_t)1 << L);  // sum over levels l < L of 2^l = 2^L - 1
-  if (gid >= total - 1) return;
-  // level l holds gids [2^l - 1, 2^{l+1} - 1)
-  const int l = 63 - __clzll(gid + 1);
-  const uint64_t q = gid + 1 - ((uint64_t)1 << l);
-  if (q == 0) return;
-  if (digits && (l & 1)) return;
-  const uint64_t s = C[q << (L - l)];
-  const uint64_t bp = digits ? 2 * s : s;
-  if ((bp & 63) && s < n) bits[lvl_off[digits ? l / 2 : l] + (bp >> 6)] = 0;
-}
-
-__global__ void k_zero_padding(uint64_t* bits, const uint64_t* lvl_off, const uint64_t* lvl_len,
-                               int nlev, int bpe) {
-  const int l = blockIdx.x;
-  if (l >= nlev) return;
-  const uint64_t used = (lvl_len[l] * bpe + 63) >> 6;
-  const uint64_t W = lvl_off[l + 1] - lvl_off[l];
-  for (uint64_t w = used + threadIdx.x; w < W; w += blockDim.x) bits[lvl_off[l] + w] = 0;
-}
-
-__global__ void k_reset_tickets(uint32_t* tickets) {
-  for (int g = threadIdx.x; g < 32; g += blockDim.x) tickets[g] = 0;
 }
 
 // Node-aligned tiles over T_a: node p spans [bnd[p*stride], bnd[(p+1)*stride]).
@@ -740,13 +827,17 @@ __global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ Pas
 }
 
 // Prefix sums of the tiles' counts, per digit value: exclusive inside each
-// chunk of TCHUNK tiles (in place, u32), and the chunks' totals.
+// chunk of 2^chsh tiles (in place, u32), and the chunks' totals.  When there
+// is one chunk only (ONE), the whole scan and the pass's plan are this
+// launch: its totals are the grand totals (row 1), and row 0 is zero.
+template <bool ONE>
 __global__ void __launch_bounds__(256) k_tile_scan_chunk(uint32_t* tcnt, const uint32_t* ntiles_dev,
-                                                         uint32_t ntiles_host, uint64_t* tchunk) {
+                                                         uint32_t ntiles_host, uint32_t chsh,
+                                                         uint64_t* tchunk, const PassPlan plan) {
   const uint32_t nt = ntiles_dev ? *ntiles_dev : ntiles_host;
   const uint32_t c = blockIdx.x, r = threadIdx.x, S = blockDim.x;  // one thread per digit
-  const uint64_t t0 = (uint64_t)c * TCHUNK;
-  const uint64_t t1 = t0 + TCHUNK < nt ? t0 + TCHUNK : nt;
+  const uint64_t t0 = (uint64_t)c << chsh;
+  const uint64_t t1 = t0 + (1u << chsh) < nt ? t0 + (1u << chsh) : nt;
   uint32_t run = 0;
   // sixteen loads in flight before their stores (in place: the stores
   // would otherwise wait for each load in turn)
@@ -761,42 +852,62 @@ __global__ void __launch_bounds__(256) k_tile_scan_chunk(uint32_t* tcnt, const u
       run += v[k];
     }
   }
-  tchunk[(uint64_t)c * S + r] = run;
+  if constexpr (ONE) {
+    __shared__ uint64_t cnt[2 * TC_STRIDE];
+    tchunk[r] = 0;
+    tchunk[S + r] = run;
+    if (plan.kind != PLAN_NONE) {
+      if (r < (1u << plan.t)) cnt[(1u << plan.t) - 1 + r] = run;
+      plan_pass(cnt, plan);
+    }
+  } else {
+    tchunk[(uint64_t)c * S + r] = run;
+  }
 }
 
 // ... and the exclusive prefix of the chunks' totals (u64), with the grand
-// total after the last chunk: one warp per digit value, 32 chunks per step
-__global__ void __launch_bounds__(32) k_tile_scan_top(uint64_t* tchunk, uint32_t nchunk) {
-  const uint32_t r = blockIdx.x, lane = threadIdx.x, S = gridDim.x;  // one warp per digit
-  uint64_t carry = 0;
-  for (uint32_t c0 = 0; c0 < nchunk; c0 += 32) {
-    const uint32_t c = c0 + lane;
-    const uint64_t v = c < nchunk ? tchunk[(uint64_t)c * S + r] : 0ull;
-    uint64_t x = v;
+// total after the last chunk: one block per 32 digit values, a lane per digit
+// value (256-byte rows), warp w scanning the w-th of 32 runs of chunks after
+// their sums are known.  (One warp per digit value, 8 bytes of each row at a
+// time, took 26 us for 1024 chunks and 95 us for 4096.)
+__global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32_t nchunk,
+                                                        uint32_t S) {
+  __shared__ uint64_t sums[32][33];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
+  const uint32_t per = (nchunk + 31) / 32;
+  const uint32_t c0 = min(w * per, nchunk), c1 = min(c0 + per, nchunk);
+  constexpr int B = 16;
+  uint64_t sum = 0;
+  for (uint32_t c = c0; c < c1; c += B) {
+    uint64_t v[B];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(FULL, x, o);
-      if ((int)lane >= o) x += y;
-    }
-    if (c < nchunk) tchunk[(uint64_t)c * S + r] = carry + x - v;
-    carry += __shfl_sync(FULL, x, 31);
+    for (int k = 0; k < B; k++) v[k] = c + k < c1 ? tchunk[(uint64_t)(c + k) * S + r] : 0ull;
+#pragma unroll
+    for (int k = 0; k < B; k++) sum += v[k];
   }
-  if (lane == 0) tchunk[(uint64_t)nchunk * S + r] = carry;
+  sums[w][lane] = sum;
+  __syncthreads();
+  uint64_t run = 0;
+  for (uint32_t k = 0; k < w; k++) run += sums[k][lane];
+  for (uint32_t c = c0; c < c1; c += B) {
+    uint64_t v[B];
+#pragma unroll
+    for (int k = 0; k < B; k++) v[k] = c + k < c1 ? tchunk[(uint64_t)(c + k) * S + r] : 0ull;
+#pragma unroll
+    for (int k = 0; k < B; k++) {
+      if (c + k < c1) tchunk[(uint64_t)(c + k) * S + r] = run;
+      run += v[k];
+    }
+  }
+  if (w == 31) tchunk[(uint64_t)nchunk * S + r] = run;
 }
 
-// A wavelet-matrix pass planned from its own tiles' digit counts: class
-// starts of its levels into cls, their zero counts into zeros.
-struct PassPlan {
-  uint64_t* cls;
-  uint64_t* zeros;
-};
-
 // tcnt_pre: the tiles' digit counts when already taken (else counted here);
-// plan: the pass's plan, made here from the totals of those counts
+// plan: what to plan from the totals of those counts
 template <typename E, bool DIG, bool BATCH = false, int TT = PT, int TNT = PNT>
 static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt_build_opts* o,
                                cudaStream_t st, uint32_t* tcnt_pre = nullptr,
-                               const PassPlan* plan = nullptr) {
+                               const PassPlan& plan = PassPlan{}) {
   using SM = PassSmem<E, TT, TNT, DIG>;
   auto kern = k_pass<E, TT, TNT, DIG, BATCH>;
   static bool attr = false;
@@ -813,8 +924,9 @@ static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt
   if (grid > max_tiles) grid = std::max<uint64_t>(max_tiles, 1);
   // every tile's digit counts and their prefix sums across the tiles
   const uint64_t mt = std::max<uint64_t>(max_tiles, 1);
-  const uint32_t nchunk = (uint32_t)((mt + TCHUNK - 1) / TCHUNK);
   PassParams Q = P;
+  Q.chsh = (uint32_t)chunk_shift(mt);
+  const uint32_t nchunk = (uint32_t)((mt + (1u << Q.chsh) - 1) >> Q.chsh);
   Q.tcs = P.tcs ? P.tcs : tc_stride(P.t);  // batched passes give the widest digit's
   Work wk{st, {}};
   uint32_t* tcnt = tcnt_pre;
@@ -826,18 +938,22 @@ static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt
     count_launch();
   }
   TRY(wk.get(&tchunk, ((uint64_t)nchunk + 1) * Q.tcs));
-  k_tile_scan_chunk<<<nchunk, Q.tcs, 0, st>>>(tcnt, P.tiles ? P.ntiles_dev : nullptr, P.ntiles,
-                                              tchunk);
+  const uint32_t* nt_dev = P.tiles ? P.ntiles_dev : nullptr;
+  if (nchunk == 1)
+    k_tile_scan_chunk<true><<<1, Q.tcs, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk, plan);
+  else
+    k_tile_scan_chunk<false><<<nchunk, Q.tcs, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk, plan);
   count_launch();
-  k_tile_scan_top<<<Q.tcs, 32, 0, st>>>(tchunk, nchunk);
-  count_launch();
-  if (plan) {
-    k_plan_wm_pass<<<1, 256, 0, st>>>(tchunk + (uint64_t)nchunk * Q.tcs, P.a, P.t, plan->cls,
-                                      plan->zeros);
+  if (nchunk > 1) {
+    k_tile_scan_top<<<Q.tcs / 32, 1024, 0, st>>>(tchunk, nchunk, Q.tcs);
     count_launch();
+    if (plan.kind != PLAN_NONE) {
+      k_plan_pass<<<1, 288, 0, st>>>(tchunk + (uint64_t)nchunk * Q.tcs, plan);
+      count_launch();
+    }
   }
   if (BATCH) {
-    k_plan_batch_pass<<<P.nsegs, 256, 0, st>>>(P.segs, tcnt, tchunk, Q.tcs, (uint32_t)mt);
+    k_plan_batch_pass<<<P.nsegs, 288, 0, st>>>(P.segs, tcnt, tchunk, Q.tcs, (uint32_t)mt, Q.chsh);
     count_launch();
   }
   Q.tcnt = tcnt;
@@ -866,7 +982,7 @@ static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt
 // wavelet matrix, the 8192-symbol tile with 512 worker threads)
 static wt_status launch_pass(const PassParams& P, bool wide, bool dig, uint64_t max_tiles,
                              const wt_build_opts* o, cudaStream_t st,
-                             uint32_t* tcnt_pre = nullptr, const PassPlan* plan = nullptr,
+                             uint32_t* tcnt_pre = nullptr, const PassPlan& plan = PassPlan{},
                              uint32_t tile = PT) {
   if (dig) return wide ? launch_pass_t<uint32_t, true>(P, max_tiles, o, st, tcnt_pre, plan)
                        : launch_pass_t<uint16_t, true>(P, max_tiles, o, st, tcnt_pre, plan);
@@ -1059,48 +1175,24 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   std::vector<PassGeom> ps = make_passes(L, tau, w);
   const int G = (int)ps.size();
   const uint32_t T = o->tile_symbols;
-  uint64_t *hist, *cls, *d_off, *d_len;
+  uint64_t *cls, *d_off, *d_len;
   uint32_t* tickets;
-  int nh = 0, ncls = 0;
-  for (auto& p : ps) {
-    nh += 1 << p.t;
-    ncls += (2 << p.t) + p.t + 1;
-  }
-  TRY(wk.get(&hist, nh));
+  int ncls = 0;
+  for (auto& p : ps) ncls += (2 << p.t) + p.t + 1;
   TRY(wk.get(&cls, ncls));
   TRY(wk.get(&tickets, 32));
   TRY(wk.get(&d_off, L + 1));
   TRY(wk.get(&d_len, L));
   TRY(upload(d_off, h->level_off.data(), (L + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), L * 8, st));
-  CK(cudaMemsetAsync(hist, 0, nh * 8, st));
-  // the first pass's digit histogram and per-tile counts (with validation)
+  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
+  // the first pass's per-tile digit counts (with validation)
   uint32_t* tcnt0;
   const uint64_t ntiles0 = (n + T - 1) / T;
   TRY(wk.get(&tcnt0, (size_t)ntiles0 * tc_stride(ps[0].t)));
-  {
-    const uint32_t blocks = (uint32_t)std::min<uint64_t>((uint64_t)num_sms() * 8, ntiles0);
-    const int t0 = ps[0].t;
-    // the first pass's levels: W * t0 words, a share per tile
-    uint4* const cl0 = (uint4*)h->d_bits;
-    const uint64_t cu0 = W * (uint64_t)t0 / 2, cp0 = (cu0 + ntiles0 - 1) / ntiles0;
-    if (w == 1)
-      k_hist_digits_tiles<1><<<blocks, 256, 0, st>>>(d_seq, n, sigma, L, t0, hist, h->d_err, tcnt0,
-                                                     tc_stride(t0), T, cl0, cu0, cp0);
-    else if (w == 2)
-      k_hist_digits_tiles<2><<<blocks, 256, 0, st>>>(d_seq, n, sigma, L, t0, hist, h->d_err, tcnt0,
-                                                     tc_stride(t0), T, cl0, cu0, cp0);
-    else
-      k_hist_digits_tiles<4><<<blocks, 256, 0, st>>>(d_seq, n, sigma, L, t0, hist, h->d_err, tcnt0,
-                                                     tc_stride(t0), T, cl0, cu0, cp0);
-    count_launch();
-    CK(cudaGetLastError());
-  }
-  // pass 0 planned from the histogram; the later passes from their own
-  // tiles' digit counts, just before they run
-  k_plan_wm<<<1, 1024, 0, st>>>(hist, L, tau, 1, cls, h->d_zeros, tickets);
-  count_launch();
-  CK(cudaGetLastError());
+  // ... zeroing the first pass's levels on the way
+  TRY(launch_first_counts(d_seq, w, n, sigma, L, ps[0].t, T, h->d_err, tcnt0, h->d_bits,
+                          W * (uint64_t)ps[0].t / 2, st));
   // intermediate sequences
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
@@ -1133,9 +1225,9 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
       P.clear_units = W * (uint64_t)ps[g + 1].t / 2;
       P.clear_per = (P.clear_units + ntiles - 1) / ntiles;
     }
-    const PassPlan plan{cls + coff, h->d_zeros};
-    TRY(launch_pass(P, pg.wide, false, ntiles, o, st, g == 0 ? tcnt0 : nullptr,
-                    g == 0 ? nullptr : &plan, T));
+    // every pass is planned from its own tiles' digit counts
+    const PassPlan plan{PLAN_WM, pg.a, pg.t, cls + coff, nullptr, h->d_zeros};
+    TRY(launch_pass(P, pg.wide, false, ntiles, o, st, g == 0 ? tcnt0 : nullptr, plan, T));
     coff += (2 << pg.t) + pg.t + 1;
     in = P.out;
   }
@@ -1156,42 +1248,52 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   h->levels = multiary ? (uint32_t)((L + 1) / 2) : (uint32_t)L;
   h->bpe = multiary ? 2 : 1;
   set_uniform_levels(h, n);
-  TRY(alloc_outputs(h, h->level_off.back()));
-  Work wk{st, {}};
-  if (n == 0) return build_directories(h);
   const int tau = pick_tau(o, L, multiary);
   std::vector<PassGeom> ps = make_passes(L, tau, w);
   const int G = (int)ps.size();
+  // a tree of one pass needs no symbol histogram: its nodes' starts follow
+  // from the tiles' digit counts, whose kernel also zeroes the level buffer
+  const bool one = G == 1;
+  TRY(alloc_outputs(h, h->level_off.back(), !one || n == 0));
+  Work wk{st, {}};
+  if (n == 0) return build_directories(h);
   const uint32_t T = PT;
   const uint64_t V = (uint64_t)1 << L;
-  uint64_t *hist, *C, *scr, *d_off, *d_len, *tcnt, *toff;
-  uint32_t *tickets, *d_ntiles;
-  TileDesc* tiles;
-  uint64_t max_nodes = (uint64_t)1 << ps.back().a;
-  const uint64_t max_tiles = (n + T - 1) / T + max_nodes + 1;
-  TRY(wk.get(&hist, V));
+  const uint64_t ntiles0 = (n + T - 1) / T;
+  uint64_t *C, *d_off, *d_len;
+  uint32_t* tickets;
+  uint32_t* tcnt0 = nullptr;
   TRY(wk.get(&C, V + 1));
-  TRY(wk.get(&scr, scan_scratch(std::max(V, max_nodes))));
   TRY(wk.get(&tickets, 32));
   TRY(wk.get(&d_off, h->levels + 1));
   TRY(wk.get(&d_len, h->levels));
-  TRY(wk.get(&tcnt, max_nodes));
-  TRY(wk.get(&toff, max_nodes + 1));
-  TRY(wk.get(&tiles, max_tiles));
-  TRY(wk.get(&d_ntiles, 1));
   TRY(upload(d_off, h->level_off.data(), (h->levels + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), h->levels * 8, st));
-  CK(cudaMemsetAsync(hist, 0, V * 8, st));
-  TRY(launch_hist_full(d_seq, w, n, sigma, hist, h->d_err, st));
-  TRY(scan_excl_u64(hist, C, V, scr, st));
-  if (!multiary) {
-    k_wt_zeros<<<L, 1024, 0, st>>>(C, L, h->d_zeros);
-    count_launch();
-    CK(cudaGetLastError());
+  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
+  uint64_t *hist, *scr = nullptr, *tcnt = nullptr, *toff = nullptr;
+  uint32_t* d_ntiles = nullptr;
+  TileDesc* tiles = nullptr;
+  if (one) {
+    TRY(wk.get(&tcnt0, (size_t)ntiles0 * tc_stride(L)));
+    TRY(launch_first_counts(d_seq, w, n, sigma, L, L, T, h->d_err, tcnt0, h->d_bits,
+                            h->level_off.back() / 2, st));
+  } else {
+    const uint64_t max_nodes = (uint64_t)1 << ps.back().a;
+    TRY(wk.get(&hist, V));
+    TRY(wk.get(&scr, scan_scratch(std::max(V, max_nodes))));
+    TRY(wk.get(&tcnt, max_nodes));
+    TRY(wk.get(&toff, max_nodes + 1));
+    TRY(wk.get(&tiles, ntiles0 + max_nodes + 1));
+    TRY(wk.get(&d_ntiles, 1));
+    CK(cudaMemsetAsync(hist, 0, V * 8, st));
+    TRY(launch_hist_full(d_seq, w, n, sigma, hist, h->d_err, st));
+    TRY(scan_excl_u64(hist, C, V, scr, st));
+    if (!multiary) {
+      k_wt_zeros<<<L, 1024, 0, st>>>(C, L, h->d_zeros);
+      count_launch();
+      CK(cudaGetLastError());
+    }
   }
-  k_reset_tickets<<<1, 32, 0, st>>>(tickets);
-  count_launch();
-  CK(cudaGetLastError());
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
     if (!seqbuf[g & 1]) {
@@ -1203,19 +1305,24 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   const void* in = d_seq;
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
-    const uint64_t nn = (uint64_t)1 << pg.a;
-    const uint64_t stride = (uint64_t)1 << (L - pg.a);
-    k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(C, stride, nn, T, tcnt);
-    count_launch();
-    TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
-    {
-      const uint64_t mt = (n + T - 1) / T + nn;
+    PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
+    uint64_t mt = ntiles0;
+    if (g > 0) {
+      // tiles inside the nodes of the pass's first level (the first pass has
+      // one node, the whole sequence)
+      const uint64_t nn = (uint64_t)1 << pg.a;
+      const uint64_t stride = (uint64_t)1 << (L - pg.a);
+      k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(C, stride, nn, T, tcnt);
+      count_launch();
+      TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
+      mt = ntiles0 + nn;
       k_tiles_write<<<(unsigned)((mt + 255) / 256), 256, 0, st>>>(C, stride, nn, T, 0, toff, tiles,
                                                                  d_ntiles, mt);
       count_launch();
+      CK(cudaGetLastError());
+      P.tiles = tiles;
+      P.ntiles_dev = d_ntiles;
     }
-    CK(cudaGetLastError());
-    PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
     P.in = in;
     P.in_w = pg.in_w;
     P.out = (g + 1 < G) ? seqbuf[g & 1] : nullptr;
@@ -1227,11 +1334,11 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     P.shape = SHAPE_WT;
     P.digits = multiary ? 1 : 0;
     P.wt_C = C;
-    P.tiles = tiles;
-    P.ntiles_dev = d_ntiles;
+    P.ntiles = (uint32_t)ntiles0;
     P.n_in = n;
-    const uint64_t mt = (n + T - 1) / T + nn;
-    TRY(launch_pass(P, pg.wide, multiary, mt, o, st));
+    const PassPlan plan{one ? PLAN_WT : PLAN_NONE, 0, pg.t, nullptr, C,
+                        multiary ? nullptr : h->d_zeros};
+    TRY(launch_pass(P, pg.wide, multiary, mt, o, st, tcnt0, plan));
     in = P.out;
   }
   if (o && (o->flags & WT_FLAG_NO_DIRECTORY)) return WT_OK;
@@ -1241,11 +1348,6 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
 // ---------------------------------------------------------------------------
 // Huffman-shaped wavelet tree
 // ---------------------------------------------------------------------------
-__global__ void k_clear_words(uint64_t* bits, const uint64_t* idx, uint64_t m) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) bits[idx[i]] = 0;
-}
-
 uint32_t huffman_lengths(const uint64_t* hist, uint32_t sigma, uint32_t cap, uint8_t* len);
 void canonical_codes(const uint8_t* len, uint32_t sigma, uint32_t* code);
 
@@ -1535,9 +1637,7 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
   TRY(wk.get(&d_ntiles, 1));
   TRY(upload(d_off, h->level_off.data(), (Lm + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), Lm * 8, st));
-  k_reset_tickets<<<1, 32, 0, st>>>(tickets);
-  count_launch();
-  CK(cudaGetLastError());
+  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
     if (!seqbuf[g & 1]) {
@@ -1550,20 +1650,29 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
     const uint64_t nn = node_lvl[3 * pg.a + 2];
-    if (nn) {
-      const uint64_t* bnd = h->d_node + node_lvl[3 * pg.a];
-      k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(bnd, 1, nn, T, tcnt);
-      count_launch();
-      TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
-      const uint64_t mtw = (h->level_len[pg.a] + T - 1) / T + nn;
-      k_tiles_write<<<(unsigned)((mtw + 255) / 256), 256, 0, st>>>(
-          bnd, 1, nn, T, node_lvl[3 * pg.a + 1], toff, tiles, d_ntiles, mtw);
-      count_launch();
-    } else {
-      CK(cudaMemsetAsync(d_ntiles, 0, 4, st));
-    }
-    CK(cudaGetLastError());
     PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
+    P.n_in = h->level_len[pg.a];
+    P.ntiles = (uint32_t)((P.n_in + T - 1) / T);
+    uint64_t mt = P.ntiles;
+    if (g > 0) {
+      // tiles inside the nodes of the pass's first level (the first pass has
+      // one node, the whole sequence)
+      if (nn) {
+        const uint64_t* bnd = h->d_node + node_lvl[3 * pg.a];
+        mt += nn;
+        k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(bnd, 1, nn, T, tcnt);
+        count_launch();
+        TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
+        k_tiles_write<<<(unsigned)((mt + 255) / 256), 256, 0, st>>>(
+            bnd, 1, nn, T, node_lvl[3 * pg.a + 1], toff, tiles, d_ntiles, mt);
+        count_launch();
+      } else {
+        CK(cudaMemsetAsync(d_ntiles, 0, 4, st));
+      }
+      CK(cudaGetLastError());
+      P.tiles = tiles;
+      P.ntiles_dev = d_ntiles;
+    }
     P.in = in;
     P.in_w = g == 0 ? w : pg.in_w;
     P.code_map = g == 0 ? d_left : nullptr;
@@ -1576,10 +1685,6 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
     P.shape = SHAPE_HUFF;
     P.hf_node = h->d_node;
     P.hf_lvl = h->d_node_lvl;
-    P.tiles = tiles;
-    P.ntiles_dev = d_ntiles;
-    P.n_in = h->level_len[pg.a];
-    const uint64_t mt = (P.n_in + T - 1) / T + nn;
     TRY(launch_pass(P, pg.wide, false, mt, o, st));
     in = P.out;
   }

@@ -388,19 +388,19 @@ __global__ void __launch_bounds__(NT + 32, PassCtas<E, T, BATCH>::value) k_pass(
       // this tile's count of every digit value in the earlier tiles of its
       // sequence or node: the prefix sums of the per-tile counts (Section
       // 4.2, prefix sums across the K sub-problems), taken before the pass
-      // (the tables are exclusive inside chunks of TCHUNK tiles, with the
+      // (the tables are exclusive inside chunks of tiles, with the
       // chunks' exclusive prefixes and their total after the last chunk: the
       // tile's own digit counts are the difference to the next tile, or to
       // the next chunk for the last tile of a chunk)
       uint64_t* const exd = ex_cnt + cls_idx(t, 0);  // exclusive digit counts
       {
-        const uint32_t ch = ti / TCHUNK;
+        const uint32_t ch = ti >> P0.chsh;
         const uint32_t S = P0.tcs;
         const uint64_t* ca = P0.tchunk + (uint64_t)ch * S;
-        const uint64_t* cb = P0.tchunk + (uint64_t)(seg0 / TCHUNK) * S;
+        const uint64_t* cb = P0.tchunk + (uint64_t)(seg0 >> P0.chsh) * S;
         const uint32_t* ta = P0.tcnt + (uint64_t)ti * S;
         const uint32_t* tb = P0.tcnt + (uint64_t)seg0 * S;
-        const bool last = (ti + 1) % TCHUNK == 0 || ti + 1 >= ntiles;
+        const bool last = ((ti + 1) >> P0.chsh) != ch || ti + 1 >= ntiles;
         uint32_t sum = 0;
         for (int r = lane; r < nd; r += 32) {
           const uint32_t a = ta[r];

@@ -29,14 +29,21 @@ struct TileDesc {
 };
 
 // Per-tile digit counts of a pass (the K sub-problems' per-node counts of
-// Section 4.2) and their prefix sums across tiles: tile ti's counts sit at
-// tcnt[ti * tcs + r] (u32, exclusive within its chunk of TCHUNK tiles
-// after the scan) and the chunk's exclusive counts at tchunk[c * tcs + r]
-// (u64).
+// Section 4.2) and their prefix sums across tiles, in chunks of 2^chsh tiles:
+// tile ti's counts sit at tcnt[ti * tcs + r] (u32, exclusive within its chunk
+// after the scan) and chunk c's exclusive counts at tchunk[c * tcs + r]
+// (u64), the totals after the last chunk.
 constexpr int TC_STRIDE = 256;  // the largest stride (t = 8)
 // the stride of a pass's tables: its digit values, at least one warp's worth
 __host__ __device__ inline uint32_t tc_stride(int t) { return t >= 5 ? (1u << t) : 32u; }
-constexpr uint32_t TCHUNK = 256;
+// Tiles per chunk: 64, so that a short table is scanned in four rounds of 16
+// loads, and more from 2^17 tiles on, so that the scan over the chunks stays
+// below 2048 of them (its blocks walk them one after another).
+inline int chunk_shift(uint64_t tiles) {
+  int s = 6;
+  while ((tiles >> s) > 2048) s++;
+  return s;
+}
 
 // Symbols per tile of the partition pass.
 #ifndef WT_PASS_T
@@ -103,6 +110,7 @@ struct PassParams {
   const uint32_t* tcnt;
   const uint64_t* tchunk;
   uint32_t tcs;          // their stride (tc_stride of the largest digit width)
+  uint32_t chsh;         // log2 of the tiles per chunk
   uint32_t* ticket;      // tiles are taken in order from this counter
   uint32_t* err;
   // 16-byte units of a later pass's levels to zero, `clear_per` of them per
