@@ -18,9 +18,8 @@
  *    (wt_sync, wt_export, wt_export_select, wt_dd_merge for its parts,
  *    wt_free, wm_autotune, wm_autotune_config) synchronise the handle's stream themselves.  Device-side errors found during
  *    a build (a symbol >= sigma: WT_ERR_SYMBOL_GE_SIGMA; an internal table
- *    that disagrees with the data, which leaves the affected bits unwritten,
- *    or a tile's bulk copy into shared memory that did not complete within
- *    about a second, after which the waiting block stops: WT_ERR_CUDA) are
+ *    that disagrees with the data, which leaves the affected bits unwritten:
+ *    WT_ERR_CUDA) are
  *    reported by wt_sync() or by the next call on the handle.
  *  * Symbol sequences are contiguous arrays of width_bytes = 1, 2 or 4
  *    (little-endian unsigned), read-only, borrowed for the duration of the
@@ -64,7 +63,8 @@ typedef struct wt_struct* wt_handle;
 typedef void* wt_stream;
 
 /* Build options; a zero field means "choose automatically".
- *  tau           levels per partition pass (1..8); the paper's tau (Sections 3, 4.1).
+ *  tau           levels per partition pass (1..8; more than 4 run as passes of 4);
+ *                the paper's tau (Sections 3, 4.1).
  *  tile_symbols  symbols per tile; the paper's sub-sequence size n/K (Section 4.2).
  *                wm_build: 2048, 4096 or 8192; the trees, 4-ary trees and batched
  *                builds: 4096 only.  Other values return WT_ERR_UNSUPPORTED.
@@ -74,7 +74,7 @@ typedef void* wt_stream;
  *                supported.
  *  wm_build fills tau, tile_symbols and ctas_per_sm left at 0 from the
  *  autotuner's record for the sequence's (L, ceil(log2 n)), if any (see
- *  wm_autotune_config), else tau 8, 4096 symbols and the occupancy limit.
+ *  wm_autotune_config), else tau 4, 4096 symbols and the occupancy limit.
  *  select_sample sampling period of the select directory; only 4096 is supported.
  *  flags         WT_FLAG_* below. */
 typedef struct {
@@ -225,7 +225,7 @@ typedef struct {
  * outs[i] receives the handle of items[i], exactly the structure wm_build
  * returns for it; the m handles share one device allocation, released when
  * the last of them is freed.  opts->tau == 0 takes each sequence's levels
- * per pass from the autotuner's table (8 when not tuned).  Each sequence has
+ * per pass from the autotuner's table (4 when not tuned).  Each sequence has
  * its own error word: a symbol >= sigma (WT_ERR_SYMBOL_GE_SIGMA), or a failed
  * internal consistency check of its tiles (WT_ERR_CUDA; never for consistent
  * tables), is reported on that sequence's handle only.  A failed call
@@ -254,7 +254,7 @@ wt_status wt_batch_free(wt_batch b);
 /* Autotuner for the levels per pass tau (Section 4.2: fewer, wider passes
  * against more work per pass).  Times wavelet-matrix builds of d_seq
  * (without directories; one untimed and the best of two timed builds) for
- * tau = 1 .. min(8, L), writes the fastest to *best_tau and the times to
+ * tau = 1 .. min(8, L), writes the fastest (at most 4) to *best_tau and the times to
  * ms_out[tau-1] (ms_out may be NULL; 0 where not tried), and records it (with
  * the default tile and occupancy) for every later wm_build / wm_batch_build
  * with opts->tau == 0 of a sequence with the same L and ceil(log2 n).
@@ -275,7 +275,7 @@ typedef struct {
  * sub-problems K against the per-sub-problem work, and tau against the
  * number of passes).  Times wavelet-matrix builds of d_seq (without
  * directories; one untimed and the best of two timed builds per
- * configuration): first tau = 1 .. min(8, L) at 4096-symbol tiles and full
+ * configuration): first tau = 1 .. min(4, L) at 4096-symbol tiles and full
  * occupancy, then, for the two fastest tau, tiles of 2048 / 4096 / 8192
  * symbols at full occupancy and at 4 and 3 CTAs per SM.  Writes the fastest
  * to *out and records it for every later wm_build with zero options (and the

@@ -107,8 +107,7 @@ wt_status sync_handle(wt_struct* h) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->deferred = WT_ERR_CUDA;
   if (err & ERR_SYMBOL) return h->deferred = WT_ERR_SYMBOL_GE_SIGMA;
-  // ERR_INTERNAL (a table disagreed with a tile) or ERR_STALL (a tile load
-  // that did not complete in time)
+  // ERR_INTERNAL: a table disagreed with a tile
   if (err) return h->deferred = WT_ERR_CUDA;
   if (!h->zeros_valid) {
     h->zeros.assign(h->levels, 0);
@@ -254,7 +253,7 @@ wt_status seq_build(int kind, const void* d_seq, uint64_t n, uint32_t sigma, uin
     case WT_KIND_WM: s = build_wm(d_seq, n, sigma, (int)width, opts, h); break;
     case WT_KIND_WT: s = build_wt(d_seq, n, sigma, (int)width, opts, h, false); break;
     case WT_KIND_MULTI: s = build_wt(d_seq, n, sigma, (int)width, opts, h, true); break;
-    default: s = build_huff(d_seq, n, sigma, (int)width, h_len, opts, h); break;
+    default: s = WT_ERR_INVALID_ARG; break;
   }
   return finish(h, s, out);
 }

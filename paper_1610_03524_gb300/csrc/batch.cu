@@ -24,8 +24,7 @@
 
 namespace wtk {
 
-wt_status launch_pass_batch(const PassParams& P, bool wide, const wt_build_opts* o,
-                            cudaStream_t st);
+wt_status launch_pass_batch(const PassParams& P, const wt_build_opts* o, cudaStream_t st);
 wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32_t nlev,
                            const std::vector<uint64_t>& sb_first, uint64_t* dir, uint64_t* samp,
                            uint64_t* zeros, int write_zeros, cudaStream_t st,
@@ -95,7 +94,6 @@ namespace {
 
 struct Pass1 {
   int a, t, rbits, in_w, out_w;
-  bool wide;
 };
 
 struct SeqPlan {
@@ -107,7 +105,7 @@ struct SeqPlan {
   // arena offsets (u64 units inside each region)
   uint64_t bits_base, dir_base, samp_base, zeros_base, meta_base;
   // workspace offsets
-  uint64_t cls_off, lvl_base, seq_off;  // seq_off: bytes in each ping-pong buffer
+  uint64_t cls_off, seq_off;  // seq_off: bytes in each ping-pong buffer
   uint64_t seq_bytes;
 };
 
@@ -123,7 +121,6 @@ void plan_seq(SeqPlan& p, const wt_build_opts* o) {
     q.rbits = p.L - a;
     q.in_w = a == 0 ? p.w : width_for_bits_b(p.L - a);
     q.out_w = (a + q.t < p.L) ? width_for_bits_b(p.L - a - q.t) : 0;
-    q.wide = q.rbits > 16;
     p.ps.push_back(q);
   }
   p.G = (int)p.ps.size();
@@ -157,7 +154,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
                          cudaStream_t st, wt_struct** hs) {
   std::vector<SeqPlan> sp(m);
   uint64_t nbits = 0, ndir = 0, nsamp = 0, nzeros = 0, nmeta = 0;
-  uint64_t ncls = 0, nlvl = 0, nseq = 0;
+  uint64_t ncls = 0, nseq = 0;
   uint64_t nlev_tot = 0;
   int Gmax = 0;
   for (uint32_t i = 0; i < m; i++) {
@@ -178,8 +175,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     nmeta += p.L;
     p.cls_off = ncls;
     for (const Pass1& q : p.ps) ncls += (2u << q.t) + q.t + 1;
-    p.lvl_base = nlvl;
-    nlvl += 2 * (uint64_t)p.L + 1;  // L+1 word offsets, then L lengths
     p.seq_off = nseq;
     nseq += p.G > 1 ? p.seq_bytes : 0;
     nlev_tot += p.L;
@@ -246,28 +241,23 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     for (uint32_t i = 0; i < m; i++)
       if (sp[i].n && g < sp[i].G) nsegs_tot++;
   const uint64_t w_cls = 0;
-  const uint64_t w_lvl = up(w_cls + 8 * ncls, 256);
-  const uint64_t w_gmeta = up(w_lvl + 8 * nlvl, 256);
+  const uint64_t w_gmeta = up(w_cls + 8 * ncls, 256);
   const uint64_t w_sseg = up(w_gmeta + sizeof(LevelMeta) * nlev_tot, 256);
   const uint64_t w_tab_end = up(w_sseg + sizeof(SegDesc) * std::max<uint64_t>(nsegs_tot, 1), 256);
-  const uint64_t w_tick = w_tab_end;
-  const uint64_t w_seq0 = up(w_tick + 4 * 64, 256);
+  const uint64_t w_seq0 = w_tab_end;
   const uint64_t w_seq1 = up(w_seq0 + nseq, 256);
   const uint64_t ws_bytes = up(w_seq1 + nseq, 256);
   void* wsv = nullptr;
   CK(dmalloc(&wsv, ws_bytes, st));
   uint8_t* Wd = (uint8_t*)wsv;
   uint64_t* d_cls = (uint64_t*)(Wd + w_cls);
-  uint64_t* d_lvl = (uint64_t*)(Wd + w_lvl);
   LevelMeta* d_gmeta = (LevelMeta*)(Wd + w_gmeta);
   SegDesc* d_sseg = (SegDesc*)(Wd + w_sseg);
-  uint32_t* d_tick = (uint32_t*)(Wd + w_tick);
   uint8_t* d_seq[2] = {Wd + w_seq0, Wd + w_seq1};
 
-  // host image of the tables [w_lvl, w_tab_end)
-  std::vector<uint8_t> img(w_tab_end - w_lvl, 0);
-  auto at = [&](uint64_t off) { return img.data() + (off - w_lvl); };
-  uint64_t* h_lvl = (uint64_t*)at(w_lvl);
+  // host image of the tables [w_gmeta, w_tab_end)
+  std::vector<uint8_t> img(w_tab_end - w_gmeta, 0);
+  auto at = [&](uint64_t off) { return img.data() + (off - w_gmeta); };
   LevelMeta* h_gmeta = (LevelMeta*)at(w_gmeta);
   SegDesc* h_sseg = (SegDesc*)at(w_sseg);
   std::vector<uint64_t> sb_first(nlev_tot + 1, 0);
@@ -276,10 +266,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     uint64_t lev = 0;
     for (uint32_t i = 0; i < m; i++) {
       const SeqPlan& p = sp[i];
-      uint64_t* lo = h_lvl + p.lvl_base;
-      uint64_t* ll = lo + p.L + 1;
-      for (int l = 0; l <= p.L; l++) lo[l] = (uint64_t)l * p.W;
-      for (int l = 0; l < p.L; l++) ll[l] = p.n;
       for (int l = 0; l < p.L; l++, lev++) {
         LevelMeta mt = meta_of(p, l);
         h_meta_all[p.meta_base + l] = mt;
@@ -292,23 +278,22 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
       }
     }
   }
-  // per-launch segment lists: pass g, narrow (E = u16) then wide (E = u32)
+  // per-launch segment lists: pass g, by the width of its elements
   struct Launch {
     uint64_t first;
     uint32_t nsegs, ntiles;
-    bool wide;
-    int tmax;  // widest digit of its segments
+    int in_w;
   };
   std::vector<Launch> launches;
   {
     uint64_t k = 0;
     for (int g = 0; g < Gmax; g++) {
-      for (int wide = 0; wide < 2; wide++) {
-        Launch L0{k, 0, 0, wide != 0, 1};
+      for (int in_w = 1; in_w <= 4; in_w *= 2) {
+        Launch L0{k, 0, 0, in_w};
         uint32_t tiles = 0;
         for (uint32_t i = 0; i < m; i++) {
           const SeqPlan& p = sp[i];
-          if (!p.n || g >= p.G || p.ps[g].wide != (wide != 0)) continue;
+          if (!p.n || g >= p.G || p.ps[g].in_w != in_w) continue;
           const Pass1& q = p.ps[g];
           uint64_t coff = p.cls_off;
           for (int g2 = 0; g2 < g; g2++) coff += (2u << p.ps[g2].t) + p.ps[g2].t + 1;
@@ -316,8 +301,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
           d.in = g == 0 ? items[i].d_seq : (const void*)(d_seq[(g - 1) & 1] + p.seq_off);
           d.out = (g + 1 < p.G) ? (void*)(d_seq[g & 1] + p.seq_off) : nullptr;
           d.bits = a_bits + p.bits_base;
-          d.lvl_off = d_lvl + p.lvl_base;
-          d.lvl_len = d_lvl + p.lvl_base + p.L + 1;
           d.wm_cls = d_cls + coff;
           d.zeros = a_zeros + p.zeros_base;
           d.err = a_err + i;
@@ -332,7 +315,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
           d.rbits = q.rbits;
           tiles += (uint32_t)((p.n + PASS_T - 1) / PASS_T);
           L0.nsegs++;
-          L0.tmax = std::max(L0.tmax, q.t);
         }
         L0.ntiles = tiles;
         if (L0.nsegs) launches.push_back(L0);
@@ -343,21 +325,19 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   if (nbits) CK(cudaMemsetAsync(a_bits, 0, 8 * nbits, st));
   CK(cudaMemsetAsync(a_err, 0, 4 * (uint64_t)m, st));
   if (nzeros) CK(cudaMemsetAsync(a_zeros, 0, 8 * nzeros, st));  // empty sequences plan nothing
-  CK(cudaMemsetAsync(d_tick, 0, 4 * 64, st));
   wt_status s = nmeta ? upload(a_meta, h_meta_all.data(), sizeof(LevelMeta) * nmeta, st) : WT_OK;
-  if (s == WT_OK) s = upload(Wd + w_lvl, img.data(), img.size(), st);
+  if (s == WT_OK) s = upload(Wd + w_gmeta, img.data(), img.size(), st);
   for (size_t li = 0; li < launches.size() && s == WT_OK; li++) {
     const Launch& L0 = launches[li];
     PassParams P;
     memset(&P, 0, sizeof(P));
     P.shape = SHAPE_WM;
-    P.ticket = d_tick + li;
     P.err = a_err;  // replaced per tile by the sequence's own word
+    P.in_w = L0.in_w;
     P.ntiles = L0.ntiles;
     P.segs = d_sseg + L0.first;
     P.nsegs = L0.nsegs;
-    P.tcs = tc_stride(L0.tmax);
-    s = launch_pass_batch(P, L0.wide, o, st);
+    s = launch_pass_batch(P, o, st);
   }
   if (s == WT_OK && !(o && (o->flags & WT_FLAG_NO_DIRECTORY)))
     s = dir_build_levels(a_bits, d_gmeta, (uint32_t)nlev_tot, sb_first, a_dir, a_samp, nullptr,
@@ -540,9 +520,9 @@ extern "C" wt_status wm_autotune(const void* d_seq, uint64_t n, uint32_t sigma,
   if (width_bytes != 1 && width_bytes != 2 && width_bytes != 4) return WT_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const uint32_t L = levels_of_b(sigma);
-  const uint32_t tmax = std::min<uint32_t>(L, TAU_MAX);
+  const uint32_t tmax = std::min<uint32_t>(L, 8);  // above TAU_MAX: passes of TAU_MAX levels
   if (ms_out)
-    for (int i = 0; i < TAU_MAX; i++) ms_out[i] = 0.f;
+    for (int i = 0; i < 8; i++) ms_out[i] = 0.f;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -577,8 +557,8 @@ extern "C" wt_status wm_autotune(const void* d_seq, uint64_t n, uint32_t sigma,
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (s != WT_OK) return s;
-  *best_tau = bt;
-  record_config(L, n, (int)bt, 0, 0);
+  *best_tau = std::min<uint32_t>(bt, TAU_MAX);
+  record_config(L, n, (int)*best_tau, 0, 0);
   return WT_OK;
 }
 

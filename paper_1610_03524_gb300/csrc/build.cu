@@ -126,73 +126,145 @@ __device__ __forceinline__ void for_each_symbol(const void* seq, uint64_t n, uin
   for (uint64_t i = nvec * PER + gtid; i < n; i += gstride) f((uint32_t)s[i]);
 }
 
-// Digit counts of the first pass (levels 0 .. t0-1): its digit is the top t0
-// bits, its sort key the digit reversed (Section 4.3: the reverse of the tau
-// bits).
-// Validation and the first pass's digit counts, walked tile by tile (tiles
-// of `tile` symbols, as the first partition pass sees them): each tile's
-// counts of the first pass's reversed digit, from one read of the sequence.
-// The later passes take their counts from their own tiles (k_tile_counts).
-template <int WB>
-__global__ void __launch_bounds__(256) k_hist_digits_tiles(const void* seq, uint64_t n,
-                                                           uint32_t sigma, int L, int t0,
-                                                           uint32_t* err, uint32_t* tcnt,
-                                                           uint32_t tcs, uint32_t tile, uint4* clear,
-                                                           uint64_t clear_units,
-                                                           uint64_t clear_per) {
-  using T = typename std::conditional<WB == 1, uint8_t,
-                                      typename std::conditional<WB == 2, uint16_t, uint32_t>::type>::type;
-  __shared__ uint32_t th[2][TC_STRIDE];
-  const int tid = threadIdx.x;
-  th[0][tid] = 0;
-  th[1][tid] = 0;
-  __syncthreads();
-  const uint32_t rmask = (1u << t0) - 1u;
-  const int rsh = 32 - L;
-  const uint64_t ntiles = (n + tile - 1) / tile;
-  const T* s = (const T*)seq;
-  const bool vec = (((uintptr_t)seq) & 15) == 0;
-  bool bad = false;
-  int buf = 0;
-  auto count = [&](uint32_t x) {
-    bad |= x >= sigma;
-    atomicAdd(&th[buf][(__brev(x) >> rsh) & rmask], 1u);
-  };
-  for (uint64_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-    // the first pass's levels start at zero: this tile's share of them
-    if (clear) clear_share(clear, clear_units, clear_per, ti, tid, blockDim.x);
-    const uint64_t i0 = ti * tile;
-    const uint64_t i1 = i0 + tile < n ? i0 + tile : n;
-    if (vec && i1 - i0 == tile) {
-      constexpr int PER = 16 / WB;
-      const uint4* v = (const uint4*)(s + i0);
-      for (int k = tid; k < (int)(tile / PER); k += blockDim.x) {
-        const uint4 q = __ldcs(v + k);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+// Digit counts of every tile of a pass (the K sub-problems' per-class counts
+// of Section 4.2), by key (the digit reversed): one warp per tile, the same
+// tiles and digits as k_pass.  A lane takes 32 elements a step as bit planes
+// (bitplane.cuh; their order does not matter) and counts each key's
+// indicator word; the lanes' sums, two 16-bit counts a word, by eight warp
+// reductions a tile.  No atomics and no barriers: about 4 instructions per
+// 32 elements, so that DRAM is the bound, where a shared-memory atomic per
+// element was.  First passes also check the symbols against sigma and zero
+// their share of the pass's levels.
+template <int EW, bool BATCH>
+__global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ PassParams P0,
+                                                     uint32_t* tcnt, uint32_t tile) {
+  __shared__ PassParams s_P[BATCH ? 8 : 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
+  const uint32_t nw = gridDim.x * 8;
+  if (BATCH && lane == 0) s_P[warp] = P0;
+  for (uint32_t ti = blockIdx.x * 8 + warp; ti < ntiles; ti += nw) {
+    if (BATCH) {
+      __syncwarp();
+      if (lane == 0) fill_seg(s_P[warp], P0, ti);
+      __syncwarp();
+    }
+    const PassParams& P = BATCH ? s_P[warp] : P0;
+    if (!BATCH && P.clear) clear_share(P.clear, P.clear_units, P.clear_per, ti, lane, 32);
+    const TileInfo I = tile_info(P, ti, tile);
+    const int t = P.t;
+    const uint32_t sigma = P.sigma;
+    // every value of the element's width is below sigma: nothing to check
+    const bool check = sigma != 0u && (EW == 4 || sigma < (1u << (8 * (EW & 3))));
+    uint32_t acc[8] = {};
+    uint32_t top[2] = {0u, 0u};  // running maxima (of 16-bit halves below 4 bytes)
+    auto count = [&](uint32_t p[4], uint32_t v) {
+      if (t < 2) p[1] = 0u;
+      if (t < 3) p[2] = 0u;
+      if (t < 4) p[3] = 0u;
+      uint32_t c[8];
+      key_counts(p, v, c);
 #pragma unroll
-        for (int m = 0; m < 4; m++) {
-          if (WB == 1) {
+      for (int k = 0; k < 8; k++) acc[k] += c[k];
+    };
+    bool bad = false;
+    constexpr int PV = 16 / EW;  // elements a vector
+    {
+      // 16-byte vectors from the aligned one that holds the tile's first
+      // element, 2 EW of them a lane and step; the ends' other elements masked
+      const int skew = (int)(((uintptr_t)I.src & 15) / EW);
+      const uint4* const src = (const uint4*)((uintptr_t)I.src & ~(uintptr_t)15);
+      const uint4* const in0 = (const uint4*)(((uintptr_t)P.in + 15) & ~(uintptr_t)15);
+      const uint4* const in1 = (const uint4*)(((uintptr_t)P.in + P.n_in * (uint64_t)EW) & ~(uintptr_t)15);
+      const int nvec = (skew + I.cnt + PV - 1) / PV;
+      const bool inside = skew == 0 && I.cnt == (int)tile;
+      for (int i0 = 0; i0 < nvec; i0 += 64 * EW) {
+        uint4 q[2 * EW];
+        uint32_t v = FULL;
+        if (inside) {
 #pragma unroll
-            for (int b = 0; b < 4; b++) count((w[m] >> (8 * b)) & 0xffu);
-          } else if (WB == 2) {
-            count(w[m] & 0xffffu);
-            count(w[m] >> 16);
-          } else {
-            count(w[m]);
+          for (int i = 0; i < 2 * EW; i++) q[i] = __ldcs(src + i0 + 32 * i + lane);
+        } else {
+          v = 0u;
+#pragma unroll
+          for (int i = 0; i < 2 * EW; i++) {
+            const int at = i0 + 32 * i + lane;
+            q[i] = make_uint4(0u, 0u, 0u, 0u);
+            // elements lo .. hi - 1 of the vector are the tile's
+            const int lo = max(skew - PV * at, 0), hi = min(skew + I.cnt - PV * at, PV);
+            if (lo < hi) {
+              if (src + at >= in0 && src + at < in1) {
+                q[i] = __ldcs(src + at);
+              } else {  // a vector that reaches past the sequence
+                for (int e = lo; e < hi; e++) {
+                  const uint32_t x = load_elem(src + at, EW, (uint64_t)e);
+                  const uint32_t y = x << (8 * ((e * EW) & 3));
+                  const int k = (e * EW) >> 2;
+                  if (k == 0) q[i].x |= y;
+                  else if (k == 1) q[i].y |= y;
+                  else if (k == 2) q[i].z |= y;
+                  else q[i].w |= y;
+                }
+              }
+              v |= (low_mask((uint32_t)hi) & ~low_mask((uint32_t)lo)) << (PV * i);
+              if (check && (lo > 0 || hi < PV)) {
+                // the neighbours' elements out of the running maxima
+                const uint32_t w[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+                for (int e = lo; e < hi; e++) {
+                  uint32_t x = w[0];
+                  const int k = (e * EW) >> 2;
+                  x = k == 1 ? w[1] : (k == 2 ? w[2] : (k == 3 ? w[3] : x));
+                  x >>= 8 * ((e * EW) & 3);
+                  if (EW == 1) x &= 0xffu;
+                  if (EW == 2) x &= 0xffffu;
+                  bad |= x >= sigma;
+                }
+              }
+            }
           }
         }
+        if (check) {
+#pragma unroll
+          for (int i = 0; i < 2 * EW; i++) {
+            const uint32_t w[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+            // whole vectors only
+            if (!inside && ((v >> (PV * i)) & low_mask(PV)) != low_mask(PV)) continue;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+              if (EW == 4) {
+                top[0] = max(top[0], w[k]);
+              } else if (EW == 2) {
+                top[0] = __vmaxu2(top[0], w[k]);
+              } else {
+                top[0] = __vmaxu2(top[0], w[k] & 0x00FF00FFu);
+                top[1] = __vmaxu2(top[1], (w[k] >> 8) & 0x00FF00FFu);
+              }
+            }
+          }
+        }
+        uint32_t p[4];
+        planes_of<EW>([&](int i, uint32_t* w) {
+          w[0] = q[i].x;
+          w[1] = q[i].y;
+          w[2] = q[i].z;
+          w[3] = q[i].w;
+        }, P.rbits, p);
+        count(p, v);
       }
-    } else {
-      for (uint64_t i = i0 + tid; i < i1; i += blockDim.x) count((uint32_t)s[i]);
+      if (check) {
+        if (EW == 4) bad |= top[0] >= sigma;
+        else bad |= max(max(top[0] & 0xffffu, top[0] >> 16), max(top[1] & 0xffffu, top[1] >> 16)) >= sigma;
+      }
     }
-    __syncthreads();
-    // the other buffer was written out one tile ago; this one now
-    const uint32_t c = th[buf][tid];
-    if (tid < (int)tcs) tcnt[ti * tcs + tid] = c;
-    th[buf][tid] = 0;
-    buf ^= 1;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const uint32_t sum = __reduce_add_sync(FULL, acc[k]);
+      if ((lane >> 1) == k) mine = (sum >> (16 * (lane & 1))) & 0xffffu;
+    }
+    if (lane < TC_STRIDE) tcnt[(uint64_t)ti * TC_STRIDE + lane] = mine;
+    if (__any_sync(FULL, bad) && lane == 0) atomicOr(P.err, ERR_SYMBOL);
   }
-  if (bad) atomicOr(err, ERR_SYMBOL);
 }
 
 // The same counts for bytes over SIG = 2 .. 8 values in a single pass
@@ -207,8 +279,8 @@ __global__ void __launch_bounds__(256) k_hist_digits_tiles(const void* seq, uint
 template <int SIG>
 __global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, uint64_t n,
                                                            uint32_t* err, uint32_t* tcnt,
-                                                           uint32_t tcs, uint32_t tile,
-                                                           uint4* clear, uint64_t clear_units,
+                                                           uint32_t tile, uint4* clear,
+                                                           uint64_t clear_units,
                                                            uint64_t clear_per) {
   constexpr int NV = SIG - 1, T0 = SIG <= 2 ? 1 : (SIG <= 4 ? 2 : 3);
   constexpr uint32_t M = 0x11111111u;
@@ -267,25 +339,24 @@ __global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, u
       if (s + 1 < NV && lane == (int)rev_bits((uint32_t)(s + 2), T0)) mine = hi;
     }
     if (lane == 0) mine = rest;
-    tcnt[ti * tcs + lane] = mine;
+    if (lane < TC_STRIDE) tcnt[ti * TC_STRIDE + lane] = mine;
   }
   if (__any_sync(FULL, bad != 0u) && lane == 0) atomicOr(err, ERR_SYMBOL);
 }
 
-// Launch of the first pass's tile counts (t0 levels of L, tiles of T), which
-// also zero `clear_units` 16-byte units at `clear`, a share per tile.
-static wt_status launch_first_counts(const void* seq, int w, uint64_t n, uint32_t sigma, int L,
-                                     int t0, uint32_t T, uint32_t* err, uint32_t* tcnt,
-                                     uint64_t* clear, uint64_t clear_units, cudaStream_t st) {
-  const uint64_t ntiles = (n + T - 1) / T, per = (clear_units + ntiles - 1) / ntiles;
-  const uint32_t tcs = tc_stride(t0);
-  uint4* const cl = (uint4*)clear;
-  if (w == 1 && L == t0 && sigma >= 2 && sigma <= 8) {
-    const uint8_t* sb = (const uint8_t*)seq;
-    const unsigned grid = (unsigned)std::min<uint64_t>((ntiles + 7) / 8, (uint64_t)num_sms() * 32);
-#define WT_COUNT_BYTES(S) \
-  case S: k_count_tiles_bytes<S><<<grid, 256, 0, st>>>(sb, n, err, tcnt, tcs, T, cl, clear_units, per); break
-    switch (sigma) {
+// Launch of a pass's tile counts into tcnt (mt tiles at most).
+template <bool BATCH>
+static wt_status launch_counts(const PassParams& P, uint32_t T, uint64_t mt, uint32_t* tcnt,
+                               cudaStream_t st) {
+  const unsigned grid = (unsigned)std::min<uint64_t>((mt + 7) / 8, (uint64_t)num_sms() * 32);
+  if (!BATCH && P.in_w == 1 && !P.tiles && P.sigma >= 2 && P.sigma <= 8 && P.t == P.L) {
+    const uint8_t* sb = (const uint8_t*)P.in;
+#define WT_COUNT_BYTES(S)                                                                          \
+  case S:                                                                                          \
+    k_count_tiles_bytes<S><<<grid, 256, 0, st>>>(sb, P.n_in, P.err, tcnt, T, P.clear,              \
+                                                 P.clear_units, P.clear_per);                      \
+    break
+    switch (P.sigma) {
       WT_COUNT_BYTES(2);
       WT_COUNT_BYTES(3);
       WT_COUNT_BYTES(4);
@@ -295,17 +366,12 @@ static wt_status launch_first_counts(const void* seq, int w, uint64_t n, uint32_
       WT_COUNT_BYTES(8);
     }
 #undef WT_COUNT_BYTES
+  } else if (P.in_w == 1) {
+    k_tile_counts<1, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
+  } else if (P.in_w == 2) {
+    k_tile_counts<2, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
   } else {
-    const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)num_sms() * 8, ntiles);
-    if (w == 1)
-      k_hist_digits_tiles<1><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
-                                                   clear_units, per);
-    else if (w == 2)
-      k_hist_digits_tiles<2><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
-                                                   clear_units, per);
-    else
-      k_hist_digits_tiles<4><<<grid, 256, 0, st>>>(seq, n, sigma, L, t0, err, tcnt, tcs, T, cl,
-                                                   clear_units, per);
+    k_tile_counts<4, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
   }
   count_launch();
   CK(cudaGetLastError());
@@ -583,7 +649,6 @@ static uint64_t scan_scratch(uint64_t n) { return n / SCAN_CH + 2; }
 // ---------------------------------------------------------------------------
 struct PassGeom {
   int a, t, rbits, in_w, out_w;
-  bool wide;  // 32-bit working elements
 };
 
 // bytes per element of the widest intermediate sequence
@@ -602,100 +667,112 @@ static std::vector<PassGeom> make_passes(int L, int tau, int first_w) {
     p.rbits = L - a;
     p.in_w = a == 0 ? first_w : width_for_bits(L - a);
     p.out_w = (a + p.t < L) ? width_for_bits(L - a - p.t) : 0;
-    p.wide = p.rbits > 16;
     ps.push_back(p);
   }
   return ps;
 }
 
-// What a pass's plan gives, from the totals of its tiles' digit counts
-// (indexed by reversed digit, the key of the splits): for the wavelet matrix
-// the class starts of its levels a .. a+t (level a+j's classes are the values
-// of the key's low j bits) into cls, for a balanced tree of one pass the
-// symbol starts C[0 .. 2^t]; for both every level's zero count (the start of
-// class 2^(j-1) after split j: a level's zeros are the same in either order).
+// What a pass's plan gives, from the totals of its tiles' digit counts by key
+// (the digit reversed): for the wavelet matrix the class starts of its levels
+// a .. a+t (level a+j's classes are the values of the key's low j bits) into
+// cls and every level's zero count (the start of class 2^(j-1) after split j);
+// for a balanced tree's first pass the starts of the nodes of level t.
 enum PlanKind : int { PLAN_NONE = 0, PLAN_WM = 1, PLAN_WT = 2 };
 struct PassPlan {
   int kind;
   int a, t;
   uint64_t* cls;    // WM
-  uint64_t* C;      // WT
-  uint64_t* zeros;  // nullptr: not wanted (digit levels)
+  uint64_t* C;      // WT: 2^t + 1
+  uint64_t* zeros;  // WM
 };
 
-// exclusive scan of n entries of v by one warp, written to out[0..n]; at
-// entry `mark` also to *at_mark
-__device__ __forceinline__ void warp_scan_to(const uint64_t* v, int n, uint64_t* out, int mark,
-                                             uint64_t* at_mark, int rev_t) {
+// exclusive prefix sums of one value a lane over the first n lanes
+__device__ __forceinline__ uint64_t warp_scan_excl(uint64_t v, uint64_t& total) {
   const int lane = threadIdx.x & 31;
-  uint64_t carry = 0;
-  for (int k0 = 0; k0 < n; k0 += 32) {
-    const int k = k0 + lane;
-    const uint64_t c = k < n ? v[rev_t ? rev_bits((uint32_t)k, rev_t) : (uint32_t)k] : 0ull;
-    uint64_t x = c;
+  uint64_t x = v;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(FULL, x, o);
-      if (lane >= o) x += y;
-    }
-    if (k < n) {
-      if (out) out[k] = carry + x - c;
-      if (k == mark) *at_mark = carry + x - c;
-    }
-    carry += __shfl_sync(FULL, x, 31);
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
   }
-  if (lane == 0 && out) out[n] = carry;
+  total = __shfl_sync(FULL, x, 31);
+  return x - v;
 }
 
-// One block: the plan from the totals in cnt[2^t - 1 + r] (shared memory).
-// The levels' counts are folded from the deepest up, then each level is
-// scanned by a warp of its own (one thread scanning 2^j entries for every
-// level in turn took 40-55 us, more than any other kernel of a small build).
-__device__ void plan_pass(uint64_t* cnt, const PassPlan& p) {
-  const int t = p.t, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int j = t - 1; j >= 0; j--) {
-    __syncthreads();
+// One warp: the plan from the totals, lane r < 2^t holding key r's.  Level j's
+// counts are folded from level j+1's.  (A thread scanning each level in turn
+// took 40-55 us for eight levels, more than any other kernel of a small
+// build.)
+__device__ void plan_pass(uint64_t tot, const PassPlan& p) {
+  const int lane = threadIdx.x & 31, t = p.t;
+  uint64_t c = lane < (1 << t) ? tot : 0ull, all;
+  if (p.kind == PLAN_WT) {
+    // in order of the digit: lane v takes the count of key rev(v)
+    const uint64_t d = __shfl_sync(FULL, c, (int)rev_bits((uint32_t)lane & ((1u << t) - 1u), t));
+    const uint64_t start = warp_scan_excl(lane < (1 << t) ? d : 0ull, all);
+    if (lane <= (1 << t)) p.C[lane] = start;
+    return;
+  }
+  for (int j = t; j >= 0; j--) {
     const int nk = 1 << j;
-    for (int k = threadIdx.x; k < nk; k += blockDim.x)
-      cnt[nk - 1 + k] = cnt[2 * nk - 1 + k] + cnt[2 * nk - 1 + k + nk];
+    const uint64_t start = warp_scan_excl(lane < nk ? c : 0ull, all);
+    uint64_t* const out = p.cls + (nk - 1 + j);
+    if (lane <= nk) out[lane] = start;  // the lane after the last class: the total
+    if (j > 0 && lane == nk / 2) p.zeros[p.a + j - 1] = start;
+    const uint64_t up = __shfl_down_sync(FULL, c, nk / 2);
+    c += lane < nk / 2 ? up : 0ull;
   }
-  __syncthreads();
-  for (int j = warp; j <= t; j += nwarps) {
-    const int nk = 1 << j;
-    warp_scan_to(cnt + nk - 1, nk, p.kind == PLAN_WM ? p.cls + (nk - 1 + j) : nullptr,
-                 j && p.zeros ? nk >> 1 : -1, p.zeros + (j ? p.a + j - 1 : 0), 0);
-  }
-  if (p.kind == PLAN_WT && warp == nwarps - 1)
-    warp_scan_to(cnt + (1 << t) - 1, 1 << t, p.C, -1, nullptr, t);
 }
 
-// the plan of one pass from the totals of its tiles' digit counts (the last
-// row of the scanned chunk table)
-__global__ void __launch_bounds__(288) k_plan_pass(const uint64_t* totals, const PassPlan p) {
-  __shared__ uint64_t cnt[2 * TC_STRIDE];
-  for (int r = threadIdx.x; r < (1 << p.t); r += blockDim.x) cnt[(1 << p.t) - 1 + r] = totals[r];
-  plan_pass(cnt, p);
-}
-
-// Batched builds, one block per sequence of the launch: the plan of its pass
+// Batched builds, one warp per sequence of the launch: the plan of its pass
 // from the totals of its own tiles' digit counts, i.e. the difference of the
 // scanned tables' prefixes at its last and first tile (tcnt exclusive within
 // chunks of 2^chsh tiles, tchunk the chunks' exclusive prefixes with the
 // total after the last chunk).
-__global__ void __launch_bounds__(288) k_plan_batch_pass(const SegDesc* segs, const uint32_t* tcnt,
-                                                         const uint64_t* tchunk, uint32_t tcs,
-                                                         uint32_t ntiles, uint32_t chsh) {
-  __shared__ uint64_t cnt[2 * TC_STRIDE];
-  const SegDesc& d = segs[blockIdx.x];
+__device__ __forceinline__ uint64_t tile_prefix(const uint32_t* tcnt, const uint64_t* tchunk,
+                                                uint32_t ntiles, uint32_t nchunk, uint32_t chsh,
+                                                uint32_t ti, uint32_t r) {
+  if (ti >= ntiles) return tchunk[(uint64_t)nchunk * TC_STRIDE + r];
+  return tchunk[(uint64_t)(ti >> chsh) * TC_STRIDE + r] + tcnt[(uint64_t)ti * TC_STRIDE + r];
+}
+
+__global__ void __launch_bounds__(256) k_plan_batch_pass(const SegDesc* segs, uint32_t nsegs,
+                                                         const uint32_t* tcnt,
+                                                         const uint64_t* tchunk, uint32_t ntiles,
+                                                         uint32_t nchunk, uint32_t chsh) {
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, r = threadIdx.x & 31;
+  if (i >= nsegs) return;
+  const SegDesc& d = segs[i];
   const uint32_t t0 = d.tile0, t1 = t0 + (uint32_t)((d.n + PASS_T - 1) / PASS_T);
-  const uint64_t last = (uint64_t)((ntiles + (1u << chsh) - 1) >> chsh) * tcs;
-  auto prefix = [&](uint32_t ti, uint32_t r) -> uint64_t {
-    if (ti >= ntiles) return tchunk[last + r];
-    return tchunk[(uint64_t)(ti >> chsh) * tcs + r] + tcnt[(uint64_t)ti * tcs + r];
-  };
-  for (uint32_t r = threadIdx.x; r < (1u << d.t); r += blockDim.x)
-    cnt[(1u << d.t) - 1 + r] = prefix(t1, r) - prefix(t0, r);
-  plan_pass(cnt, PassPlan{PLAN_WM, d.a, d.t, d.wm_cls, nullptr, d.zeros});
+  uint64_t tot = 0;
+  if (r < (1u << d.t))
+    tot = tile_prefix(tcnt, tchunk, ntiles, nchunk, chsh, t1, r) -
+          tile_prefix(tcnt, tchunk, ntiles, nchunk, chsh, t0, r);
+  plan_pass(tot, PassPlan{PLAN_WM, d.a, d.t, d.wm_cls, nullptr, d.zeros});
+}
+
+// Balanced trees, passes after the first, one warp per node q of level a: the
+// starts of its descendants on level a + t, C[q 2^t .. (q+1) 2^t), from the
+// totals of the node's tiles toff[q] .. toff[q+1] - 1 (and C's last entry, n).
+__global__ void __launch_bounds__(256) k_plan_nodes(const uint64_t* Ca, const uint64_t* toff,
+                                                    uint64_t nn, int t, uint64_t n,
+                                                    const uint32_t* tcnt, const uint64_t* tchunk,
+                                                    const uint32_t* ntiles_dev, uint32_t nchunk,
+                                                    uint32_t chsh, uint64_t* C) {
+  const uint64_t q = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t v = threadIdx.x & 31;
+  if (q >= nn) return;
+  const uint32_t ntiles = *ntiles_dev;
+  const uint32_t t0 = (uint32_t)toff[q], t1 = (uint32_t)toff[q + 1];
+  uint64_t tot = 0, all;
+  if (v < (1u << t) && t1 > t0) {
+    const uint32_t r = rev_bits(v, t);
+    tot = tile_prefix(tcnt, tchunk, ntiles, nchunk, chsh, t1, r) -
+          tile_prefix(tcnt, tchunk, ntiles, nchunk, chsh, t0, r);
+  }
+  const uint64_t start = Ca[q] + warp_scan_excl(tot, all);
+  if (v < (1u << t)) C[(q << t) + v] = start;
+  if (q + 1 == nn && v == 0) C[nn << t] = n;
 }
 
 // Balanced-tree helpers over C (C[v] = number of symbols < v, v in [0, 2^L]).
@@ -712,20 +789,38 @@ __global__ void k_wt_zeros(const uint64_t* C, int L, uint64_t* zeros) {
   if (threadIdx.x == 0) zeros[l] = tot;
 }
 
-// Node-aligned tiles over T_a: node p spans [bnd[p*stride], bnd[(p+1)*stride]).
-__global__ void k_tiles_count(const uint64_t* bnd, uint64_t stride, uint64_t nn, uint32_t T,
-                              uint64_t* tcnt) {
+// Node-aligned tiles over T_a: node p spans [bnd[p], bnd[p+1]).
+__global__ void k_tiles_count(const uint64_t* bnd, uint64_t nn, uint32_t T, uint64_t* tcnt) {
   const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= nn) return;
-  const uint64_t sz = bnd[(p + 1) * stride] - bnd[p * stride];
+  const uint64_t sz = bnd[p + 1] - bnd[p];
   tcnt[p] = (sz + T - 1) / T;
+}
+
+// The tile counts' and offsets of up to 4096 nodes by one block (one launch
+// instead of four).
+__global__ void __launch_bounds__(1024) k_tiles_offsets(const uint64_t* bnd, uint32_t nn, uint32_t T,
+                                                        uint64_t* toff) {
+  uint64_t c[4], sum = 0;
+  const uint32_t p0 = threadIdx.x * 4;
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    c[k] = p0 + k < nn ? (bnd[p0 + k + 1] - bnd[p0 + k] + T - 1) / T : 0ull;
+    sum += c[k];
+  }
+  uint64_t tot, ex = block_scan_excl_u64(sum, &tot);
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    if (p0 + k < nn) toff[p0 + k] = ex;
+    ex += c[k];
+  }
+  if (threadIdx.x == 0) toff[nn] = tot;
 }
 
 // One thread per tile: tile i belongs to the node p with toff[p] <= i <
 // toff[p+1] (nodes without tiles share their toff with the next node, so the
 // last p with toff[p] <= i is the right one).
-__global__ void k_tiles_write(const uint64_t* bnd, uint64_t stride, uint64_t nn, uint32_t T,
-                              uint64_t node_base, const uint64_t* toff, TileDesc* tiles,
+__global__ void k_tiles_write(const uint64_t* bnd, uint64_t nn, uint32_t T, uint64_t node_base, const uint64_t* toff, TileDesc* tiles,
                               uint32_t* ntiles, uint64_t max_tiles) {
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t total = toff[nn];
@@ -738,7 +833,7 @@ __global__ void k_tiles_write(const uint64_t* bnd, uint64_t stride, uint64_t nn,
     else hi = mid - 1;
   }
   const uint64_t p = lo, k = i - toff[p];
-  const uint64_t s = bnd[p * stride] + k * T, e = bnd[(p + 1) * stride];
+  const uint64_t s = bnd[p] + k * T, e = bnd[p + 1];
   TileDesc d;
   d.start = s;
   d.count = (uint32_t)std::min<uint64_t>(T, e - s);
@@ -748,94 +843,43 @@ __global__ void k_tiles_write(const uint64_t* bnd, uint64_t stride, uint64_t nn,
   tiles[i] = d;
 }
 
+// The node-aligned tiles of a pass: node p of nn spans [bnd[p], bnd[p+1]).
+static wt_status launch_node_tiles(const uint64_t* bnd, uint64_t nn, uint32_t T, uint64_t node_base,
+                                   uint64_t mt, uint64_t* tcnt, uint64_t* toff, uint64_t* scr,
+                                   TileDesc* tiles, uint32_t* d_ntiles, cudaStream_t st) {
+  if (nn <= 4096) {
+    k_tiles_offsets<<<1, 1024, 0, st>>>(bnd, (uint32_t)nn, T, toff);
+    count_launch();
+  } else {
+    k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(bnd, nn, T, tcnt);
+    count_launch();
+    TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
+  }
+  k_tiles_write<<<(unsigned)((mt + 255) / 256), 256, 0, st>>>(bnd, nn, T, node_base, toff, tiles,
+                                                             d_ntiles, mt);
+  count_launch();
+  CK(cudaGetLastError());
+  return WT_OK;
+}
+
 // ---------------------------------------------------------------------------
 // 3. pass launch
 // ---------------------------------------------------------------------------
-#ifndef WT_PASS_NT
-#define WT_PASS_NT 256
-#endif
-constexpr int PT = PASS_T, PNT = WT_PASS_NT;
+constexpr int PT = PASS_T;
 
-// Digit counts of every tile of a pass (the K sub-problems' per-class counts
-// of Section 4.2): one block per tile, the same tiles and digits as k_pass.
-template <typename E, bool BATCH>
-__global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ PassParams P0,
-                                                     uint32_t* tcnt, uint32_t tile) {
-  __shared__ uint32_t h[TC_STRIDE];
-  __shared__ PassParams s_P;
-  const PassParams& P = BATCH ? s_P : P0;
-  const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
-  const int tid = threadIdx.x;
-  if (BATCH && tid == 0) s_P = P0;
-  for (uint32_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-    if (BATCH && tid == 0) fill_seg(s_P, P0, ti);
-    h[tid] = 0;
-    __syncthreads();
-    uint64_t ts;
-    int cnt;
-    if (P.tiles) {
-      const TileDesc d = P.tiles[ti];
-      ts = d.start;
-      cnt = (int)d.count;
-    } else {
-      ts = (uint64_t)(ti - P.tile0) * tile;
-      const uint64_t rem = P.n_in - ts;
-      cnt = (int)(rem < (uint64_t)tile ? rem : (uint64_t)tile);
-    }
-    const uint32_t rmask = (1u << P.t) - 1u;
-    const int rsh = 32 - P.rbits;
-    // batched first passes also check the symbols (the single builds check
-    // them in their histogram kernel)
-    const uint32_t sigma = BATCH ? P.sigma : 0u;
-    bool bad = false;
-    auto count = [&](uint32_t x) {
-      if (BATCH) bad |= sigma != 0u && x >= sigma;
-      atomicAdd(&h[(__brev(x) >> rsh) & rmask], 1u);
-    };
-    const uintptr_t a = (uintptr_t)P.in + ts * (uint64_t)P.in_w;
-    if (P.code_map) {
-      for (int i = tid; i < cnt; i += 256) count(P.code_map[load_elem(P.in, P.in_w, ts + i)]);
-    } else if (P.in_w == 2 && cnt == (int)tile && (a & 15) == 0) {
-      const uint4* src = (const uint4*)a;
-      for (int i = tid; i < (int)tile / 8; i += 256) {
-        const uint4 q = __ldcs(src + i);
-        const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          count(w4[k] & 0xffffu);
-          count(w4[k] >> 16);
-        }
-      }
-    } else if (P.in_w == 1 && cnt == (int)tile && (a & 15) == 0) {
-      const uint4* src = (const uint4*)a;
-      for (int i = tid; i < (int)tile / 16; i += 256) {
-        const uint4 q = __ldcs(src + i);
-        const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-#pragma unroll
-          for (int b = 0; b < 4; b++) count((w4[k] >> (8 * b)) & 0xffu);
-      }
-    } else {
-      for (int i = tid; i < cnt; i += 256) count(load_elem(P.in, P.in_w, ts + i));
-    }
-    if (BATCH && bad) atomicOr(P.err, ERR_SYMBOL);
-    __syncthreads();
-    if (tid < (int)P0.tcs) tcnt[(uint64_t)ti * P0.tcs + tid] = h[tid];
-    __syncthreads();
-  }
-}
-
-// Prefix sums of the tiles' counts, per digit value: exclusive inside each
-// chunk of 2^chsh tiles (in place, u32), and the chunks' totals.  When there
-// is one chunk only (ONE), the whole scan and the pass's plan are this
-// launch: its totals are the grand totals (row 1), and row 0 is zero.
+// Prefix sums of the tiles' counts, per key: exclusive inside each chunk of
+// 2^chsh tiles (in place, u32), and the chunks' totals; a thread per chunk and
+// key.  When there is one chunk only (ONE), the whole scan and the pass's plan
+// are this launch: its totals are the grand totals (row 1), row 0 is zero.
 template <bool ONE>
 __global__ void __launch_bounds__(256) k_tile_scan_chunk(uint32_t* tcnt, const uint32_t* ntiles_dev,
                                                          uint32_t ntiles_host, uint32_t chsh,
-                                                         uint64_t* tchunk, const PassPlan plan) {
+                                                         uint32_t nchunk, uint64_t* tchunk,
+                                                         const PassPlan plan) {
+  constexpr int S = TC_STRIDE;
   const uint32_t nt = ntiles_dev ? *ntiles_dev : ntiles_host;
-  const uint32_t c = blockIdx.x, r = threadIdx.x, S = blockDim.x;  // one thread per digit
+  const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) / S, r = threadIdx.x % S;
+  if (c >= (ONE ? 2u : nchunk)) return;  // ONE: the plan is made by a whole warp
   const uint64_t t0 = (uint64_t)c << chsh;
   const uint64_t t1 = t0 + (1u << chsh) < nt ? t0 + (1u << chsh) : nt;
   uint32_t run = 0;
@@ -853,28 +897,26 @@ __global__ void __launch_bounds__(256) k_tile_scan_chunk(uint32_t* tcnt, const u
     }
   }
   if constexpr (ONE) {
-    __shared__ uint64_t cnt[2 * TC_STRIDE];
-    tchunk[r] = 0;
-    tchunk[S + r] = run;
-    if (plan.kind != PLAN_NONE) {
-      if (r < (1u << plan.t)) cnt[(1u << plan.t) - 1 + r] = run;
-      plan_pass(cnt, plan);
+    if (c == 0) {
+      tchunk[r] = 0;
+      tchunk[S + r] = run;
     }
+    if (plan.kind != PLAN_NONE) plan_pass(run, plan);
   } else {
     tchunk[(uint64_t)c * S + r] = run;
   }
 }
 
 // ... and the exclusive prefix of the chunks' totals (u64), with the grand
-// total after the last chunk: one block per 32 digit values, a lane per digit
-// value (256-byte rows), warp w scanning the w-th of 32 runs of chunks after
-// their sums are known.  (One warp per digit value, 8 bytes of each row at a
-// time, took 26 us for 1024 chunks and 95 us for 4096.)
+// total after the last chunk, and the pass's plan from it: one block, 64 runs
+// of chunks side by side whose sums are known before they are scanned.
 __global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32_t nchunk,
-                                                        uint32_t S) {
-  __shared__ uint64_t sums[32][33];
-  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
-  const uint32_t per = (nchunk + 31) / 32;
+                                                        const PassPlan plan) {
+  constexpr int S = TC_STRIDE, RUN = 1024 / S;
+  __shared__ uint64_t sums[RUN][S];
+  __shared__ uint64_t total[S];
+  const uint32_t r = threadIdx.x % S, w = threadIdx.x / S;
+  const uint32_t per = (nchunk + RUN - 1) / RUN;
   const uint32_t c0 = min(w * per, nchunk), c1 = min(c0 + per, nchunk);
   constexpr int B = 16;
   uint64_t sum = 0;
@@ -885,10 +927,10 @@ __global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32
 #pragma unroll
     for (int k = 0; k < B; k++) sum += v[k];
   }
-  sums[w][lane] = sum;
+  sums[w][r] = sum;
   __syncthreads();
   uint64_t run = 0;
-  for (uint32_t k = 0; k < w; k++) run += sums[k][lane];
+  for (uint32_t k = 0; k < w; k++) run += sums[k][r];
   for (uint32_t c = c0; c < c1; c += B) {
     uint64_t v[B];
 #pragma unroll
@@ -899,65 +941,33 @@ __global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32
       run += v[k];
     }
   }
-  if (w == 31) tchunk[(uint64_t)nchunk * S + r] = run;
+  if (w == RUN - 1) {
+    tchunk[(uint64_t)nchunk * S + r] = run;
+    total[r] = run;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32 && plan.kind != PLAN_NONE)
+    plan_pass(threadIdx.x < S ? total[threadIdx.x] : 0ull, plan);
 }
 
-// tcnt_pre: the tiles' digit counts when already taken (else counted here);
-// plan: what to plan from the totals of those counts
-template <typename E, bool DIG, bool BATCH = false, int TT = PT, int TNT = PNT>
-static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt_build_opts* o,
-                               cudaStream_t st, uint32_t* tcnt_pre = nullptr,
-                               const PassPlan& plan = PassPlan{}) {
-  using SM = PassSmem<E, TT, TNT, DIG>;
-  auto kern = k_pass<E, TT, TNT, DIG, BATCH>;
+template <int EW, bool DIG, bool BATCH, int NT>
+static wt_status launch_pass_t(const PassParams& Q, uint64_t mt, const wt_build_opts* o,
+                               cudaStream_t st) {
+  using E = typename std::conditional<EW == 1, uint8_t,
+                                      typename std::conditional<EW == 2, uint16_t, uint32_t>::type>::type;
+  using SM = PassSmem<EW, NT>;
+  auto kern = k_pass<E, DIG, BATCH, NT>;
   static bool attr = false;
   static int occ = 0;
   if (!attr) {
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes));
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, TNT + 32, SM::bytes));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, SM::bytes));
     if (occ < 1) occ = 1;
     attr = true;
   }
   int per_sm = occ;
   if (o && o->ctas_per_sm) per_sm = std::min<int>(occ, (int)o->ctas_per_sm);
-  uint64_t grid = (uint64_t)num_sms() * per_sm;
-  if (grid > max_tiles) grid = std::max<uint64_t>(max_tiles, 1);
-  // every tile's digit counts and their prefix sums across the tiles
-  const uint64_t mt = std::max<uint64_t>(max_tiles, 1);
-  PassParams Q = P;
-  Q.chsh = (uint32_t)chunk_shift(mt);
-  const uint32_t nchunk = (uint32_t)((mt + (1u << Q.chsh) - 1) >> Q.chsh);
-  Q.tcs = P.tcs ? P.tcs : tc_stride(P.t);  // batched passes give the widest digit's
-  Work wk{st, {}};
-  uint32_t* tcnt = tcnt_pre;
-  uint64_t* tchunk = nullptr;
-  if (!tcnt) {
-    TRY(wk.get(&tcnt, mt * Q.tcs));
-    k_tile_counts<E, BATCH><<<(unsigned)std::min<uint64_t>(mt, (uint64_t)num_sms() * 16), 256, 0,
-                              st>>>(Q, tcnt, (uint32_t)TT);
-    count_launch();
-  }
-  TRY(wk.get(&tchunk, ((uint64_t)nchunk + 1) * Q.tcs));
-  const uint32_t* nt_dev = P.tiles ? P.ntiles_dev : nullptr;
-  if (nchunk == 1)
-    k_tile_scan_chunk<true><<<1, Q.tcs, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk, plan);
-  else
-    k_tile_scan_chunk<false><<<nchunk, Q.tcs, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk, plan);
-  count_launch();
-  if (nchunk > 1) {
-    k_tile_scan_top<<<Q.tcs / 32, 1024, 0, st>>>(tchunk, nchunk, Q.tcs);
-    count_launch();
-    if (plan.kind != PLAN_NONE) {
-      k_plan_pass<<<1, 288, 0, st>>>(tchunk + (uint64_t)nchunk * Q.tcs, plan);
-      count_launch();
-    }
-  }
-  if (BATCH) {
-    k_plan_batch_pass<<<P.nsegs, 288, 0, st>>>(P.segs, tcnt, tchunk, Q.tcs, (uint32_t)mt, Q.chsh);
-    count_launch();
-  }
-  Q.tcnt = tcnt;
-  Q.tchunk = tchunk;
+  const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms() * per_sm, std::max<uint64_t>(mt, 1));
   Prof& pf = prof();
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (pf.on) {
@@ -965,7 +975,7 @@ static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt
     cudaEventCreate(&e1);
     cudaEventRecord(e0, st);
   }
-  kern<<<(unsigned)grid, TNT + 32, SM::bytes, st>>>(Q);
+  kern<<<(unsigned)grid, NT, SM::bytes, st>>>(Q);
   CK(cudaGetLastError());
   count_launch();
   if (pf.on) {
@@ -978,34 +988,94 @@ static wt_status launch_pass_t(const PassParams& P, uint64_t max_tiles, const wt
   return WT_OK;
 }
 
+// Nodes of a tree pass after the first, planned from its own tiles' counts.
+struct NodePlan {
+  const uint64_t* Ca = nullptr;  // starts of the nodes of level a
+  const uint64_t* toff = nullptr;
+  uint64_t nn = 0;
+  uint64_t* C = nullptr;  // starts of the nodes of level a + t
+};
+
+// One pass over at most mt tiles: every tile's digit counts, their prefix
+// sums across the tiles, what is planned from their totals, and the pass.
+template <bool BATCH, typename Launch>
+static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const PassPlan& plan,
+                          const NodePlan& np, cudaStream_t st, Launch&& launch) {
+  mt = std::max<uint64_t>(mt, 1);
+  PassParams Q = P;
+  Q.chsh = (uint32_t)chunk_shift(mt);
+  const uint32_t nchunk = (uint32_t)((mt + (1u << Q.chsh) - 1) >> Q.chsh);
+  Work wk{st, {}};
+  uint32_t* tcnt;
+  uint64_t* tchunk;
+  TRY(wk.get(&tcnt, mt * TC_STRIDE));
+  TRY(wk.get(&tchunk, ((uint64_t)nchunk + 1) * TC_STRIDE));
+  // the zeroing belongs to the counts of a first pass (sigma set), else to
+  // the pass
+  if (!P.sigma) Q.clear = nullptr;
+  TRY(launch_counts<BATCH>(Q, T, mt, tcnt, st));
+  const uint32_t* nt_dev = P.tiles ? P.ntiles_dev : nullptr;
+  if (nchunk == 1) {
+    k_tile_scan_chunk<true><<<1, 32, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, 1, tchunk, plan);
+    count_launch();
+  } else {
+    k_tile_scan_chunk<false><<<(nchunk * TC_STRIDE + 255) / 256, 256, 0, st>>>(
+        tcnt, nt_dev, P.ntiles, Q.chsh, nchunk, tchunk, plan);
+    k_tile_scan_top<<<1, 1024, 0, st>>>(tchunk, nchunk, plan);
+    count_launch(2);
+  }
+  if (BATCH) {
+    k_plan_batch_pass<<<(P.nsegs + 7) / 8, 256, 0, st>>>(P.segs, P.nsegs, tcnt, tchunk,
+                                                         (uint32_t)mt, nchunk, Q.chsh);
+    count_launch();
+  }
+  if (np.nn) {
+    k_plan_nodes<<<(unsigned)((np.nn + 7) / 8), 256, 0, st>>>(np.Ca, np.toff, np.nn, P.t, P.n_in,
+                                                              tcnt, tchunk, P.ntiles_dev, nchunk,
+                                                              Q.chsh, np.C);
+    count_launch();
+  }
+  CK(cudaGetLastError());
+  Q.tcnt = tcnt;
+  Q.tchunk = tchunk;
+  Q.clear = P.sigma ? nullptr : P.clear;
+  return launch(Q, mt);
+}
+
 // tile: symbols per tile (PT for the trees; 2048, 4096 or 8192 for the
-// wavelet matrix, the 8192-symbol tile with 512 worker threads)
-static wt_status launch_pass(const PassParams& P, bool wide, bool dig, uint64_t max_tiles,
-                             const wt_build_opts* o, cudaStream_t st,
-                             uint32_t* tcnt_pre = nullptr, const PassPlan& plan = PassPlan{},
-                             uint32_t tile = PT) {
-  if (dig) return wide ? launch_pass_t<uint32_t, true>(P, max_tiles, o, st, tcnt_pre, plan)
-                       : launch_pass_t<uint16_t, true>(P, max_tiles, o, st, tcnt_pre, plan);
-  if (tile == 2048)
-    return wide ? launch_pass_t<uint32_t, false, false, 2048, 256>(P, max_tiles, o, st, tcnt_pre, plan)
-                : launch_pass_t<uint16_t, false, false, 2048, 256>(P, max_tiles, o, st, tcnt_pre, plan);
-  if (tile == 8192)
-    return wide ? launch_pass_t<uint32_t, false, false, 8192, 512>(P, max_tiles, o, st, tcnt_pre, plan)
-                : launch_pass_t<uint16_t, false, false, 8192, 512>(P, max_tiles, o, st, tcnt_pre, plan);
-  return wide ? launch_pass_t<uint32_t, false>(P, max_tiles, o, st, tcnt_pre, plan)
-              : launch_pass_t<uint16_t, false>(P, max_tiles, o, st, tcnt_pre, plan);
+// wavelet matrix)
+template <int EW>
+static wt_status launch_pass_w(const PassParams& Q, bool dig, uint64_t mt, const wt_build_opts* o,
+                               cudaStream_t st, uint32_t tile) {
+  if (dig) return launch_pass_t<EW, true, false, PT / 32>(Q, mt, o, st);
+  if (tile == 2048) return launch_pass_t<EW, false, false, 64>(Q, mt, o, st);
+  if (tile == 8192) return launch_pass_t<EW, false, false, 256>(Q, mt, o, st);
+  return launch_pass_t<EW, false, false, PT / 32>(Q, mt, o, st);
+}
+static wt_status launch_pass(const PassParams& P, bool dig, uint64_t mt, const wt_build_opts* o,
+                             cudaStream_t st, const PassPlan& plan = PassPlan{},
+                             const NodePlan& np = NodePlan{}, uint32_t tile = PT) {
+  const int ew = P.in_w;
+  return run_pass<false>(P, mt, tile, plan, np, st, [&](const PassParams& Q, uint64_t m) {
+    if (ew == 1) return launch_pass_w<1>(Q, dig, m, o, st, tile);
+    if (ew == 2) return launch_pass_w<2>(Q, dig, m, o, st, tile);
+    return launch_pass_w<4>(Q, dig, m, o, st, tile);
+  });
 }
 
 // Batched wavelet matrices: one launch over the tiles of every sequence in
-// P.segs (P.ntiles tiles in total).
-wt_status launch_pass_batch(const PassParams& P, bool wide, const wt_build_opts* o,
-                            cudaStream_t st) {
-  return wide ? launch_pass_t<uint32_t, false, true>(P, P.ntiles, o, st)
-              : launch_pass_t<uint16_t, false, true>(P, P.ntiles, o, st);
+// P.segs (P.ntiles tiles in total), whose elements all have P.in_w bytes.
+wt_status launch_pass_batch(const PassParams& P, const wt_build_opts* o, cudaStream_t st) {
+  return run_pass<true>(P, P.ntiles, PT, PassPlan{}, NodePlan{}, st,
+                        [&](const PassParams& Q, uint64_t m) {
+                          if (Q.in_w == 1) return launch_pass_t<1, false, true, PT / 32>(Q, m, o, st);
+                          if (Q.in_w == 2) return launch_pass_t<2, false, true, PT / 32>(Q, m, o, st);
+                          return launch_pass_t<4, false, true, PT / 32>(Q, m, o, st);
+                        });
 }
 
 static int pick_tau(const wt_build_opts* o, int L, bool even, uint64_t n = 0) {
-  int tau = (o && o->tau) ? (int)o->tau : (even ? 8 : tuned_tau((uint32_t)L, n));
+  int tau = (o && o->tau) ? (int)o->tau : (even ? TAU_MAX : tuned_tau((uint32_t)L, n));
   if (tau < 1) tau = 1;
   if (tau > TAU_MAX) tau = TAU_MAX;
   if (even && (tau & 1)) tau = tau > 1 ? tau - 1 : 2;
@@ -1034,16 +1104,11 @@ static void set_uniform_levels(wt_struct* h, uint64_t elems_per_level) {
     h->level_off[l + 1] = h->level_off[l] + level_words(elems_per_level * h->bpe);
 }
 
-static PassParams base_params(wt_struct* h, Work& wk, uint32_t* tickets,
-                              const uint64_t* d_lvl_off, const uint64_t* d_lvl_len) {
+static PassParams base_params(wt_struct* h) {
   PassParams P;
   memset(&P, 0, sizeof(P));
   P.bits = h->d_bits;
-  P.lvl_off = d_lvl_off;
-  P.lvl_len = d_lvl_len;
-  P.ticket = tickets;
   P.err = h->d_err;
-  (void)wk;
   return P;
 }
 
@@ -1164,7 +1229,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   Work wk{st, {}};
   if (n == 0) return build_directories(h);
   // levels per pass, symbols per tile and CTAs per SM: the caller's, else
-  // the autotuner's for (L, ceil(log2 n)), else 8 / 4096 / the occupancy limit
+  // the autotuner's for (L, ceil(log2 n)), else 4 / 4096 / the occupancy limit
   const TuneConfig tc = tuned_config((uint32_t)L, n);
   wt_build_opts eo = o ? *o : wt_build_opts{};
   if (!eo.tau) eo.tau = (uint32_t)tc.tau;
@@ -1175,24 +1240,10 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   std::vector<PassGeom> ps = make_passes(L, tau, w);
   const int G = (int)ps.size();
   const uint32_t T = o->tile_symbols;
-  uint64_t *cls, *d_off, *d_len;
-  uint32_t* tickets;
+  uint64_t* cls;
   int ncls = 0;
   for (auto& p : ps) ncls += (2 << p.t) + p.t + 1;
   TRY(wk.get(&cls, ncls));
-  TRY(wk.get(&tickets, 32));
-  TRY(wk.get(&d_off, L + 1));
-  TRY(wk.get(&d_len, L));
-  TRY(upload(d_off, h->level_off.data(), (L + 1) * 8, st));
-  TRY(upload(d_len, h->level_len.data(), L * 8, st));
-  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
-  // the first pass's per-tile digit counts (with validation)
-  uint32_t* tcnt0;
-  const uint64_t ntiles0 = (n + T - 1) / T;
-  TRY(wk.get(&tcnt0, (size_t)ntiles0 * tc_stride(ps[0].t)));
-  // ... zeroing the first pass's levels on the way
-  TRY(launch_first_counts(d_seq, w, n, sigma, L, ps[0].t, T, h->d_err, tcnt0, h->d_bits,
-                          W * (uint64_t)ps[0].t / 2, st));
   // intermediate sequences
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
@@ -1207,7 +1258,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   const uint64_t ntiles = (n + T - 1) / T;
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
-    PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
+    PassParams P = base_params(h);
     P.in = in;
     P.in_w = pg.in_w;
     P.out = (g + 1 < G) ? seqbuf[g & 1] : nullptr;
@@ -1220,14 +1271,19 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     P.wm_cls = cls + coff;
     P.ntiles = (uint32_t)ntiles;
     P.n_in = n;
-    if (g + 1 < G) {
-      P.clear = (uint4*)(h->d_bits + W * (uint64_t)ps[g + 1].a);
-      P.clear_units = W * (uint64_t)ps[g + 1].t / 2;
+    // the first pass's counts check the symbols and zero the levels of the
+    // first two passes, every later pass zeroes the next pass's
+    const int z0 = g == 0 ? 0 : (g + 1 < G ? ps[g + 1].a : L);
+    const int z1 = g == 0 ? (G > 1 ? ps[1].a + ps[1].t : L) : (g + 1 < G ? z0 + ps[g + 1].t : L);
+    if (g == 0) P.sigma = sigma;
+    if (z1 > z0) {
+      P.clear = (uint4*)(h->d_bits + W * (uint64_t)z0);
+      P.clear_units = W * (uint64_t)(z1 - z0) / 2;
       P.clear_per = (P.clear_units + ntiles - 1) / ntiles;
     }
     // every pass is planned from its own tiles' digit counts
     const PassPlan plan{PLAN_WM, pg.a, pg.t, cls + coff, nullptr, h->d_zeros};
-    TRY(launch_pass(P, pg.wide, false, ntiles, o, st, g == 0 ? tcnt0 : nullptr, plan, T));
+    TRY(launch_pass(P, false, ntiles, o, st, plan, NodePlan{}, T));
     coff += (2 << pg.t) + pg.t + 1;
     in = P.out;
   }
@@ -1251,48 +1307,23 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   const int tau = pick_tau(o, L, multiary);
   std::vector<PassGeom> ps = make_passes(L, tau, w);
   const int G = (int)ps.size();
-  // a tree of one pass needs no symbol histogram: its nodes' starts follow
-  // from the tiles' digit counts, whose kernel also zeroes the level buffer
+  // a tree of one pass has its level buffer zeroed by the counting kernel
   const bool one = G == 1;
   TRY(alloc_outputs(h, h->level_off.back(), !one || n == 0));
   Work wk{st, {}};
   if (n == 0) return build_directories(h);
   const uint32_t T = PT;
-  const uint64_t V = (uint64_t)1 << L;
   const uint64_t ntiles0 = (n + T - 1) / T;
-  uint64_t *C, *d_off, *d_len;
-  uint32_t* tickets;
-  uint32_t* tcnt0 = nullptr;
-  TRY(wk.get(&C, V + 1));
-  TRY(wk.get(&tickets, 32));
-  TRY(wk.get(&d_off, h->levels + 1));
-  TRY(wk.get(&d_len, h->levels));
-  TRY(upload(d_off, h->level_off.data(), (h->levels + 1) * 8, st));
-  TRY(upload(d_len, h->level_len.data(), h->levels * 8, st));
-  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
-  uint64_t *hist, *scr = nullptr, *tcnt = nullptr, *toff = nullptr;
+  uint64_t *scr = nullptr, *tcnt = nullptr, *toff = nullptr;
   uint32_t* d_ntiles = nullptr;
   TileDesc* tiles = nullptr;
-  if (one) {
-    TRY(wk.get(&tcnt0, (size_t)ntiles0 * tc_stride(L)));
-    TRY(launch_first_counts(d_seq, w, n, sigma, L, L, T, h->d_err, tcnt0, h->d_bits,
-                            h->level_off.back() / 2, st));
-  } else {
+  if (!one) {
     const uint64_t max_nodes = (uint64_t)1 << ps.back().a;
-    TRY(wk.get(&hist, V));
-    TRY(wk.get(&scr, scan_scratch(std::max(V, max_nodes))));
+    TRY(wk.get(&scr, scan_scratch(max_nodes)));
     TRY(wk.get(&tcnt, max_nodes));
     TRY(wk.get(&toff, max_nodes + 1));
     TRY(wk.get(&tiles, ntiles0 + max_nodes + 1));
     TRY(wk.get(&d_ntiles, 1));
-    CK(cudaMemsetAsync(hist, 0, V * 8, st));
-    TRY(launch_hist_full(d_seq, w, n, sigma, hist, h->d_err, st));
-    TRY(scan_excl_u64(hist, C, V, scr, st));
-    if (!multiary) {
-      k_wt_zeros<<<L, 1024, 0, st>>>(C, L, h->d_zeros);
-      count_launch();
-      CK(cudaGetLastError());
-    }
   }
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
@@ -1302,26 +1333,37 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
       seqbuf[g & 1] = b;
     }
   }
+  // Every pass is planned from its own tiles' digit counts (no histogram of
+  // the symbols): C holds the starts of the nodes of level a, and the totals
+  // of each node's tiles give those of level a + t.
+  uint64_t* C = nullptr;
   const void* in = d_seq;
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
-    PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
+    PassParams P = base_params(h);
+    const uint64_t nn = (uint64_t)1 << pg.a;
+    uint64_t* Cn;
+    TRY(wk.get(&Cn, (nn << pg.t) + 1));
     uint64_t mt = ntiles0;
+    NodePlan np;
     if (g > 0) {
       // tiles inside the nodes of the pass's first level (the first pass has
       // one node, the whole sequence)
-      const uint64_t nn = (uint64_t)1 << pg.a;
-      const uint64_t stride = (uint64_t)1 << (L - pg.a);
-      k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(C, stride, nn, T, tcnt);
-      count_launch();
-      TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
       mt = ntiles0 + nn;
-      k_tiles_write<<<(unsigned)((mt + 255) / 256), 256, 0, st>>>(C, stride, nn, T, 0, toff, tiles,
-                                                                 d_ntiles, mt);
-      count_launch();
-      CK(cudaGetLastError());
+      TRY(launch_node_tiles(C, nn, T, 0, mt, tcnt, toff, scr, tiles, d_ntiles, st));
       P.tiles = tiles;
       P.ntiles_dev = d_ntiles;
+      np.Ca = C;
+      np.toff = toff;
+      np.nn = nn;
+      np.C = Cn;
+    } else {
+      P.sigma = sigma;
+      if (one) {
+        P.clear = (uint4*)h->d_bits;
+        P.clear_units = h->level_off.back() / 2;
+        P.clear_per = (P.clear_units + ntiles0 - 1) / ntiles0;
+      }
     }
     P.in = in;
     P.in_w = pg.in_w;
@@ -1333,13 +1375,18 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     P.rbits = pg.rbits;
     P.shape = SHAPE_WT;
     P.digits = multiary ? 1 : 0;
-    P.wt_C = C;
+    P.wt_C = Cn;
     P.ntiles = (uint32_t)ntiles0;
     P.n_in = n;
-    const PassPlan plan{one ? PLAN_WT : PLAN_NONE, 0, pg.t, nullptr, C,
-                        multiary ? nullptr : h->d_zeros};
-    TRY(launch_pass(P, pg.wide, multiary, mt, o, st, tcnt0, plan));
+    const PassPlan plan{g == 0 ? PLAN_WT : PLAN_NONE, 0, pg.t, nullptr, Cn, nullptr};
+    TRY(launch_pass(P, multiary, mt, o, st, plan, np));
     in = P.out;
+    C = Cn;
+  }
+  if (!multiary) {
+    k_wt_zeros<<<L, 1024, 0, st>>>(C, L, h->d_zeros);
+    count_launch();
+    CK(cudaGetLastError());
   }
   if (o && (o->flags & WT_FLAG_NO_DIRECTORY)) return WT_OK;
   return build_directories(h);
@@ -1348,10 +1395,44 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
 // ---------------------------------------------------------------------------
 // Huffman-shaped wavelet tree
 // ---------------------------------------------------------------------------
+// The symbols' left-aligned codewords, four bytes each, which every pass then
+// reads as elements (mapping the symbols in the first pass's counts and again
+// in the pass itself took two gathers per symbol through their slowest
+// loads).  in == out for 4-byte symbols; both 16-byte aligned.
+template <int W>
+__global__ void __launch_bounds__(256) k_map_codes(const void* in, uint64_t n, const uint32_t* map,
+                                                   uint32_t* out) {
+  const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, nv = n / 4;
+  for (uint64_t i = i0; i < nv; i += stride) {
+    uint32_t x[4];
+    if (W == 4) {
+      const uint4 q = ((const uint4*)in)[i];
+      x[0] = q.x;
+      x[1] = q.y;
+      x[2] = q.z;
+      x[3] = q.w;
+    } else if (W == 2) {
+      const uint2 q = ((const uint2*)in)[i];
+      x[0] = q.x & 0xffffu;
+      x[1] = q.x >> 16;
+      x[2] = q.y & 0xffffu;
+      x[3] = q.y >> 16;
+    } else {
+      const uint32_t q = ((const uint32_t*)in)[i];
+#pragma unroll
+      for (int k = 0; k < 4; k++) x[k] = (q >> (8 * k)) & 0xffu;
+    }
+    ((uint4*)out)[i] = make_uint4(map[x[0]], map[x[1]], map[x[2]], map[x[3]]);
+  }
+  for (uint64_t i = nv * 4 + i0; i < n; i += stride) out[i] = map[load_elem(in, W, i)];
+}
+
 uint32_t huffman_lengths(const uint64_t* hist, uint32_t sigma, uint32_t cap, uint8_t* len);
 void canonical_codes(const uint8_t* len, uint32_t sigma, uint32_t* code);
 
-wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
+// d_seq: the library's own copy of the sequence (16-byte aligned), overwritten
+wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
                      const wt_build_opts* o, wt_struct* h) {
   cudaStream_t st = h->stream;
   if (sigma > (1u << 24)) return WT_ERR_UNSUPPORTED;
@@ -1622,12 +1703,11 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
   const int G = (int)ps.size();
   const uint32_t T = PT;
   uint64_t *d_off, *d_len, *scr, *tcnt, *toff;
-  uint32_t *tickets, *d_ntiles;
+  uint32_t* d_ntiles;
   TileDesc* tiles;
   uint64_t max_nodes = 1;
   for (int l = 0; l < Lm; l++) max_nodes = std::max<uint64_t>(max_nodes, node_lvl[3 * l + 2]);
   const uint64_t max_tiles = (n + T - 1) / T + max_nodes + 1;
-  TRY(wk.get(&tickets, 32));
   TRY(wk.get(&d_off, Lm + 1));
   TRY(wk.get(&d_len, Lm));
   TRY(wk.get(&scr, scan_scratch(max_nodes)));
@@ -1637,7 +1717,6 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
   TRY(wk.get(&d_ntiles, 1));
   TRY(upload(d_off, h->level_off.data(), (Lm + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), Lm * 8, st));
-  CK(cudaMemsetAsync(tickets, 0, 32 * 4, st));
   void* seqbuf[2] = {nullptr, nullptr};
   for (int g = 0; g + 1 < G; g++) {
     if (!seqbuf[g & 1]) {
@@ -1646,11 +1725,23 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
       seqbuf[g & 1] = b;
     }
   }
-  const void* in = d_seq;
+  uint32_t* codes = (uint32_t*)d_seq;
+  if (w < 4) TRY(wk.get(&codes, n));
+  {
+    const unsigned grid = (unsigned)std::min<uint64_t>((n / 4 + 255) / 256 + 1, (uint64_t)num_sms() * 16);
+    if (w == 1) k_map_codes<1><<<grid, 256, 0, st>>>(d_seq, n, d_left, codes);
+    else if (w == 2) k_map_codes<2><<<grid, 256, 0, st>>>(d_seq, n, d_left, codes);
+    else k_map_codes<4><<<grid, 256, 0, st>>>(d_seq, n, d_left, codes);
+    count_launch();
+    CK(cudaGetLastError());
+  }
+  const void* in = codes;
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
     const uint64_t nn = node_lvl[3 * pg.a + 2];
-    PassParams P = base_params(h, wk, tickets + g, d_off, d_len);
+    PassParams P = base_params(h);
+    P.lvl_off = d_off;
+    P.lvl_len = d_len;
     P.n_in = h->level_len[pg.a];
     P.ntiles = (uint32_t)((P.n_in + T - 1) / T);
     uint64_t mt = P.ntiles;
@@ -1660,12 +1751,8 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
       if (nn) {
         const uint64_t* bnd = h->d_node + node_lvl[3 * pg.a];
         mt += nn;
-        k_tiles_count<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(bnd, 1, nn, T, tcnt);
-        count_launch();
-        TRY(scan_excl_u64(tcnt, toff, nn, scr, st));
-        k_tiles_write<<<(unsigned)((mt + 255) / 256), 256, 0, st>>>(
-            bnd, 1, nn, T, node_lvl[3 * pg.a + 1], toff, tiles, d_ntiles, mt);
-        count_launch();
+        TRY(launch_node_tiles(bnd, nn, T, node_lvl[3 * pg.a + 1], mt, tcnt, toff, scr, tiles,
+                              d_ntiles, st));
       } else {
         CK(cudaMemsetAsync(d_ntiles, 0, 4, st));
       }
@@ -1674,8 +1761,7 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
       P.ntiles_dev = d_ntiles;
     }
     P.in = in;
-    P.in_w = g == 0 ? w : pg.in_w;
-    P.code_map = g == 0 ? d_left : nullptr;
+    P.in_w = pg.in_w;
     P.out = (g + 1 < G) ? seqbuf[g & 1] : nullptr;
     P.out_w = pg.out_w;
     P.L = Lm;
@@ -1685,7 +1771,7 @@ wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const
     P.shape = SHAPE_HUFF;
     P.hf_node = h->d_node;
     P.hf_lvl = h->d_node_lvl;
-    TRY(launch_pass(P, pg.wide, false, mt, o, st));
+    TRY(launch_pass(P, false, mt, o, st));
     in = P.out;
   }
   if (o && (o->flags & WT_FLAG_NO_DIRECTORY)) return WT_OK;

@@ -1,48 +1,47 @@
-// k_pass.cuh -- the level-group partition kernel (one pass = t levels).
+// k_pass.cuh -- the level-group partition kernel (one pass = t <= 4 levels).
 //
-// One CTA processes one tile of T_a at a time (tiles taken from an atomic
-// ticket; no CTA waits on another).  A whole, aligned tile arrives by one
-// bulk copy (TMA) into shared memory, issued while the previous tile is still
-// being processed.  For a tile it computes, in shared memory:
-//   * the tile's bits of levels a..a+t-1, each in the order that level has
-//     inside the tile, by t stable 1-bit splits of the tile (Section 4.1: the
-//     descendants' sub-sequences are a stable integer sort on the next tau
-//     bits; Section 4.3: for the wavelet matrix the key is the reversed
-//     digit, i.e. the splits run from the level-a bit up).  Level j's bits
-//     are the ballot words of b_j in the order after j splits;
-//   * the element count of every class (node) of every level, folded from
-//     the tile's digit counts.
-// The tile's digit counts and those of all earlier tiles of its sequence or
-// node come from prefix sums, taken before the pass, of every tile's digit
-// counts: the domain decomposition of Section 4.2 with K = number of tiles
-// and per-node offsets by prefix sums across the K sub-problems.  The
-// tile's level bits leave as runs, one per (level, class); the runs' output
-// words form one list, written by lanes in windows of 32 consecutive
-// entries.  Words copied whole are stored; the "boundary" words that several
-// tiles or nodes share (Section 4.2) are merged with atomicOr into the level
-// buffer, which is zero before the pass (in a wavelet-matrix build each tile
-// zeroes its share of the next pass's levels).  Finally the tile scatters its
-// elements, narrowed to the bits still needed, to T_{a+t}: the stable
-// partition on the t-bit digit (big nodes, Section 3).
+// One CTA processes one tile of T_a at a time; no CTA waits on another.  A
+// thread holds 32 consecutive elements of the tile as bit planes (bitplane.cuh),
+// in which t - 1 stable 1-bit splits (Section 4.1: the descendants'
+// sub-sequences are a stable integer sort on the next tau bits; Section 4.3:
+// for the wavelet matrix the key is the reversed digit, i.e. the splits run
+// from the level-a bit up) give its bits of levels a .. a+t-1, each in the
+// order that level has inside the 32 elements, with every class's bits
+// together.  The counts of the 2^t keys in the earlier threads (a prefix sum
+// over the tile, two 16-bit counts a word) place those pieces in the tile's
+// runs, one per (level, class), which are assembled in shared memory at the
+// bit alignment they have in the output and leave as whole words; words that
+// several tiles or nodes share (the "boundary" words of Section 4.2) are
+// merged with atomicOr into the level buffer, which is zero before the pass
+// (in a wavelet-matrix build each tile zeroes its share of the next pass's
+// levels).  The same counts give every element's place in the tile's stable
+// order by key: each thread walks its elements once with a pointer per key,
+// and the runs of T_{a+t}, again assembled at their output alignment, leave in
+// 16-byte stores (big nodes, Section 3), narrowed to the bits still needed.
+//
+// The digit counts of all earlier tiles of a tile's sequence or node come from
+// prefix sums, taken before the pass, of every tile's digit counts: the
+// domain decomposition of Section 4.2 with K = number of tiles and per-node
+// offsets by prefix sums across the K sub-problems.
+//
+// What bounds it: instructions, most of them on the integer logic pipe (65% of
+// it used, 2.45 instructions per cycle and SM; DRAM below 15%).  An earlier
+// form moved the elements once per level through shared memory (a ballot, a
+// rank and a store per 32 elements and level): 231 and 198 warp instructions
+// per 32 elements for its two passes of 8 levels, 14.3 ms for the 2^30 16-bit
+// symbols of 16 levels; the four passes here take 69 (46 the last) and 10.8 ms.
 #pragma once
 #include <type_traits>
 
+#include "bitplane.cuh"
 #include "wt_internal.cuh"
 
 namespace wtk {
-
-__device__ __forceinline__ int cls_idx(int j, int k) { return (1 << j) - 1 + k; }
 
 __device__ __forceinline__ uint32_t load_elem(const void* p, int w, uint64_t i) {
   if (w == 1) return ((const uint8_t*)p)[i];
   if (w == 2) return ((const uint16_t*)p)[i];
   return ((const uint32_t*)p)[i];
-}
-
-__device__ __forceinline__ void store_elem(void* p, int w, uint64_t i, uint32_t v) {
-  if (w == 1) ((uint8_t*)p)[i] = (uint8_t)v;
-  else if (w == 2) ((uint16_t*)p)[i] = (uint16_t)v;
-  else ((uint32_t*)p)[i] = v;
 }
 
 // Batched builds: tile ti's sequence, the last segment with tile0 <= ti.
@@ -69,8 +68,6 @@ __device__ __forceinline__ void fill_seg(PassParams& D, const PassParams& P0, ui
   D.t = d.t;
   D.rbits = d.rbits;
   D.bits = d.bits;
-  D.lvl_off = d.lvl_off;
-  D.lvl_len = d.lvl_len;
   D.wm_cls = d.wm_cls;
   D.err = d.err;
   D.n_in = d.n;
@@ -78,43 +75,74 @@ __device__ __forceinline__ void fill_seg(PassParams& D, const PassParams& P0, ui
   D.sigma = d.sigma;
 }
 
-// Global class range [cs, ce) of level a+j, class k (k = the tile-local key
-// whose bit i is digit bit i, i.e. the LSD order of the splits), for a tile
-// inside node `node` of level a.  `dead` marks Huffman prefixes that are not
-// internal nodes at that level (their elements have left the tree).
-__device__ __forceinline__ void class_range(const PassParams& P, int j, uint32_t k,
-                                            uint32_t node, uint64_t& cs, uint64_t& ce,
-                                            bool& dead) {
-  dead = false;
-  if (P.shape == SHAPE_WM) {
-    const uint64_t* z = P.wm_cls + ((1u << j) - 1u + (uint32_t)j);
-    cs = z[k];
-    ce = z[k + 1];
-    return;
+// A tile: where its elements are and which part of the pass it belongs to.
+struct TileInfo {
+  const unsigned char* src;
+  uint64_t ts;          // its first element's index
+  int cnt;
+  uint32_t node, seg0;  // node of level a; first tile of its sequence or node
+};
+
+__device__ __forceinline__ TileInfo tile_info(const PassParams& P, uint32_t ti, uint32_t tile) {
+  TileInfo I;
+  if (P.tiles) {
+    const TileDesc d = P.tiles[ti];
+    I.ts = d.start;
+    I.cnt = (int)d.count;
+    I.node = d.node;
+    I.seg0 = d.seg0;
+  } else {
+    I.ts = (uint64_t)(ti - P.tile0) * tile;
+    const uint64_t rem = P.n_in - I.ts;
+    I.cnt = (int)(rem < tile ? rem : tile);
+    I.node = 0;
+    I.seg0 = P.tile0;
   }
-  const int l = P.a + j;
-  const uint64_t q = ((uint64_t)node << j) | rev_bits(k, j);
-  if (P.shape == SHAPE_WT) {
-    const int sh = P.L - l;
-    cs = P.wt_C[q << sh];
-    ce = P.wt_C[(q + 1) << sh];
-    return;
-  }
-  const uint64_t off = P.hf_lvl[3 * l], first = P.hf_lvl[3 * l + 1], num = P.hf_lvl[3 * l + 2];
-  if (q < first || q >= first + num) {
-    dead = true;
-    cs = ce = 0;
-    return;
-  }
-  cs = P.hf_node[off + (q - first)];
-  ce = P.hf_node[off + (q - first) + 1];
+  I.src = (const unsigned char*)P.in + I.ts * (uint64_t)P.in_w;
+  return I;
 }
 
-// store the low sizeof(E) bytes of v at shared-memory byte address a
-template <typename E>
+// Where the start of class k of level a+j stands (k = the tile-local key whose
+// bit i is digit bit i, i.e. the LSD order of the splits), for a tile inside
+// node `node` of level a; nullptr for Huffman prefixes that are not internal
+// nodes at that level (their elements have left the tree).  hf: the pass's
+// rows of hf_lvl.
+__device__ __forceinline__ const uint64_t* class_start(const PassParams& P, int j, uint32_t k,
+                                                       uint32_t node, const uint64_t* hf) {
+  if (P.shape == SHAPE_WM) return P.wm_cls + ((1u << j) - 1u + (uint32_t)j) + k;
+  const uint64_t q = ((uint64_t)node << j) | rev_bits(k, j);
+  if (P.shape == SHAPE_WT) return P.wt_C + (q << (P.t - j));  // wt_C: node starts of level a + t
+  const uint64_t off = hf[3 * j], first = hf[3 * j + 1], num = hf[3 * j + 2];
+  return q < first || q >= first + num ? nullptr : P.hf_node + off + (q - first);
+}
+
+// 16-byte asynchronous copies into shared memory (each thread's own, complete
+// for it after cp_async_wait and for the block after the next barrier)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+template <int B>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {  // 4 or 8 bytes
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(B) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ uint32_t ld_shared_u16(uint32_t a) {
+  unsigned short v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+  return v;
+}
+template <int W>
 __device__ __forceinline__ void st_shared(uint32_t a, uint32_t v) {
-  if (sizeof(E) == 2) asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v));
-  else asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v));
+  if (W == 1) asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+  else if (W == 2) asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+  else asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// set the bits v at shared-memory word a (no access when there are none)
+__device__ __forceinline__ void or_shared(uint32_t a, uint32_t v) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.or.b32 [%0], %1;\n\t}" ::"r"(a), "r"(v)
+               : "memory");
 }
 
 __device__ __forceinline__ uint64_t spread32(uint32_t v) {
@@ -127,572 +155,534 @@ __device__ __forceinline__ uint64_t spread32(uint32_t v) {
   return x;
 }
 
-template <int TW>
-__device__ __forceinline__ uint32_t get32(const uint32_t* pl, int e) {
-  const int w = e >> 5, o = e & 31;
-  const uint32_t lo = (w >= 0 && w < TW) ? pl[w] : 0u;
-  const uint32_t hi = (w + 1 >= 0 && w + 1 < TW) ? pl[w + 1] : 0u;
-  return o ? __funnelshift_r(lo, hi, o) : lo;
-}
-
-// the same over the ballot halves of a level's row words
-template <int TW>
-__device__ __forceinline__ uint32_t get32q(const uint2* pl, int e) {
-  const int w = e >> 5, o = e & 31;
-  const uint32_t lo = (w >= 0 && w < TW) ? pl[w].x : 0u;
-  const uint32_t hi = (w + 1 >= 0 && w + 1 < TW) ? pl[w + 1].x : 0u;
-  return o ? __funnelshift_r(lo, hi, o) : lo;
-}
-
-template <typename E, int T, int NT, bool DIG>
+// Shared memory of one CTA: the move's pointers, 1 KB a warp (at its own
+// alignment, so that addresses are put together by OR); the tile as loaded, a
+// row per thread padded by 16 bytes (eight lanes' 16-byte reads of their rows
+// then fall on all banks); the elements in key order, each key's run at its
+// output's 16-byte alignment (and before that the prefix sums' scratch); the
+// level bits, each run at its output's 64-bit alignment.
+template <int EW, int NT>
 struct PassSmem {
-  static constexpr int TW = T / 32;
-  static constexpr size_t off_buf = 0;                                        // 2 x T elements
-  static constexpr size_t off_lbits = off_buf + 2 * (size_t)T * sizeof(E);   // row words per level
-  static constexpr int TWS = TW + 2;  // row words per level, two zero words after them
-  static constexpr size_t off_pb1 = off_lbits + (size_t)TAU_MAX * TWS * 8;   // second digit bits
-  static constexpr size_t off_ccnt = off_pb1 + (DIG ? (size_t)(TAU_MAX / 2) * TW * 4 : 0);
-  static constexpr size_t off_cstart = off_ccnt + (size_t)NCLS * 4;
-  static constexpr size_t off_excnt = off_cstart + (size_t)NCLS * 4;  // 8-aligned
-  static constexpr size_t off_clscs = off_excnt + (size_t)NCLS * 8;
-  static constexpr size_t bytes = off_clscs + (size_t)(1 << TAU_MAX) * 8;
+  static constexpr int T = 32 * NT, RS = 32 * EW + 16;
+  static constexpr int KEYS = 1 << TAU_MAX, RUNS = KEYS - 1;
+  static constexpr int SCRW = 8 * 32 + 3 * 8;                   // scratch words per warp
+  static constexpr int AREA = TAU_MAX * T / 64 + 2 * RUNS + 2;  // 64-bit words
+  static constexpr int SRT = T * EW + 32 * KEYS > NT / 32 * SCRW * 4 ? T * EW + 32 * KEYS : NT / 32 * SCRW * 4;
+  static constexpr size_t off_ptr = 0;
+  static constexpr size_t off_in = off_ptr + (size_t)(NT / 32) * 1024;
+  static constexpr size_t off_srt = off_in + (size_t)NT * RS;
+  static constexpr size_t off_area = off_srt + (size_t)SRT;
+  static constexpr size_t bytes = off_area + (size_t)AREA * 8;
 };
 
-// resident CTAs per SM the register budget is sized for: 5 for 16-bit
-// elements (40 registers a thread at 288 threads a CTA; batched passes keep
-// their per-sequence state in shared memory and spill 12 bytes at 40, which
-// costs less than a fifth of the CTAs would); 4 for 32-bit elements, whose
-// buffers let only 4 CTAs share an SM's shared memory (56 registers); 2 for
-// the 8192-symbol tile (544 threads a CTA).  And whether a split keeps its
-// elements in registers between its two phases (else it reads them from
-// shared memory again).
-#ifndef WT_PASS_MIN_CTAS
-#define WT_PASS_MIN_CTAS 5
+// CTAs per SM the register budget is sized for, at 128 threads
+#ifndef WT_PASS_CTAS
+#define WT_PASS_CTAS 7
 #endif
-template <typename E, int T, bool BATCH>
+template <int EW, int NT>
 struct PassCtas {
-  static constexpr int value = T >= 8192 ? 2 : sizeof(E) == 4 ? 4 : WT_PASS_MIN_CTAS;
+  static constexpr int at128 = EW == 4 ? 5 : WT_PASS_CTAS;
+  static constexpr int value = NT == 64 ? 2 * at128 : (NT == 128 ? at128 : at128 / 2);
 };
-#ifndef WT_PASS_KEEP_X
-#define WT_PASS_KEEP_X 1
-#endif
 
-template <typename E, int T, int NT, bool DIG, bool BATCH>
-__global__ void __launch_bounds__(NT + 32, PassCtas<E, T, BATCH>::value) k_pass(const __grid_constant__ PassParams P0) {
-  __shared__ PassParams s_P;
-  const PassParams& P = BATCH ? s_P : P0;
-  constexpr int W = NT / 32, PW = T / W, EPW = PW / 32, TW = T / 32, NB = NT + 32, CW = W;
-  constexpr int TWS = TW + 2;
-  static_assert(EPW >= 1 && EPW <= 32, "iterations per warp must fit a warp");
-  static_assert(T % 64 == 0 && NT >= (1 << TAU_MAX), "tile geometry");
-  using SM = PassSmem<E, T, NT, DIG>;
-  extern __shared__ __align__(16) unsigned char smem[];
-  E* const buf0 = (E*)(smem + SM::off_buf);
-  E* const buf1 = buf0 + T;
-  // per level and row: (ballot of the level's bit = the level's bits in its
-  // order, ones before the row inside its warp)
-  uint2* const rowq = (uint2*)(smem + SM::off_lbits);
-  uint32_t* const pb1 = (uint32_t*)(smem + SM::off_pb1);      // b_j+1 plane of pair rounds
-  uint32_t* const ccnt = (uint32_t*)(smem + SM::off_ccnt);
-  uint32_t* const cstart = (uint32_t*)(smem + SM::off_cstart);
-  uint64_t* const ex_cnt = (uint64_t*)(smem + SM::off_excnt);
-  uint64_t* const cls_cs = (uint64_t*)(smem + SM::off_clscs);
-  uint64_t* const sbase = cls_cs;  // reused by the scatter
+// One run of a tile on its way out: units (words or chunks) first .. last - 1
+// of its area are the run's alone; unit i goes to address base + i * size
+// (base == 0: nowhere).
+struct __align__(16) Run {
+  uint64_t base;
+  uint32_t first, last;
+};
 
-  __shared__ uint32_t s_tile;
-  // the buffer holding this tile's elements as loaded (0: the first of the
-  // two) and whether they came by a bulk copy that completes on s_bar; the
-  // same for the next tile (set during this one)
-  __shared__ int s_ib, s_stg, s_nib, s_nstg, s_stall;
-  __shared__ uint32_t s_phase, s_nxt;           // s_bar's open phase; the next tile
-  __shared__ const unsigned char* s_nsrc;       // its elements if copied in bulk
-  __shared__ int s_niw;                         // and their width
-  __shared__ __align__(8) uint64_t s_bar;
-  __shared__ int s_ones[W];
-  __shared__ int s_scan[W + 1];
-  __shared__ int wst[1 << TAU_MAX];
-  __shared__ uint32_t s_dead[(1 << TAU_MAX) / 32];
-  __shared__ int s_bad;
-  __shared__ int s_oob;
-  // the writer's flattened list of run words, in windows of 32 entries
-  constexpr int WMAX = TAU_MAX * (2 * T / 64) + 2 * (1 << TAU_MAX);
-  constexpr int WWIN = (WMAX + 31) / 32;
-  __shared__ uint8_t s_g0[1 << TAU_MAX];
-  __shared__ uint32_t s_wstart[WWIN];
-  __shared__ uint8_t s_runid[WWIN * 32];
-  __shared__ uint8_t s_winrun[WWIN];
+template <typename E, bool DIG, bool BATCH, int NT>
+__global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(const __grid_constant__ PassParams P0) {
+  constexpr int EW = (int)sizeof(E), T = 32 * NT, W = NT / 32;
+  using SM = PassSmem<EW, NT>;
+  constexpr int RS = SM::RS, KEYS = SM::KEYS;
+  static_assert(TAU_MAX == 4, "planes, keys and runs are laid out for four levels");
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* const s_in = smem + SM::off_in;
+  unsigned char* const s_srt = smem + SM::off_srt;
+  uint64_t* const s_area = (uint64_t*)(smem + SM::off_area);
+
+  __shared__ PassParams s_P[BATCH ? 2 : 1];
+  __shared__ TileInfo s_info[2];
+  __shared__ __align__(16) uint32_t s_wtot[W][8];  // the warps' key counts, two a word
+  // the next tile's table rows (its own, the next tile's and its first
+  // tile's, within their chunks; the chunks' and the next chunk's) and class
+  // starts, brought in with its elements
+  __shared__ uint32_t s_ta[KEYS], s_tn[KEYS], s_tb[KEYS];
+  __shared__ uint64_t s_ca[KEYS], s_cn[KEYS], s_cb[KEYS];
+  __shared__ uint64_t s_cs[2 * KEYS - 1];
+  __shared__ uint64_t s_hf[3 * (TAU_MAX + 1)], s_lo[TAU_MAX], s_ll[TAU_MAX];  // Huffman: rows of the level tables
+  __shared__ uint32_t s_own[KEYS];  // the tile's key counts by the tables
+  __shared__ bool s_over[2];        // a run past its level's or the sequence's end
+  // the runs of level bits that are not empty, and those of the next
+  // sequence, in order: first word of the area (16-byte chunk), and the words
+  // (chunks) the run holds whole with the address word (chunk) 0 would have
+  __shared__ uint32_t s_rs[2][KEYS];
+  __shared__ Run s_run[2][KEYS];
+  __shared__ uint32_t s_n[2], s_nr;  // their words and chunks; runs of the next sequence
+  __shared__ uint32_t s_edge[KEYS];  // offset in the first chunk, bytes << 8
+  __shared__ __align__(16) uint32_t s_ab[KEYS];  // a run's first bit, from shared memory's start
+  __shared__ __align__(16) uint32_t s_sb[8];  // where a key's first element goes in s_srt, two keys a word
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* const ptr = (uint32_t*)(smem + SM::off_ptr) + warp * 256;
+  uint32_t* const scr = (uint32_t*)s_srt + warp * SM::SCRW;
   const int bpe = DIG ? 2 : 1;
   const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
-  if (BATCH && tid == 0) s_P = P0;
-  const uint32_t lt = lanemask_lt();
-  const int wbase = warp * PW;
-  // the two words after each level's rows stay zero (the writer reads past
-  // a level's last row without a bounds check)
-  for (int i = tid; i < 2 * TAU_MAX; i += NB) rowq[(i >> 1) * TWS + TW + (i & 1)] = make_uint2(0u, 0u);
 
-  auto bar_workers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
-  // block-wide exclusive scan of one int per thread
-  auto block_scan = [&](int v, int& total) -> int {
-    int si = v;
+  // tile ti's parameters into buffer b (one thread)
+  auto set_info = [&](uint32_t ti, int b) {
+    if (BATCH) fill_seg(s_P[b], P0, ti);
+    s_info[b] = tile_info(BATCH ? s_P[b] : P0, ti, T);
+  };
+  // its elements into s_in (all threads)
+  auto load_tile = [&](int b) {
+    const PassParams& P = BATCH ? s_P[b] : P0;
+    const TileInfo I = s_info[b];
+    if (I.cnt == T && ((uintptr_t)I.src & 15) == 0) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(FULL, si, o);
-      if (lane >= o) si += y;
-    }
-    if (lane == 31) s_scan[warp] = si;
-    __syncthreads();
-    const int x = lane <= W ? s_scan[lane] : 0;
-    const int base = __reduce_add_sync(FULL, lane < warp ? x : 0);
-    total = __reduce_add_sync(FULL, x);
-    __syncthreads();
-    return base + si - v;
-  };
-
-  // Tile loads by the bulk-copy unit (TMA): tile ti+1's elements are copied
-  // into the buffer tile ti no longer reads while tile ti is still being
-  // processed, so a tile's load latency hides behind the previous tile.
-  // Used for whole tiles at 16-byte aligned addresses whose elements have the
-  // buffer's width (copied as they are) or are bytes in 16-bit buffers
-  // (copied into the buffer's upper half, where the first split reads them
-  // as bytes); other tiles are loaded by the threads.
-  // tile nx's elements if they can come by one bulk copy, else nullptr
-  // (and its element width into iw)
-  auto stage_src = [&](uint32_t nx, int& iw) -> const unsigned char* {
-    if (nx >= ntiles || P0.code_map) return nullptr;
-    const void* in = P0.in;
-    iw = P0.in_w;
-    uint64_t s0;
-    if (BATCH) {
-      const SegDesc& sd = seg_of(P0, nx);
-      in = sd.in;
-      iw = sd.in_w;
-      s0 = (uint64_t)(nx - sd.tile0) * T;
-      if (s0 + T > sd.n) return nullptr;
-    } else if (P0.tiles) {
-      const TileDesc d = P0.tiles[nx];
-      if (d.count != (uint32_t)T) return nullptr;
-      s0 = d.start;
-    } else {
-      s0 = (uint64_t)(nx - P0.tile0) * T;
-      if (s0 + T > P0.n_in) return nullptr;
-    }
-    if (!(iw == (int)sizeof(E) || (iw == 1 && sizeof(E) == 2))) return nullptr;
-    const unsigned char* src = (const unsigned char*)in + s0 * (uint64_t)iw;
-    return ((uintptr_t)src & 15) ? nullptr : src;
-  };
-  // copy them into buffer X (bytes narrower than E into its upper part)
-  auto stage = [&](const unsigned char* src, int iw, E* X) {
-    bulk_load((unsigned char*)X + (size_t)T * (sizeof(E) - iw), src, (uint32_t)(T * iw), &s_bar);
-  };
-  if (tid == 0) {
-    s_stall = 0;
-    s_nib = 0;
-    s_phase = 0;
-    const uint32_t nx = atomicAdd(P0.ticket, 1u);
-    s_nxt = nx;
-    mbar_init1(&s_bar);
-    int iw;
-    const unsigned char* src = stage_src(nx, iw);
-    if (src) stage(src, iw, buf0);
-    s_nstg = src != nullptr;
-  }
-
-  for (;;) {
-    if (tid == 0) {
-      const uint32_t nx = s_nxt;
-      s_tile = nx;
-      s_ib = s_nib;
-      s_stg = s_nstg;
-      if (BATCH && nx < ntiles) fill_seg(s_P, P0, nx);
-    }
-    __syncthreads();
-    const uint32_t ti = s_tile;
-    if (ti >= ntiles) break;
-    // the tile's elements as loaded (k = 0) and the other buffer (k = 1),
-    // both from one register: the byte offset of the first of them
-    const uint32_t boff = s_ib ? (uint32_t)(T * sizeof(E)) : 0u;
-    auto buf = [&](int k) -> E* {
-      return (E*)((unsigned char*)buf0 + (boff ^ (k ? (uint32_t)(T * sizeof(E)) : 0u)));
-    };
-    // this tile's share of the zeroing of a later pass's levels (stores that
-    // use the DRAM bandwidth the tile's compute leaves idle)
-    if (!BATCH && P0.clear) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid, NB);
-    const int t = P.t;
-    const int ntl = (1 << t) - 1;
-    uint64_t ts;
-    int cnt;
-    uint32_t node, seg0;  // seg0: first tile of the tile's sequence or node
-    if (P.tiles) {
-      const TileDesc d = P.tiles[ti];
-      ts = d.start;
-      cnt = (int)d.count;
-      node = d.node;
-      seg0 = d.seg0;
-    } else {
-      ts = (uint64_t)(ti - P.tile0) * T;
-      const uint64_t rem = P.n_in - ts;
-      cnt = (int)(rem < (uint64_t)T ? rem : (uint64_t)T);
-      node = 0;
-      seg0 = P.tile0;
-    }
-    const bool full = cnt == T;
-
-    // ---- 1. load the tile (its digit counts were taken before the pass) --
-    if (s_stg) {
-      if (!mbar_wait(&s_bar, s_phase)) s_stall = 1;
-    } else {
-      E* const bufA = buf(0);
-      if (P.code_map) {
-        for (int i = tid; i < cnt; i += NB) bufA[i] = (E)P.code_map[load_elem(P.in, P.in_w, ts + i)];
-      } else if (P.in_w == 2 && sizeof(E) == 2 && full &&
-                 (((uintptr_t)P.in + 2 * ts) & 15) == 0) {
-        const uint4* src = (const uint4*)((const uint16_t*)P.in + ts);
-        uint4* dst = (uint4*)bufA;
-        for (int i = tid; i < T / 8; i += NB) dst[i] = __ldcs(src + i);
-      } else if (P.in_w == 1 && sizeof(E) == 2 && full && (((uintptr_t)P.in + ts) & 15) == 0) {
-        const uint4* src = (const uint4*)((const uint8_t*)P.in + ts);
-        for (int i = tid; i < T / 16; i += NB) {
-          const uint4 q = __ldcs(src + i);
-          const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-          uint4* d = (uint4*)(bufA + 16 * i);
-          uint32_t o[8];
-#pragma unroll
-          for (int k = 0; k < 4; k++) {
-            o[2 * k] = __byte_perm(w4[k], 0, 0x4140);
-            o[2 * k + 1] = __byte_perm(w4[k], 0, 0x4342);
-          }
-          d[0] = make_uint4(o[0], o[1], o[2], o[3]);
-          d[1] = make_uint4(o[4], o[5], o[6], o[7]);
-        }
-      } else {
-        for (int i = tid; i < cnt; i += NB) bufA[i] = (E)load_elem(P.in, P.in_w, ts + i);
+      for (int k = 0; k < 2 * EW; k++) {
+        const int i = tid + k * NT;
+        cp_async16(s_in + 16 * i + 16 * (i / (2 * EW)), I.src + 16 * i);
       }
-    }
-    __syncthreads();
-    if (s_stall) {  // uniform: a bulk copy that never completed
-      if (tid == 0) atomicOr(P.err, ERR_STALL);
       return;
     }
+    // else 4-byte words put together from the aligned words around them, as
+    // far as those lie inside the sequence, and single elements
+    int from = 0;
+    const unsigned char* const base = (const unsigned char*)((uintptr_t)I.src & ~(uintptr_t)3);
+    const uint32_t mis = (uint32_t)((uintptr_t)I.src & 3) * 8;
+    if (base >= (const unsigned char*)P.in) {
+      const uint64_t left = (uint64_t)((const unsigned char*)P.in + P.n_in * (uint64_t)EW - base) / 4;
+      const int have = left > (uint64_t)(T * EW) ? T * EW : (int)left - (mis ? 1 : 0);
+      const int nwords = min((I.cnt * EW + 3) / 4, have);
+      const uint32_t* src = (const uint32_t*)base;
+      for (int j = tid; j < nwords; j += NT) {
+        const uint32_t lo = __ldcs(src + j), hi = mis ? __ldcs(src + j + 1) : 0u;
+        *(uint32_t*)(s_in + 4 * j + 16 * (j / (8 * EW))) = __funnelshift_r(lo, hi, mis);
+      }
+      from = max(nwords, 0) * 4 / EW;
+    }
+    for (int i = from + tid; i < I.cnt; i += NT) {
+      ((E*)(s_in + (i >> 5) * RS))[i & 31] = ((const E*)I.src)[i];
+    }
+  };
 
-    int cur;
-    if (warp == CW) {
-      // ---- 3 (control warp). class counts of every level from the tile's
-      //      digit counts; counts of all earlier tiles from their prefix
-      //      sums; exclusive counts of every level -------------------------
-      // the CTA's next tile, taken now so that its latency hides behind
-      // this tile's work, and where its elements are
-      const uint32_t nx = lane == 0 ? atomicAdd(P0.ticket, 1u) : 0u;
-      const int nd = 1 << t;
-      // this tile's count of every digit value in the earlier tiles of its
-      // sequence or node: the prefix sums of the per-tile counts (Section
-      // 4.2, prefix sums across the K sub-problems), taken before the pass
-      // (the tables are exclusive inside chunks of tiles, with the
-      // chunks' exclusive prefixes and their total after the last chunk: the
-      // tile's own digit counts are the difference to the next tile, or to
-      // the next chunk for the last tile of a chunk)
-      uint64_t* const exd = ex_cnt + cls_idx(t, 0);  // exclusive digit counts
-      {
-        const uint32_t ch = ti >> P0.chsh;
-        const uint32_t S = P0.tcs;
-        const uint64_t* ca = P0.tchunk + (uint64_t)ch * S;
-        const uint64_t* cb = P0.tchunk + (uint64_t)(seg0 >> P0.chsh) * S;
-        const uint32_t* ta = P0.tcnt + (uint64_t)ti * S;
-        const uint32_t* tb = P0.tcnt + (uint64_t)seg0 * S;
-        const bool last = ((ti + 1) >> P0.chsh) != ch || ti + 1 >= ntiles;
-        uint32_t sum = 0;
-        for (int r = lane; r < nd; r += 32) {
-          const uint32_t a = ta[r];
-          const uint32_t c = last ? (uint32_t)(ca[S + r] - ca[r]) - a : ta[S + r] - a;
-          exd[r] = (ca[r] + a) - (cb[r] + tb[r]);
-          ccnt[cls_idx(t, r)] = c;
-          sum += c;
-        }
-        // a table that disagrees with the tile would misplace its bits: flag
-        // it and leave the tile's outputs alone
-        const bool bad = __reduce_add_sync(FULL, sum) != (uint32_t)cnt;
-        if (lane == 0) {
-          s_bad = bad;
-          if (bad) atomicOr(P.err, ERR_INTERNAL);
-        }
+  // the control data of the tile ti whose parameters are in buffer b (warp 0)
+  auto load_ctl = [&](uint32_t ti, int b) {
+    const PassParams& P = BATCH ? s_P[b] : P0;
+    const TileInfo I = s_info[b];
+    const int nd = 1 << P.t;
+    if (lane < nd) {
+      const uint64_t* ca = P0.tchunk + (uint64_t)(ti >> P0.chsh) * TC_STRIDE + lane;
+      const uint32_t* ta = P0.tcnt + (uint64_t)ti * TC_STRIDE + lane;
+      cp_async<8>(s_ca + lane, ca);
+      cp_async<8>(s_cn + lane, ca + TC_STRIDE);
+      cp_async<8>(s_cb + lane, P0.tchunk + (uint64_t)(I.seg0 >> P0.chsh) * TC_STRIDE + lane);
+      cp_async<4>(s_ta + lane, ta);
+      cp_async<4>(s_tn + lane, ti + 1 < ntiles ? ta + TC_STRIDE : ta);
+      cp_async<4>(s_tb + lane, P0.tcnt + (uint64_t)I.seg0 * TC_STRIDE + lane);
+    }
+    // lanes 0-14 the classes of levels a .. a+t-1, lanes 16-31 of level a+t
+    if (lane < nd - 1 || (lane >= 16 && lane - 16 < nd && P.out != nullptr)) {
+      const int ci = lane < 16 ? lane : nd - 1 + lane - 16;
+      const int j = 31 - __clz(ci + 1);
+      const uint64_t* at = class_start(P, j, (uint32_t)(ci + 1 - (1 << j)), I.node, s_hf);
+      if (at) cp_async<8>(s_cs + ci, at);
+      else s_cs[ci] = ~0ull;
+    }
+  };
+
+  for (int i = tid; i < SM::AREA; i += NT) s_area[i] = 0ull;
+  if (BATCH && tid < 2) s_P[tid] = P0;
+  if (P0.shape == SHAPE_HUFF) {
+    if (tid < 3 * (TAU_MAX + 1))
+      s_hf[tid] = P0.a + tid / 3 < P0.L ? P0.hf_lvl[3 * P0.a + tid] : 0ull;
+    if (tid < P0.t) {
+      s_lo[tid] = P0.lvl_off[P0.a + tid];
+      s_ll[tid] = P0.lvl_len[P0.a + tid];
+    }
+  }
+  __syncthreads();
+  uint32_t ti = blockIdx.x;
+  int cur = 0;
+  if (ti < ntiles) {
+    if (tid == 0) set_info(ti, 0);
+    __syncthreads();
+    load_tile(0);
+    if (warp == 0) load_ctl(ti, 0);
+  }
+  for (; ti < ntiles; ti += gridDim.x, cur ^= 1) {
+    const PassParams& P = BATCH ? s_P[cur] : P0;
+    const bool more = ti + gridDim.x < ntiles;
+    const int t = P.t, nd = 1 << t;
+    const int cnt = s_info[cur].cnt;
+    // this tile's share of the zeroing of a later pass's levels (stores that
+    // use the DRAM bandwidth the tile's compute leaves idle)
+    if (!BATCH && P0.clear) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid, NT);
+    cp_async_wait();
+    __syncthreads();
+
+    // ---- 1. where the runs go (from the tables; a warp for the level bits',
+    //      one for the next sequence's), and the next tile -------------------
+    if (warp < 2) {
+      const int half = warp;
+      // lane r < 2^t: key r's count in the tile (a difference of prefixes) and
+      // in the earlier tiles of its sequence or node
+      uint32_t c = 0;
+      uint64_t ex = 0;
+      if (lane < nd) {
+        const bool last = ((ti + 1) >> P0.chsh) != (ti >> P0.chsh) || ti + 1 >= ntiles;
+        const uint32_t a = s_ta[lane];
+        c = last ? (uint32_t)(s_cn[lane] - s_ca[lane]) - a : s_tn[lane] - a;
+        ex = (s_ca[lane] + a) - (s_cb[lane] + s_tb[lane]);
       }
-      // class counts and tile-local class starts
-      // level j classes are the digit values mod 2^j: level t holds the
-      // digit counts, level j-1 class k sums classes k and k + 2^(j-1)
-      __syncwarp();
-      for (int j = t - 1; j >= 0; j--) {
-        for (int k = lane; k < (1 << j); k += 32)
-          ccnt[cls_idx(j, k)] = ccnt[cls_idx(j + 1, k)] + ccnt[cls_idx(j + 1, k + (1 << j))];
-        __syncwarp();
-      }
-      // tile-local class starts: exclusive scan of each level's counts
-      for (int j = 0; j <= t; j++) {
-        uint32_t carry = 0;
-        for (int k0 = 0; k0 < (1 << j); k0 += 32) {
-          const int k = k0 + lane;
-          const uint32_t c = k < (1 << j) ? ccnt[cls_idx(j, k)] : 0u;
-          uint32_t ci = c;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, ci, o);
-            if (lane >= o) ci += y;
+      int j = t;
+      if (half == 0) {
+        if (lane < KEYS) s_own[lane] = c;
+        // lane i takes class k of level j, i + 1 = 2^j + k: the keys' counts
+        // folded level by level
+        const int mj = 31 - __clz(lane + 1), mk = lane + 1 - (1 << mj);
+        uint32_t fc = c, rc = 0;
+        uint64_t fx = ex, rx = 0;
+        for (int l = t - 1; l >= 0; l--) {
+          fc += __shfl_down_sync(FULL, fc, 1 << l);
+          fx += __shfl_down_sync(FULL, fx, 1 << l);
+          const uint32_t yc = __shfl_sync(FULL, fc, mk);
+          const uint64_t yx = __shfl_sync(FULL, fx, mk);
+          if (mj == l) {
+            rc = yc;
+            rx = yx;
           }
-          if (k < (1 << j)) cstart[cls_idx(j, k)] = carry + ci - c;
-          carry += __shfl_sync(FULL, ci, 31);
         }
+        c = lane < nd - 1 && (!DIG || (mj & 1) == 0) ? rc : 0u;
+        ex = rx;
+        j = mj;
+      } else if (P.out == nullptr) {
+        c = 0;
       }
-      __syncwarp();
-      // exclusive counts of every level from the exclusive digit counts
-      for (int j = t - 1; j >= 0; j--) {
-        for (int k = lane; k < (1 << j); k += 32)
-          ex_cnt[cls_idx(j, k)] = ex_cnt[cls_idx(j + 1, k)] + ex_cnt[cls_idx(j + 1, k + (1 << j))];
-        __syncwarp();
+      uint32_t n = 0, len = 0, off = 0;  // area words or chunks; bits or bytes; offset in the first
+      uint64_t where = 0;                // address of the first (0: nowhere)
+      bool over = false;
+      if (c) {
+        const uint64_t cs = s_cs[half ? nd - 1 + lane : lane], b0 = cs + ex;
+        const bool dead = cs == ~0ull;
+        if (half) {
+          over = !dead && b0 + c > P.n_in;  // never for consistent tables
+          where = (uint64_t)(uintptr_t)P.out + b0 * (uint64_t)P.out_w;
+          off = (uint32_t)(where & 15);
+          where -= off;
+          len = c * (uint32_t)P.out_w;
+          n = (off + len + 15) >> 4;
+        } else {
+          // levels of n_in elements back to back, or the Huffman tree's
+          const uint64_t lv = (uint64_t)(DIG ? (P.a + j) >> 1 : P.a + j);
+          const bool hf = P.shape == SHAPE_HUFF;
+          const uint64_t lbits = hf ? s_ll[j] : P.n_in * bpe;
+          const uint64_t lwords = hf ? s_lo[j] : lv * (((lbits + 2047) >> 11) << 5);
+          const uint64_t G0 = b0 * bpe;
+          len = c * bpe;
+          over = !dead && G0 + len > lbits;  // never for consistent tables
+          off = (uint32_t)(G0 & 63);
+          n = (off + len + 63) >> 6;
+          where = (uint64_t)(uintptr_t)(P.bits + lwords + (G0 >> 6));
+        }
+        if (dead) where = 0;
       }
+      uint32_t first = n;
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, first, o);
+        if (lane >= o) first += y;
+      }
+      const uint32_t total = __shfl_sync(FULL, first, 15);
+      first -= n;
+      const uint32_t some = __ballot_sync(FULL, n != 0u);
+      const int at = __popc(some & lanemask_lt()), runs = __popc(some);
+      if (lane >= runs && lane < KEYS) s_rs[half][lane] = ~0u;
+      if (n) {
+        const int sh = half ? 4 : 6, usz = half ? 16 : 8;  // unit: 16-byte chunk, or word of 64 bits
+        s_rs[half][at] = first;
+        Run r;
+        r.base = where ? where - (uint64_t)first * usz : 0ull;
+        r.first = where ? first + (off ? 1u : 0u) : ~0u;
+        r.last = where ? first + ((off + len) >> sh) : 0u;
+        s_run[half][at] = r;
+        if (half) s_edge[at] = where ? off | (len << 8) : 0u;
+      }
+      if (lane < KEYS) {
+        if (half) ((uint16_t*)s_sb)[lane] = (uint16_t)(16 * first + off);
+        else s_ab[lane] = 8 * smem_addr(s_area) + 64 * first + off;
+      }
+      const bool stop = __any_sync(FULL, over);
       if (lane == 0) {
-        s_nxt = nx;
-        int iw;
-        s_nsrc = stage_src(nx, iw);
-        s_niw = iw;
+        s_n[half] = total;
+        if (half) s_nr = (uint32_t)runs;
+        s_over[half] = stop;
       }
-    } else {
-      // ---- 4 (worker warps). t stable 1-bit splits in shared memory -------
-      // Warp w holds rows 16w..16w+15 of the tile (row = 32 consecutive
-      // positions, one per lane).  Each level: one ballot per row gives the
-      // level's bits in the current order (stored as they are) and, because
-      // every lane sees every ballot of its warp, the ones before each row
-      // are a running sum in uniform registers.  After one exchange of the
-      // warps' one counts, an element at position p with k ones before it
-      // goes to Z + k if its bit is 1 and to p - k otherwise.
-      // a staged tile of bytes bound for a 16-bit buffer sits, as bytes, in
-      // the buffer's upper half; the first split reads it there
-      const bool bytes0 = sizeof(E) == 2 && s_stg && P.in_w == 1;
-      auto splits = [&](auto full_c) {
-        constexpr bool F = decltype(full_c)::value;
-        const int nmove = P.out != nullptr ? t : t - 1;
-        for (int j = 0; j < t; j++) {
-          const E* src = buf(j & 1);
-          E* dst = buf((j & 1) ^ 1);
-          const uint32_t m = 1u << (P.rbits - 1 - j);
-          const bool two = DIG && (((P.a + j) & 1) == 0) && (P.a + j + 1 < P.L);
-          uint2* const Rw = rowq + j * TWS + warp * EPW;
-#if WT_PASS_KEEP_X
-          uint32_t xr[EPW];
-#endif
-          int ones = 0;
-          // ballots of the level's bit over the warp's rows, reading the
-          // elements through sp (bytes for a staged byte tile's first split)
-          auto phase1 = [&](auto* sp) {
+    }
+    if (tid == NT - 1 && more) set_info(ti + gridDim.x, cur ^ 1);
+
+    // ---- 2. planes and key counts of the thread's 32 elements -------------
+    const unsigned char* const row = s_in + tid * RS;
+    const int nv = min(max(cnt - 32 * tid, 0), 32);
+    const uint32_t v = low_mask((uint32_t)nv);
+    uint32_t p[4], C[8], X[8];
+    planes_of<EW>([&](int i, uint32_t* w) {
+      const uint4 q = *(const uint4*)(row + 16 * i);
+      w[0] = q.x;
+      w[1] = q.y;
+      w[2] = q.z;
+      w[3] = q.w;
+    }, P.rbits, p);
+    if (t < 2) p[1] = 0u;
+    if (t < 3) p[2] = 0u;
+    if (t < 4) p[3] = 0u;
+    key_counts(p, v, C);
+    // prefix sums over the warp: lane (q, k) adds up word k of eight lanes,
+    // rows of eight words, eight apart more every eight rows (no bank is hit
+    // twice by the four q)
+    {
+      uint32_t* const mine = scr + lane * 8 + (lane >> 3) * 8;
+      *(uint4*)mine = make_uint4(C[0], C[1], C[2], C[3]);
+      *(uint4*)(mine + 4) = make_uint4(C[4], C[5], C[6], C[7]);
+      __syncwarp();
+      const int k = lane & 7, q = lane >> 3;
+      uint32_t* const col = scr + q * 72 + k;
+      uint32_t c[8], sum = 0;
 #pragma unroll
-            for (int e = 0; e < EPW; e++) {
-              const int p = wbase + e * 32 + lane;
-              const uint32_t x = (F || p < cnt) ? (uint32_t)sp[p] : 0u;
-#if WT_PASS_KEEP_X
-              xr[e] = x;
-#endif
-              const uint32_t B = __ballot_sync(FULL, x & m);
-              if (lane == 0) Rw[e] = make_uint2(B, (uint32_t)ones);
-              ones += (int)sizeof(E) * __popc(B);
-              if (DIG && two) {
-                const uint32_t B2 = __ballot_sync(FULL, x & (m >> 1));
-                if (lane == 0) pb1[(j >> 1) * TW + warp * EPW + e] = B2;
-              }
-            }
+      for (int i = 0; i < 8; i++) {
+        c[i] = col[8 * i];
+        sum += c[i];
+      }
+      uint32_t inc = sum;
+      uint32_t y = __shfl_up_sync(FULL, inc, 8);
+      if (q >= 1) inc += y;
+      y = __shfl_up_sync(FULL, inc, 16);
+      if (q >= 2) inc += y;
+      if (q == 3) s_wtot[warp][k] = inc;
+      uint32_t run = inc - sum;
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        col[8 * i] = run;
+        run += c[i];
+      }
+      __syncwarp();
+      const uint4 a = *(const uint4*)mine, b = *(const uint4*)(mine + 4);
+      X[0] = a.x;
+      X[1] = a.y;
+      X[2] = a.z;
+      X[3] = a.w;
+      X[4] = b.x;
+      X[5] = b.y;
+      X[6] = b.z;
+      X[7] = b.w;
+    }
+    __syncthreads();
+
+    // ---- 3. the splits ------------------------------------------------------
+    // the tile's key counts against the tables': tables that disagree with the
+    // tile would misplace its runs, so the tile is flagged (every warp finds
+    // the same) and its outputs are left alone
+    bool bad = s_over[0] | s_over[1];
+    {
+      uint32_t tot = 0;
+      if (lane < nd) {
+#pragma unroll
+        for (int w = 0; w < W; w++) tot += s_wtot[w][lane >> 1];
+        tot = (tot >> (16 * (lane & 1))) & 0xffffu;
+      }
+      bad |= __any_sync(FULL, lane < nd && tot != s_own[lane & (KEYS - 1)]);
+      if (bad && tid == 0) atomicOr(P.err, ERR_INTERNAL);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) p[j] |= ~v;  // the bits past the tile's end stay last
+    const uint32_t d1 = p[1];  // digit levels: the second bit of the first digit
+    // (one copy of the code for every t: the last levels' splits are the same)
+    if (t >= 2) {
+      uint32_t x[4] = {p[0], p[1], p[2], p[3]};
+      if (t == 3) {
+        x[1] = p[0];
+        x[2] = p[1];
+        x[3] = p[2];
+      } else if (t == 2) {
+        x[2] = p[0];
+        x[3] = p[1];
+      }
+      if (t == 4) split_planes<3>(x[0], x + 1);
+      if (t >= 3) split_planes<2>(x[1], x + 2);
+      if (!DIG || t == 3) split_planes<1>(x[2], x + 3);
+      p[1] = t == 4 ? x[1] : (t == 3 ? x[2] : x[3]);
+      p[2] = t == 4 ? x[2] : x[3];
+      p[3] = x[3];
+    }
+
+    if (!bad) {
+      // the earlier warps' counts
+      for (int w = 0; w < warp; w++) {
+        const uint4 a = *(const uint4*)s_wtot[w], b = *(const uint4*)(s_wtot[w] + 4);
+        X[0] += a.x;
+        X[1] += a.y;
+        X[2] += a.z;
+        X[3] += a.w;
+        X[4] += b.x;
+        X[5] += b.y;
+        X[6] += b.z;
+        X[7] += b.w;
+      }
+      // ---- 4. the level bits into the runs' areas -------------------------
+      // a piece's set bits at bit q of shared memory (pieces of one thread or
+      // of several share words)
+      auto or_bits = [&](uint32_t q, uint32_t x) {
+        const uint32_t w = (q >> 3) & ~3u;
+        or_shared(w, __funnelshift_l(0u, x, q));
+        or_shared(w + 4, __funnelshift_l(x, 0u, q));
+      };
+      // level j: its bits b0 (and b1, the digit's second bit), the thread's
+      // and the earlier threads' counts of its classes
+      auto level = [&](auto jc, uint32_t b0, uint32_t b1, const uint32_t* c, const uint32_t* x) {
+        constexpr int j = decltype(jc)::value;
+        uint32_t at = 0;
+#pragma unroll
+        for (int k = 0; k < (1 << j); k++) {
+          const uint32_t n = (k & 1) ? c[k >> 1] >> 16 : c[k >> 1] & 0xffffu;
+          const uint32_t xk = (k & 1) ? x[k >> 1] >> 16 : x[k >> 1] & 0xffffu;
+          const uint32_t q = s_ab[(1 << j) - 1 + k] + xk * bpe;
+          const uint32_t w0 = __funnelshift_rc(b0, 0u, at) & low_mask(n);
+          if (!DIG) {
+            or_bits(q, w0);
+          } else {
+            const uint32_t w1 = __funnelshift_rc(b1, 0u, at) & low_mask(n);
+            const uint64_t d = P.a + j + 1 < P.L ? (spread32(w0) << 1) | spread32(w1) : spread32(w0);
+            or_bits(q, (uint32_t)d);
+            or_bits(q + 32, (uint32_t)(d >> 32));
+          }
+          at += n;
+        }
+      };
+      uint32_t c2[2], x2[2], c1, x1;
+      {
+        uint32_t c3[4], x3[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          c3[k] = C[k] + C[k + 4];
+          x3[k] = X[k] + X[k + 4];
+        }
+        if (!DIG && t > 3) level(std::integral_constant<int, 3>{}, p[3], 0u, c3, x3);
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+          c2[k] = c3[k] + c3[k + 2];
+          x2[k] = x3[k] + x3[k + 2];
+        }
+      }
+      if (t > 2) level(std::integral_constant<int, 2>{}, p[2], p[3], c2, x2);
+      c1 = c2[0] + c2[1];
+      x1 = x2[0] + x2[1];
+      if (!DIG && t > 1) level(std::integral_constant<int, 1>{}, p[1], 0u, &c1, &x1);
+      const uint32_t c0 = (uint32_t)nv, x0 = min((uint32_t)(32 * tid), (uint32_t)cnt);
+      level(std::integral_constant<int, 0>{}, p[0], d1, &c0, &x0);
+
+      // ---- 5. the elements into key order ----------------------------------
+      // a pointer per key and thread, two 16-bit ones a word: word b1 b2 b3
+      // (the digit's lower bits as they stand in the element), half b0
+      if (P.out != nullptr) {
+        const uint32_t ow = (uint32_t)P.out_w;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          const int rk = ((k & 1) << 2) | (k & 2) | (k >> 2);
+          ptr[rk * 32 + lane] = s_sb[k] + X[k] * ow;
+        }
+        // (no other thread reads them)
+        const uint32_t ptrs = smem_addr(ptr) + 4 * lane, srt = smem_addr(s_srt);
+        const uint32_t m1 = t == 4 ? 0x380u : (t == 3 ? 0x300u : (t == 2 ? 0x200u : 0u));
+        const int r1 = P.rbits - 11, r0 = P.rbits - 2;
+        auto move = [&](auto wc) {
+          constexpr int OW = decltype(wc)::value;
+          constexpr int PER = 4 / EW;  // elements a word
+          auto one = [&](uint32_t w, int sh) {
+            const uint32_t pa = (rotr32(w, r0 + sh) & 2u) | ((rotr32(w, r1 + sh) & m1) | ptrs);
+            const uint32_t to = ld_shared_u16(pa);
+            st_shared<OW>(srt + to, w >> sh);
+            st_shared<2>(pa, to + OW);
           };
-          if (sizeof(E) == 2 && j == 0 && bytes0)
-            phase1((const uint8_t*)src + T);
-          else
-            phase1(src);
-          if (j < nmove) {
-            if (lane == 0) s_ones[warp] = ones;
-            bar_workers();
-            const int v = lane < W ? s_ones[lane] : 0;
-            const int T1 = __reduce_add_sync(FULL, v);
-            const int ob = __reduce_add_sync(FULL, lane < warp ? v : 0);
-            // shared-memory byte addresses: of this warp's first one's
-            // destination, and of the lane's position minus the ones before
-            // the warp
-            const uint32_t ds = smem_addr(dst);
-            const uint32_t zb = ds + (uint32_t)((int)sizeof(E) * cnt - T1 + ob);
-            const uint32_t pl = ds + (uint32_t)((int)sizeof(E) * (wbase + lane) - ob);
+          const int whole = nv * EW / 16;
+#pragma unroll 1
+          for (int i = 0; i < whole; i++) {
+            const uint4 q = *(const uint4*)(row + 16 * i);
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int e = 0; e < EPW; e++) {
-              const uint2 R = Rw[e];
-              const uint32_t q = R.y + (uint32_t)sizeof(E) * __popc(R.x & lt);
-#if WT_PASS_KEEP_X
-              const uint32_t x = xr[e];
-#else
-              const uint32_t x = (F || wbase + e * 32 + lane < cnt) ? (uint32_t)src[wbase + e * 32 + lane] : 0u;
-#endif
-              const uint32_t dest = (x & m) ? zb + q : pl + (uint32_t)(sizeof(E) * 32 * e) - q;
-              if (F || wbase + e * 32 + lane < cnt) st_shared<E>(dest, x);
-            }
-            bar_workers();
+            for (int k = 0; k < 4; k++)
+#pragma unroll
+              for (int h = 0; h < PER; h++) one(w[k], 8 * EW * h);
           }
-        }
-      };
-      if (full) splits(std::true_type{});
-      else splits(std::false_type{});
-    }
-    fence_async_smem();  // the splits' accesses before the next bulk copy
-    __syncthreads();
-    // the final element order is in buf(1) after an odd number of moves
-    cur = (P.out != nullptr ? t : t - 1) & 1;
-    // the next tile goes to the buffer that does not hold the final order;
-    // a bulk copy consumed by this tile has closed s_bar's phase
-    if (tid == 0) {
-      const int nib = cur ? s_ib : 1 - s_ib;
-      const unsigned char* src = s_nsrc;
-      s_phase ^= (uint32_t)s_stg;
-      s_nib = nib;
-      s_nstg = src != nullptr;
-      if (src) stage(src, s_niw, nib ? buf1 : buf0);
-    }
-
-    if (s_bad) continue;  // uniform: read after the barrier above
-
-    // ---- 5. level bitmaps: whole words stored, shared words ORed ----------
-    auto emitted = [&](int j) -> bool { return !DIG || (((P.a + j) & 1) == 0); };
-    // 64 local bits of level j starting at local bit position bp
-    auto get64 = [&](int j, int bp) -> uint64_t {
-      if (!DIG) {
-        // bp >= 0 and bp < T: words bp/32 .. bp/32 + 2 exist (zero pads)
-        const uint2* r = rowq + j * TWS + (bp >> 5);
-        const int o = bp & 31;
-        const uint32_t w0 = r[0].x, w1 = r[1].x, w2 = r[2].x;
-        const uint32_t lo = __funnelshift_r(w0, w1, o), hi = __funnelshift_r(w1, w2, o);
-        return ((uint64_t)hi << 32) | lo;
-      }
-      const int e = bp >> 1;
-      const uint32_t b0 = get32q<TW>(rowq + j * TWS, e);
-      if (P.a + j + 1 < P.L) {
-        const uint32_t b1 = get32<TW>(pb1 + (j >> 1) * TW, e);
-        return (spread32(b0) << 1) | spread32(b1);
-      }
-      return spread32(b0);
-    };
-    // words of every (level, class) of this tile, one flattened list: per
-    // run its output word pointer, first bit in that word and word count
-    uint64_t* const cls_wp = cls_cs;
-    int nw = 0;
-    if (tid < ntl) {
-      const int j = 31 - __clz(tid + 1);
-      uint64_t cs = 0, ce = 0;
-      bool dead = true;
-      if (emitted(j) && ccnt[tid]) class_range(P, j, (uint32_t)(tid + 1 - (1 << j)), node, cs, ce, dead);
-      if (!dead) {
-        const uint64_t G0 = (cs + ex_cnt[tid]) * bpe;
-        const uint64_t G1 = G0 + (uint64_t)ccnt[tid] * bpe;
-        const int lo_ = DIG ? ((P.a + j) >> 1) : (P.a + j);
-        if (G1 > P.lvl_len[lo_] * (uint64_t)bpe) {
-          atomicOr(P.err, ERR_INTERNAL);  // never for consistent tables
-        } else {
-          nw = (int)(((G1 - 1) >> 6) - (G0 >> 6) + 1);
-          cls_wp[tid] = (uint64_t)(P.bits + P.lvl_off[lo_] + (G0 >> 6));
-          s_g0[tid] = (uint8_t)(G0 & 63);
-        }
-      }
-    }
-    // the list in windows of 32 entries: a bit per run start, the run of
-    // each start, and the run in force at each window's first entry
-    if (tid < WWIN) s_wstart[tid] = 0u;
-    int wtot;
-    const int wex = block_scan(nw, wtot);  // its barriers order the zeroing
-    if (tid < ntl) {
-      wst[tid] = wex;
-      if (nw > 0 && wex + nw <= WMAX) {
-        atomicOr(&s_wstart[wex >> 5], 1u << (wex & 31));
-        s_runid[wex] = (uint8_t)tid;
-        for (int w = (wex + 31) >> 5; (w << 5) < wex + nw; w++) s_winrun[w] = (uint8_t)tid;
-      }
-    }
-    __syncthreads();
-    if (wtot > WMAX) {
-      if (tid == 0) atomicOr(P.err, ERR_INTERNAL);  // never: bounded by the tile geometry
-    } else {
-      const uint32_t le = lt | (1u << lane);
-      for (int win = warp; (win << 5) < wtot; win += NB / 32) {
-        const int x = (win << 5) + lane;
-        const uint32_t mb = s_wstart[win] & le;
-        const int ci = mb ? (int)s_runid[(win << 5) + 31 - __clz(mb)] : (int)s_winrun[win];
-        if (x < wtot) {
-          const int k = x - wst[ci];  // word of the run
-          const int j = 31 - __clz(ci + 1);
-          uint64_t* const wp = (uint64_t*)cls_wp[ci];
-          const int g0 = s_g0[ci];
-          const int nbits = (int)ccnt[ci] * bpe, lb0 = (int)cstart[ci] * bpe;
-          const int lo = k ? 0 : g0;           // first bit of the word that is the run's
-          const int r0 = k ? 64 * k - g0 : 0;  // its index in the run
-          const int nb = min(64 - lo, nbits - r0);
-          uint64_t v = get64(j, lb0 + r0);
-          if (nb < 64) v &= (1ull << nb) - 1ull;
-          // stored when the run holds the whole word, else ORed
-          if (nb == 64) wp[k] = v;
-          else atomicOr((unsigned long long*)(wp + k), (unsigned long long)(v << lo));
-        }
-      }
-    }
-    __syncthreads();
-
-    // ---- 6. scatter T_{a+t}, narrowed ------------------------------------
-    if (P.out) {
-      const E* fin = buf(cur);
-      if (tid < 8) s_dead[tid] = 0;
-      if (tid == 0) s_oob = 0;
-      __syncthreads();
-      // per digit value d (the t bits above the ones still needed, i.e. the
-      // class key reversed): the byte address that tile-local position 0
-      // would have in d's output range, so that position p goes to that
-      // address + p * width (modular arithmetic: the base itself may lie
-      // outside the output)
-      for (int r = tid; r < (1 << t); r += NB) {
-        uint64_t cs, ce;
-        bool dead;
-        class_range(P, t, (uint32_t)r, node, cs, ce, dead);
-        const int ci = cls_idx(t, r);
-        const uint32_t d = rev_bits((uint32_t)r, t);
-        const uint64_t b0 = cs + ex_cnt[ci];
-        sbase[d] = (uint64_t)(uintptr_t)P.out + (b0 - cstart[ci]) * (uint64_t)P.out_w;
-        if (dead) atomicOr(&s_dead[d >> 5], 1u << (d & 31));
-        else if (ccnt[ci] && b0 + ccnt[ci] > P.n_in) s_oob = 1;  // never for consistent tables
-      }
-      __syncthreads();
-      const int nb = P.rbits - t;
-      const uint32_t mask = nb >= 32 ? 0xffffffffu : ((1u << nb) - 1u);
-      const uint32_t dmask = (1u << t) - 1u;
-      // only Huffman trees have dead classes (elements leaving the tree)
-      auto scatter = [&](auto out_t, auto huff_c) {
-        using O = decltype(out_t);
-        constexpr bool HF = decltype(huff_c)::value;
-        auto one = [&](int p) {
-          const uint32_t x = fin[p];
-          const uint32_t d = (x >> nb) & dmask;
-          if (HF && ((s_dead[d >> 5] >> (d & 31)) & 1u)) return;
-          *(O*)(uintptr_t)(sbase[d] + (uint64_t)p * sizeof(O)) = (O)(x & mask);
+#pragma unroll 1
+          for (int i = whole * 16 / EW; i < nv; i++) one((uint32_t)((const E*)row)[i], 0);
         };
-        if (full) {
-          // a whole tile: T / NT elements per worker thread, unrolled
-          if (tid < NT) {
-#pragma unroll
-            for (int k = 0; k < T / NT; k++) one(tid + k * NT);
-          }
-        } else {
-          for (int p = tid; p < cnt; p += NB) one(p);
-        }
-      };
-      if (s_oob) {
-        if (tid == 0) atomicOr(P.err, ERR_INTERNAL);
-      } else if (P.shape == SHAPE_HUFF) {
-        if (P.out_w == 1) scatter(uint8_t{}, std::true_type{});
-        else if (P.out_w == 2) scatter(uint16_t{}, std::true_type{});
-        else scatter(uint32_t{}, std::true_type{});
-      } else {
-        if (P.out_w == 1) scatter(uint8_t{}, std::false_type{});
-        else if (P.out_w == 2) scatter(uint16_t{}, std::false_type{});
-        else scatter(uint32_t{}, std::false_type{});
+        if (ow == 1) move(std::integral_constant<int, 1>{});
+        else if (EW >= 2 && ow == 2) move(std::integral_constant<int, 2>{});
+        else if (EW == 4) move(std::integral_constant<int, 4>{});
       }
     }
     __syncthreads();
+    if (more) {  // behind the stores below
+      load_tile(cur ^ 1);
+      if (warp == 0) load_ctl(ti + gridDim.x, cur ^ 1);
+    }
+    if (bad) continue;  // uniform; nothing was put into the areas
+
+    // ---- 6. level words out, and the areas back to zero; T_{a+t} out ------
+    // A warp takes 32 consecutive units; a lane's run is the last one that
+    // starts at or before its unit: the number of starts up to the window's
+    // first unit, and a bit per start inside the window.
+    auto each = [&](int half, auto&& f) {
+      const uint32_t total = s_n[half];
+      const uint32_t start = lane < 16 ? s_rs[half][lane] : ~0u;
+      for (uint32_t b = 32 * warp; b < total; b += NT) {
+        const uint32_t before = __popc(__ballot_sync(FULL, start <= b));
+        const uint32_t in = __reduce_or_sync(FULL, start > b && start < b + 32 ? 1u << (start - b) : 0u);
+        const uint32_t i = b + lane;
+        if (i < total) f(i, s_run[half][before - 1 + __popc(in << (31 - lane))]);
+      }
+    };
+    each(0, [&](uint32_t i, const Run& r) {
+      const uint64_t x = s_area[i];
+      s_area[i] = 0ull;
+      uint64_t* const wp = (uint64_t*)(uintptr_t)r.base + i;
+      // stored when the run holds the whole word, else ORed
+      if (i >= r.first && i < r.last) *wp = x;
+      else if (x && r.base) atomicOr((unsigned long long*)wp, (unsigned long long)x);
+    });
+    if (P.out != nullptr) {
+      each(1, [&](uint32_t i, const Run& r) {
+        if (i >= r.first && i < r.last)
+          *((uint4*)(uintptr_t)r.base + i) = *((const uint4*)s_srt + i);
+      });
+      // the chunks at the runs' ends that other tiles share: four bytes a
+      // thread, by elements where not all of them are the run's
+      for (uint32_t e = tid; e < 8 * s_nr; e += NT) {
+        const uint32_t at = e >> 3, b = 4 * (e & 3), oe = s_edge[at];
+        const uint32_t off = oe & 0xffu, end = off + (oe >> 8);
+        const uint32_t k = (e & 4) ? (end - 1) >> 4 : 0u;  // last chunk or first
+        const uint32_t lo = k ? 0u : off, hi = min(end - 16 * k, 16u);
+        // once only, and only if not stored whole above
+        if (oe == 0u || ((e & 4) && k == 0u) || hi - lo == 16u) continue;
+        const uint32_t i = s_rs[1][at] + k;
+        const unsigned char* from = s_srt + 16 * i + b;
+        unsigned char* to = (unsigned char*)(uintptr_t)(s_run[1][at].base + 16ull * i) + b;
+        if (lo <= b && b + 4 <= hi) {
+          *(uint32_t*)to = *(const uint32_t*)from;
+        } else if (P.out_w == 2) {
+          if (lo <= b && b + 2 <= hi) *(uint16_t*)to = *(const uint16_t*)from;
+          if (lo <= b + 2 && b + 4 <= hi) *(uint16_t*)(to + 2) = *(const uint16_t*)(from + 2);
+        } else if (P.out_w == 1) {
+#pragma unroll
+          for (uint32_t q = 0; q < 4; q++)
+            if (lo <= b + q && b + q < hi) to[q] = from[q];
+        }
+      }
+    }
   }
 }
 

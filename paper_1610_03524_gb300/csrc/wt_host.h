@@ -174,7 +174,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
                    wt_struct* h);
 wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const wt_build_opts* o,
                    wt_struct* h, bool multiary);
-wt_status build_huff(const void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
+wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
                      const wt_build_opts* o, wt_struct* h);
 wt_status launch_query(wt_struct* h, int op, const uint32_t* c, const uint64_t* x, uint64_t q,
                        uint64_t* out, cudaStream_t st);
@@ -184,7 +184,7 @@ wt_status launch_query_multi(wt_struct* const* hs, uint32_t nh, const uint32_t* 
                              const uint8_t* op, const uint32_t* c, const uint64_t* x, uint64_t q,
                              uint64_t* out, cudaStream_t st);
 // configuration of a wavelet-matrix build recorded by the autotuner for
-// (L, ceil(log2 n)): levels per pass (8 if none), symbols per tile (PASS_T if
+// (L, ceil(log2 n)): levels per pass (TAU_MAX if none), symbols per tile (PASS_T if
 // none) and CTAs per SM (0 = as many as fit)
 struct TuneConfig {
   int tau;

@@ -6,14 +6,17 @@
 
 namespace wtk {
 
-constexpr int TAU_MAX = 8;                  // levels per partition pass (upper bound)
-constexpr int NCLS = 1 << (TAU_MAX + 1);    // class-tree slots: level j class k at 2^j-1+k
+// Levels per partition pass (upper bound; a larger tau runs as passes of 4).
+// With four, a thread's 32 elements need six plane moves for their levels and
+// one element move, a tile has 15 runs of level bits and 16 of elements, and
+// its tables are 64 bytes; eight levels in one pass would halve the passes'
+// reads and writes of the elements, which are not what bounds them.
+constexpr int TAU_MAX = 4;
 constexpr uint32_t FULL = 0xffffffffu;
 
 // device error word bits
 // (ERR_INTERNAL: a prefix table disagreed with a tile; never for correct tables)
-// (ERR_STALL: a staged tile load did not complete within its time limit)
-enum : uint32_t { ERR_SYMBOL = 1u, ERR_INTERNAL = 4u, ERR_STALL = 8u };
+enum : uint32_t { ERR_SYMBOL = 1u, ERR_INTERNAL = 4u };
 
 // structure shapes handled by the partition pass
 enum Shape : int { SHAPE_WM = 0, SHAPE_WT = 1, SHAPE_HUFF = 2 };
@@ -30,18 +33,16 @@ struct TileDesc {
 
 // Per-tile digit counts of a pass (the K sub-problems' per-node counts of
 // Section 4.2) and their prefix sums across tiles, in chunks of 2^chsh tiles:
-// tile ti's counts sit at tcnt[ti * tcs + r] (u32, exclusive within its chunk
-// after the scan) and chunk c's exclusive counts at tchunk[c * tcs + r]
+// tile ti's counts sit at tcnt[ti * TC_STRIDE + r] (u32, exclusive within its chunk
+// after the scan) and chunk c's exclusive counts at tchunk[c * TC_STRIDE + r]
 // (u64), the totals after the last chunk.
-constexpr int TC_STRIDE = 256;  // the largest stride (t = 8)
-// the stride of a pass's tables: its digit values, at least one warp's worth
-__host__ __device__ inline uint32_t tc_stride(int t) { return t >= 5 ? (1u << t) : 32u; }
-// Tiles per chunk: 64, so that a short table is scanned in four rounds of 16
-// loads, and more from 2^17 tiles on, so that the scan over the chunks stays
-// below 2048 of them (its blocks walk them one after another).
+constexpr int TC_STRIDE = 1 << TAU_MAX;  // row stride of both tables
+// Tiles per chunk: 64, so that a thread scans them in four rounds of 16 loads
+// (256 of them took 197 us for 2^20 tiles, 64 take 20), and more from 2^20
+// tiles on, so that the one block that scans the chunks walks at most 16384.
 inline int chunk_shift(uint64_t tiles) {
   int s = 6;
-  while ((tiles >> s) > 2048) s++;
+  while ((tiles >> s) > 16384) s++;
   return s;
 }
 
@@ -62,8 +63,6 @@ struct SegDesc {
   const void* in;
   void* out;
   uint64_t* bits;
-  const uint64_t* lvl_off;
-  const uint64_t* lvl_len;
   uint64_t* wm_cls;
   uint64_t* zeros;
   uint32_t* err;
@@ -77,7 +76,6 @@ struct PassParams {
   // input sequence T_a (elements hold the rbits = L - a low bits still needed)
   const void* in;
   int in_w;                 // bytes per input element (1, 2, 4)
-  const uint32_t* code_map; // HUFF first pass: symbol -> left-aligned codeword
   // output sequence T_{a+t}, narrowed to rbits - t bits (nullptr on the last pass)
   void* out;
   int out_w;
@@ -89,11 +87,11 @@ struct PassParams {
   int digits;               // 1: emit 2-bit digit levels at even levels (multiary)
   // outputs
   uint64_t* bits;           // level bitmaps (or digit levels)
-  const uint64_t* lvl_off;  // word offset per output level
-  const uint64_t* lvl_len;  // elements per output level
+  const uint64_t* lvl_off;  // HUFF: word offset per level (the others' levels, of n_in
+  const uint64_t* lvl_len;  // elements each, stand back to back), and its elements
   // class starts
   const uint64_t* wm_cls;   // WM: per level j of the pass, 2^j+1 starts at 2^j-1+j
-  const uint64_t* wt_C;     // WT: C[v] = #symbols < v, v in [0, 2^L]
+  const uint64_t* wt_C;     // WT: starts of the nodes of level a + t, 2^(a+t) + 1
   const uint64_t* hf_node;  // HUFF: starts of the internal nodes, per level + sentinel
   const uint64_t* hf_lvl;   // HUFF: per level l: [3l] table offset, [3l+1] first internal prefix, [3l+2] count
   // tiles
@@ -102,16 +100,14 @@ struct PassParams {
   uint32_t ntiles;
   uint64_t n_in;
   uint32_t tile0;           // first tile of the sequence (0 unless batched)
-  uint32_t sigma;           // batched first passes: the tile counts check S[i] < sigma
+  uint32_t sigma;           // first passes: the tile counts check S[i] < sigma (0: no check)
   // batched builds: per-sequence parts, sorted by tile0
   const SegDesc* segs;
   uint32_t nsegs;
   // prefix sums of the tiles' digit counts (see TileDesc)
   const uint32_t* tcnt;
   const uint64_t* tchunk;
-  uint32_t tcs;          // their stride (tc_stride of the largest digit width)
   uint32_t chsh;         // log2 of the tiles per chunk
-  uint32_t* ticket;      // tiles are taken in order from this counter
   uint32_t* err;
   // 16-byte units of a later pass's levels to zero, `clear_per` of them per
   // tile (nullptr: none); see clear_share
@@ -139,63 +135,8 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// ---- bulk copies (TMA) into shared memory, completed on an mbarrier -------
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
-
-// an mbarrier for one arriving thread, visible to the bulk-copy unit
-__device__ __forceinline__ void mbar_init1(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Copy `bytes` (a multiple of 16; both addresses 16-byte aligned) from global
-// memory to shared memory with the bulk-copy unit; the barrier's current
-// phase completes when the bytes have landed.  One thread issues it.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
-               "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(bar))
-      : "memory");
-}
-
-// order this thread's earlier shared-memory accesses before later bulk copies
-__device__ __forceinline__ void fence_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Wait for the phase of `bar` with parity `parity` to complete: false if it
-// has not after about one second (or 2^24 polls), which a bulk copy of a few
-// KB from valid memory never takes.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const uint32_t a = smem_addr(bar);
-  uint64_t t0 = 0;
-  for (uint32_t it = 0; it < (1u << 24); it++) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (it == 0) t0 = global_ns();
-    else if (global_ns() - t0 > 1000000000ull) return false;
-  }
-  return false;
-}
-
 
 }  // namespace wtk
