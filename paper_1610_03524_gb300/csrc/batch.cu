@@ -27,8 +27,7 @@ namespace wtk {
 wt_status launch_pass_batch(const PassParams& P, const wt_build_opts* o, cudaStream_t st);
 wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32_t nlev,
                            const std::vector<uint64_t>& sb_first, uint64_t* dir, uint64_t* samp,
-                           uint64_t* zeros, int write_zeros, cudaStream_t st,
-                           const LevelMeta* h_meta = nullptr);
+                           uint64_t* zeros, cudaStream_t st, const LevelMeta* h_meta);
 
 #define CK(x)                                                   \
   do {                                                          \
@@ -341,7 +340,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   }
   if (s == WT_OK && !(o && (o->flags & WT_FLAG_NO_DIRECTORY)))
     s = dir_build_levels(a_bits, d_gmeta, (uint32_t)nlev_tot, sb_first, a_dir, a_samp, nullptr,
-                         0, st);
+                         st, nullptr);
   dfree(wsv, st);
   if (s != WT_OK) return s;
   CK(cudaGetLastError());

@@ -14,6 +14,7 @@
 // digit value (Section 5.2 generalized select: the position of every 4096th
 // occurrence of each value), four regions of n/4096 + 1 per level.
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <cstdio>
 #include <vector>
 
@@ -95,16 +96,19 @@ __device__ __forceinline__ void load_block(const uint64_t* lbits, uint64_t w0, u
 // ---------------------------------------------------------------------------
 // binary directories
 // ---------------------------------------------------------------------------
-// One block covers DIR_SB_PER_BLOCK superblocks of one level (blk_first[l]:
-// first block of level l), so the level is found once per block; each warp
-// counts DIR_SB_PER_WARP superblocks with their words loaded together.
+// Three launches build the directories of any number of levels: the counts
+// of every group of DIR_GROUP superblocks of one level with their prefix sums
+// inside the group (blk_first[l]: first group of level l), the prefix sums of
+// the group totals of each level, and the absolute counts with the select
+// samples.  One launch does when no level has more than one group.
 #ifndef WT_DIR_SB_PER_WARP
 #define WT_DIR_SB_PER_WARP 8
 #endif
 constexpr int DIR_SB_PER_WARP = WT_DIR_SB_PER_WARP;
 constexpr int DIR_SB_PER_BLOCK = 8 * DIR_SB_PER_WARP;  // 256 threads
+constexpr int DIR_GROUP = DIR_SB_PER_BLOCK;
 
-// Up to DIR_SMALL levels: their first blocks, first superblocks and
+// Up to DIR_SMALL levels: their first groups, first superblocks and
 // metadata ride in the kernel parameters, so a block finds its level without
 // a dependent load (else the tables are searched in global memory).
 constexpr int DIR_SMALL = 32;
@@ -115,105 +119,42 @@ struct DirLevels {
   LevelMeta meta[DIR_SMALL];
 };
 
-template <bool SMALL>
-__global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const LevelMeta* meta,
-                                                   int nlev, const uint64_t* sb_first,
-                                                   const uint64_t* blk_first, uint64_t* dir,
-                                                   uint64_t* sbz, const __grid_constant__ DirLevels dl) {
-  __shared__ LevelMeta sm;
-  __shared__ uint64_t s_sb0, s_g0;
-  LevelMeta m;
-  uint64_t sb0, g0;
-  if (SMALL) {
-    int l = 0;
-    while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= blockIdx.x) l++;
-    m = dl.meta[l];
-    sb0 = (blockIdx.x - dl.blk_first[l]) * DIR_SB_PER_BLOCK;
-    g0 = dl.sb_first[l];
-  } else {
-    if (threadIdx.x == 0) {
-      const int l = find_level(blk_first, nlev, blockIdx.x);
-      sm = meta[l];
-      s_sb0 = (blockIdx.x - blk_first[l]) * DIR_SB_PER_BLOCK;
-      s_g0 = sb_first[l];
-    }
-    __syncthreads();
-    m = sm;
-    sb0 = s_sb0;
-    g0 = s_g0;
+// the last level whose first group is at most b, found by the whole warp: 32
+// entries a step (a binary search over the 39000 levels of a batch of 4096
+// sequences is 16 dependent loads)
+__device__ __forceinline__ int warp_find_level(const uint64_t* first, int nlev, uint64_t b) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = nlev - 1;
+  while (lo < hi) {
+    const int step = (hi - lo + 31) >> 5;
+    const int at = lo + (lane + 1) * step;
+    const uint32_t c = (uint32_t)__popc(__ballot_sync(FULL, at <= hi && first[at] <= b));
+    lo += (int)c * step;
+    if (c < 32 && lo + step - 1 < hi) hi = lo + step - 1;
   }
-  // two superblocks at a time: lanes 0-15 the first, 16-31 the second, each
-  // lane two consecutive words (one 16-byte load where aligned)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int hl = lane & 15, half = lane >> 4;
-  const uint64_t s0 = sb0 + (uint64_t)warp * DIR_SB_PER_WARP;
-  const uint64_t* lb = bits + m.bit_off;
-  const bool vec = (((uintptr_t)lb) & 15) == 0;
-  constexpr int NP = DIR_SB_PER_WARP / 2;
-  uint64_t w0[NP], w1[NP];
-  int v0[NP], v1[NP];
-#pragma unroll
-  for (int u = 0; u < NP; u++) {
-    const uint64_t s = s0 + 2 * u + half;
-    const int64_t rem = (int64_t)m.n - (int64_t)(2048 * s + 128 * (uint64_t)hl);
-    const bool live = s < m.nsb && rem > 0;
-    v0[u] = !live ? 0 : (rem >= 64 ? 64 : (int)rem);
-    v1[u] = (!live || rem <= 64) ? 0 : (rem >= 128 ? 64 : (int)(rem - 64));
-    const uint64_t* p = lb + 32 * s + 2 * hl;
-    // words past the last valid bit are not read (a caller bitvector may end there)
-    if (v1[u] && vec) {
-      const ulonglong2 q = __ldcs((const ulonglong2*)p);
-      w0[u] = q.x;
-      w1[u] = q.y;
-    } else {
-      w0[u] = v0[u] ? __ldcs(p) : 0ull;
-      w1[u] = v1[u] ? __ldcs(p + 1) : 0ull;
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < NP; u++) {
-    const uint64_t s = s0 + 2 * u + half;
-    const int z = v0[u] + v1[u] - __popcll(w0[u]) - __popcll(w1[u]);
-    int zi = z;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-      const int y = __shfl_up_sync(FULL, zi, o, 16);
-      if (hl >= o) zi += y;
-    }
-    // zeros of 512-bit blocks 0, 1, 2 of the superblock: lanes 3, 7, 11 of its half
-    const uint64_t r1 = (uint64_t)__shfl_sync(FULL, zi, 3, 16);
-    const uint64_t r2 = (uint64_t)__shfl_sync(FULL, zi, 7, 16);
-    const uint64_t r3 = (uint64_t)__shfl_sync(FULL, zi, 11, 16);
-    if (s < m.nsb) {
-      if (hl == 0) dir[m.dir_off + 2 * s + 1] = (r1 << 16) | (r2 << 32) | (r3 << 48);
-      if (hl == 15) sbz[g0 + s] = (uint64_t)zi;
-    }
-  }
+  return lo;
 }
 
-__global__ void k_dir_finish(const LevelMeta* meta, int nlev, const uint64_t* sb_first,
-                             uint64_t total_sb, const uint64_t* sbx, uint64_t* dir,
-                             uint64_t* zeros, int write_zeros) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < total_sb) {
-    const int l = find_level(sb_first, nlev, g);
-    const uint64_t s = g - sb_first[l];
-    dir[meta[l].dir_off + 2 * s] = sbx[g] - sbx[sb_first[l]];
-  } else if (g < total_sb + nlev) {
-    const int l = (int)(g - total_sb);
-    const LevelMeta m = meta[l];
-    const uint64_t tot = sbx[sb_first[l + 1]] - sbx[sb_first[l]];
-    dir[m.dir_off + 2 * m.nsb] = tot;
-    dir[m.dir_off + 2 * m.nsb + 1] = 0;
-    if (write_zeros) zeros[l] = tot;
+// idx-th (0-based) set bit of m
+__device__ __forceinline__ int nth_bit(uint32_t m, uint32_t idx) {
+  int at = 0;
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) {
+    const uint32_t c = __popc(m & ((1u << w) - 1u));
+    if (idx >= c) {
+      idx -= c;
+      m >>= w;
+      at += w;
+    }
   }
+  return at;
 }
 
 // position (inside superblock s, relative to its start) of the r-th
-// (0-based) bit equal to bv, which lies in s; nw as for load_block
-__device__ uint32_t find_in_sb(const uint64_t* lbits, const uint64_t* ldir, uint64_t s, int bv,
+// (0-based) bit equal to bv, which lies in s; rel: the second word of its
+// record; nw as for load_block
+__device__ uint32_t find_in_sb(const uint64_t* lbits, uint64_t rel, uint64_t s, int bv,
                                uint32_t r, uint64_t nw) {
-  const uint64_t rel = ldir[2 * s + 1];
   int b = 3;
   for (; b > 0; b--) {
     const uint32_t z = (uint32_t)((rel >> (16 * b)) & 0xffffu);
@@ -243,41 +184,296 @@ __device__ uint32_t find_in_sb(const uint64_t* lbits, const uint64_t* ldir, uint
   return (uint32_t)((8 * b + at) * 64) + sel64(word, r);
 }
 
-template <bool SMALL>
-__global__ void k_select_samples(const uint64_t* bits, const LevelMeta* meta, int nlev,
-                                 const uint64_t* sb_first, uint64_t total_sb,
-                                 const uint64_t* dir, uint64_t* samp,
-                                 const __grid_constant__ DirLevels dl) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total_sb) return;
+// Select samples of 32 consecutive superblocks of a level, one per lane (live;
+// superblock s0 + lane, zeros zb before it and zs in it, rel the second word
+// of its record): every 4096th zero and one.  About half of the superblocks of
+// a dense level hold a sample, so the warp's searches are dealt to its lanes
+// in one go instead of the zeros' and the ones' in turn with half of the lanes
+// idle.
+__device__ __forceinline__ void warp_samples(bool live, uint64_t s0, uint64_t zb, uint32_t zs,
+                                             uint64_t rel, const LevelMeta& m, const uint64_t* lb,
+                                             bool aligned, uint64_t* samp) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t s = s0 + lane;
+  const uint64_t nvalid = live ? std::min<uint64_t>(2048, m.n - 2048 * s) : 0;
+  const uint64_t ob = 2048 * s - zb;
+  const bool h0 = live && ((zb + 4095) & ~4095ull) < zb + zs;
+  const bool h1 = live && ((ob + 4095) & ~4095ull) < ob + (nvalid - zs);
+  const uint32_t m0 = __ballot_sync(FULL, h0), m1 = __ballot_sync(FULL, h1);
+  const uint32_t n0 = __popc(m0), total = n0 + __popc(m1);
+  for (uint32_t b = 0; b < total; b += 32) {
+    const uint32_t task = b + lane;
+    const bool on = task < total;
+    const int bv = task >= n0 ? 1 : 0;
+    const int src = on ? nth_bit(bv ? m1 : m0, bv ? task - n0 : task) : 0;
+    const uint64_t szb = __shfl_sync(FULL, zb, src), srel = __shfl_sync(FULL, rel, src);
+    if (on) {
+      const uint64_t ss = s0 + src;
+      const uint64_t before = bv ? 2048 * ss - szb : szb, k = (before + 4095) >> 12;
+      // a whole superblock's words can all be read; the last one's, and those
+      // of a caller's bitvector off a 16-byte boundary, one by one up to the end
+      const uint64_t nw = ss + 1 < m.nsb && aligned ? PADDED : (m.n + 63) / 64;
+      samp[(bv ? m.s1_off : m.s0_off) + k] =
+          2048 * ss + find_in_sb(lb, srel, ss, bv, (uint32_t)(4096 * k - before), nw);
+    }
+  }
+}
+
+// Counts of one group: a record per superblock with the zeros before it in
+// the group; the group's total into blk_tot.  ONE: the group is the whole
+// level (block l = level l): its records are final, and its total record, zero
+// count and samples are written too.
+template <bool SMALL, bool ONE>
+__global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const LevelMeta* meta,
+                                                   int nlev, const uint64_t* blk_first,
+                                                   uint64_t* dir, uint64_t* blk_tot, uint64_t* samp,
+                                                   uint64_t* zeros,
+                                                   const __grid_constant__ DirLevels dl) {
+  __shared__ LevelMeta sm;
+  __shared__ uint64_t s_sb0;
+  __shared__ uint32_t s_z[DIR_GROUP];
+  __shared__ uint64_t s_rel[ONE ? DIR_GROUP : 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   LevelMeta m;
-  uint64_t s;
+  uint64_t sb0;
   if (SMALL) {
     int l = 0;
-    while (l + 1 < dl.nlev && dl.sb_first[l + 1] <= g) l++;
+    if (ONE) l = (int)blockIdx.x;
+    else
+      while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= blockIdx.x) l++;
     m = dl.meta[l];
-    s = g - dl.sb_first[l];
+    sb0 = ONE ? 0 : (blockIdx.x - dl.blk_first[l]) * DIR_GROUP;
   } else {
-    const int l = find_level(sb_first, nlev, g);
-    m = meta[l];
-    s = g - sb_first[l];
+    if (warp == 0) {
+      const int l = warp_find_level(blk_first, nlev, blockIdx.x);
+      if (lane == 0) {
+        sm = meta[l];
+        s_sb0 = (blockIdx.x - blk_first[l]) * DIR_GROUP;
+      }
+    }
+    __syncthreads();
+    m = sm;
+    sb0 = s_sb0;
   }
-  const uint64_t* ld = dir + m.dir_off;
+  // two superblocks at a time: lanes 0-15 the first, 16-31 the second, each
+  // lane two consecutive words (one 16-byte load where aligned)
+  const int hl = lane & 15, half = lane >> 4;
+  const uint64_t s0 = sb0 + (uint64_t)warp * DIR_SB_PER_WARP;
   const uint64_t* lb = bits + m.bit_off;
-  const uint64_t zb = ld[2 * s], ze = ld[2 * s + 2];
-  const uint64_t zs = ze - zb;
-  const uint64_t nvalid = std::min<uint64_t>(2048, m.n - 2048 * s);
-  const uint64_t ob = 2048 * s - zb, os = nvalid - zs;
-  // a whole superblock's words can all be read; the last one's, and those of a
-  // caller's bitvector off a 16-byte boundary, one by one up to the end
-  const bool whole = s + 1 < m.nsb && (((uintptr_t)lb) & 15) == 0;
-  const uint64_t nw = whole ? PADDED : (m.n + 63) / 64;
-  const uint64_t k0 = (zb + 4095) / 4096;
-  if (4096 * k0 < zb + zs)
-    samp[m.s0_off + k0] = 2048 * s + find_in_sb(lb, ld, s, 0, (uint32_t)(4096 * k0 - zb), nw);
-  const uint64_t k1 = (ob + 4095) / 4096;
-  if (4096 * k1 < ob + os)
-    samp[m.s1_off + k1] = 2048 * s + find_in_sb(lb, ld, s, 1, (uint32_t)(4096 * k1 - ob), nw);
+  const bool vec = (((uintptr_t)lb) & 15) == 0;
+  constexpr int NP = DIR_SB_PER_WARP / 2;
+  uint64_t w0[NP], w1[NP];
+  int v0[NP], v1[NP];
+#pragma unroll
+  for (int u = 0; u < NP; u++) {
+    const uint64_t s = s0 + 2 * u + half;
+    const int64_t rem = (int64_t)m.n - (int64_t)(2048 * s + 128 * (uint64_t)hl);
+    const bool live = s < m.nsb && rem > 0;
+    v0[u] = !live ? 0 : (rem >= 64 ? 64 : (int)rem);
+    v1[u] = (!live || rem <= 64) ? 0 : (rem >= 128 ? 64 : (int)(rem - 64));
+    const uint64_t* p = lb + 32 * s + 2 * hl;
+    // words past the last valid bit are not read (a caller bitvector may end there)
+    if (v1[u] && vec) {
+      const ulonglong2 q = __ldcs((const ulonglong2*)p);
+      w0[u] = q.x;
+      w1[u] = q.y;
+    } else {
+      w0[u] = v0[u] ? __ldcs(p) : 0ull;
+      w1[u] = v1[u] ? __ldcs(p + 1) : 0ull;
+    }
+  }
+  uint64_t rel[NP];
+#pragma unroll
+  for (int u = 0; u < NP; u++) {
+    const int z = v0[u] + v1[u] - __popcll(w0[u]) - __popcll(w1[u]);
+    int zi = z;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, zi, o, 16);
+      if (hl >= o) zi += y;
+    }
+    // zeros of 512-bit blocks 0, 1, 2 of the superblock: lanes 3, 7, 11 of its half
+    const uint64_t r1 = (uint64_t)__shfl_sync(FULL, zi, 3, 16);
+    const uint64_t r2 = (uint64_t)__shfl_sync(FULL, zi, 7, 16);
+    const uint64_t r3 = (uint64_t)__shfl_sync(FULL, zi, 11, 16);
+    rel[u] = (r1 << 16) | (r2 << 32) | (r3 << 48);
+    if (hl == 15) s_z[warp * DIR_SB_PER_WARP + 2 * u + half] = (uint32_t)zi;
+  }
+  __syncthreads();
+  // zeros before each of the warp's superblocks in the group: lane i the sum
+  // of the earlier warps' and of the warp's first i
+  static_assert(DIR_GROUP == 64, "two superblocks a lane");
+  const uint32_t a = s_z[2 * lane], b = s_z[2 * lane + 1];
+  uint32_t inc = a + b;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, inc, o);
+    if (lane >= o) inc += y;
+  }
+  const uint32_t total = __shfl_sync(FULL, inc, 31);
+#pragma unroll
+  for (int u = 0; u < NP; u++) {
+    const uint64_t s = s0 + 2 * u + half;
+    // superblock warp * 8 + 2 u + half of the group: lane warp * 4 + u holds its pair
+    const uint32_t pair = __shfl_sync(FULL, inc - a - b, warp * NP + u);
+    const uint32_t prev = __shfl_sync(FULL, a, warp * NP + u);
+    const uint32_t before = pair + (half ? prev : 0u);
+    if (hl == 0 && s < m.nsb) {
+      *(ulonglong2*)(dir + m.dir_off + 2 * s) = make_ulonglong2(before, rel[u]);
+      if (ONE) s_rel[warp * DIR_SB_PER_WARP + 2 * u + half] = rel[u];
+    }
+  }
+  if (!ONE) {
+    if (threadIdx.x == 0) blk_tot[blockIdx.x] = total;
+  } else {
+    if (threadIdx.x == 0) {
+      *(ulonglong2*)(dir + m.dir_off + 2 * m.nsb) = make_ulonglong2(total, 0ull);
+      if (zeros) zeros[blockIdx.x] = total;
+    }
+    __syncthreads();
+    if (warp < 2) {
+      const uint64_t i = 32 * warp + lane;
+      const uint32_t at = __shfl_sync(FULL, inc - a - b, 16 * warp + (lane >> 1));
+      const uint32_t pa = __shfl_sync(FULL, a, 16 * warp + (lane >> 1));
+      warp_samples(i < m.nsb, 32 * warp, at + ((lane & 1) ? pa : 0u), s_z[i], s_rel[i], m, lb, vec, samp);
+    }
+  }
+}
+
+// Exclusive prefix sums of tot[0 .. n) in place by the warps of a cluster of CL
+// blocks, each a contiguous range, four values a lane and step; returns the
+// grand total (to every thread).  (One block alone takes 36 us for the 65536
+// groups of 2^33 bits: an SM's loads in flight bound it; eight take 14.)
+template <int CL>
+__device__ uint64_t cluster_scan_range(uint64_t* tot, uint64_t n) {
+  namespace cg = cooperative_groups;
+  __shared__ uint64_t ws[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  const uint64_t per = ((n + nw * CL - 1) / (nw * CL) + 127) & ~127ull;
+  const uint64_t b0 = std::min<uint64_t>(per * (rank * nw + warp), n), b1 = std::min<uint64_t>(b0 + per, n);
+  uint64_t sum = 0;
+#pragma unroll 8
+  for (uint64_t i = b0 + lane; i < b1; i += 32) sum += tot[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+  if (lane == 0) ws[warp] = sum;
+  if (CL > 1) cg::this_cluster().sync();
+  else __syncthreads();
+  // lane w: warp w's sum of each block
+  uint64_t carry = 0, all = 0;
+  for (int r = 0; r < CL; r++) {
+    const uint64_t* rs = CL > 1 ? cg::this_cluster().map_shared_rank(ws, r) : ws;
+    const uint64_t x = lane < nw ? rs[lane] : 0ull;
+    uint64_t before = r < rank || (r == rank && lane < warp) ? x : 0ull, every = x;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      before += __shfl_xor_sync(FULL, before, o);
+      every += __shfl_xor_sync(FULL, every, o);
+    }
+    carry += before;
+    all += every;
+  }
+  if (CL > 1) cg::this_cluster().sync();  // the sums are read before a block ends
+  for (uint64_t i0 = b0; i0 < b1; i0 += 128) {
+    const uint64_t i = i0 + 4 * lane;
+    uint64_t v[4], x = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      v[k] = i + k < b1 ? tot[i + k] : 0ull;
+      x += v[k];
+    }
+    const uint64_t mine = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    uint64_t at = carry + x - mine;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (i + k < b1) tot[i + k] = at;
+      at += v[k];
+    }
+    carry += __shfl_sync(FULL, x, 31);
+  }
+  return all;
+}
+
+// The group totals of every level to prefix sums, and the level's total
+// record: SMALL a cluster of DIR_CLUSTER blocks per level, else one warp.
+constexpr int DIR_CLUSTER = 8;
+template <bool SMALL>
+__device__ __forceinline__ void dir_groups(int l, int rank, const LevelMeta* meta,
+                                           const uint64_t* blk_first, uint64_t* blk_tot,
+                                           uint64_t* dir, uint64_t* zeros, const DirLevels& dl) {
+  const uint64_t b0 = SMALL ? dl.blk_first[l] : blk_first[l];
+  const uint64_t b1 = SMALL ? dl.blk_first[l + 1] : blk_first[l + 1];
+  const uint64_t total = cluster_scan_range<SMALL ? DIR_CLUSTER : 1>(blk_tot + b0, b1 - b0);
+  if (rank == 0 && threadIdx.x == 0) {
+    const uint64_t off = SMALL ? dl.meta[l].dir_off + 2 * dl.meta[l].nsb
+                               : meta[l].dir_off + 2 * meta[l].nsb;
+    *(ulonglong2*)(dir + off) = make_ulonglong2(total, 0ull);
+    if (zeros) zeros[l] = total;
+  }
+}
+
+__global__ void __cluster_dims__(DIR_CLUSTER, 1, 1) __launch_bounds__(512)
+    k_dir_groups_small(uint64_t* blk_tot, uint64_t* dir, uint64_t* zeros,
+                       const __grid_constant__ DirLevels dl) {
+  dir_groups<true>((int)blockIdx.x / DIR_CLUSTER, (int)blockIdx.x % DIR_CLUSTER, nullptr, nullptr,
+                   blk_tot, dir, zeros, dl);
+}
+
+__global__ void __launch_bounds__(32) k_dir_groups(const LevelMeta* meta, const uint64_t* blk_first,
+                                                   uint64_t* blk_tot, uint64_t* dir, uint64_t* zeros,
+                                                   const __grid_constant__ DirLevels dl) {
+  dir_groups<false>((int)blockIdx.x, 0, meta, blk_first, blk_tot, dir, zeros, dl);
+}
+
+// Absolute counts and select samples: 64 threads per group.
+template <bool SMALL>
+__global__ void __launch_bounds__(256) k_dir_finish(const uint64_t* bits, const LevelMeta* meta,
+                                                    int nlev, const uint64_t* blk_first,
+                                                    uint64_t ngroups, const uint64_t* blk,
+                                                    uint64_t* dir, uint64_t* samp,
+                                                    const __grid_constant__ DirLevels dl) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t g = (uint64_t)blockIdx.x * (256 / DIR_GROUP) + threadIdx.x / DIR_GROUP;
+  const bool in = g < ngroups;
+  LevelMeta m;
+  uint64_t s0;
+  if (SMALL) {
+    int l = 0;
+    while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= g) l++;
+    m = dl.meta[l];
+    s0 = (g - dl.blk_first[l]) * DIR_GROUP;
+  } else {
+    const int l = warp_find_level(blk_first, nlev, g);
+    m = meta[l];
+    s0 = (g - blk_first[l]) * DIR_GROUP;
+  }
+  s0 += threadIdx.x % DIR_GROUP - lane;  // the warp's first superblock
+  const uint64_t s = s0 + lane;
+  const bool live = in && s < m.nsb;
+  uint64_t* const ld = dir + m.dir_off;
+  ulonglong2 rec = make_ulonglong2(0, 0);
+  uint64_t end = 0;  // zeros before the next superblock
+  if (live) {
+    rec = *(const ulonglong2*)(ld + 2 * s);
+    rec.x += blk[g];
+    // the last superblock of the level, and of the group
+    if (s + 1 == m.nsb) end = ld[2 * m.nsb];
+    else if ((s + 1) % DIR_GROUP == 0) end = blk[g + 1];
+    else if (lane == 31) end = blk[g] + ld[2 * s + 2];
+  }
+  const uint64_t next = __shfl_down_sync(FULL, rec.x, 1);
+  if (live && lane < 31 && s + 1 < m.nsb && (s + 1) % DIR_GROUP) end = next;
+  // the middle of a group is read by one warp and written by the other
+  __syncthreads();
+  if (live) ld[2 * s] = rec.x;
+  const uint64_t* lb = bits + m.bit_off;
+  warp_samples(live, s0, rec.x, (uint32_t)(end - rec.x), rec.y, m, lb, (((uintptr_t)lb) & 15) == 0, samp);
 }
 
 // ---------------------------------------------------------------------------
@@ -472,71 +668,66 @@ wt_status upload_meta(wt_struct* h) {
 }
 
 // Binary directories and select samples of nlev levels described by d_meta
-// (offsets relative to bits / dir / samp); sb_first: first superblock of each
-// level in one numbering, its first nlev + 1 entries used.  write_zeros: also store each
-// level's zero count in zeros[l].
+// or, when not null, by h_meta (offsets relative to bits / dir / samp); sb_first: first
+// superblock of each level in one numbering, its first nlev + 1 entries used.
+// zeros: when not null, each level's zero count is stored in zeros[l].
 wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32_t nlev,
                            const std::vector<uint64_t>& sb_first, uint64_t* dir, uint64_t* samp,
-                           uint64_t* zeros, int write_zeros, cudaStream_t st,
-                           const LevelMeta* h_meta) {
+                           uint64_t* zeros, cudaStream_t st, const LevelMeta* h_meta) {
   if (nlev == 0) return WT_OK;
-  const uint64_t total_sb = sb_first[nlev];
-  // blocks of the counting kernel: DIR_SB_PER_BLOCK superblocks of one level each
-  std::vector<uint64_t> firsts(2 * ((size_t)nlev + 1), 0);
-  std::copy(sb_first.begin(), sb_first.begin() + nlev + 1, firsts.begin());
-  uint64_t* blk_first = firsts.data() + nlev + 1;
-  for (uint32_t l = 0; l < nlev; l++) {
-    const uint64_t nsb = sb_first[l + 1] - sb_first[l];
-    blk_first[l + 1] = blk_first[l] + (nsb + DIR_SB_PER_BLOCK - 1) / DIR_SB_PER_BLOCK;
-  }
-  const uint64_t nblk = blk_first[nlev];
-  Work wk{st, {}};
-  uint64_t *d_first, *sbz, *sbx, *scr;
-  TRY(wk.get(&d_first, 2 * ((size_t)nlev + 1)));
-  TRY(wk.get(&sbz, std::max<uint64_t>(total_sb, 1)));
-  TRY(wk.get(&sbx, total_sb + 1));
-  TRY(wk.get(&scr, scan_scratch_pub(total_sb)));
-  TRY(upload(d_first, firsts.data(), firsts.size() * 8, st));
-  const unsigned fgrid = (unsigned)((total_sb + nlev + 255) / 256);
   // few levels with host metadata: the level tables go in the parameters
   const bool small = h_meta && nlev <= (uint32_t)DIR_SMALL;
+  std::vector<uint64_t> blk_first((size_t)nlev + 1, 0);
+  bool one = small;
+  for (uint32_t l = 0; l < nlev; l++) {
+    const uint64_t nsb = sb_first[l + 1] - sb_first[l];
+    blk_first[l + 1] = blk_first[l] + (nsb + DIR_GROUP - 1) / DIR_GROUP;
+    one = one && nsb <= (uint64_t)DIR_GROUP;
+  }
+  const uint64_t nblk = blk_first[nlev];
   DirLevels dl;
   memset(&dl, 0, sizeof(dl));
   if (small) {
     dl.nlev = (int)nlev;
-    for (uint32_t l = 0; l <= nlev; l++) {
-      dl.blk_first[l] = blk_first[l];
-      dl.sb_first[l] = sb_first[l];
-    }
+    for (uint32_t l = 0; l <= nlev; l++) dl.blk_first[l] = blk_first[l];
     for (uint32_t l = 0; l < nlev; l++) dl.meta[l] = h_meta[l];
   }
-  if (total_sb) {
-    if (small)
-      k_dir_count<true><<<(unsigned)nblk, 256, 0, st>>>(bits, d_meta, (int)nlev, d_first,
-                                                       d_first + nlev + 1, dir, sbz, dl);
-    else
-      k_dir_count<false><<<(unsigned)nblk, 256, 0, st>>>(bits, d_meta, (int)nlev, d_first,
-                                                        d_first + nlev + 1, dir, sbz, dl);
+  if (one) {
+    k_dir_count<true, true><<<nlev, 256, 0, st>>>(bits, nullptr, (int)nlev, nullptr, dir, nullptr,
+                                                  samp, zeros, dl);
     count_launch();
+    CK(cudaGetLastError());
+    return WT_OK;
   }
-  wt_status s = scan_excl_u64_pub(sbz, sbx, total_sb, scr, st);
-  if (s == WT_OK) {
-    k_dir_finish<<<fgrid, 256, 0, st>>>(d_meta, (int)nlev, d_first, total_sb, sbx, dir, zeros,
-                                        write_zeros);
+  Work wk{st, {}};
+  uint64_t *d_first = nullptr, *blk;
+  TRY(wk.get(&blk, nblk + 1));
+  const unsigned fgrid = (unsigned)((nblk + 256 / DIR_GROUP - 1) / (256 / DIR_GROUP));
+  if (small) {
+    k_dir_count<true, false><<<(unsigned)nblk, 256, 0, st>>>(bits, nullptr, (int)nlev, nullptr, dir,
+                                                            blk, samp, nullptr, dl);
+    k_dir_groups_small<<<nlev * DIR_CLUSTER, 512, 0, st>>>(blk, dir, zeros, dl);
+    k_dir_finish<true><<<fgrid, 256, 0, st>>>(bits, nullptr, (int)nlev, nullptr, nblk, blk, dir,
+                                              samp, dl);
+    count_launch(3);
+  } else {
+    TRY(wk.get(&d_first, (size_t)nlev + 1));
+    TRY(upload(d_first, blk_first.data(), blk_first.size() * 8, st));
+    if (nblk) {
+      k_dir_count<false, false><<<(unsigned)nblk, 256, 0, st>>>(bits, d_meta, (int)nlev, d_first, dir,
+                                                               blk, samp, nullptr, dl);
+      count_launch();
+    }
+    k_dir_groups<<<nlev, 32, 0, st>>>(d_meta, d_first, blk, dir, zeros, dl);
     count_launch();
-    if (total_sb) {
-      if (small)
-        k_select_samples<true><<<(unsigned)((total_sb + 255) / 256), 256, 0, st>>>(
-            bits, d_meta, (int)nlev, d_first, total_sb, dir, samp, dl);
-      else
-        k_select_samples<false><<<(unsigned)((total_sb + 255) / 256), 256, 0, st>>>(
-            bits, d_meta, (int)nlev, d_first, total_sb, dir, samp, dl);
+    if (nblk) {
+      k_dir_finish<false><<<fgrid, 256, 0, st>>>(bits, d_meta, (int)nlev, d_first, nblk, blk, dir,
+                                                 samp, dl);
       count_launch();
     }
   }
-  cudaError_t e = cudaGetLastError();
-  if (s != WT_OK) return s;
-  return e == cudaSuccess ? WT_OK : WT_ERR_CUDA;
+  CK(cudaGetLastError());
+  return WT_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -578,7 +769,7 @@ __device__ uint64_t dir_select(const uint64_t* lbits, const uint64_t* ldir, int 
   }
   const uint32_t r = (uint32_t)(q - occ_before<DIG>(ldir, b, lo));
   if (DIG) return 1024 * lo + find_in_dsb(lbits, ldir, lo, (uint32_t)b, r);
-  return 2048 * lo + find_in_sb(lbits, ldir, lo, b, r, nw);
+  return 2048 * lo + find_in_sb(lbits, ldir[2 * lo + 1], lo, b, r, nw);
 }
 
 // one (level, bit or digit value) of the directory build
@@ -871,12 +1062,14 @@ wt_status build_directories(wt_struct* h) {
   const uint64_t total_sb = sb_first[nlev];
   CK(dmalloc((void**)&h->d_dir, std::max<uint64_t>(h->dir_off[nlev], 1) * 8, st));
   CK(dmalloc((void**)&h->d_samp, std::max<uint64_t>(h->samp_off[NV * nlev], 1) * 8, st));
-  wt_status s = upload_meta(h);
+  // (queries on the uniform levels of a wavelet matrix or a balanced tree
+  // compute the offsets)
+  wt_status s = h->kind == WT_KIND_WM || h->kind == WT_KIND_WT ? WT_OK : upload_meta(h);
   if (s != WT_OK) return s;
   if (nlev == 0) return WT_OK;
   if (!dig) {
     s = dir_build_levels(h->d_bits_ro, h->d_meta, nlev, sb_first, h->d_dir, h->d_samp,
-                         h->d_zeros, h->kind == WT_KIND_RS ? 1 : 0, st, h->meta.data());
+                         h->kind == WT_KIND_RS ? h->d_zeros : nullptr, st, h->meta.data());
     if (s == WT_OK && (h->flags & WT_FLAG_SELECT_O1)) s = build_clark(h);
     return s;
   }
