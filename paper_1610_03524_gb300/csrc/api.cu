@@ -1,6 +1,7 @@
 // api.cu -- the C ABI (include/wavelet.h): argument checks, handle lifetime,
 // export.  Every computational step runs in the kernels of build.cu and
 // dirq.cu.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -28,14 +29,12 @@ wt_status check_opts(const wt_build_opts* o) {
   return WT_OK;
 }
 
-// sync: first wait for the work queued on the handle's stream (queries on
-// other streams included, through the caller's ordering), as wt_free does
+// sync: for an arena, wait for the release (wt_free waits for the others)
 void free_arrays(wt_struct* h, bool sync = false) {
   cudaStream_t st = h->stream;
   if (h->arena) {
     // the last handle of a batch returns the shared allocation
     if (h->arena->refs.fetch_sub(1) == 1) {
-      if (sync) cudaStreamSynchronize(st);
       dfree(h->arena->base, st);
       delete h->arena;
       // the memory is back in the pool, for allocations on any stream
@@ -44,11 +43,8 @@ void free_arrays(wt_struct* h, bool sync = false) {
     h->arena = nullptr;
     return;
   }
-  if (sync) cudaStreamSynchronize(st);
   dfree(h->d_bits, st);
   dfree(h->d_dir, st);
-  dfree(h->d_samp, st);
-  dfree(h->d_zeros, st);
   dfree(h->d_err, st);
   dfree(h->d_meta, st);
   dfree(h->d_code, st);
@@ -69,12 +65,14 @@ wt_status new_handle(wt_stream stream, uint64_t n, uint32_t sigma, wt_struct** o
   h->n = n;
   h->sigma = sigma;
   cudaGetDevice(&h->device);
-  if (dmalloc((void**)&h->d_err, 8, h->stream) != cudaSuccess) {
+  constexpr size_t bytes = 8 + 8 * MAX_LEVELS;
+  if (dmalloc((void**)&h->d_err, bytes, h->stream) != cudaSuccess) {
     free_arrays(h);
     delete h;
     return WT_ERR_NO_MEMORY;
   }
-  cudaMemsetAsync(h->d_err, 0, 8, h->stream);
+  h->d_zeros = (uint64_t*)h->d_err + 1;
+  cudaMemsetAsync(h->d_err, 0, bytes, h->stream);
   *out = h;
   return WT_OK;
 }
@@ -98,25 +96,24 @@ wt_status finish(wt_struct* h, wt_status s, wt_handle* out) {
 
 wt_status sync_handle(wt_struct* h) {
   if (h->deferred != WT_OK) return h->deferred;
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return h->deferred = WT_ERR_CUDA;
-  // small reads on the handle's own stream (not the legacy stream, which
-  // would wait for every other blocking stream of the device)
-  uint32_t err = 0;
-  e = cudaMemcpyAsync(&err, h->d_err, 4, cudaMemcpyDeviceToHost, h->stream);
+  // the error word and, the first time, the zero counts that follow it, read
+  // by one copy on the handle's own stream (not the legacy stream, which would
+  // wait for every other blocking stream of the device)
+  const bool zeros = !h->zeros_valid && h->bpe == 1 && h->levels;
+  uint64_t buf[1 + MAX_LEVELS] = {0};
+  cudaError_t e = cudaMemcpyAsync(buf, h->d_err, zeros && !h->arena ? 8 + 8 * (size_t)h->levels : 4,
+                                  cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess && zeros && h->arena)
+    e = cudaMemcpyAsync(buf + 1, h->d_zeros, 8 * (size_t)h->levels, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->deferred = WT_ERR_CUDA;
+  const uint32_t err = (uint32_t)buf[0];
   if (err & ERR_SYMBOL) return h->deferred = WT_ERR_SYMBOL_GE_SIGMA;
   // ERR_INTERNAL: a table disagreed with a tile
   if (err) return h->deferred = WT_ERR_CUDA;
   if (!h->zeros_valid) {
     h->zeros.assign(h->levels, 0);
-    if (h->levels && h->bpe == 1) {
-      e = cudaMemcpyAsync(h->zeros.data(), h->d_zeros, h->levels * 8, cudaMemcpyDeviceToHost,
-                          h->stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-      if (e != cudaSuccess) return h->deferred = WT_ERR_CUDA;
-    }
+    if (zeros) std::copy(buf + 1, buf + 1 + h->levels, h->zeros.begin());
     h->zeros_valid = true;
   }
   return WT_OK;
@@ -352,8 +349,7 @@ wt_status rs_build(const uint64_t* d_bits, uint64_t nbits, const wt_build_opts* 
   h->level_len.assign(1, nbits);
   h->level_off.assign(2, 0);
   h->level_off[1] = ((nbits + 2047) / 2048) * 32;
-  if (dmalloc((void**)&h->d_zeros, 8, h->stream) != cudaSuccess) s = WT_ERR_NO_MEMORY;
-  if (s == WT_OK) s = build_directories(h);
+  s = build_directories(h);
   return finish(h, s, out);
 }
 

@@ -517,7 +517,7 @@ static wt_status launch_hist_full(const void* seq, int w, uint64_t n, uint32_t s
   uint32_t ncopy = 1;
   uint64_t* dst = hist;
   uint32_t* dst32 = nullptr;
-  Work wk{st, {}};
+  Work wk{st};
   const bool narrow = n < (1ull << 32);
   if (!use_smem) {
     const uint64_t c32 = HIST_COPY_BYTES / (4ull * sigma);
@@ -996,20 +996,29 @@ struct NodePlan {
   uint64_t* C = nullptr;  // starts of the nodes of level a + t
 };
 
+// Count tables of the passes of a build with at most mt tiles each.
+struct PassTables {
+  uint32_t* tcnt = nullptr;
+  uint64_t* tchunk = nullptr;
+  void want(Work& wk, uint64_t mt) {
+    mt = std::max<uint64_t>(mt, 1);
+    wk.want(&tcnt, mt * TC_STRIDE);
+    wk.want(&tchunk, (std::min<uint64_t>((mt + 63) / 64, MAX_CHUNKS) + 1) * TC_STRIDE);
+  }
+};
+
 // One pass over at most mt tiles: every tile's digit counts, their prefix
 // sums across the tiles, what is planned from their totals, and the pass.
 template <bool BATCH, typename Launch>
-static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const PassPlan& plan,
-                          const NodePlan& np, cudaStream_t st, Launch&& launch) {
+static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const PassTables& tb,
+                          const PassPlan& plan, const NodePlan& np, cudaStream_t st,
+                          Launch&& launch) {
   mt = std::max<uint64_t>(mt, 1);
   PassParams Q = P;
   Q.chsh = (uint32_t)chunk_shift(mt);
   const uint32_t nchunk = (uint32_t)((mt + (1u << Q.chsh) - 1) >> Q.chsh);
-  Work wk{st, {}};
-  uint32_t* tcnt;
-  uint64_t* tchunk;
-  TRY(wk.get(&tcnt, mt * TC_STRIDE));
-  TRY(wk.get(&tchunk, ((uint64_t)nchunk + 1) * TC_STRIDE));
+  uint32_t* const tcnt = tb.tcnt;
+  uint64_t* const tchunk = tb.tchunk;
   // the zeroing belongs to the counts of a first pass (sigma set), else to
   // the pass
   if (!P.sigma) Q.clear = nullptr;
@@ -1052,11 +1061,12 @@ static wt_status launch_pass_w(const PassParams& Q, bool dig, uint64_t mt, const
   if (tile == 8192) return launch_pass_t<EW, false, false, 256>(Q, mt, o, st);
   return launch_pass_t<EW, false, false, PT / 32>(Q, mt, o, st);
 }
-static wt_status launch_pass(const PassParams& P, bool dig, uint64_t mt, const wt_build_opts* o,
-                             cudaStream_t st, const PassPlan& plan = PassPlan{},
+static wt_status launch_pass(const PassParams& P, bool dig, uint64_t mt, const PassTables& tb,
+                             const wt_build_opts* o, cudaStream_t st,
+                             const PassPlan& plan = PassPlan{},
                              const NodePlan& np = NodePlan{}, uint32_t tile = PT) {
   const int ew = P.in_w;
-  return run_pass<false>(P, mt, tile, plan, np, st, [&](const PassParams& Q, uint64_t m) {
+  return run_pass<false>(P, mt, tile, tb, plan, np, st, [&](const PassParams& Q, uint64_t m) {
     if (ew == 1) return launch_pass_w<1>(Q, dig, m, o, st, tile);
     if (ew == 2) return launch_pass_w<2>(Q, dig, m, o, st, tile);
     return launch_pass_w<4>(Q, dig, m, o, st, tile);
@@ -1066,7 +1076,11 @@ static wt_status launch_pass(const PassParams& P, bool dig, uint64_t mt, const w
 // Batched wavelet matrices: one launch over the tiles of every sequence in
 // P.segs (P.ntiles tiles in total), whose elements all have P.in_w bytes.
 wt_status launch_pass_batch(const PassParams& P, const wt_build_opts* o, cudaStream_t st) {
-  return run_pass<true>(P, P.ntiles, PT, PassPlan{}, NodePlan{}, st,
+  Work wk{st};
+  PassTables tb;
+  tb.want(wk, P.ntiles);
+  TRY(wk.take());
+  return run_pass<true>(P, P.ntiles, PT, tb, PassPlan{}, NodePlan{}, st,
                         [&](const PassParams& Q, uint64_t m) {
                           if (Q.in_w == 1) return launch_pass_t<1, false, true, PT / 32>(Q, m, o, st);
                           if (Q.in_w == 2) return launch_pass_t<2, false, true, PT / 32>(Q, m, o, st);
@@ -1092,8 +1106,6 @@ static wt_status alloc_outputs(wt_struct* h, uint64_t total_words, bool zero_bit
   // the partition passes store whole words and OR the words shared by
   // several tiles or nodes, so the level buffer starts at zero
   if (zero_bits) CK(cudaMemsetAsync(h->d_bits, 0, total_words * 8, h->stream));
-  CK(dmalloc((void**)&h->d_zeros, std::max<uint32_t>(h->levels, 1) * 8, h->stream));
-  CK(cudaMemsetAsync(h->d_zeros, 0, std::max<uint32_t>(h->levels, 1) * 8, h->stream));
   return WT_OK;
 }
 
@@ -1226,7 +1238,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   // the level buffer is zeroed by the build's kernels (the histogram kernel
   // the first pass's levels, each pass the next pass's), not by a memset
   TRY(alloc_outputs(h, W * L, n == 0));
-  Work wk{st, {}};
+  Work wk{st};
   if (n == 0) return build_directories(h);
   // levels per pass, symbols per tile and CTAs per SM: the caller's, else
   // the autotuner's for (L, ceil(log2 n)), else 4 / 4096 / the occupancy limit
@@ -1243,19 +1255,15 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   uint64_t* cls;
   int ncls = 0;
   for (auto& p : ps) ncls += (2 << p.t) + p.t + 1;
-  TRY(wk.get(&cls, ncls));
-  // intermediate sequences
-  void* seqbuf[2] = {nullptr, nullptr};
-  for (int g = 0; g + 1 < G; g++) {
-    if (!seqbuf[g & 1]) {
-      uint8_t* b;
-      TRY(wk.get(&b, (size_t)n * max_out_w(ps)));
-      seqbuf[g & 1] = b;
-    }
-  }
+  const uint64_t ntiles = (n + T - 1) / T;
+  PassTables tb;
+  uint8_t* seqbuf[2] = {nullptr, nullptr};  // intermediate sequences
+  wk.want(&cls, ncls);
+  tb.want(wk, ntiles);
+  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  TRY(wk.take());
   const void* in = d_seq;
   int coff = 0;
-  const uint64_t ntiles = (n + T - 1) / T;
   for (int g = 0; g < G; g++) {
     const PassGeom& pg = ps[g];
     PassParams P = base_params(h);
@@ -1283,7 +1291,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     }
     // every pass is planned from its own tiles' digit counts
     const PassPlan plan{PLAN_WM, pg.a, pg.t, cls + coff, nullptr, h->d_zeros};
-    TRY(launch_pass(P, false, ntiles, o, st, plan, NodePlan{}, T));
+    TRY(launch_pass(P, false, ntiles, tb, o, st, plan, NodePlan{}, T));
     coff += (2 << pg.t) + pg.t + 1;
     in = P.out;
   }
@@ -1310,29 +1318,28 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   // a tree of one pass has its level buffer zeroed by the counting kernel
   const bool one = G == 1;
   TRY(alloc_outputs(h, h->level_off.back(), !one || n == 0));
-  Work wk{st, {}};
+  Work wk{st};
   if (n == 0) return build_directories(h);
   const uint32_t T = PT;
   const uint64_t ntiles0 = (n + T - 1) / T;
   uint64_t *scr = nullptr, *tcnt = nullptr, *toff = nullptr;
   uint32_t* d_ntiles = nullptr;
   TileDesc* tiles = nullptr;
+  PassTables tb;
+  uint8_t* seqbuf[2] = {nullptr, nullptr};
+  std::vector<uint64_t*> Cs(G, nullptr);
+  const uint64_t max_nodes = (uint64_t)1 << ps.back().a;
+  for (int g = 0; g < G; g++) wk.want(&Cs[g], ((uint64_t)1 << (ps[g].a + ps[g].t)) + 1);
+  tb.want(wk, ntiles0 + (one ? 0 : max_nodes));
   if (!one) {
-    const uint64_t max_nodes = (uint64_t)1 << ps.back().a;
-    TRY(wk.get(&scr, scan_scratch(max_nodes)));
-    TRY(wk.get(&tcnt, max_nodes));
-    TRY(wk.get(&toff, max_nodes + 1));
-    TRY(wk.get(&tiles, ntiles0 + max_nodes + 1));
-    TRY(wk.get(&d_ntiles, 1));
+    wk.want(&scr, scan_scratch(max_nodes));
+    wk.want(&tcnt, max_nodes);
+    wk.want(&toff, max_nodes + 1);
+    wk.want(&tiles, ntiles0 + max_nodes + 1);
+    wk.want(&d_ntiles, 1);
   }
-  void* seqbuf[2] = {nullptr, nullptr};
-  for (int g = 0; g + 1 < G; g++) {
-    if (!seqbuf[g & 1]) {
-      uint8_t* b;
-      TRY(wk.get(&b, (size_t)n * max_out_w(ps)));
-      seqbuf[g & 1] = b;
-    }
-  }
+  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  TRY(wk.take());
   // Every pass is planned from its own tiles' digit counts (no histogram of
   // the symbols): C holds the starts of the nodes of level a, and the totals
   // of each node's tiles give those of level a + t.
@@ -1342,8 +1349,7 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     const PassGeom& pg = ps[g];
     PassParams P = base_params(h);
     const uint64_t nn = (uint64_t)1 << pg.a;
-    uint64_t* Cn;
-    TRY(wk.get(&Cn, (nn << pg.t) + 1));
+    uint64_t* const Cn = Cs[g];
     uint64_t mt = ntiles0;
     NodePlan np;
     if (g > 0) {
@@ -1379,7 +1385,7 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     P.ntiles = (uint32_t)ntiles0;
     P.n_in = n;
     const PassPlan plan{g == 0 ? PLAN_WT : PLAN_NONE, 0, pg.t, nullptr, Cn, nullptr};
-    TRY(launch_pass(P, multiary, mt, o, st, plan, np));
+    TRY(launch_pass(P, multiary, mt, tb, o, st, plan, np));
     in = P.out;
     C = Cn;
   }
@@ -1438,7 +1444,7 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
   if (sigma > (1u << 24)) return WT_ERR_UNSUPPORTED;
   h->kind = WT_KIND_HUFF;
   h->bpe = 1;
-  Work wk{st, {}};
+  Work wk{st};
   uint64_t* hist;
   TRY(wk.get(&hist, sigma));
   CK(cudaMemsetAsync(hist, 0, (size_t)sigma * 8, st));
@@ -1708,25 +1714,25 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
   uint64_t max_nodes = 1;
   for (int l = 0; l < Lm; l++) max_nodes = std::max<uint64_t>(max_nodes, node_lvl[3 * l + 2]);
   const uint64_t max_tiles = (n + T - 1) / T + max_nodes + 1;
-  TRY(wk.get(&d_off, Lm + 1));
-  TRY(wk.get(&d_len, Lm));
-  TRY(wk.get(&scr, scan_scratch(max_nodes)));
-  TRY(wk.get(&tcnt, max_nodes));
-  TRY(wk.get(&toff, max_nodes + 1));
-  TRY(wk.get(&tiles, max_tiles));
-  TRY(wk.get(&d_ntiles, 1));
+  PassTables tb;
+  uint8_t* seqbuf[2] = {nullptr, nullptr};
+  uint32_t* codes = (uint32_t*)d_seq;
+  uint64_t most = 0;  // tiles of a pass: by its elements and nodes
+  for (const PassGeom& p : ps)
+    most = std::max<uint64_t>(most, (h->level_len[p.a] + T - 1) / T + node_lvl[3 * p.a + 2]);
+  wk.want(&d_off, Lm + 1);
+  wk.want(&d_len, Lm);
+  wk.want(&scr, scan_scratch(max_nodes));
+  wk.want(&tcnt, max_nodes);
+  wk.want(&toff, max_nodes + 1);
+  wk.want(&tiles, max_tiles);
+  wk.want(&d_ntiles, 1);
+  tb.want(wk, most);
+  if (w < 4) wk.want(&codes, n);
+  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  TRY(wk.take());
   TRY(upload(d_off, h->level_off.data(), (Lm + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), Lm * 8, st));
-  void* seqbuf[2] = {nullptr, nullptr};
-  for (int g = 0; g + 1 < G; g++) {
-    if (!seqbuf[g & 1]) {
-      uint8_t* b;
-      TRY(wk.get(&b, (size_t)n * max_out_w(ps)));
-      seqbuf[g & 1] = b;
-    }
-  }
-  uint32_t* codes = (uint32_t*)d_seq;
-  if (w < 4) TRY(wk.get(&codes, n));
   {
     const unsigned grid = (unsigned)std::min<uint64_t>((n / 4 + 255) / 256 + 1, (uint64_t)num_sms() * 16);
     if (w == 1) k_map_codes<1><<<grid, 256, 0, st>>>(d_seq, n, d_left, codes);
@@ -1771,7 +1777,7 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
     P.shape = SHAPE_HUFF;
     P.hf_node = h->d_node;
     P.hf_lvl = h->d_node_lvl;
-    TRY(launch_pass(P, false, mt, o, st));
+    TRY(launch_pass(P, false, mt, tb, o, st));
     in = P.out;
   }
   if (o && (o->flags & WT_FLAG_NO_DIRECTORY)) return WT_OK;

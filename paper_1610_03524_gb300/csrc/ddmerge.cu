@@ -213,7 +213,6 @@ wt_status dd_merge(wt_struct* const* parts, uint32_t R, wt_struct* h) {
   for (int l = 0; l < L; l++) h->level_off[l + 1] = h->level_off[l] + W;
   CK(dmalloc((void**)&h->d_bits, std::max<uint64_t>(W * L, 1) * 8, st));
   h->d_bits_ro = h->d_bits;
-  CK(dmalloc((void**)&h->d_zeros, std::max(L, 1) * 8, st));
   // zero counts: the parts' sums
   h->zeros.assign(L, 0);
   for (uint32_t p = 0; p < R; p++)
@@ -230,7 +229,7 @@ wt_status dd_merge(wt_struct* const* parts, uint32_t R, wt_struct* h) {
     }
   const uint64_t stride = ((uint64_t)1 << L) - 1;  // nodes of levels 0 .. L-1
   const uint64_t nseg = (uint64_t)R * stride;
-  Work wk{st, {}};
+  Work wk{st};
   DdLevel* d_lv;
   uint64_t *cnt, *cs, *dst, *npc, *tot, *X, *PS, *scr;
   TRY(wk.get(&d_lv, hl.size()));

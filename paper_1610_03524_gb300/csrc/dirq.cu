@@ -39,18 +39,6 @@ wt_status scan_excl_u64_pub(const uint64_t* in, uint64_t* out, uint64_t n, uint6
                             cudaStream_t st);
 uint64_t scan_scratch_pub(uint64_t n);
 
-// the level holding superblock g: last l with first[l] <= g (levels with no
-// superblock share their first with the next level and are skipped)
-__device__ __forceinline__ int find_level(const uint64_t* first, int nlev, uint64_t g) {
-  int lo = 0, hi = nlev - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (first[mid] <= g) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 // r-th (0-based) set bit of v, by halving (__fns steps bit by bit)
 __device__ __forceinline__ uint32_t sel64(uint64_t v, uint32_t r) {
   uint32_t x = (uint32_t)v, at = 0;
@@ -108,14 +96,12 @@ constexpr int DIR_SB_PER_WARP = WT_DIR_SB_PER_WARP;
 constexpr int DIR_SB_PER_BLOCK = 8 * DIR_SB_PER_WARP;  // 256 threads
 constexpr int DIR_GROUP = DIR_SB_PER_BLOCK;
 
-// Up to DIR_SMALL levels: their first groups, first superblocks and
-// metadata ride in the kernel parameters, so a block finds its level without
+// Up to DIR_SMALL levels: their first groups and metadata ride in the kernel parameters, so a block finds its level without
 // a dependent load (else the tables are searched in global memory).
 constexpr int DIR_SMALL = 32;
 struct DirLevels {
   int nlev;
   uint64_t blk_first[DIR_SMALL + 1];
-  uint64_t sb_first[DIR_SMALL + 1];
   LevelMeta meta[DIR_SMALL];
 };
 
@@ -484,24 +470,24 @@ __device__ __forceinline__ uint64_t digit_match(uint64_t w, uint32_t d) {
   return ~(x | (x >> 1)) & 0x5555555555555555ull;
 }
 
-// The same counts, laid out like k_dir_count for up to DIR_SMALL levels:
-// DIR_SB_PER_BLOCK superblocks of one level per block, two superblocks per
-// warp step (each half-warp one: 16 lanes x two words = 1024 digits), 16-byte
-// loads.  A lane holds 64 digits, so the 256-digit blocks end at lanes 3, 7,
-// 11 of its half.
-__global__ void __launch_bounds__(256) k_mdir_count_blk(const uint64_t* bits, uint64_t total_sb,
-                                                        uint64_t* dir, uint64_t* sbz,
-                                                        const __grid_constant__ DirLevels dl) {
+// The same three launches for digit levels (there are never more than
+// DIR_SMALL): a group's records with the four values' counts before each
+// superblock in the group, two superblocks per warp step (each half-warp one:
+// 16 lanes x two words = 1024 digits).  A lane holds 64 digits, so the
+// 256-digit blocks end at lanes 3, 7, 11 of its half.  The group's totals of
+// value d into blk_tot[d * ngroups + group].
+__global__ void __launch_bounds__(256) k_mdir_count(const uint64_t* bits, uint64_t ngroups,
+                                                    uint64_t* dir, uint64_t* blk_tot,
+                                                    const __grid_constant__ DirLevels dl) {
+  __shared__ uint32_t s_z[4][DIR_GROUP];
   int l = 0;
   while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= blockIdx.x) l++;
   const LevelMeta m = dl.meta[l];
-  const uint64_t sb0 = (blockIdx.x - dl.blk_first[l]) * DIR_SB_PER_BLOCK;
-  const uint64_t g0 = dl.sb_first[l];
+  const uint64_t sb0 = (blockIdx.x - dl.blk_first[l]) * DIR_GROUP;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int hl = lane & 15, half = lane >> 4;
   const uint64_t s0 = sb0 + (uint64_t)warp * DIR_SB_PER_WARP;
   const uint64_t* lb = bits + m.bit_off;
-  const bool vec = (((uintptr_t)lb) & 15) == 0;
   constexpr int NP = DIR_SB_PER_WARP / 2;
   uint64_t w0[NP], w1[NP];
   int v0[NP], v1[NP];  // valid digits of the two words
@@ -512,22 +498,17 @@ __global__ void __launch_bounds__(256) k_mdir_count_blk(const uint64_t* bits, ui
     const bool live = s < m.nsb && rem > 0;
     v0[u] = !live ? 0 : (rem >= 32 ? 32 : (int)rem);
     v1[u] = (!live || rem <= 32) ? 0 : (rem >= 64 ? 32 : (int)(rem - 32));
-    const uint64_t* p = lb + 32 * s + 2 * hl;
-    if (v1[u] && vec) {
-      const ulonglong2 q = __ldcs((const ulonglong2*)p);
-      w0[u] = q.x;
-      w1[u] = q.y;
-    } else {
-      w0[u] = v0[u] ? __ldcs(p) : 0ull;
-      w1[u] = v1[u] ? __ldcs(p + 1) : 0ull;
-    }
+    ulonglong2 q = make_ulonglong2(0, 0);
+    if (live) q = __ldcs((const ulonglong2*)(lb + 32 * s + 2 * hl));  // levels are padded
+    w0[u] = q.x;
+    w1[u] = q.y;
   }
+  uint64_t rec[NP];  // lane hl < 4: the four values' counts before block hl
 #pragma unroll
   for (int u = 0; u < NP; u++) {
-    const uint64_t s = s0 + 2 * u + half;
     const uint64_t vm0 = v0[u] >= 32 ? ~0ull : ((1ull << (2 * v0[u])) - 1ull);
     const uint64_t vm1 = v1[u] >= 32 ? ~0ull : ((1ull << (2 * v1[u])) - 1ull);
-    uint64_t rec = 0;  // lane hl < 4: the four values' counts before block hl
+    rec[u] = 0;
 #pragma unroll
     for (int d = 0; d < 4; d++) {
       int ci = __popcll(digit_match(w0[u], d) & vm0) + __popcll(digit_match(w1[u], d) & vm1);
@@ -540,73 +521,54 @@ __global__ void __launch_bounds__(256) k_mdir_count_blk(const uint64_t* bits, ui
       const uint32_t r2 = (uint32_t)__shfl_sync(FULL, ci, 7, 16);
       const uint32_t r3 = (uint32_t)__shfl_sync(FULL, ci, 11, 16);
       const uint32_t rb = hl == 1 ? r1 : (hl == 2 ? r2 : (hl == 3 ? r3 : 0u));
-      rec |= (uint64_t)rb << (16 * d);
-      if (hl == 15 && s < m.nsb) sbz[(uint64_t)d * total_sb + g0 + s] = (uint64_t)ci;
+      rec[u] |= (uint64_t)rb << (16 * d);
+      if (hl == 15) s_z[d][warp * DIR_SB_PER_WARP + 2 * u + half] = (uint32_t)ci;
     }
-    if (hl < 4 && s < m.nsb) dir[m.dir_off + 8 * s + 4 + hl] = rec;
   }
-}
-
-__global__ void k_mdir_count(const uint64_t* bits, const LevelMeta* meta, int nlev,
-                             const uint64_t* sb_first, uint64_t total_sb, uint64_t* dir,
-                             uint64_t* sbz /* 4 x total_sb */) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t g = gw; g < total_sb; g += nw) {
-    const int l = find_level(sb_first, nlev, g);
-    const LevelMeta m = meta[l];
-    const uint64_t s = g - sb_first[l];
-    const int64_t rem = (int64_t)m.n - (int64_t)(1024 * s + 32 * (uint64_t)lane);
-    const int valid = rem <= 0 ? 0 : (rem >= 32 ? 32 : (int)rem);
-    const uint64_t w = valid ? bits[m.bit_off + 32 * s + lane] : 0ull;
-    const uint64_t vm = valid == 32 ? ~0ull : ((1ull << (2 * valid)) - 1ull);
-    uint64_t packed[4];
+  __syncthreads();
+  uint32_t before[NP];  // lane hl < 4: value hl before superblock u of its half
 #pragma unroll
-    for (int d = 0; d < 4; d++) {
-      int c = __popcll(digit_match(w, d) & vm);
-      int ci = c;
+  for (int u = 0; u < NP; u++) before[u] = 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, ci, o);
-        if (lane >= o) ci += y;
-      }
-      const uint64_t r1 = (uint64_t)__shfl_sync(FULL, ci, 7);
-      const uint64_t r2 = (uint64_t)__shfl_sync(FULL, ci, 15);
-      const uint64_t r3 = (uint64_t)__shfl_sync(FULL, ci, 23);
-      packed[d] = (r1 << 16) | (r2 << 32) | (r3 << 48);  // rel of blocks 1..3 for value d
-      if (lane == 31) sbz[(uint64_t)d * total_sb + g] = (uint64_t)ci;
+  for (int d = 0; d < 4; d++) {
+    const uint32_t a = s_z[d][2 * lane], b = s_z[d][2 * lane + 1];
+    uint32_t inc = a + b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL, inc, o);
+      if (lane >= o) inc += y;
     }
-    if (lane < 4) {
-      // record word 4+b holds the four values' counts of block b
-      const int b = lane;
-      uint64_t v = 0;
+    if (threadIdx.x == 31) blk_tot[(uint64_t)d * ngroups + blockIdx.x] = inc;
 #pragma unroll
-      for (int d = 0; d < 4; d++) v |= ((packed[d] >> (16 * b)) & 0xffffull) << (16 * d);
-      dir[m.dir_off + 8 * s + 4 + b] = v;
+    for (int u = 0; u < NP; u++) {
+      const uint32_t pair = __shfl_sync(FULL, inc - a - b, warp * NP + u);
+      const uint32_t prev = __shfl_sync(FULL, a, warp * NP + u);
+      if (hl == d) before[u] = pair + (half ? prev : 0u);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NP; u++) {
+    const uint64_t s = s0 + 2 * u + half;
+    if (hl < 4 && s < m.nsb) {
+      uint64_t* const r = dir + m.dir_off + 8 * s;
+      r[hl] = before[u];
+      r[4 + hl] = rec[u];
     }
   }
 }
 
-__global__ void k_mdir_finish(const LevelMeta* meta, int nlev, const uint64_t* sb_first,
-                              uint64_t total_sb, const uint64_t* sbx /* 4 x (total_sb+1) */,
-                              uint64_t* dir) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < total_sb) {
-    const int l = find_level(sb_first, nlev, g);
-    const uint64_t s = g - sb_first[l];
-    for (int d = 0; d < 4; d++) {
-      const uint64_t* x = sbx + (uint64_t)d * (total_sb + 1);
-      dir[meta[l].dir_off + 8 * s + d] = x[g] - x[sb_first[l]];
-    }
-  } else if (g < total_sb + nlev) {
-    const int l = (int)(g - total_sb);
-    const LevelMeta m = meta[l];
-    for (int d = 0; d < 4; d++) {
-      const uint64_t* x = sbx + (uint64_t)d * (total_sb + 1);
-      dir[m.dir_off + 8 * m.nsb + d] = x[sb_first[l + 1]] - x[sb_first[l]];
-      dir[m.dir_off + 8 * m.nsb + 4 + d] = 0;
-    }
+// The groups' totals of every level and value to prefix sums, and the
+// level's total record: a cluster per level and value.
+__global__ void __cluster_dims__(DIR_CLUSTER, 1, 1) __launch_bounds__(512)
+    k_mdir_groups(uint64_t ngroups, uint64_t* blk_tot, uint64_t* dir,
+                  const __grid_constant__ DirLevels dl) {
+  const int c = (int)blockIdx.x / DIR_CLUSTER, l = c >> 2, d = c & 3;
+  const uint64_t total = cluster_scan_range<DIR_CLUSTER>(
+      blk_tot + (uint64_t)d * ngroups + dl.blk_first[l], dl.blk_first[l + 1] - dl.blk_first[l]);
+  if (blockIdx.x % DIR_CLUSTER == 0 && threadIdx.x == 0) {
+    uint64_t* const r = dir + dl.meta[l].dir_off + 8 * dl.meta[l].nsb;
+    r[d] = total;
+    r[4 + d] = 0;
   }
 }
 
@@ -639,24 +601,67 @@ __device__ uint32_t find_in_dsb(const uint64_t* lbits, const uint64_t* ldir, uin
   return (uint32_t)((8 * b + at) * 32) + sel64(word, r) / 2;
 }
 
-// every 4096th occurrence of each digit value: one thread per superblock
-// (a superblock of 1024 digits holds at most one sample per value)
-__global__ void k_mdigit_samples(const uint64_t* bits, const LevelMeta* meta, int nlev,
-                                 const uint64_t* sb_first, uint64_t total_sb,
-                                 const uint64_t* dir, uint64_t* samp) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total_sb) return;
-  const int l = find_level(sb_first, nlev, g);
-  const LevelMeta m = meta[l];
-  const uint64_t s = g - sb_first[l];
-  const uint64_t* ld = dir + m.dir_off;
+// Absolute counts and the samples of each value (the position of every
+// 4096th occurrence): 64 threads per group, the warp's searches dealt to its
+// lanes.
+__global__ void __launch_bounds__(256) k_mdir_finish(const uint64_t* bits, uint64_t ngroups,
+                                                     const uint64_t* blk, uint64_t* dir,
+                                                     uint64_t* samp,
+                                                     const __grid_constant__ DirLevels dl) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t g = (uint64_t)blockIdx.x * (256 / DIR_GROUP) + threadIdx.x / DIR_GROUP;
+  const bool in = g < ngroups;
+  int l = 0;
+  while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= g) l++;
+  const LevelMeta m = dl.meta[l];
+  const uint64_t s0 = (g - dl.blk_first[l]) * DIR_GROUP + threadIdx.x % DIR_GROUP - lane;
+  const uint64_t s = s0 + lane;
+  const bool live = in && s < m.nsb;
+  uint64_t* const ld = dir + m.dir_off;
+  const bool lastsb = s + 1 == m.nsb, lastg = (s + 1) % DIR_GROUP == 0;
+  uint64_t at[4], end[4];
+#pragma unroll
+  for (int d = 0; d < 4; d++) {
+    const uint64_t* const bd = blk + (uint64_t)d * ngroups;
+    at[d] = end[d] = 0;
+    if (live) {
+      at[d] = bd[g] + ld[8 * s + d];
+      if (lastsb) end[d] = ld[8 * m.nsb + d];
+      else if (lastg) end[d] = bd[g + 1];
+      else if (lane == 31) end[d] = bd[g] + ld[8 * s + 8 + d];
+    }
+    const uint64_t next = __shfl_down_sync(FULL, at[d], 1);
+    if (live && lane < 31 && !lastsb && !lastg) end[d] = next;
+  }
+  // the middle of a group is read by one warp and written by the other
+  __syncthreads();
+  uint32_t has[4], first[5] = {0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int d = 0; d < 4; d++) {
+    if (live) ld[8 * s + d] = at[d];
+    has[d] = __ballot_sync(FULL, live && ((at[d] + 4095) & ~4095ull) < end[d]);
+    first[d + 1] = first[d] + __popc(has[d]);
+  }
   const uint64_t* lb = bits + m.bit_off;
   const uint64_t cap = m.n / 4096 + 1;
-  for (uint32_t d = 0; d < 4; d++) {
-    const uint64_t before = ld[8 * s + d], in = ld[8 * (s + 1) + d] - before;
-    const uint64_t k = (before + 4095) / 4096;
-    if (4096 * k < before + in)
-      samp[m.s0_off + d * cap + k] = 1024 * s + find_in_dsb(lb, ld, s, d, (uint32_t)(4096 * k - before));
+  for (uint32_t b = 0; b < first[4]; b += 32) {
+    const uint32_t task = b + lane;
+    const bool on = task < first[4];
+    const int d = task >= first[3] ? 3 : (task >= first[2] ? 2 : (task >= first[1] ? 1 : 0));
+    const uint32_t mask = d == 3 ? has[3] : (d == 2 ? has[2] : (d == 1 ? has[1] : has[0]));
+    const uint32_t f = d == 3 ? first[3] : (d == 2 ? first[2] : (d == 1 ? first[1] : 0u));
+    const int src = on ? nth_bit(mask, task - f) : 0;
+    uint64_t before = 0;
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const uint64_t x = __shfl_sync(FULL, at[e], src);
+      if (e == d) before = x;
+    }
+    if (on) {
+      const uint64_t ss = s0 + src, k = (before + 4095) >> 12;
+      samp[m.s0_off + (uint64_t)d * cap + k] =
+          1024 * ss + find_in_dsb(lb, ld, ss, (uint32_t)d, (uint32_t)(4096 * k - before));
+    }
   }
 }
 
@@ -699,7 +704,7 @@ wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32
     CK(cudaGetLastError());
     return WT_OK;
   }
-  Work wk{st, {}};
+  Work wk{st};
   uint64_t *d_first = nullptr, *blk;
   TRY(wk.get(&blk, nblk + 1));
   const unsigned fgrid = (unsigned)((nblk + 256 / DIR_GROUP - 1) / (256 / DIR_GROUP));
@@ -897,7 +902,7 @@ static wt_status build_clark(wt_struct* h) {
       std::vector<uint64_t> idx(occ.size());
       for (uint32_t l = 0; l < nlev; l++)
         for (int d = 0; d < 4; d++) idx[4 * l + d] = h->meta[l].dir_off + 8 * h->meta[l].nsb + d;
-      Work wk0{st, {}};
+      Work wk0{st};
       uint64_t *d_idx, *d_got;
       TRY(wk0.get(&d_idx, idx.size()));
       TRY(wk0.get(&d_got, idx.size()));
@@ -941,7 +946,7 @@ static wt_status build_clark(wt_struct* h) {
     }
   }
   const uint32_t nseg = (uint32_t)segs.size();
-  Work wk{st, {}};
+  Work wk{st};
   uint64_t *d_kind, *d_nh, *d_ns, *d_gh, *d_gs, *scr;
   CkSeg* d_segs;
   uint32_t* d_sub;
@@ -1059,12 +1064,13 @@ wt_status build_directories(wt_struct* h) {
     m.s0_off = h->samp_off[NV * l];
     m.s1_off = h->samp_off[NV * l + 1];
   }
-  const uint64_t total_sb = sb_first[nlev];
-  CK(dmalloc((void**)&h->d_dir, std::max<uint64_t>(h->dir_off[nlev], 1) * 8, st));
-  CK(dmalloc((void**)&h->d_samp, std::max<uint64_t>(h->samp_off[NV * nlev], 1) * 8, st));
-  // (queries on the uniform levels of a wavelet matrix or a balanced tree
-  // compute the offsets)
-  wt_status s = h->kind == WT_KIND_WM || h->kind == WT_KIND_WT ? WT_OK : upload_meta(h);
+  {
+    const uint64_t dir = (h->dir_off[nlev] + 31) / 32 * 32, samp = h->samp_off[NV * nlev];
+    CK(dmalloc((void**)&h->d_dir, std::max<uint64_t>(dir + samp, 1) * 8, st));
+    h->d_samp = h->d_dir + dir;
+  }
+  // (queries compute the offsets of levels of equal length)
+  wt_status s = h->kind == WT_KIND_HUFF ? upload_meta(h) : WT_OK;
   if (s != WT_OK) return s;
   if (nlev == 0) return WT_OK;
   if (!dig) {
@@ -1073,51 +1079,30 @@ wt_status build_directories(wt_struct* h) {
     if (s == WT_OK && (h->flags & WT_FLAG_SELECT_O1)) s = build_clark(h);
     return s;
   }
-  Work wk{st, {}};
-  uint64_t *d_first, *sbz, *sbx, *scr;
-  TRY(wk.get(&d_first, nlev + 1));
-  TRY(wk.get(&sbz, std::max<uint64_t>(total_sb, 1) * 4));
-  TRY(wk.get(&sbx, (total_sb + 1) * 4));
-  TRY(wk.get(&scr, scan_scratch_pub(total_sb)));
-  TRY(upload(d_first, sb_first.data(), (nlev + 1) * 8, st));
-  const unsigned fgrid = (unsigned)((total_sb + nlev + 255) / 256);
-  if (total_sb && nlev <= (uint32_t)DIR_SMALL) {
-    // blocks of DIR_SB_PER_BLOCK superblocks of one level, the level tables
-    // in the parameters
-    DirLevels dl;
-    memset(&dl, 0, sizeof(dl));
-    dl.nlev = (int)nlev;
-    for (uint32_t l = 0; l < nlev; l++) {
-      dl.blk_first[l + 1] =
-          dl.blk_first[l] + (h->meta[l].nsb + DIR_SB_PER_BLOCK - 1) / DIR_SB_PER_BLOCK;
-      dl.sb_first[l + 1] = sb_first[l + 1];
-      dl.meta[l] = h->meta[l];
-    }
-    k_mdir_count_blk<<<(unsigned)dl.blk_first[nlev], 256, 0, st>>>(h->d_bits_ro, total_sb,
-                                                                  h->d_dir, sbz, dl);
-    count_launch();
-  } else if (total_sb) {
-    // one warp per superblock: enough loads in flight to stream the bitmaps
-    const unsigned cgrid = (unsigned)std::min<uint64_t>((total_sb * 32 + 255) / 256 + 1, 1u << 24);
-    k_mdir_count<<<cgrid, 256, 0, st>>>(h->d_bits_ro, h->d_meta, nlev, d_first, total_sb,
-                                        h->d_dir, sbz);
+  DirLevels dl;
+  memset(&dl, 0, sizeof(dl));
+  dl.nlev = (int)nlev;
+  for (uint32_t l = 0; l < nlev; l++) {
+    dl.blk_first[l + 1] = dl.blk_first[l] + (h->meta[l].nsb + DIR_GROUP - 1) / DIR_GROUP;
+    dl.meta[l] = h->meta[l];
+  }
+  const uint64_t ng = dl.blk_first[nlev];
+  Work wk{st};
+  uint64_t* blk;
+  TRY(wk.get(&blk, 4 * ng + 1));
+  if (ng) {
+    k_mdir_count<<<(unsigned)ng, 256, 0, st>>>(h->d_bits_ro, ng, h->d_dir, blk, dl);
     count_launch();
   }
-  for (int d = 0; d < 4 && s == WT_OK; d++)
-    s = scan_excl_u64_pub(sbz + (uint64_t)d * total_sb, sbx + (uint64_t)d * (total_sb + 1),
-                          total_sb, scr, st);
-  if (s == WT_OK) {
-    k_mdir_finish<<<fgrid, 256, 0, st>>>(h->d_meta, nlev, d_first, total_sb, sbx, h->d_dir);
+  k_mdir_groups<<<nlev * 4 * DIR_CLUSTER, 512, 0, st>>>(ng, blk, h->d_dir, dl);
+  count_launch();
+  if (ng) {
+    constexpr int per = 256 / DIR_GROUP;
+    k_mdir_finish<<<(unsigned)((ng + per - 1) / per), 256, 0, st>>>(h->d_bits_ro, ng, blk, h->d_dir,
+                                                                    h->d_samp, dl);
     count_launch();
-    if (total_sb) {
-      k_mdigit_samples<<<(unsigned)((total_sb + 255) / 256), 256, 0, st>>>(
-          h->d_bits_ro, h->d_meta, nlev, d_first, total_sb, h->d_dir, h->d_samp);
-      count_launch();
-    }
   }
-  cudaError_t e = cudaGetLastError();
-  if (s != WT_OK) return s;
-  if (e != cudaSuccess) return WT_ERR_CUDA;
+  CK(cudaGetLastError());
   if (h->flags & WT_FLAG_SELECT_O1) return build_clark(h);
   return WT_OK;
 }
@@ -1164,15 +1149,15 @@ __device__ __forceinline__ BinLevel bin_level(const QStruct& S, int l) {
   v.n = m.n;
   v.nsb = m.nsb;
   v.zeros = S.zeros[l];
-  v.nw = S.kind == WT_KIND_RS ? (m.n + 63) / 64 : PADDED;
+  v.nw = PADDED;
   v.cm = S.cmeta ? S.cmeta + l : nullptr;
   v.ck64 = S.ck64;
   v.ck32 = S.ck32;
   return v;
 }
 
-// The same for a wavelet matrix or a balanced tree, whose levels all have n
-// bits: the offsets follow from n and l, so that no table read stands before
+// The same for a wavelet matrix, a balanced tree or a bitvector, whose levels
+// all have n bits: the offsets follow from n and l, so that no table read stands before
 // a level's first access.
 __device__ __forceinline__ BinLevel uniform_level(const QStruct& S, int l) {
   const uint64_t nsb = (S.n + 2047) >> 11, cap = (S.n >> 12) + 1;
@@ -1463,13 +1448,13 @@ struct DigLevel {
 };
 
 __device__ __forceinline__ DigLevel dig_level(const QStruct& S, int l) {
-  const LevelMeta m = S.meta[l];
+  const uint64_t nsb = (S.n + 1023) >> 10;  // digit levels all have n digits
   DigLevel v;
-  v.bits = S.bits + m.bit_off;
-  v.dir = S.dir + m.dir_off;
-  v.samp = S.samp + m.s0_off;
-  v.n = m.n;
-  v.nsb = m.nsb;
+  v.bits = S.bits + (uint64_t)l * 32 * nsb;
+  v.dir = S.dir + (uint64_t)l * 8 * (nsb + 1);
+  v.samp = S.samp + (uint64_t)l * 4 * ((S.n >> 12) + 1);
+  v.n = S.n;
+  v.nsb = nsb;
   v.cm = S.cmeta ? S.cmeta + l : nullptr;
   v.ck64 = S.ck64;
   v.ck32 = S.ck32;
@@ -1614,7 +1599,8 @@ __device__ uint64_t q_multi(const QStruct& S, int op, uint32_t c, uint64_t x) {
 }
 
 __device__ uint64_t q_rs(const QStruct& S, int op, uint32_t c, uint64_t x) {
-  const BinLevel v = bin_level(S, 0);
+  BinLevel v = uniform_level(S, 0);
+  v.nw = (S.n + 63) / 64;  // the caller's words
   if (op == 0) return x < S.n ? (uint64_t)get_bit(v, x) : NONE;
   if (c > 1) return NONE;
   if (op == 1) {
@@ -1716,7 +1702,7 @@ wt_status launch_query_multi(wt_struct* const* hs, uint32_t nh, const uint32_t* 
   if (q == 0) return WT_OK;
   std::vector<QStruct> tab(std::max<uint32_t>(nh, 1));
   for (uint32_t i = 0; i < nh; i++) fill_qstruct(hs[i], tab[i]);
-  Work wk{st, {}};
+  Work wk{st};
   QStruct* d_tab = nullptr;
   TRY(wk.get(&d_tab, tab.size()));
   TRY(upload(d_tab, tab.data(), tab.size() * sizeof(QStruct), st));

@@ -13,6 +13,8 @@
 
 namespace wtk {
 
+constexpr uint32_t MAX_LEVELS = 32;  // of any structure (symbols and codes have at most 32 bits)
+
 // One device allocation shared by the handles of a batched build; freed when
 // the last of them is freed.
 struct Arena {
@@ -70,9 +72,9 @@ struct wt_struct {
   uint64_t* d_bits = nullptr;
   const uint64_t* d_bits_ro = nullptr;  // == d_bits, or the caller's bitvector (RS)
   uint64_t* d_dir = nullptr;
-  uint64_t* d_samp = nullptr;
-  uint64_t* d_zeros = nullptr;   // [levels]
-  uint32_t* d_err = nullptr;     // device error word
+  uint64_t* d_samp = nullptr;    // in d_dir's allocation
+  uint32_t* d_err = nullptr;     // device error word (8 bytes), zeroed with the handle,
+  uint64_t* d_zeros = nullptr;   // and after it the levels' zero counts (batched: elsewhere)
   wtk::LevelMeta* d_meta = nullptr;
   // Huffman tables (device)
   uint32_t* d_code = nullptr;
@@ -140,6 +142,28 @@ struct Work {
     if (e != cudaSuccess) return WT_ERR_NO_MEMORY;
     bufs.push_back(q);
     *p = (T*)q;
+    return WT_OK;
+  }
+  // several buffers by one allocation: want() each, then take() them all (an
+  // allocation and its release cost the host about as much as a launch)
+  struct Want {
+    void** p;
+    size_t at;
+  };
+  std::vector<Want> wants;
+  size_t wanted = 0;
+  template <typename T>
+  void want(T** p, size_t count) {
+    wants.push_back(Want{(void**)p, wanted});
+    wanted += (count * sizeof(T) + 255) / 256 * 256;
+  }
+  wt_status take() {
+    uint8_t* b = nullptr;
+    const wt_status s = get(&b, wanted);
+    if (s != WT_OK) return s;
+    for (const Want& w : wants) *w.p = b + w.at;
+    wants.clear();
+    wanted = 0;
     return WT_OK;
   }
 };

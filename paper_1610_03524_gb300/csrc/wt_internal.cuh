@@ -40,9 +40,10 @@ constexpr int TC_STRIDE = 1 << TAU_MAX;  // row stride of both tables
 // Tiles per chunk: 64, so that a thread scans them in four rounds of 16 loads
 // (256 of them took 197 us for 2^20 tiles, 64 take 20), and more from 2^20
 // tiles on, so that the one block that scans the chunks walks at most 16384.
+constexpr uint64_t MAX_CHUNKS = 16384;
 inline int chunk_shift(uint64_t tiles) {
   int s = 6;
-  while ((tiles >> s) > 16384) s++;
+  while (((tiles + ((uint64_t)1 << s) - 1) >> s) > MAX_CHUNKS) s++;
   return s;
 }
 

@@ -69,3 +69,22 @@ def test_many_short_levels(wt):
         assert np.array_equal(ex.bits.reshape(ob.shape), ob) and np.array_equal(ex.zeros, oz)
         check_binary_dirs(ex, list(ob), [n] * ob.shape[0])
         h.free()
+
+
+@pytest.mark.parametrize("n", [0, 1, 1023, 1025, 32 * 1024 + 1, 64 * 1024 - 1, 64 * 1024,
+                               64 * 1024 + 1, 333333, 70 * 64 * 1024 + 9])
+@pytest.mark.parametrize("sigma", [2, 4, 77])
+def test_digit_directory(wt, n, sigma):
+    """Records and samples of every value of every digit level of a 4-ary tree."""
+    rng = np.random.default_rng(n + sigma)
+    S = np.where(rng.random(n) < 0.6, sigma - 1, rng.integers(0, sigma, n)).astype(np.uint8)
+    d = to_dev(S if n else np.zeros(1, np.uint8))
+    h = wt.multiary_build(d, sigma, n=n)
+    ex = h.export()
+    om = oracle.mwt_build(S, sigma)
+    assert ex.levels == om.shape[0]
+    for b in range(ex.levels):
+        assert np.array_equal(ex.level_dir(b), oracle.mwt_dir(om[b], n)), b
+        for v in range(4):
+            assert np.array_equal(ex.samples(b, v), oracle.digit_samples(om[b], n, v)), (b, v)
+    h.free()
