@@ -1038,6 +1038,12 @@ static wt_status build_clark(wt_struct* h) {
   return e == cudaSuccess ? WT_OK : WT_ERR_CUDA;
 }
 
+// A wavelet matrix keeps its symbols' starts (k_wm_starts) where the sequence
+// has at least START_MIN elements per entry, so that their walks (20 us for
+// 2^16 symbols) are a small part of a build.
+constexpr uint64_t START_MIN = 256;
+static wt_status build_starts(wt_struct* h);
+
 wt_status build_directories(wt_struct* h) {
   cudaStream_t st = h->stream;
   const uint32_t nlev = h->levels;
@@ -1065,9 +1071,12 @@ wt_status build_directories(wt_struct* h) {
     m.s1_off = h->samp_off[NV * l + 1];
   }
   {
-    const uint64_t dir = (h->dir_off[nlev] + 31) / 32 * 32, samp = h->samp_off[NV * nlev];
-    CK(dmalloc((void**)&h->d_dir, std::max<uint64_t>(dir + samp, 1) * 8, st));
+    const uint64_t dir = (h->dir_off[nlev] + 31) / 32 * 32, samp = (h->samp_off[NV * nlev] + 31) / 32 * 32;
+    const bool starts = h->kind == WT_KIND_WM && h->L <= 24 && h->n >> h->L >= START_MIN;
+    const uint64_t ns = starts ? ((uint64_t)1 << h->L) + 1 : 0;
+    CK(dmalloc((void**)&h->d_dir, std::max<uint64_t>(dir + samp + ns, 1) * 8, st));
     h->d_samp = h->d_dir + dir;
+    if (starts) h->d_start = h->d_samp + samp;
   }
   // (queries compute the offsets of levels of equal length)
   wt_status s = h->kind == WT_KIND_HUFF ? upload_meta(h) : WT_OK;
@@ -1076,6 +1085,7 @@ wt_status build_directories(wt_struct* h) {
   if (!dig) {
     s = dir_build_levels(h->d_bits_ro, h->d_meta, nlev, sb_first, h->d_dir, h->d_samp,
                          h->kind == WT_KIND_RS ? h->d_zeros : nullptr, st, h->meta.data());
+    if (s == WT_OK && h->d_start) s = build_starts(h);
     if (s == WT_OK && (h->flags & WT_FLAG_SELECT_O1)) s = build_clark(h);
     return s;
   }
@@ -1121,6 +1131,7 @@ struct QStruct {
   const uint64_t* samp;
   const LevelMeta* meta;
   const uint64_t* zeros;
+  const uint64_t* start;  // wavelet matrix: see k_wm_starts, or null
   HuffQuery hq;
   const ClarkMeta* cmeta;  // constant-time select directory, or null
   const uint64_t* ck64;
@@ -1270,27 +1281,37 @@ __device__ uint64_t select_b(const BinLevel& v, int bv, uint64_t k) {
 // Wavelet matrix.  The three operations walk down together, so that a warp
 // with a mixture of them walks once: rank and select carry the start s and
 // the end p of the symbol's class, access the position p alone.  Select then
-// walks up.
+// walks up.  Where the structure keeps the symbols' starts (k_wm_starts),
+// rank carries its position alone and select does not walk down: half of the
+// lines of a rank (2^22 of them on n = 2^30: 1.79 -> 1.50 ms), and of the
+// latency of a select.
 __device__ uint64_t q_wm(const QStruct& S, int op, uint32_t c, uint64_t x) {
   const int L = S.L;
   if (op == 2 ? x == 0 : x >= S.n) return NONE;
   if (op != 0 && c >= S.sigma) return NONE;
   uint64_t s = 0, p = op == 0 ? x : (op == 1 ? x + 1 : S.n);
+  const bool starts = S.start != nullptr, both = op != 0 && !starts;
   uint32_t sym = 0;
-  for (int l = 0; l < L; l++) {
-    const BinLevel v = uniform_level(S, l);
-    const Line lp = load_line(v, p);
-    Line ls;
-    int b = (int)((c >> (L - 1 - l)) & 1u);
-    if (op == 0) b = get_bit(v, p);
-    else ls = load_line(v, s);
-    const uint64_t zp = zeros_before(lp, p);
-    p = b ? v.zeros + (p - zp) : zp;
-    if (op == 0) {
-      sym = (sym << 1) | (uint32_t)b;
-    } else {
-      const uint64_t zs = zeros_before(ls, s);
-      s = b ? v.zeros + (s - zs) : zs;
+  if (starts && op != 0) {
+    const uint32_t r = rev_bits(c, L);
+    s = S.start[r];
+    if (op == 2) p = S.start[r + 1];
+  }
+  if (!(starts && op == 2)) {
+    for (int l = 0; l < L; l++) {
+      const BinLevel v = uniform_level(S, l);
+      const Line lp = load_line(v, p);
+      Line ls;
+      int b = (int)((c >> (L - 1 - l)) & 1u);
+      if (op == 0) b = get_bit(v, p);
+      if (both) ls = load_line(v, s);
+      const uint64_t zp = zeros_before(lp, p);
+      p = b ? v.zeros + (p - zp) : zp;
+      if (op == 0) sym = (sym << 1) | (uint32_t)b;
+      if (both) {
+        const uint64_t zs = zeros_before(ls, s);
+        s = b ? v.zeros + (s - zs) : zs;
+      }
     }
   }
   if (op == 0) return sym;
@@ -1303,6 +1324,22 @@ __device__ uint64_t q_wm(const QStruct& S, int op, uint32_t c, uint64_t x) {
     pos = select_b(v, b, b ? pos - v.zeros : pos);
   }
   return pos;
+}
+
+// Wavelet matrix: the start of every symbol's class in the order after the
+// last level (ascending in the symbol's L bits reversed), entry r for the
+// symbol rev(r), and n at the end: one walk down per symbol.
+__global__ void __launch_bounds__(64) k_wm_starts(const QStruct S, uint64_t* start) {
+  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x, nr = 1u << S.L;
+  if (r == 0) start[nr] = S.n;
+  if (r >= nr) return;
+  uint64_t s = 0;
+  for (int l = 0; l < S.L; l++) {
+    const BinLevel v = uniform_level(S, l);
+    const uint64_t z = rank0(v, s);
+    s = (r >> l) & 1u ? v.zeros + (s - z) : z;
+  }
+  start[r] = s;
 }
 
 // Balanced tree: the node's start s and end e, and the position p in it
@@ -1640,6 +1677,7 @@ static void fill_qstruct(const wt_struct* h, QStruct& S) {
   S.samp = h->d_samp;
   S.meta = h->d_meta;
   S.zeros = h->d_zeros;
+  S.start = h->d_start;
   S.hq.code = h->d_code;
   S.hq.len = h->d_len;
   S.hq.sym_by_rank = h->d_sym_by_rank;
@@ -1656,6 +1694,15 @@ static void fill_qstruct(const wt_struct* h, QStruct& S) {
 // Threads per block: single warps while they all fit on the SMs at once, so
 // that a small batch spreads over all of them.
 static unsigned query_block(uint64_t q) { return q <= (uint64_t)num_sms() * 512 ? 32u : 128u; }
+
+static wt_status build_starts(wt_struct* h) {
+  QStruct S;
+  fill_qstruct(h, S);
+  k_wm_starts<<<((1u << h->L) + 63) / 64, 64, 0, h->stream>>>(S, h->d_start);
+  count_launch();
+  CK(cudaGetLastError());
+  return WT_OK;
+}
 
 wt_status launch_query(wt_struct* h, int op, const uint32_t* c, const uint64_t* x, uint64_t q,
                        uint64_t* out, cudaStream_t st) {

@@ -73,6 +73,7 @@ struct wt_struct {
   const uint64_t* d_bits_ro = nullptr;  // == d_bits, or the caller's bitvector (RS)
   uint64_t* d_dir = nullptr;
   uint64_t* d_samp = nullptr;    // in d_dir's allocation
+  uint64_t* d_start = nullptr;   // (there too) wavelet matrix: the symbols' starts, or null
   uint32_t* d_err = nullptr;     // device error word (8 bytes), zeroed with the handle,
   uint64_t* d_zeros = nullptr;   // and after it the levels' zero counts (batched: elsewhere)
   wtk::LevelMeta* d_meta = nullptr;
@@ -144,27 +145,39 @@ struct Work {
     *p = (T*)q;
     return WT_OK;
   }
-  // several buffers by one allocation: want() each, then take() them all (an
-  // allocation and its release cost the host about as much as a launch)
+  // several buffers: want() each, then take() them all; the small ones by one
+  // allocation (an allocation and its release cost the host about as much as a
+  // launch), the large ones each by its own, so that the pool finds blocks of
+  // their sizes again in the next build (one 4 GB block for all of them was
+  // split by the next build's levels and mapped anew: 0.3 ms)
+  static constexpr size_t LARGE = 32u << 20;
   struct Want {
     void** p;
-    size_t at;
+    size_t bytes;
   };
   std::vector<Want> wants;
-  size_t wanted = 0;
   template <typename T>
   void want(T** p, size_t count) {
-    wants.push_back(Want{(void**)p, wanted});
-    wanted += (count * sizeof(T) + 255) / 256 * 256;
+    wants.push_back(Want{(void**)p, (count * sizeof(T) + 255) / 256 * 256});
   }
   wt_status take() {
+    size_t small = 0, at = 0;
+    for (const Want& w : wants) small += w.bytes < LARGE ? w.bytes : 0;
     uint8_t* b = nullptr;
-    const wt_status s = get(&b, wanted);
-    if (s != WT_OK) return s;
-    for (const Want& w : wants) *w.p = b + w.at;
+    wt_status s = get(&b, small);
+    for (const Want& w : wants) {
+      if (s != WT_OK) return s;
+      if (w.bytes >= LARGE) {
+        uint8_t* q = nullptr;
+        s = get(&q, w.bytes);
+        *w.p = q;
+      } else {
+        *w.p = b + at;
+        at += w.bytes;
+      }
+    }
     wants.clear();
-    wanted = 0;
-    return WT_OK;
+    return s;
   }
 };
 

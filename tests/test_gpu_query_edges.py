@@ -91,3 +91,31 @@ def test_one_launch_mixes_the_operations(wt, kind, n, sigma):
     wt.query_multi([h], to_dev(np.zeros(q, np.uint32)), to_dev(op), to_dev(c), to_dev(x), out)
     assert np.array_equal(from_dev_u64(out), exp)
     h.free()
+
+
+@pytest.mark.parametrize("sigma", [2, 3, 256, 300])
+@pytest.mark.parametrize("per", [255, 256, 257])
+def test_matrix_queries_with_and_without_starts(wt, sigma, per):
+    """Rank and select of every symbol (present or not) on both sides of the
+    length from which a matrix keeps its symbols' starts."""
+    import torch
+    L = max(1, (sigma - 1).bit_length())
+    n = per << L
+    rng = np.random.default_rng(n)
+    S = (rng.integers(0, sigma, n) // 2 * 2 % sigma).astype(np.uint16)  # odd symbols absent
+    h = wt.wm_build(to_dev(S), sigma)
+    c = np.repeat(np.arange(sigma + 1, dtype=np.uint32), 6)
+    x = np.tile(np.array([0, 1, n // 3, n - 1, n, per], np.uint64), sigma + 1)
+    out = torch.empty(c.size, dtype=torch.int64, device="cuda")
+    h.rank(to_dev(c), to_dev(x), out)
+    rank = from_dev_u64(out).copy()
+    h.select(to_dev(c), to_dev(x), out)
+    sel = from_dev_u64(out)
+    pos = [np.flatnonzero(S == v) for v in range(sigma + 1)]
+    for t in range(c.size):
+        v, a = int(c[t]), int(x[t])
+        ok = v < sigma and a < n
+        assert rank[t] == (np.searchsorted(pos[v], a, side="right") if ok else UMAX)
+        ok = v < sigma and 1 <= a <= pos[v].size
+        assert sel[t] == (pos[v][a - 1] if ok else UMAX)
+    h.free()
