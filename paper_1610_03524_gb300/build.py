@@ -18,7 +18,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwavelet.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["build.cu", "dirq.cu", "api.cu", "huffman.cpp", "noalloc.cu", "batch.cu", "server.cu",
-           "ddmerge.cu"]
+           "ddmerge.cu", "huffdev.cu"]
 
 
 def nvcc() -> str:

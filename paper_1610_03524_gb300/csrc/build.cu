@@ -1437,18 +1437,11 @@ __global__ void __launch_bounds__(256) k_map_codes(const void* in, uint64_t n, c
 uint32_t huffman_lengths(const uint64_t* hist, uint32_t sigma, uint32_t cap, uint8_t* len);
 void canonical_codes(const uint8_t* len, uint32_t sigma, uint32_t* code);
 
-// d_seq: the library's own copy of the sequence (16-byte aligned), overwritten
-wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
-                     const wt_build_opts* o, wt_struct* h) {
+// The code tables from the symbol counts (or the caller's lengths), on the
+// host: codes, node table, zero counts, level lengths.
+static wt_status huff_tables_host(const uint64_t* hist, uint32_t sigma, const uint8_t* h_len,
+                                  wt_struct* h, uint32_t* d_left, std::vector<uint64_t>& node_lvl) {
   cudaStream_t st = h->stream;
-  if (sigma > (1u << 24)) return WT_ERR_UNSUPPORTED;
-  h->kind = WT_KIND_HUFF;
-  h->bpe = 1;
-  Work wk{st};
-  uint64_t* hist;
-  TRY(wk.get(&hist, sigma));
-  CK(cudaMemsetAsync(hist, 0, (size_t)sigma * 8, st));
-  TRY(launch_hist_full(d_seq, w, n, sigma, hist, h->d_err, st));
   std::vector<uint64_t> hh(sigma);
   uint32_t err = 0;
   CK(cudaMemcpyAsync(hh.data(), hist, (size_t)sigma * 8, cudaMemcpyDeviceToHost, st));
@@ -1611,7 +1604,7 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
     for (int l = 0; l <= Lw; l++) first_gt[l] = std::min<uint64_t>(first_gt[l], np);
   }
   h->level_len.assign(Lm, 0);
-  std::vector<uint64_t> node_lvl(3 * (size_t)Lw, 0);
+  node_lvl.assign(3 * (size_t)Lw, 0);
   std::vector<uint64_t> zc(Lw, 0);
   std::vector<uint64_t> node;
   {
@@ -1664,9 +1657,6 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
     zc[l] = h->level_len[l] - ones[l];
     node[node_lvl[3 * l] + nn[l]] = h->level_len[l];  // sentinel = level length
   }
-  h->level_off.assign(Lm + 1, 0);
-  for (int l = 0; l < Lm; l++) h->level_off[l + 1] = h->level_off[l] + level_words(h->level_len[l]);
-  TRY(alloc_outputs(h, std::max<uint64_t>(h->level_off.back(), 1)));
   // zero counts per level: elements whose code bit l is 0
   h->zeros.assign(zc.begin(), zc.begin() + Lm);
   if (Lm) CK(cudaMemcpyAsync(h->d_zeros, h->zeros.data(), Lm * 8, cudaMemcpyHostToDevice, st));
@@ -1689,8 +1679,6 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
   CK(dmalloc((void**)&h->d_len_tab, lentab.size() * 8, st));
   CK(dmalloc((void**)&h->d_node, std::max<size_t>(node.size(), 1) * 8, st));
   CK(dmalloc((void**)&h->d_node_lvl, node_lvl.size() * 8, st));
-  uint32_t* d_left;
-  TRY(wk.get(&d_left, sigma));
   CK(cudaMemcpyAsync(h->d_code, h->code.data(), (size_t)sigma * 4, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(h->d_len, h->code_len.data(), sigma, cudaMemcpyHostToDevice, st));
   if (!order.empty())
@@ -1701,6 +1689,71 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
   CK(cudaMemcpyAsync(h->d_node_lvl, node_lvl.data(), node_lvl.size() * 8, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_left, left.data(), (size_t)sigma * 4, cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));  // host vectors above are pageable and local
+  return WT_OK;
+}
+
+wt_status huff_tables_device(const uint64_t* hist, uint64_t n, uint32_t sigma, wt_struct* h,
+                             uint32_t* d_left, std::vector<uint64_t>& node_lvl, bool* done);
+
+// Alphabets from which the code is built on the device: its launches take
+// about 0.6 ms whatever the alphabet, the host about 1 ms for 2^16 symbols and
+// 16 ms for 2^20 (and no time of the device's, if another build has it).
+constexpr uint32_t HUFF_DEVICE_MIN = 1u << 16;
+
+// Copies of h->d_len and h->d_code into the handle's host vectors, ordered after
+// what is on its stream at begin(), made by finish() on another stream.
+struct HostCopies {
+  cudaEvent_t ready = nullptr;
+  cudaStream_t xs = nullptr;
+  wt_status begin(wt_struct* h) {
+    CK(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+    CK(cudaEventRecord(ready, h->stream));
+    return WT_OK;
+  }
+  wt_status finish(wt_struct* h) {
+    if (!ready) return WT_OK;
+    CK(cudaStreamCreateWithFlags(&xs, cudaStreamNonBlocking));
+    CK(cudaStreamWaitEvent(xs, ready, 0));
+    h->code_len.resize(h->sigma);
+    h->code.resize(h->sigma);
+    CK(cudaMemcpyAsync(h->code_len.data(), h->d_len, h->sigma, cudaMemcpyDeviceToHost, xs));
+    CK(cudaMemcpyAsync(h->code.data(), h->d_code, (size_t)h->sigma * 4, cudaMemcpyDeviceToHost, xs));
+    CK(cudaStreamSynchronize(xs));
+    return WT_OK;
+  }
+  ~HostCopies() {
+    if (xs) cudaStreamDestroy(xs);
+    if (ready) cudaEventDestroy(ready);
+  }
+};
+
+// d_seq: the library's own copy of the sequence (16-byte aligned), overwritten
+wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8_t* h_len,
+                     const wt_build_opts* o, wt_struct* h) {
+  cudaStream_t st = h->stream;
+  if (sigma > (1u << 24)) return WT_ERR_UNSUPPORTED;
+  h->kind = WT_KIND_HUFF;
+  h->bpe = 1;
+  Work wk{st};
+  uint64_t* hist;
+  TRY(wk.get(&hist, sigma));
+  CK(cudaMemsetAsync(hist, 0, (size_t)sigma * 8, st));
+  TRY(launch_hist_full(d_seq, w, n, sigma, hist, h->d_err, st));
+  uint32_t* d_left;
+  TRY(wk.get(&d_left, sigma));
+  std::vector<uint64_t> node_lvl;
+  bool dev = false;
+  if (!h_len && n && n < (1ull << 32) && sigma >= HUFF_DEVICE_MIN)
+    TRY(huff_tables_device(hist, n, sigma, h, d_left, node_lvl, &dev));
+  if (!dev) TRY(huff_tables_host(hist, sigma, h_len, h, d_left, node_lvl));
+  const int Lm = (int)h->max_code_len;
+  h->level_off.assign(Lm + 1, 0);
+  for (int l = 0; l < Lm; l++) h->level_off[l + 1] = h->level_off[l] + level_words(h->level_len[l]);
+  TRY(alloc_outputs(h, std::max<uint64_t>(h->level_off.back(), 1)));
+  // the handle's host copies of device-built codes: by a stream of their own,
+  // while the passes run
+  HostCopies copies;
+  if (dev) TRY(copies.begin(h));
   if (n == 0 || Lm == 0) return build_directories(h);
   // the pass kernel wants hf_lvl as [off, first] pairs plus the count; use a
   // 3-wide table and read [3l], [3l+1], [3l+2]
@@ -1780,8 +1833,8 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
     TRY(launch_pass(P, false, mt, tb, o, st));
     in = P.out;
   }
-  if (o && (o->flags & WT_FLAG_NO_DIRECTORY)) return WT_OK;
-  return build_directories(h);
+  if (!(o && (o->flags & WT_FLAG_NO_DIRECTORY))) TRY(build_directories(h));
+  return copies.finish(h);
 }
 
 
