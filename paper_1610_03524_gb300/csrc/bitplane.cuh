@@ -118,9 +118,12 @@ WT_HD int pop32(uint32_t x) {
 #endif
 }
 
-// The moves of a compress within each byte (Hacker's Delight, 2nd edition,
-// section 7-4, on four bytes at once): the bits at the set positions of m to
-// their byte's low end, in order, in conditional shifts by 1, 2 and 4.
+// The moves of a compress within each byte (after Hacker's Delight, 2nd
+// edition, section 7-4, on four bytes at once): the bits at the set positions of
+// m to their byte's high end, in order, in conditional shifts by 1, 2 and 4.  A
+// shift to the left of the bits t of x, whose places are free, is the
+// multiplication-addition x + t (2^s - 1): half of the work goes to the
+// multipliers instead of the logic pipe that bounds the pass.
 struct ByteCompress {
   uint32_t m, mv[3];
 };
@@ -128,15 +131,15 @@ struct ByteCompress {
 WT_HD ByteCompress byte_compress_plan(uint32_t m) {
   ByteCompress c;
   c.m = m;
-  uint32_t mk = (~m << 1) & 0xFEFEFEFEu;
+  uint32_t mk = (~m >> 1) & 0x7F7F7F7Fu;
 #pragma unroll
   for (int i = 0; i < 3; i++) {
-    uint32_t mp = mk ^ ((mk << 1) & 0xFEFEFEFEu);
-    mp ^= (mp << 2) & 0xFCFCFCFCu;
-    mp ^= (mp << 4) & 0xF0F0F0F0u;
+    uint32_t mp = mk ^ ((mk >> 1) & 0x7F7F7F7Fu);
+    mp ^= (mp >> 2) & 0x3F3F3F3Fu;
+    mp ^= (mp >> 4) & 0x0F0F0F0Fu;
     const uint32_t mv = mp & m;
     c.mv[i] = mv;
-    m = (m ^ mv) | (mv >> (1 << i));
+    m += mv * ((1u << (1 << i)) - 1u);
     mk &= ~mp;
   }
   return c;
@@ -145,43 +148,54 @@ WT_HD ByteCompress byte_compress_plan(uint32_t m) {
 WT_HD uint32_t byte_compress(const ByteCompress& c, uint32_t x) {
   x &= c.m;
 #pragma unroll
-  for (int i = 0; i < 3; i++) {
-    const uint32_t t = x & c.mv[i];
-    x = (x ^ t) | (t >> (1 << i));
-  }
+  for (int i = 0; i < 3; i++) x += (x & c.mv[i]) * ((1u << (1 << i)) - 1u);
   return x;
 }
 
-// The stable split of 32 elements by plane b: the planes x[0..N) with the
-// zeros' bits first, the ones' bits after them.  Each byte is split by
-// itself, then the eight pieces are put together by multiplications with
-// powers of two: five stages on whole words would take half as many masks
-// again and all of them on the logic pipe.  (Fewer than 32 elements: the
-// bits past them set in every plane keep them behind the others.)
+WT_HD uint32_t reverse32(uint32_t x) {
+#ifdef __CUDA_ARCH__
+  return __brev(x);
+#else
+  uint32_t r = 0;
+  for (int i = 0; i < 32; i++) r |= ((x >> i) & 1u) << (31 - i);
+  return r;
+#endif
+}
+
+// The stable split of 32 elements by plane b, the first element in the top bit
+// here: the planes x[0..N) with the zeros' bits first (on top), the ones' bits
+// after them.  Each byte is split by itself, then its two pieces move up by the
+// bits of the other kind above it.  (Fewer than 32 elements: the bits past them
+// set in every plane keep them behind the others.)
 template <int N>
 WT_HD void split_planes(uint32_t b, uint32_t* x) {
   const ByteCompress c0 = byte_compress_plan(~b), c1 = byte_compress_plan(b);
-  // zeros per byte; where each byte's zeros and ones go
+  // zeros per byte; zeros above each byte, and ones
   uint32_t n = ~b - ((~b >> 1) & 0x55555555u);
   n = (n & 0x33333333u) + ((n >> 2) & 0x33333333u);
   n = (n + (n >> 4)) & 0x0F0F0F0Fu;
-  const uint32_t z = (n * 0x01010101u) >> 24;
-  const uint32_t pz = n * 0x01010100u, po = z * 0x01010101u + 0x18100800u - pz;
-  uint32_t fz[4], fo[4];
+  const uint32_t q = n * 0x01010101u, z = q >> 24;
+  const uint32_t zeros = z * 0x01010101u - q, ones = 0x00081018u - zeros;
+  uint32_t fz[3], fo[3];
 #pragma unroll
-  for (int k = 0; k < 4; k++) {
-    fz[k] = 1u << ((pz >> (8 * k)) & 31u);
-    fo[k] = 1u << ((po >> (8 * k)) & 31u);  // 32: no ones there
+  for (int k = 0; k < 3; k++) {
+    fz[k] = low_mask((ones >> (8 * k)) & 31u);
+    fo[k] = low_mask((zeros >> (8 * k)) & 31u);
   }
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const uint32_t l = byte_compress(c0, x[i]), h = byte_compress(c1, x[i]);
-    uint32_t r = l & 0xffu;
+    uint32_t l = byte_compress(c0, x[i]), h = byte_compress(c1, x[i]);
+    const uint32_t l0 = l, h0 = h;
 #pragma unroll
-    for (int k = 1; k < 4; k++) r += ((l >> (8 * k)) & 0xffu) * fz[k];
-#pragma unroll
-    for (int k = 0; k < 4; k++) r += ((h >> (8 * k)) & 0xffu) * fo[k];
-    x[i] = r;
+    for (int k = 0; k < 3; k++) {
+      l += (l0 & (0xffu << (8 * k))) * fz[k];
+      h += (h0 & (0xffu << (8 * k))) * fo[k];
+    }
+#ifdef __CUDA_ARCH__
+    x[i] = l | __funnelshift_rc(h, 0u, z);
+#else
+    x[i] = l | (z < 32 ? h >> z : 0u);
+#endif
   }
 }
 

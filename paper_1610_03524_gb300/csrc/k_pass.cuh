@@ -29,7 +29,10 @@
 // form moved the elements once per level through shared memory (a ballot, a
 // rank and a store per 32 elements and level): 231 and 198 warp instructions
 // per 32 elements for its two passes of 8 levels, 14.3 ms for the 2^30 16-bit
-// symbols of 16 levels; the four passes here take 69 (46 the last) and 10.8 ms.
+// symbols of 16 levels.  The four passes here took 69 (46 the last) and 10.8 ms
+// with the first element in a plane's low bit; with it in the top bit, where
+// half of a split's moves are multiplications, they take 10.1 ms (2^28 symbols:
+// 2.74 and 2.53 ms; 2^26 32-bit ones 0.93 and 0.86).
 #pragma once
 #include <type_traits>
 
@@ -177,7 +180,7 @@ struct PassSmem {
 
 // CTAs per SM the register budget is sized for, at 128 threads
 #ifndef WT_PASS_CTAS
-#define WT_PASS_CTAS 7
+#define WT_PASS_CTAS 8
 #endif
 template <int EW, int NT>
 struct PassCtas {
@@ -502,21 +505,21 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     const uint32_t d1 = p[1];  // digit levels: the second bit of the first digit
     // (one copy of the code for every t: the last levels' splits are the same)
     if (t >= 2) {
-      uint32_t x[4] = {p[0], p[1], p[2], p[3]};
-      if (t == 3) {
-        x[1] = p[0];
-        x[2] = p[1];
-        x[3] = p[2];
-      } else if (t == 2) {
-        x[2] = p[0];
-        x[3] = p[1];
+      uint32_t x[4];  // the first element in the top bit
+      if (t == 4) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) x[j] = reverse32(p[j]);
+      } else {
+        x[1] = reverse32(p[0]);
+        x[2] = t == 3 ? reverse32(p[1]) : x[1];
+        x[3] = reverse32(t == 3 ? p[2] : p[1]);
       }
       if (t == 4) split_planes<3>(x[0], x + 1);
       if (t >= 3) split_planes<2>(x[1], x + 2);
       if (!DIG || t == 3) split_planes<1>(x[2], x + 3);
-      p[1] = t == 4 ? x[1] : (t == 3 ? x[2] : x[3]);
-      p[2] = t == 4 ? x[2] : x[3];
-      p[3] = x[3];
+      p[1] = reverse32(t == 4 ? x[1] : (t == 3 ? x[2] : x[3]));
+      p[2] = reverse32(t == 4 ? x[2] : x[3]);
+      p[3] = reverse32(x[3]);
     }
 
     if (!bad) {
