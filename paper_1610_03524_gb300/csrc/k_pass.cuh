@@ -10,14 +10,16 @@
 // together.  The counts of the 2^t keys in the earlier threads (a prefix sum
 // over the tile, two 16-bit counts a word) place those pieces in the tile's
 // runs, one per (level, class), which are assembled in shared memory at the
-// bit alignment they have in the output and leave as whole words; words that
-// several tiles or nodes share (the "boundary" words of Section 4.2) are
-// merged with atomicOr into the level buffer, which is zero before the pass
+// alignment they have in the output's 16-byte units; units that several tiles
+// or nodes share (the "boundary" words of Section 4.2) are merged with
+// atomicOr into the level buffer, which is zero before the pass
 // (in a wavelet-matrix build each tile zeroes its share of the next pass's
 // levels).  The same counts give every element's place in the tile's stable
 // order by key: each thread walks its elements once with a pointer per key,
-// and the runs of T_{a+t}, again assembled at their output alignment, leave in
-// 16-byte stores (big nodes, Section 3), narrowed to the bits still needed.
+// and the runs of T_{a+t} (big nodes, Section 3), narrowed to the bits still
+// needed, are again assembled at their output alignment.  One bulk copy takes
+// each run out, behind the loads of the next tile; its first and last unit, if
+// not the run's alone, are written piecewise.
 //
 // The digit counts of all earlier tiles of a tile's sequence or node come from
 // prefix sums, taken before the pass, of every tile's digit counts: the
@@ -31,8 +33,10 @@
 // per 32 elements for its two passes of 8 levels, 14.3 ms for the 2^30 16-bit
 // symbols of 16 levels.  The four passes here took 69 (46 the last) and 10.8 ms
 // with the first element in a plane's low bit; with it in the top bit, where
-// half of a split's moves are multiplications, they take 10.1 ms (2^28 symbols:
-// 2.74 and 2.53 ms; 2^26 32-bit ones 0.93 and 0.86).
+// half of a split's moves are multiplications, 10.1 ms (2^28 symbols: 2.74 and
+// 2.53 ms; 2^26 32-bit ones 0.93 and 0.86), and with the runs taken out by bulk
+// copies instead of a search for the run and a store for every word 64 (43) and
+// 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).
 #pragma once
 #include <type_traits>
 
@@ -130,6 +134,20 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {  // 4 or 
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Bulk copies from shared to global memory (both 16-byte aligned, a multiple
+// of 16 bytes): issued by one thread, which waits until its copies have read
+// their source; other threads' writes to the source are fenced before the
+// barrier that precedes the copy.
+__device__ __forceinline__ void bulk_store(uint64_t dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_addr(src)),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t a) {
   unsigned short v;
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
@@ -163,19 +181,19 @@ __device__ __forceinline__ uint64_t spread32(uint32_t v) {
 // row per thread padded by 16 bytes (eight lanes' 16-byte reads of their rows
 // then fall on all banks); the elements in key order, each key's run at its
 // output's 16-byte alignment (and before that the prefix sums' scratch); the
-// level bits, each run at its output's 64-bit alignment.
+// level bits, each run at its output's 16-byte alignment too.
 template <int EW, int NT>
 struct PassSmem {
   static constexpr int T = 32 * NT, RS = 32 * EW + 16;
   static constexpr int KEYS = 1 << TAU_MAX, RUNS = KEYS - 1;
   static constexpr int SCRW = 8 * 32 + 3 * 8;                   // scratch words per warp
-  static constexpr int AREA = TAU_MAX * T / 64 + 2 * RUNS + 2;  // 64-bit words
+  static constexpr int AREA = TAU_MAX * T / 128 + 2 * RUNS + 2;  // 16-byte units
   static constexpr int SRT = T * EW + 32 * KEYS > NT / 32 * SCRW * 4 ? T * EW + 32 * KEYS : NT / 32 * SCRW * 4;
   static constexpr size_t off_ptr = 0;
   static constexpr size_t off_in = off_ptr + (size_t)(NT / 32) * 1024;
   static constexpr size_t off_srt = off_in + (size_t)NT * RS;
   static constexpr size_t off_area = off_srt + (size_t)SRT;
-  static constexpr size_t bytes = off_area + (size_t)AREA * 8;
+  static constexpr size_t bytes = off_area + (size_t)AREA * 16;
 };
 
 // CTAs per SM the register budget is sized for, at 128 threads
@@ -188,12 +206,12 @@ struct PassCtas {
   static constexpr int value = NT == 64 ? 2 * at128 : (NT == 128 ? at128 : at128 / 2);
 };
 
-// One run of a tile on its way out: units (words or chunks) first .. last - 1
-// of its area are the run's alone; unit i goes to address base + i * size
-// (base == 0: nowhere).
+// One run of a tile on its way out: the 16-byte units first .. last - 1 of its
+// area are the run's alone, its area has n units from unit `at` on; unit i goes
+// to address base + 16 i (base == 0: nowhere).
 struct __align__(16) Run {
   uint64_t base;
-  uint32_t first, last;
+  uint32_t first, last, at, n;
 };
 
 template <typename E, bool DIG, bool BATCH, int NT>
@@ -220,12 +238,10 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   __shared__ uint32_t s_own[KEYS];  // the tile's key counts by the tables
   __shared__ bool s_over[2];        // a run past its level's or the sequence's end
   // the runs of level bits that are not empty, and those of the next
-  // sequence, in order: first word of the area (16-byte chunk), and the words
-  // (chunks) the run holds whole with the address word (chunk) 0 would have
-  __shared__ uint32_t s_rs[2][KEYS];
+  // sequence; the latter's offset in the first unit, bytes << 8
   __shared__ Run s_run[2][KEYS];
-  __shared__ uint32_t s_n[2], s_nr;  // their words and chunks; runs of the next sequence
-  __shared__ uint32_t s_edge[KEYS];  // offset in the first chunk, bytes << 8
+  __shared__ uint32_t s_nr[2];
+  __shared__ uint32_t s_edge[KEYS];
   __shared__ __align__(16) uint32_t s_ab[KEYS];  // a run's first bit, from shared memory's start
   __shared__ __align__(16) uint32_t s_sb[8];  // where a key's first element goes in s_srt, two keys a word
 
@@ -298,7 +314,6 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     }
   };
 
-  for (int i = tid; i < SM::AREA; i += NT) s_area[i] = 0ull;
   if (BATCH && tid < 2) s_P[tid] = P0;
   if (P0.shape == SHAPE_HUFF) {
     if (tid < 3 * (TAU_MAX + 1))
@@ -326,7 +341,9 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     // use the DRAM bandwidth the tile's compute leaves idle)
     if (!BATCH && P0.clear) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid, NT);
     cp_async_wait();
+    if (warp < 2) bulk_wait_read();  // the last tile's runs have left
     __syncthreads();
+    for (int i = tid; i < SM::AREA; i += NT) ((uint4*)s_area)[i] = make_uint4(0u, 0u, 0u, 0u);
 
     // ---- 1. where the runs go (from the tables; a warp for the level bits',
     //      one for the next sequence's), and the next tile -------------------
@@ -366,7 +383,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       } else if (P.out == nullptr) {
         c = 0;
       }
-      uint32_t n = 0, len = 0, off = 0;  // area words or chunks; bits or bytes; offset in the first
+      uint32_t n = 0, len = 0, off = 0;  // 16-byte units; bits or bytes; offset in the first
       uint64_t where = 0;                // address of the first (0: nowhere)
       bool over = false;
       if (c) {
@@ -388,9 +405,9 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
           const uint64_t G0 = b0 * bpe;
           len = c * bpe;
           over = !dead && G0 + len > lbits;  // never for consistent tables
-          off = (uint32_t)(G0 & 63);
-          n = (off + len + 63) >> 6;
-          where = (uint64_t)(uintptr_t)(P.bits + lwords + (G0 >> 6));
+          off = (uint32_t)(G0 & 127);
+          n = (off + len + 127) >> 7;
+          where = (uint64_t)(uintptr_t)(P.bits + lwords + 2 * (G0 >> 7));
         }
         if (dead) where = 0;
       }
@@ -400,29 +417,26 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
         const uint32_t y = __shfl_up_sync(FULL, first, o);
         if (lane >= o) first += y;
       }
-      const uint32_t total = __shfl_sync(FULL, first, 15);
       first -= n;
       const uint32_t some = __ballot_sync(FULL, n != 0u);
-      const int at = __popc(some & lanemask_lt()), runs = __popc(some);
-      if (lane >= runs && lane < KEYS) s_rs[half][lane] = ~0u;
       if (n) {
-        const int sh = half ? 4 : 6, usz = half ? 16 : 8;  // unit: 16-byte chunk, or word of 64 bits
-        s_rs[half][at] = first;
+        const int at = __popc(some & lanemask_lt()), sh = half ? 4 : 7;  // a unit's bytes or bits
         Run r;
-        r.base = where ? where - (uint64_t)first * usz : 0ull;
+        r.base = where ? where - 16ull * first : 0ull;
         r.first = where ? first + (off ? 1u : 0u) : ~0u;
         r.last = where ? first + ((off + len) >> sh) : 0u;
+        r.at = first;
+        r.n = n;
         s_run[half][at] = r;
         if (half) s_edge[at] = where ? off | (len << 8) : 0u;
       }
       if (lane < KEYS) {
         if (half) ((uint16_t*)s_sb)[lane] = (uint16_t)(16 * first + off);
-        else s_ab[lane] = 8 * smem_addr(s_area) + 64 * first + off;
+        else s_ab[lane] = 8 * smem_addr(s_area) + 128 * first + off;
       }
       const bool stop = __any_sync(FULL, over);
       if (lane == 0) {
-        s_n[half] = total;
-        if (half) s_nr = (uint32_t)runs;
+        s_nr[half] = (uint32_t)__popc(some);
         s_over[half] = stop;
       }
     }
@@ -628,6 +642,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
         else if (EW == 4) move(std::integral_constant<int, 4>{});
       }
     }
+    fence_async_smem();
     __syncthreads();
     if (more) {  // behind the stores below
       load_tile(cur ^ 1);
@@ -635,43 +650,36 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     }
     if (bad) continue;  // uniform; nothing was put into the areas
 
-    // ---- 6. level words out, and the areas back to zero; T_{a+t} out ------
-    // A warp takes 32 consecutive units; a lane's run is the last one that
-    // starts at or before its unit: the number of starts up to the window's
-    // first unit, and a bit per start inside the window.
-    auto each = [&](int half, auto&& f) {
-      const uint32_t total = s_n[half];
-      const uint32_t start = lane < 16 ? s_rs[half][lane] : ~0u;
-      for (uint32_t b = 32 * warp; b < total; b += NT) {
-        const uint32_t before = __popc(__ballot_sync(FULL, start <= b));
-        const uint32_t in = __reduce_or_sync(FULL, start > b && start < b + 32 ? 1u << (start - b) : 0u);
-        const uint32_t i = b + lane;
-        if (i < total) f(i, s_run[half][before - 1 + __popc(in << (31 - lane))]);
+    // ---- 6. the runs out: whole 16-byte units by bulk copies, a lane per run
+    //      (one warp for the level bits', one for the next sequence's) --------
+    if (warp < 2) {
+      if (lane < (int)s_nr[warp]) {
+        const Run r = s_run[warp][lane];
+        const unsigned char* const from = warp == 0 ? (const unsigned char*)s_area : s_srt;
+        if (r.last > r.first && r.base)
+          bulk_store(r.base + 16ull * r.first, from + 16 * r.first, 16 * (r.last - r.first));
       }
-    };
-    each(0, [&](uint32_t i, const Run& r) {
-      const uint64_t x = s_area[i];
-      s_area[i] = 0ull;
-      uint64_t* const wp = (uint64_t*)(uintptr_t)r.base + i;
-      // stored when the run holds the whole word, else ORed
-      if (i >= r.first && i < r.last) *wp = x;
-      else if (x && r.base) atomicOr((unsigned long long*)wp, (unsigned long long)x);
-    });
+      bulk_commit();
+    }
+    // the units at the runs' ends, shared with other tiles: level words ORed ...
+    for (uint32_t e = tid; e < 4 * s_nr[0]; e += NT) {
+      const Run r = s_run[0][e >> 2];
+      const uint32_t u = r.at + ((e & 2) ? r.n - 1 : 0u);
+      if (((e & 2) && r.n == 1) || (u >= r.first && u < r.last)) continue;
+      const uint64_t x = s_area[2 * u + (e & 1)];
+      if (x && r.base)
+        atomicOr((unsigned long long*)(uintptr_t)(r.base + 16ull * u + 8 * (e & 1)), (unsigned long long)x);
+    }
+    // ... and elements four bytes a thread, one by one where not all are the run's
     if (P.out != nullptr) {
-      each(1, [&](uint32_t i, const Run& r) {
-        if (i >= r.first && i < r.last)
-          *((uint4*)(uintptr_t)r.base + i) = *((const uint4*)s_srt + i);
-      });
-      // the chunks at the runs' ends that other tiles share: four bytes a
-      // thread, by elements where not all of them are the run's
-      for (uint32_t e = tid; e < 8 * s_nr; e += NT) {
+      for (uint32_t e = tid; e < 8 * s_nr[1]; e += NT) {
         const uint32_t at = e >> 3, b = 4 * (e & 3), oe = s_edge[at];
         const uint32_t off = oe & 0xffu, end = off + (oe >> 8);
-        const uint32_t k = (e & 4) ? (end - 1) >> 4 : 0u;  // last chunk or first
+        const uint32_t k = (e & 4) ? (end - 1) >> 4 : 0u;  // last unit or first
         const uint32_t lo = k ? 0u : off, hi = min(end - 16 * k, 16u);
         // once only, and only if not stored whole above
         if (oe == 0u || ((e & 4) && k == 0u) || hi - lo == 16u) continue;
-        const uint32_t i = s_rs[1][at] + k;
+        const uint32_t i = s_run[1][at].at + k;
         const unsigned char* from = s_srt + 16 * i + b;
         unsigned char* to = (unsigned char*)(uintptr_t)(s_run[1][at].base + 16ull * i) + b;
         if (lo <= b && b + 4 <= hi) {
@@ -687,6 +695,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       }
     }
   }
+  if (warp < 2) bulk_wait();
 }
 
 }  // namespace wtk
