@@ -128,21 +128,33 @@ struct ByteCompress {
   uint32_t m, mv[3];
 };
 
-WT_HD ByteCompress byte_compress_plan(uint32_t m) {
-  ByteCompress c;
-  c.m = m;
-  uint32_t mk = (~m >> 1) & 0x7F7F7F7Fu;
+// The moves for the bits at m (c1) and for the others (c0).  Bit i of a byte
+// has 7 - i bits above it, so whether the zeros above it are odd in number
+// gives the same of the ones: one prefix parity serves both first shifts.
+WT_HD void byte_compress_plans(uint32_t m, ByteCompress& c0, ByteCompress& c1) {
+  const uint32_t mk0 = (m >> 1) & 0x7F7F7F7Fu;
+  uint32_t par = mk0 ^ ((mk0 >> 1) & 0x7F7F7F7Fu);
+  par ^= (par >> 2) & 0x3F3F3F3Fu;
+  par ^= (par >> 4) & 0x0F0F0F0Fu;
 #pragma unroll
-  for (int i = 0; i < 3; i++) {
-    uint32_t mp = mk ^ ((mk >> 1) & 0x7F7F7F7Fu);
-    mp ^= (mp >> 2) & 0x3F3F3F3Fu;
-    mp ^= (mp >> 4) & 0x0F0F0F0Fu;
-    const uint32_t mv = mp & m;
-    c.mv[i] = mv;
-    m += mv * ((1u << (1 << i)) - 1u);
-    mk &= ~mp;
+  for (int h = 0; h < 2; h++) {
+    ByteCompress& c = h ? c1 : c0;
+    uint32_t x = h ? m : ~m, mk = h ? (~m >> 1) & 0x7F7F7F7Fu : mk0;
+    c.m = x;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      uint32_t mp = h ? par ^ 0x55555555u : par;
+      if (i) {
+        mp = mk ^ ((mk >> 1) & 0x7F7F7F7Fu);
+        mp ^= (mp >> 2) & 0x3F3F3F3Fu;
+        mp ^= (mp >> 4) & 0x0F0F0F0Fu;
+      }
+      const uint32_t mv = mp & x;
+      c.mv[i] = mv;
+      x += mv * ((1u << (1 << i)) - 1u);
+      mk &= ~mp;
+    }
   }
-  return c;
 }
 
 WT_HD uint32_t byte_compress(const ByteCompress& c, uint32_t x) {
@@ -169,7 +181,8 @@ WT_HD uint32_t reverse32(uint32_t x) {
 // set in every plane keep them behind the others.)
 template <int N>
 WT_HD void split_planes(uint32_t b, uint32_t* x) {
-  const ByteCompress c0 = byte_compress_plan(~b), c1 = byte_compress_plan(b);
+  ByteCompress c0, c1;
+  byte_compress_plans(b, c0, c1);
   // zeros per byte; zeros above each byte, and ones
   uint32_t n = ~b - ((~b >> 1) & 0x55555555u);
   n = (n & 0x33333333u) + ((n >> 2) & 0x33333333u);

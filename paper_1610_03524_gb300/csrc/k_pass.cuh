@@ -36,7 +36,9 @@
 // half of a split's moves are multiplications, 10.1 ms (2^28 symbols: 2.74 and
 // 2.53 ms; 2^26 32-bit ones 0.93 and 0.86), and with the runs taken out by bulk
 // copies instead of a search for the run and a store for every word 64 (43) and
-// 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).
+// 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).  One warp's lanes for both kinds of
+// runs, pieces masked in place and the splits' shared parities: 9.5 ms (2^28:
+// 2.37 ms; 32-bit 0.82).
 #pragma once
 #include <type_traits>
 
@@ -198,7 +200,7 @@ struct PassSmem {
 
 // CTAs per SM the register budget is sized for, at 128 threads
 #ifndef WT_PASS_CTAS
-#define WT_PASS_CTAS 8
+#define WT_PASS_CTAS 7
 #endif
 template <int EW, int NT>
 struct PassCtas {
@@ -211,7 +213,7 @@ struct PassCtas {
 // to address base + 16 i (base == 0: nowhere).
 struct __align__(16) Run {
   uint64_t base;
-  uint32_t first, last, at, n;
+  uint16_t first, last, at, n;
 };
 
 template <typename E, bool DIG, bool BATCH, int NT>
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   __shared__ uint64_t s_cs[2 * KEYS - 1];
   __shared__ uint64_t s_hf[3 * (TAU_MAX + 1)], s_lo[TAU_MAX], s_ll[TAU_MAX];  // Huffman: rows of the level tables
   __shared__ uint32_t s_own[KEYS];  // the tile's key counts by the tables
-  __shared__ bool s_over[2];        // a run past its level's or the sequence's end
+  __shared__ bool s_over;           // a run past its level's or the sequence's end
   // the runs of level bits that are not empty, and those of the next
   // sequence; the latter's offset in the first unit, bytes << 8
   __shared__ Run s_run[2][KEYS];
@@ -341,30 +343,30 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     // use the DRAM bandwidth the tile's compute leaves idle)
     if (!BATCH && P0.clear) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid, NT);
     cp_async_wait();
-    if (warp < 2) bulk_wait_read();  // the last tile's runs have left
+    if (warp == 0) bulk_wait_read();  // the last tile's runs have left
     __syncthreads();
     for (int i = tid; i < SM::AREA; i += NT) ((uint4*)s_area)[i] = make_uint4(0u, 0u, 0u, 0u);
 
-    // ---- 1. where the runs go (from the tables; a warp for the level bits',
-    //      one for the next sequence's), and the next tile -------------------
-    if (warp < 2) {
-      const int half = warp;
-      // lane r < 2^t: key r's count in the tile (a difference of prefixes) and
+    // ---- 1. where the runs go (from the tables; warp 0, lanes 0-15 the level
+    //      bits', lanes 16-31 the next sequence's), and the next tile ---------
+    if (warp == 0) {
+      const int half = lane >> 4, l16 = lane & 15;
+      // l16 = r < 2^t: key r's count in the tile (a difference of prefixes) and
       // in the earlier tiles of its sequence or node
       uint32_t c = 0;
       uint64_t ex = 0;
-      if (lane < nd) {
+      if (l16 < nd) {
         const bool last = ((ti + 1) >> P0.chsh) != (ti >> P0.chsh) || ti + 1 >= ntiles;
-        const uint32_t a = s_ta[lane];
-        c = last ? (uint32_t)(s_cn[lane] - s_ca[lane]) - a : s_tn[lane] - a;
-        ex = (s_ca[lane] + a) - (s_cb[lane] + s_tb[lane]);
+        const uint32_t a = s_ta[l16];
+        c = last ? (uint32_t)(s_cn[l16] - s_ca[l16]) - a : s_tn[l16] - a;
+        ex = (s_ca[l16] + a) - (s_cb[l16] + s_tb[l16]);
       }
-      int j = t;
-      if (half == 0) {
-        if (lane < KEYS) s_own[lane] = c;
-        // lane i takes class k of level j, i + 1 = 2^j + k: the keys' counts
-        // folded level by level
-        const int mj = 31 - __clz(lane + 1), mk = lane + 1 - (1 << mj);
+      if (half == 0) s_own[l16] = c;
+      // lanes 0-15: lane i takes class k of level j, i + 1 = 2^j + k: the keys'
+      // counts folded level by level
+      int j = 31 - __clz(l16 + 1);
+      {
+        const int mk = l16 + 1 - (1 << j);
         uint32_t fc = c, rc = 0;
         uint64_t fx = ex, rx = 0;
         for (int l = t - 1; l >= 0; l--) {
@@ -372,22 +374,23 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
           fx += __shfl_down_sync(FULL, fx, 1 << l);
           const uint32_t yc = __shfl_sync(FULL, fc, mk);
           const uint64_t yx = __shfl_sync(FULL, fx, mk);
-          if (mj == l) {
+          if (j == l) {
             rc = yc;
             rx = yx;
           }
         }
-        c = lane < nd - 1 && (!DIG || (mj & 1) == 0) ? rc : 0u;
-        ex = rx;
-        j = mj;
-      } else if (P.out == nullptr) {
-        c = 0;
+        if (half == 0) {
+          c = l16 < nd - 1 && (!DIG || (j & 1) == 0) ? rc : 0u;
+          ex = rx;
+        } else if (P.out == nullptr) {
+          c = 0;
+        }
       }
       uint32_t n = 0, len = 0, off = 0;  // 16-byte units; bits or bytes; offset in the first
       uint64_t where = 0;                // address of the first (0: nowhere)
       bool over = false;
       if (c) {
-        const uint64_t cs = s_cs[half ? nd - 1 + lane : lane], b0 = cs + ex;
+        const uint64_t cs = s_cs[half ? nd - 1 + l16 : l16], b0 = cs + ex;
         const bool dead = cs == ~0ull;
         if (half) {
           over = !dead && b0 + c > P.n_in;  // never for consistent tables
@@ -414,31 +417,27 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       uint32_t first = n;
 #pragma unroll
       for (int o = 1; o < 16; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, first, o);
-        if (lane >= o) first += y;
+        const uint32_t y = __shfl_up_sync(FULL, first, o, 16);
+        if (l16 >= o) first += y;
       }
       first -= n;
-      const uint32_t some = __ballot_sync(FULL, n != 0u);
+      const uint32_t some = __ballot_sync(FULL, n != 0u) & (half ? 0xffff0000u : 0xffffu);
       if (n) {
         const int at = __popc(some & lanemask_lt()), sh = half ? 4 : 7;  // a unit's bytes or bits
         Run r;
         r.base = where ? where - 16ull * first : 0ull;
-        r.first = where ? first + (off ? 1u : 0u) : ~0u;
-        r.last = where ? first + ((off + len) >> sh) : 0u;
-        r.at = first;
-        r.n = n;
+        r.first = (uint16_t)(first + (off ? 1u : 0u));
+        r.last = (uint16_t)(where ? first + ((off + len) >> sh) : 0u);
+        r.at = (uint16_t)first;
+        r.n = (uint16_t)n;
         s_run[half][at] = r;
         if (half) s_edge[at] = where ? off | (len << 8) : 0u;
       }
-      if (lane < KEYS) {
-        if (half) ((uint16_t*)s_sb)[lane] = (uint16_t)(16 * first + off);
-        else s_ab[lane] = 8 * smem_addr(s_area) + 128 * first + off;
-      }
+      if (half) ((uint16_t*)s_sb)[l16] = (uint16_t)(16 * first + off);
+      else s_ab[l16] = 8 * smem_addr(s_area) + 128 * first + off;
+      if (l16 == 0) s_nr[half] = (uint32_t)__popc(some);
       const bool stop = __any_sync(FULL, over);
-      if (lane == 0) {
-        s_nr[half] = (uint32_t)__popc(some);
-        s_over[half] = stop;
-      }
+      if (lane == 0) s_over = stop;
     }
     if (tid == NT - 1 && more) set_info(ti + gridDim.x, cur ^ 1);
 
@@ -503,7 +502,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     // the tile's key counts against the tables': tables that disagree with the
     // tile would misplace its runs, so the tile is flagged (every warp finds
     // the same) and its outputs are left alone
-    bool bad = s_over[0] | s_over[1];
+    bool bad = s_over;
     {
       uint32_t tot = 0;
       if (lane < nd) {
@@ -561,16 +560,19 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       // and the earlier threads' counts of its classes
       auto level = [&](auto jc, uint32_t b0, uint32_t b1, const uint32_t* c, const uint32_t* x) {
         constexpr int j = decltype(jc)::value;
-        uint32_t at = 0;
+        uint32_t at = 0, below = 0;  // bits of the classes before k, as a mask
 #pragma unroll
         for (int k = 0; k < (1 << j); k++) {
           const uint32_t n = (k & 1) ? c[k >> 1] >> 16 : c[k >> 1] & 0xffffu;
           const uint32_t xk = (k & 1) ? x[k >> 1] >> 16 : x[k >> 1] & 0xffffu;
           const uint32_t q = s_ab[(1 << j) - 1 + k] + xk * bpe;
-          const uint32_t w0 = __funnelshift_rc(b0, 0u, at) & low_mask(n);
           if (!DIG) {
-            or_bits(q, w0);
+            // shifted as they stand, from at bits before their place on
+            const uint32_t upto = low_mask(at + n);
+            or_bits(q - at, b0 & upto & ~below);
+            below = upto;
           } else {
+            const uint32_t w0 = __funnelshift_rc(b0, 0u, at) & low_mask(n);
             const uint32_t w1 = __funnelshift_rc(b1, 0u, at) & low_mask(n);
             const uint64_t d = P.a + j + 1 < P.L ? (spread32(w0) << 1) | spread32(w1) : spread32(w0);
             or_bits(q, (uint32_t)d);
@@ -651,11 +653,11 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     if (bad) continue;  // uniform; nothing was put into the areas
 
     // ---- 6. the runs out: whole 16-byte units by bulk copies, a lane per run
-    //      (one warp for the level bits', one for the next sequence's) --------
-    if (warp < 2) {
-      if (lane < (int)s_nr[warp]) {
-        const Run r = s_run[warp][lane];
-        const unsigned char* const from = warp == 0 ? (const unsigned char*)s_area : s_srt;
+    if (warp == 0) {
+      const int half = lane >> 4;
+      if ((uint32_t)(lane & 15) < s_nr[half]) {
+        const Run r = s_run[half][lane & 15];
+        const unsigned char* const from = half ? s_srt : (const unsigned char*)s_area;
         if (r.last > r.first && r.base)
           bulk_store(r.base + 16ull * r.first, from + 16 * r.first, 16 * (r.last - r.first));
       }
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       }
     }
   }
-  if (warp < 2) bulk_wait();
+  if (warp == 0) bulk_wait();
 }
 
 }  // namespace wtk
