@@ -65,13 +65,14 @@ wt_status new_handle(wt_stream stream, uint64_t n, uint32_t sigma, wt_struct** o
   h->n = n;
   h->sigma = sigma;
   cudaGetDevice(&h->device);
-  constexpr size_t bytes = 8 + 8 * MAX_LEVELS;
+  constexpr size_t bytes = 8 + 8 * MAX_LEVELS + 4 * (1 + SCAN_CHUNKS);
   if (dmalloc((void**)&h->d_err, bytes, h->stream) != cudaSuccess) {
     free_arrays(h);
     delete h;
     return WT_ERR_NO_MEMORY;
   }
   h->d_zeros = (uint64_t*)h->d_err + 1;
+  h->d_tick = (uint32_t*)(h->d_zeros + MAX_LEVELS);
   cudaMemsetAsync(h->d_err, 0, bytes, h->stream);
   *out = h;
   return WT_OK;

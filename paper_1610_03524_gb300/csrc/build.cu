@@ -126,6 +126,161 @@ __device__ __forceinline__ void for_each_symbol(const void* seq, uint64_t n, uin
   for (uint64_t i = nvec * PER + gtid; i < n; i += gstride) f((uint32_t)s[i]);
 }
 
+// What a pass's plan gives, from the totals of its tiles' digit counts by key
+// (the digit reversed): for the wavelet matrix the class starts of its levels
+// a .. a+t (level a+j's classes are the values of the key's low j bits) into
+// cls and every level's zero count (the start of class 2^(j-1) after split j);
+// for a balanced tree's first pass the starts of the nodes of level t.
+enum PlanKind : int { PLAN_NONE = 0, PLAN_WM = 1, PLAN_WT = 2 };
+struct PassPlan {
+  int kind;
+  int a, t;
+  uint64_t* cls;    // WM
+  uint64_t* C;      // WT: 2^t + 1
+  uint64_t* zeros;  // WM
+};
+
+// exclusive prefix sums of one value a lane over the first n lanes
+__device__ __forceinline__ uint64_t warp_scan_excl(uint64_t v, uint64_t& total) {
+  const int lane = threadIdx.x & 31;
+  uint64_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  total = __shfl_sync(FULL, x, 31);
+  return x - v;
+}
+
+// One warp: the plan from the totals, lane r < 2^t holding key r's.  Level j's
+// counts are folded from level j+1's.  (A thread scanning each level in turn
+// took 40-55 us for eight levels, more than any other kernel of a small
+// build.)
+__device__ void plan_pass(uint64_t tot, const PassPlan& p) {
+  const int lane = threadIdx.x & 31, t = p.t;
+  uint64_t c = lane < (1 << t) ? tot : 0ull, all;
+  if (p.kind == PLAN_WT) {
+    // in order of the digit: lane v takes the count of key rev(v)
+    const uint64_t d = __shfl_sync(FULL, c, (int)rev_bits((uint32_t)lane & ((1u << t) - 1u), t));
+    const uint64_t start = warp_scan_excl(lane < (1 << t) ? d : 0ull, all);
+    if (lane <= (1 << t)) p.C[lane] = start;
+    return;
+  }
+  for (int j = t; j >= 0; j--) {
+    const int nk = 1 << j;
+    const uint64_t start = warp_scan_excl(lane < nk ? c : 0ull, all);
+    uint64_t* const out = p.cls + (nk - 1 + j);
+    if (lane <= nk) out[lane] = start;  // the lane after the last class: the total
+    if (j > 0 && lane == nk / 2) p.zeros[p.a + j - 1] = start;
+    const uint64_t up = __shfl_down_sync(FULL, c, nk / 2);
+    c += lane < nk / 2 ? up : 0ull;
+  }
+}
+
+// The prefix sums of the tiles' counts and the pass's plan as the tail of the
+// counting kernel, for passes of at most SCAN_TILES tiles, which run one tile a
+// warp: the block that is the last of its chunk's eight to finish scans the
+// chunk's 64 tiles, and the one that finishes the last chunk scans the chunks
+// and makes the plan (a block takes a ticket when it is done; no block waits
+// for another).  A block's 256 threads hold a chunk's, or the chunks', counts
+// in one round of loads.  A wavelet matrix of 12.3 million 32-bit symbols (5
+// passes of 3015 tiles) went from 454 to 419 us with two launches less a pass,
+// one of 50 million 16-bit ones (4 passes of 12208) from 1290 to 1258 us, a
+// tree of 2^20 bytes from 184 to 167 us.  Above that the fence and the ticket
+// of every block meet a kernel that DRAM bounds, and the launches no longer
+// count.
+constexpr uint32_t SCAN_TILES = 64 * SCAN_CHUNKS;
+struct TileScan {
+  uint32_t* tick;  // finished chunks, then every chunk's finished blocks: zero before and after
+  uint32_t nchunk;
+  uint64_t* tchunk;
+  PassPlan plan;
+};
+
+// Whether the block is the last of n to come here; what the others wrote
+// before is then visible to all its threads.
+__device__ __forceinline__ bool last_block(uint32_t* tick, uint32_t n) {
+  __shared__ bool s_last;
+  __syncthreads();
+  if (n == 1) return true;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const bool last = atomicAdd(tick, 1u) == n - 1;
+    if (last) *tick = 0;
+    __threadfence();
+    s_last = last;
+  }
+  __syncthreads();
+  return s_last;
+}
+
+__device__ __noinline__ void scan_tail(uint32_t* tcnt, uint32_t ntiles, const TileScan& sc) {
+  constexpr int S = TC_STRIDE;
+  static_assert(S == 16 && SCAN_CHUNKS == 256, "four threads a tile, a warp per two keys");
+  __shared__ uint4 s_half[4];
+  __shared__ uint64_t s_tot[S];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t c = blockIdx.x >> 3;
+  if (!last_block(sc.tick + 1 + c, min(8u, gridDim.x - 8 * c))) return;
+  {
+    // warp (h, q): keys 4 q .. 4 q + 3 of the chunk's tiles 32 h + lane
+    const int q = warp & 3, h = warp >> 2;
+    const uint32_t ti = 64 * c + 32 * h + lane;
+    uint4* const row = (uint4*)(tcnt + (uint64_t)ti * S) + q;
+    const uint4 v = ti < ntiles ? __ldcg(row) : make_uint4(0u, 0u, 0u, 0u);
+    uint4 x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint4 y = make_uint4(__shfl_up_sync(FULL, x.x, o), __shfl_up_sync(FULL, x.y, o),
+                                 __shfl_up_sync(FULL, x.z, o), __shfl_up_sync(FULL, x.w, o));
+      if (lane >= o) x = make_uint4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
+    }
+    if (h == 0 && lane == 31) s_half[q] = x;
+    __syncthreads();
+    if (h) {
+      const uint4 y = s_half[q];
+      x = make_uint4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
+    }
+    if (ti < ntiles) *row = make_uint4(x.x - v.x, x.y - v.y, x.z - v.z, x.w - v.w);
+    if (h && lane == 31) {
+      uint64_t* const to = sc.tchunk + (uint64_t)c * S + 4 * q;
+      *(ulonglong2*)to = make_ulonglong2(x.x, x.y);
+      *(ulonglong2*)(to + 2) = make_ulonglong2(x.z, x.w);
+    }
+  }
+  if (!last_block(sc.tick, sc.nchunk)) return;
+  {
+    // warp w: keys 2 w and 2 w + 1, lanes the chunks
+    ulonglong2 v[8];
+#pragma unroll
+    for (int g = 0; g < 8; g++) {
+      const uint32_t i = 32 * g + lane;
+      v[g] = i < sc.nchunk ? __ldcg((const ulonglong2*)(sc.tchunk + (uint64_t)i * S + 2 * warp))
+                           : make_ulonglong2(0ull, 0ull);
+    }
+    uint64_t a = 0, b = 0;  // before the group
+#pragma unroll
+    for (int g = 0; g < 8; g++) {
+      if (32u * g >= sc.nchunk) break;
+      const uint32_t i = 32 * g + lane;
+      uint64_t ta, tb;
+      const uint64_t xa = warp_scan_excl(v[g].x, ta), xb = warp_scan_excl(v[g].y, tb);
+      if (i < sc.nchunk)
+        *(ulonglong2*)(sc.tchunk + (uint64_t)i * S + 2 * warp) = make_ulonglong2(a + xa, b + xb);
+      a += ta;
+      b += tb;
+    }
+    if (lane == 0) {
+      *(ulonglong2*)(sc.tchunk + (uint64_t)sc.nchunk * S + 2 * warp) = make_ulonglong2(a, b);
+      s_tot[2 * warp] = a;
+      s_tot[2 * warp + 1] = b;
+    }
+  }
+  __syncthreads();
+  if (warp == 0 && sc.plan.kind != PLAN_NONE) plan_pass(lane < S ? s_tot[lane] : 0ull, sc.plan);
+}
+
 // Digit counts of every tile of a pass (the K sub-problems' per-class counts
 // of Section 4.2), by key (the digit reversed): one warp per tile, the same
 // tiles and digits as k_pass.  A lane takes 32 elements a step as bit planes
@@ -135,9 +290,10 @@ __device__ __forceinline__ void for_each_symbol(const void* seq, uint64_t n, uin
 // 32 elements, so that DRAM is the bound, where a shared-memory atomic per
 // element was.  First passes also check the symbols against sigma and zero
 // their share of the pass's levels.
-template <int EW, bool BATCH>
+template <int EW, bool BATCH, bool SCAN>
 __global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ PassParams P0,
-                                                     uint32_t* tcnt, uint32_t tile) {
+                                                     uint32_t* tcnt, uint32_t tile,
+                                                     const __grid_constant__ TileScan sc) {
   __shared__ PassParams s_P[BATCH ? 8 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
@@ -265,6 +421,7 @@ __global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ Pas
     if (lane < TC_STRIDE) tcnt[(uint64_t)ti * TC_STRIDE + lane] = mine;
     if (__any_sync(FULL, bad) && lane == 0) atomicOr(P.err, ERR_SYMBOL);
   }
+  if (SCAN) scan_tail(tcnt, ntiles, sc);
 }
 
 // The same counts for bytes over SIG = 2 .. 8 values in a single pass
@@ -345,11 +502,25 @@ __global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, u
 }
 
 // Launch of a pass's tile counts into tcnt (mt tiles at most).
+// counts by k_count_tiles_bytes
+static bool byte_counts(const PassParams& P) {
+  return P.in_w == 1 && !P.tiles && P.sigma >= 2 && P.sigma <= 8 && P.t == P.L;
+}
+
+template <bool BATCH, bool SCAN>
+static void launch_tile_counts(const PassParams& P, uint32_t T, unsigned grid, uint32_t* tcnt,
+                               const TileScan& sc, cudaStream_t st) {
+  if (P.in_w == 1) k_tile_counts<1, BATCH, SCAN><<<grid, 256, 0, st>>>(P, tcnt, T, sc);
+  else if (P.in_w == 2) k_tile_counts<2, BATCH, SCAN><<<grid, 256, 0, st>>>(P, tcnt, T, sc);
+  else k_tile_counts<4, BATCH, SCAN><<<grid, 256, 0, st>>>(P, tcnt, T, sc);
+}
+
+// sc: the scans and the plan too (at most SCAN_TILES tiles)
 template <bool BATCH>
 static wt_status launch_counts(const PassParams& P, uint32_t T, uint64_t mt, uint32_t* tcnt,
-                               cudaStream_t st) {
+                               const TileScan* sc, cudaStream_t st) {
   const unsigned grid = (unsigned)std::min<uint64_t>((mt + 7) / 8, (uint64_t)num_sms() * 32);
-  if (!BATCH && P.in_w == 1 && !P.tiles && P.sigma >= 2 && P.sigma <= 8 && P.t == P.L) {
+  if (!BATCH && byte_counts(P)) {
     const uint8_t* sb = (const uint8_t*)P.in;
 #define WT_COUNT_BYTES(S)                                                                          \
   case S:                                                                                          \
@@ -366,12 +537,10 @@ static wt_status launch_counts(const PassParams& P, uint32_t T, uint64_t mt, uin
       WT_COUNT_BYTES(8);
     }
 #undef WT_COUNT_BYTES
-  } else if (P.in_w == 1) {
-    k_tile_counts<1, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
-  } else if (P.in_w == 2) {
-    k_tile_counts<2, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
+  } else if (!BATCH && sc) {
+    launch_tile_counts<false, true>(P, T, (unsigned)((mt + 7) / 8), tcnt, *sc, st);
   } else {
-    k_tile_counts<4, BATCH><<<grid, 256, 0, st>>>(P, tcnt, T);
+    launch_tile_counts<BATCH, false>(P, T, grid, tcnt, TileScan{}, st);
   }
   count_launch();
   CK(cudaGetLastError());
@@ -672,58 +841,6 @@ static std::vector<PassGeom> make_passes(int L, int tau, int first_w) {
   return ps;
 }
 
-// What a pass's plan gives, from the totals of its tiles' digit counts by key
-// (the digit reversed): for the wavelet matrix the class starts of its levels
-// a .. a+t (level a+j's classes are the values of the key's low j bits) into
-// cls and every level's zero count (the start of class 2^(j-1) after split j);
-// for a balanced tree's first pass the starts of the nodes of level t.
-enum PlanKind : int { PLAN_NONE = 0, PLAN_WM = 1, PLAN_WT = 2 };
-struct PassPlan {
-  int kind;
-  int a, t;
-  uint64_t* cls;    // WM
-  uint64_t* C;      // WT: 2^t + 1
-  uint64_t* zeros;  // WM
-};
-
-// exclusive prefix sums of one value a lane over the first n lanes
-__device__ __forceinline__ uint64_t warp_scan_excl(uint64_t v, uint64_t& total) {
-  const int lane = threadIdx.x & 31;
-  uint64_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(FULL, x, o);
-    if (lane >= o) x += y;
-  }
-  total = __shfl_sync(FULL, x, 31);
-  return x - v;
-}
-
-// One warp: the plan from the totals, lane r < 2^t holding key r's.  Level j's
-// counts are folded from level j+1's.  (A thread scanning each level in turn
-// took 40-55 us for eight levels, more than any other kernel of a small
-// build.)
-__device__ void plan_pass(uint64_t tot, const PassPlan& p) {
-  const int lane = threadIdx.x & 31, t = p.t;
-  uint64_t c = lane < (1 << t) ? tot : 0ull, all;
-  if (p.kind == PLAN_WT) {
-    // in order of the digit: lane v takes the count of key rev(v)
-    const uint64_t d = __shfl_sync(FULL, c, (int)rev_bits((uint32_t)lane & ((1u << t) - 1u), t));
-    const uint64_t start = warp_scan_excl(lane < (1 << t) ? d : 0ull, all);
-    if (lane <= (1 << t)) p.C[lane] = start;
-    return;
-  }
-  for (int j = t; j >= 0; j--) {
-    const int nk = 1 << j;
-    const uint64_t start = warp_scan_excl(lane < nk ? c : 0ull, all);
-    uint64_t* const out = p.cls + (nk - 1 + j);
-    if (lane <= nk) out[lane] = start;  // the lane after the last class: the total
-    if (j > 0 && lane == nk / 2) p.zeros[p.a + j - 1] = start;
-    const uint64_t up = __shfl_down_sync(FULL, c, nk / 2);
-    c += lane < nk / 2 ? up : 0ull;
-  }
-}
-
 // Batched builds, one warp per sequence of the launch: the plan of its pass
 // from the totals of its own tiles' digit counts, i.e. the difference of the
 // scanned tables' prefixes at its last and first tile (tcnt exclusive within
@@ -1022,9 +1139,13 @@ static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const Pa
   // the zeroing belongs to the counts of a first pass (sigma set), else to
   // the pass
   if (!P.sigma) Q.clear = nullptr;
-  TRY(launch_counts<BATCH>(Q, T, mt, tcnt, st));
+  // up to SCAN_TILES tiles one launch counts, scans and plans, else three
+  const TileScan sc{P.tick, nchunk, tchunk, plan};
+  const bool tail = !BATCH && P.tick && mt <= SCAN_TILES && !byte_counts(P);
+  TRY(launch_counts<BATCH>(Q, T, mt, tcnt, tail ? &sc : nullptr, st));
   const uint32_t* nt_dev = P.tiles ? P.ntiles_dev : nullptr;
-  if (nchunk == 1) {
+  if (tail) {
+  } else if (nchunk == 1) {
     k_tile_scan_chunk<true><<<1, 32, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, 1, tchunk, plan);
     count_launch();
   } else {
@@ -1121,6 +1242,7 @@ static PassParams base_params(wt_struct* h) {
   memset(&P, 0, sizeof(P));
   P.bits = h->d_bits;
   P.err = h->d_err;
+  P.tick = h->d_tick;
   return P;
 }
 

@@ -76,6 +76,7 @@ struct wt_struct {
   uint64_t* d_start = nullptr;   // (there too) wavelet matrix: the symbols' starts, or null
   uint32_t* d_err = nullptr;     // device error word (8 bytes), zeroed with the handle,
   uint64_t* d_zeros = nullptr;   // and after it the levels' zero counts (batched: elsewhere)
+  uint32_t* d_tick = nullptr;    // and tickets of the build's kernels, or null
   wtk::LevelMeta* d_meta = nullptr;
   // Huffman tables (device)
   uint32_t* d_code = nullptr;

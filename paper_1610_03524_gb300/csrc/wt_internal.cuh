@@ -47,6 +47,9 @@ inline int chunk_shift(uint64_t tiles) {
   return s;
 }
 
+// Chunks of the passes whose counting kernel also scans the counts.
+constexpr uint32_t SCAN_CHUNKS = 256;
+
 // Symbols per tile of the partition pass.
 #ifndef WT_PASS_T
 #define WT_PASS_T 4096
@@ -109,6 +112,7 @@ struct PassParams {
   const uint32_t* tcnt;
   const uint64_t* tchunk;
   uint32_t chsh;         // log2 of the tiles per chunk
+  uint32_t* tick;           // zeroed tickets of the counts' scans, or nullptr
   uint32_t* err;
   // 16-byte units of a later pass's levels to zero, `clear_per` of them per
   // tile (nullptr: none); see clear_share

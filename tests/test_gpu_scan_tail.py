@@ -1,0 +1,35 @@
+"""Passes whose counting kernel also scans the counts: tile numbers at the
+edges of a block (8), of a chunk (64) and of the range (256 chunks) on both
+sides, for sequences cut into equal tiles and into the nodes' tiles; every bit
+against the oracle (integer, tolerance 0)."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("tiles", [1, 7, 8, 9, 63, 64, 65, 128, 513, 16383, 16384, 16385])
+@pytest.mark.parametrize("short", [0, 1, 2047])
+def test_tiles_at_chunk_edges(tiles, short):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1610_03524_gb300 as wt
+    if tiles > 1000 and short == 2047:
+        pytest.skip("as with 1, at a few seconds more")
+    n, sigma = tiles * 2048 - short, 20
+    S = np.random.default_rng(tiles).integers(0, sigma, n).astype(np.uint8)
+    d = to_dev(S)
+    ob, oz = oracle.wm_build(S, sigma)
+    h = wt.wm_build(d, sigma, tile_symbols=2048)
+    ex = h.export()
+    assert np.array_equal(ex.bits.reshape(ob.shape), ob) and np.array_equal(ex.zeros, oz)
+    h.free()
+    ot = oracle.wt_build(S, sigma)
+    h = wt.wt_build(d, sigma)
+    ex = h.export()
+    assert np.array_equal(ex.bits.reshape(ot.shape), ot) and np.array_equal(ex.zeros, oz)
+    h.free()
