@@ -208,7 +208,10 @@ __device__ __forceinline__ void warp_samples(bool live, uint64_t s0, uint64_t zb
 // Counts of one group: a record per superblock with the zeros before it in
 // the group; the group's total into blk_tot.  ONE: the group is the whole
 // level (block l = level l): its records are final, and its total record, zero
-// count and samples are written too.
+// count and samples are written too.  DRAM is the bound where all of a group's
+// words are there: 2^33 bits in 148 us, 7.7 TB/s with the records, against 194
+// us with a prefix sum per superblock and every word's bounds checked (16
+// levels of 2^30 bits: 311 and 436 us).
 template <bool SMALL, bool ONE>
 __global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const LevelMeta* meta,
                                                    int nlev, const uint64_t* blk_first,
@@ -248,42 +251,59 @@ __global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const L
   const uint64_t* lb = bits + m.bit_off;
   const bool vec = (((uintptr_t)lb) & 15) == 0;
   constexpr int NP = DIR_SB_PER_WARP / 2;
-  uint64_t w0[NP], w1[NP];
-  int v0[NP], v1[NP];
+  static_assert(NP == 4, "four counts in two words");
+  uint32_t z[NP];  // zeros of the lane's words
+  if (vec && 2048 * (sb0 + DIR_GROUP) <= m.n) {
+    const ulonglong2* const p = (const ulonglong2*)(lb + 32 * (s0 + half) + 2 * hl);
+    ulonglong2 q[NP];
 #pragma unroll
-  for (int u = 0; u < NP; u++) {
-    const uint64_t s = s0 + 2 * u + half;
-    const int64_t rem = (int64_t)m.n - (int64_t)(2048 * s + 128 * (uint64_t)hl);
-    const bool live = s < m.nsb && rem > 0;
-    v0[u] = !live ? 0 : (rem >= 64 ? 64 : (int)rem);
-    v1[u] = (!live || rem <= 64) ? 0 : (rem >= 128 ? 64 : (int)(rem - 64));
-    const uint64_t* p = lb + 32 * s + 2 * hl;
-    // words past the last valid bit are not read (a caller bitvector may end there)
-    if (v1[u] && vec) {
-      const ulonglong2 q = __ldcs((const ulonglong2*)p);
-      w0[u] = q.x;
-      w1[u] = q.y;
-    } else {
-      w0[u] = v0[u] ? __ldcs(p) : 0ull;
-      w1[u] = v1[u] ? __ldcs(p + 1) : 0ull;
+    for (int u = 0; u < NP; u++) q[u] = __ldcs(p + 32 * u);
+#pragma unroll
+    for (int u = 0; u < NP; u++) z[u] = 128 - __popcll(q[u].x) - __popcll(q[u].y);
+  } else {
+#pragma unroll
+    for (int u = 0; u < NP; u++) {
+      const uint64_t s = s0 + 2 * u + half;
+      const int64_t rem = (int64_t)m.n - (int64_t)(2048 * s + 128 * (uint64_t)hl);
+      const bool live = s < m.nsb && rem > 0;
+      const int v0 = !live ? 0 : (rem >= 64 ? 64 : (int)rem);
+      const int v1 = (!live || rem <= 64) ? 0 : (rem >= 128 ? 64 : (int)(rem - 64));
+      const uint64_t* p = lb + 32 * s + 2 * hl;
+      // words past the last valid bit are not read (a caller bitvector may end there)
+      ulonglong2 q = make_ulonglong2(0ull, 0ull);
+      if (v1 && vec) {
+        q = __ldcs((const ulonglong2*)p);
+      } else {
+        if (v0) q.x = __ldcs(p);
+        if (v1) q.y = __ldcs(p + 1);
+      }
+      z[u] = v0 + v1 - __popcll(q.x) - __popcll(q.y);
     }
   }
-  uint64_t rel[NP];
+  // all four superblocks' prefix sums over the half's lanes at once, two 16-bit
+  // counts a word; then lane u < 4 of the half has superblock u's record
+  uint32_t za = z[0] | (z[1] << 16), zb = z[2] | (z[3] << 16);
 #pragma unroll
-  for (int u = 0; u < NP; u++) {
-    const int z = v0[u] + v1[u] - __popcll(w0[u]) - __popcll(w1[u]);
-    int zi = z;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-      const int y = __shfl_up_sync(FULL, zi, o, 16);
-      if (hl >= o) zi += y;
+  for (int o = 1; o < 16; o <<= 1) {
+    const uint32_t ya = __shfl_up_sync(FULL, za, o, 16), yb = __shfl_up_sync(FULL, zb, o, 16);
+    if (hl >= o) {
+      za += ya;
+      zb += yb;
     }
-    // zeros of 512-bit blocks 0, 1, 2 of the superblock: lanes 3, 7, 11 of its half
-    const uint64_t r1 = (uint64_t)__shfl_sync(FULL, zi, 3, 16);
-    const uint64_t r2 = (uint64_t)__shfl_sync(FULL, zi, 7, 16);
-    const uint64_t r3 = (uint64_t)__shfl_sync(FULL, zi, 11, 16);
-    rel[u] = (r1 << 16) | (r2 << 32) | (r3 << 48);
-    if (hl == 15) s_z[warp * DIR_SB_PER_WARP + 2 * u + half] = (uint32_t)zi;
+  }
+  // zeros before 512-bit blocks 1, 2, 3 of the superblock, and in all: lanes 3, 7, 11, 15
+  const int u = hl & 3;
+  uint32_t at[4];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const uint32_t xa = __shfl_sync(FULL, za, 4 * k + 3, 16), xb = __shfl_sync(FULL, zb, 4 * k + 3, 16);
+    at[k] = ((u & 2 ? xb : xa) >> (16 * (u & 1))) & 0xffffu;
+  }
+  const uint64_t rel = ((uint64_t)(at[1] | (at[2] << 16)) << 32) | (at[0] << 16);
+  const int i = warp * DIR_SB_PER_WARP + 2 * u + half;  // in the group
+  if (hl < 4) {
+    s_z[i] = at[3];
+    if (ONE) s_rel[i] = rel;
   }
   __syncthreads();
   // zeros before each of the warp's superblocks in the group: lane i the sum
@@ -297,17 +317,13 @@ __global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const L
     if (lane >= o) inc += y;
   }
   const uint32_t total = __shfl_sync(FULL, inc, 31);
-#pragma unroll
-  for (int u = 0; u < NP; u++) {
-    const uint64_t s = s0 + 2 * u + half;
-    // superblock warp * 8 + 2 u + half of the group: lane warp * 4 + u holds its pair
+  {
+    // lane i / 2 holds the pair of superblock i
     const uint32_t pair = __shfl_sync(FULL, inc - a - b, warp * NP + u);
     const uint32_t prev = __shfl_sync(FULL, a, warp * NP + u);
-    const uint32_t before = pair + (half ? prev : 0u);
-    if (hl == 0 && s < m.nsb) {
-      *(ulonglong2*)(dir + m.dir_off + 2 * s) = make_ulonglong2(before, rel[u]);
-      if (ONE) s_rel[warp * DIR_SB_PER_WARP + 2 * u + half] = rel[u];
-    }
+    const uint64_t s = s0 + 2 * u + half;
+    if (hl < 4 && s < m.nsb)
+      *(ulonglong2*)(dir + m.dir_off + 2 * s) = make_ulonglong2(pair + (half ? prev : 0u), rel);
   }
   if (!ONE) {
     if (threadIdx.x == 0) blk_tot[blockIdx.x] = total;
