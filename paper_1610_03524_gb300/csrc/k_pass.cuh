@@ -38,7 +38,8 @@
 // copies instead of a search for the run and a store for every word 64 (43) and
 // 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).  One warp's lanes for both kinds of
 // runs, pieces masked in place and the splits' shared parities: 9.5 ms (2^28:
-// 2.37 ms; 32-bit 0.82).
+// 2.37 ms; 32-bit 0.82).  The other warps take the work that warp 0, which
+// they wait for, had beside the runs' layout: 9.3 ms (2.32; 0.80).
 #pragma once
 #include <type_traits>
 
@@ -200,7 +201,7 @@ struct PassSmem {
 
 // CTAs per SM the register budget is sized for, at 128 threads
 #ifndef WT_PASS_CTAS
-#define WT_PASS_CTAS 7
+#define WT_PASS_CTAS 8
 #endif
 template <int EW, int NT>
 struct PassCtas {
@@ -341,11 +342,14 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     const int cnt = s_info[cur].cnt;
     // this tile's share of the zeroing of a later pass's levels (stores that
     // use the DRAM bandwidth the tile's compute leaves idle)
-    if (!BATCH && P0.clear) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid, NT);
+    if (!BATCH && P0.clear && warp) clear_share(P0.clear, P0.clear_units, P0.clear_per, ti, tid - 32, NT - 32);
     cp_async_wait();
     if (warp == 0) bulk_wait_read();  // the last tile's runs have left
     __syncthreads();
-    for (int i = tid; i < SM::AREA; i += NT) ((uint4*)s_area)[i] = make_uint4(0u, 0u, 0u, 0u);
+    // (this, the zeroing above and the runs' ends are left to the other warps:
+    // warp 0 has the runs to lay out, and the others wait for it)
+    if (warp)
+      for (int i = tid - 32; i < SM::AREA; i += NT - 32) ((uint4*)s_area)[i] = make_uint4(0u, 0u, 0u, 0u);
 
     // ---- 1. where the runs go (from the tables; warp 0, lanes 0-15 the level
     //      bits', lanes 16-31 the next sequence's), and the next tile ---------
@@ -662,9 +666,10 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
           bulk_store(r.base + 16ull * r.first, from + 16 * r.first, 16 * (r.last - r.first));
       }
       bulk_commit();
+      continue;
     }
     // the units at the runs' ends, shared with other tiles: level words ORed ...
-    for (uint32_t e = tid; e < 4 * s_nr[0]; e += NT) {
+    for (uint32_t e = tid - 32; e < 4 * s_nr[0]; e += NT - 32) {
       const Run r = s_run[0][e >> 2];
       const uint32_t u = r.at + ((e & 2) ? r.n - 1 : 0u);
       if (((e & 2) && r.n == 1) || (u >= r.first && u < r.last)) continue;
@@ -674,7 +679,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
     }
     // ... and elements four bytes a thread, one by one where not all are the run's
     if (P.out != nullptr) {
-      for (uint32_t e = tid; e < 8 * s_nr[1]; e += NT) {
+      for (uint32_t e = tid - 32; e < 8 * s_nr[1]; e += NT - 32) {
         const uint32_t at = e >> 3, b = 4 * (e & 3), oe = s_edge[at];
         const uint32_t off = oe & 0xffu, end = off + (oe >> 8);
         const uint32_t k = (e & 4) ? (end - 1) >> 4 : 0u;  // last unit or first
