@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ Pas
   for (uint32_t ti = blockIdx.x * 8 + warp; ti < ntiles; ti += nw) {
     if (BATCH) {
       __syncwarp();
-      if (lane == 0) fill_seg(s_P[warp], P0, ti);
+      fill_seg(s_P[warp], P0, ti);
       __syncwarp();
     }
     const PassParams& P = BATCH ? s_P[warp] : P0;

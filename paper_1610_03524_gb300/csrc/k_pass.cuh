@@ -54,21 +54,26 @@ __device__ __forceinline__ uint32_t load_elem(const void* p, int w, uint64_t i) 
   return ((const uint32_t*)p)[i];
 }
 
-// Batched builds: tile ti's sequence, the last segment with tile0 <= ti.
+// Batched builds: tile ti's sequence, the last segment with tile0 <= ti, found
+// by a whole warp, 32 segments a step (a binary search over 4096 sequences is
+// twelve dependent loads).
 __device__ __forceinline__ const SegDesc& seg_of(const PassParams& P0, uint32_t ti) {
+  const uint32_t lane = threadIdx.x & 31;
   uint32_t lo = 0, hi = P0.nsegs - 1;
   while (lo < hi) {
-    const uint32_t mid = (lo + hi + 1) >> 1;
-    if (P0.segs[mid].tile0 <= ti) lo = mid;
-    else hi = mid - 1;
+    const uint32_t step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step;
+    const bool before = at <= hi && P0.segs[at].tile0 <= ti;
+    lo += step * (uint32_t)__popc(__ballot_sync(FULL, before));
+    hi = min(hi, lo + step - 1);
   }
   return P0.segs[lo];
 }
 
 // Batched builds: the part of the parameters that belongs to tile ti's
-// sequence into D.
+// sequence into D (a whole warp; its first lane writes).
 __device__ __forceinline__ void fill_seg(PassParams& D, const PassParams& P0, uint32_t ti) {
   const SegDesc& d = seg_of(P0, ti);
+  if (threadIdx.x & 31) return;
   D.in = d.in;
   D.in_w = d.in_w;
   D.out = d.out;
@@ -254,10 +259,10 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   const int bpe = DIG ? 2 : 1;
   const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
 
-  // tile ti's parameters into buffer b (one thread)
+  // tile ti's parameters into buffer b (the last warp)
   auto set_info = [&](uint32_t ti, int b) {
     if (BATCH) fill_seg(s_P[b], P0, ti);
-    s_info[b] = tile_info(BATCH ? s_P[b] : P0, ti, T);
+    if (lane == 0) s_info[b] = tile_info(BATCH ? s_P[b] : P0, ti, T);
   };
   // its elements into s_in (all threads)
   auto load_tile = [&](int b) {
@@ -330,7 +335,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   uint32_t ti = blockIdx.x;
   int cur = 0;
   if (ti < ntiles) {
-    if (tid == 0) set_info(ti, 0);
+    if (warp == W - 1) set_info(ti, 0);
     __syncthreads();
     load_tile(0);
     if (warp == 0) load_ctl(ti, 0);
@@ -443,7 +448,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       const bool stop = __any_sync(FULL, over);
       if (lane == 0) s_over = stop;
     }
-    if (tid == NT - 1 && more) set_info(ti + gridDim.x, cur ^ 1);
+    if (warp == W - 1 && more) set_info(ti + gridDim.x, cur ^ 1);
 
     // ---- 2. planes and key counts of the thread's 32 elements -------------
     const unsigned char* const row = s_in + tid * RS;
