@@ -259,10 +259,11 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   const int bpe = DIG ? 2 : 1;
   const uint32_t ntiles = P0.tiles ? *P0.ntiles_dev : P0.ntiles;
 
-  // tile ti's parameters into buffer b (the last warp)
+  // tile ti's parameters into buffer b (the last thread; batched builds its warp)
+  const bool sets = BATCH ? warp == W - 1 : tid == NT - 1;
   auto set_info = [&](uint32_t ti, int b) {
     if (BATCH) fill_seg(s_P[b], P0, ti);
-    if (lane == 0) s_info[b] = tile_info(BATCH ? s_P[b] : P0, ti, T);
+    if (!BATCH || lane == 0) s_info[b] = tile_info(BATCH ? s_P[b] : P0, ti, T);
   };
   // its elements into s_in (all threads)
   auto load_tile = [&](int b) {
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
   uint32_t ti = blockIdx.x;
   int cur = 0;
   if (ti < ntiles) {
-    if (warp == W - 1) set_info(ti, 0);
+    if (sets) set_info(ti, 0);
     __syncthreads();
     load_tile(0);
     if (warp == 0) load_ctl(ti, 0);
@@ -448,7 +449,7 @@ __global__ void __launch_bounds__(NT, (PassCtas<sizeof(E), NT>::value)) k_pass(c
       const bool stop = __any_sync(FULL, over);
       if (lane == 0) s_over = stop;
     }
-    if (warp == W - 1 && more) set_info(ti + gridDim.x, cur ^ 1);
+    if (sets && more) set_info(ti + gridDim.x, cur ^ 1);
 
     // ---- 2. planes and key counts of the thread's 32 elements -------------
     const unsigned char* const row = s_in + tid * RS;
