@@ -178,6 +178,44 @@ __device__ void plan_pass(uint64_t tot, const PassPlan& p) {
   }
 }
 
+// Prefix sums of the tiles' counts of chunk c (2^chsh tiles), per key, in place,
+// and the chunk's totals, by a block of 256: 64 tiles a step, warp (h, q) keys
+// 4 q .. 4 q + 3 of tiles 32 h + lane.
+__device__ __forceinline__ void scan_chunk(uint32_t* tcnt, uint32_t ntiles, uint32_t c, uint32_t chsh,
+                                           uint64_t* tchunk) {
+  constexpr int S = TC_STRIDE;
+  static_assert(S == 16, "four threads a tile");
+  __shared__ uint4 s_half[2][4];
+  const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) & 3, h = threadIdx.x >> 7;
+  auto add = [](uint4 a, uint4 b) { return make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+  uint4 carry = make_uint4(0u, 0u, 0u, 0u);
+  for (uint32_t g = 0; g < 1u << (chsh - 6); g++) {
+    const uint32_t ti = (c << chsh) + 64 * g + 32 * h + lane;
+    uint4* const row = (uint4*)(tcnt + (uint64_t)ti * S) + q;
+    const uint4 v = ti < ntiles ? __ldcg(row) : make_uint4(0u, 0u, 0u, 0u);
+    uint4 x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint4 y = make_uint4(__shfl_up_sync(FULL, x.x, o), __shfl_up_sync(FULL, x.y, o),
+                                 __shfl_up_sync(FULL, x.z, o), __shfl_up_sync(FULL, x.w, o));
+      if (lane >= o) x = add(x, y);
+    }
+    if (g) __syncthreads();
+    if (lane == 31) s_half[h][q] = x;
+    __syncthreads();
+    const uint4 lo = s_half[0][q];
+    if (h) x = add(x, lo);
+    x = add(x, carry);
+    if (ti < ntiles) *row = make_uint4(x.x - v.x, x.y - v.y, x.z - v.z, x.w - v.w);
+    carry = add(carry, add(lo, s_half[1][q]));
+  }
+  if (h && lane == 31) {
+    uint64_t* const to = tchunk + (uint64_t)c * S + 4 * q;
+    *(ulonglong2*)to = make_ulonglong2(carry.x, carry.y);
+    *(ulonglong2*)(to + 2) = make_ulonglong2(carry.z, carry.w);
+  }
+}
+
 // The prefix sums of the tiles' counts and the pass's plan as the tail of the
 // counting kernel, for passes of at most SCAN_TILES tiles, which run one tile a
 // warp: the block that is the last of its chunk's eight to finish scans the
@@ -217,38 +255,12 @@ __device__ __forceinline__ bool last_block(uint32_t* tick, uint32_t n) {
 
 __device__ __noinline__ void scan_tail(uint32_t* tcnt, uint32_t ntiles, const TileScan& sc) {
   constexpr int S = TC_STRIDE;
-  static_assert(S == 16 && SCAN_CHUNKS == 256, "four threads a tile, a warp per two keys");
-  __shared__ uint4 s_half[4];
+  static_assert(S == 16 && SCAN_CHUNKS == 256, "a warp per two keys, eight chunks a lane");
   __shared__ uint64_t s_tot[S];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t c = blockIdx.x >> 3;
   if (!last_block(sc.tick + 1 + c, min(8u, gridDim.x - 8 * c))) return;
-  {
-    // warp (h, q): keys 4 q .. 4 q + 3 of the chunk's tiles 32 h + lane
-    const int q = warp & 3, h = warp >> 2;
-    const uint32_t ti = 64 * c + 32 * h + lane;
-    uint4* const row = (uint4*)(tcnt + (uint64_t)ti * S) + q;
-    const uint4 v = ti < ntiles ? __ldcg(row) : make_uint4(0u, 0u, 0u, 0u);
-    uint4 x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint4 y = make_uint4(__shfl_up_sync(FULL, x.x, o), __shfl_up_sync(FULL, x.y, o),
-                                 __shfl_up_sync(FULL, x.z, o), __shfl_up_sync(FULL, x.w, o));
-      if (lane >= o) x = make_uint4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
-    }
-    if (h == 0 && lane == 31) s_half[q] = x;
-    __syncthreads();
-    if (h) {
-      const uint4 y = s_half[q];
-      x = make_uint4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
-    }
-    if (ti < ntiles) *row = make_uint4(x.x - v.x, x.y - v.y, x.z - v.z, x.w - v.w);
-    if (h && lane == 31) {
-      uint64_t* const to = sc.tchunk + (uint64_t)c * S + 4 * q;
-      *(ulonglong2*)to = make_ulonglong2(x.x, x.y);
-      *(ulonglong2*)(to + 2) = make_ulonglong2(x.z, x.w);
-    }
-  }
+  scan_chunk(tcnt, ntiles, c, 6, sc.tchunk);
   if (!last_block(sc.tick, sc.nchunk)) return;
   {
     // warp w: keys 2 w and 2 w + 1, lanes the chunks
@@ -1083,43 +1095,42 @@ static wt_status launch_node_tiles(const uint64_t* bnd, uint64_t nn, uint32_t T,
 constexpr int PT = PASS_T;
 
 // Prefix sums of the tiles' counts, per key: exclusive inside each chunk of
-// 2^chsh tiles (in place, u32), and the chunks' totals; a thread per chunk and
-// key.  When there is one chunk only (ONE), the whole scan and the pass's plan
-// are this launch: its totals are the grand totals (row 1), row 0 is zero.
-template <bool ONE>
+// 2^chsh tiles (in place, u32), and the chunks' totals, a block per chunk.
+// (2^18 tiles: 11 us; 50 with a thread per chunk and key, too few loads in
+// flight.)
 __global__ void __launch_bounds__(256) k_tile_scan_chunk(uint32_t* tcnt, const uint32_t* ntiles_dev,
                                                          uint32_t ntiles_host, uint32_t chsh,
-                                                         uint32_t nchunk, uint64_t* tchunk,
-                                                         const PassPlan plan) {
+                                                         uint64_t* tchunk) {
+  scan_chunk(tcnt, ntiles_dev ? *ntiles_dev : ntiles_host, blockIdx.x, chsh, tchunk);
+}
+
+// The whole scan and the pass's plan where there is one chunk: its totals are
+// the grand totals (row 1), row 0 is zero.  One warp.
+__global__ void __launch_bounds__(32) k_tile_scan_one(uint32_t* tcnt, const uint32_t* ntiles_dev,
+                                                      uint32_t ntiles_host, uint64_t* tchunk,
+                                                      const PassPlan plan) {
   constexpr int S = TC_STRIDE;
-  const uint32_t nt = ntiles_dev ? *ntiles_dev : ntiles_host;
-  const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) / S, r = threadIdx.x % S;
-  if (c >= (ONE ? 2u : nchunk)) return;  // ONE: the plan is made by a whole warp
-  const uint64_t t0 = (uint64_t)c << chsh;
-  const uint64_t t1 = t0 + (1u << chsh) < nt ? t0 + (1u << chsh) : nt;
+  const uint32_t nt = ntiles_dev ? *ntiles_dev : ntiles_host, r = threadIdx.x % S;
   uint32_t run = 0;
-  // sixteen loads in flight before their stores (in place: the stores
-  // would otherwise wait for each load in turn)
-  constexpr int B = 16;
-  for (uint64_t ti = t0; ti < t1; ti += B) {
-    uint32_t v[B];
+  if (threadIdx.x < S) {
+    // sixteen loads in flight before their stores (in place: the stores would
+    // otherwise wait for each load in turn)
+    constexpr int B = 16;
+    for (uint32_t ti = 0; ti < nt; ti += B) {
+      uint32_t v[B];
 #pragma unroll
-    for (int k = 0; k < B; k++) v[k] = ti + k < t1 ? tcnt[(ti + k) * S + r] : 0u;
+      for (int k = 0; k < B; k++) v[k] = ti + k < nt ? tcnt[(uint64_t)(ti + k) * S + r] : 0u;
 #pragma unroll
-    for (int k = 0; k < B; k++) {
-      if (ti + k < t1) tcnt[(ti + k) * S + r] = run;
-      run += v[k];
+      for (int k = 0; k < B; k++) {
+        if (ti + k < nt) tcnt[(uint64_t)(ti + k) * S + r] = run;
+        run += v[k];
+      }
     }
+    tchunk[r] = 0;
+    tchunk[S + r] = run;
   }
-  if constexpr (ONE) {
-    if (c == 0) {
-      tchunk[r] = 0;
-      tchunk[S + r] = run;
-    }
-    if (plan.kind != PLAN_NONE) plan_pass(run, plan);
-  } else {
-    tchunk[(uint64_t)c * S + r] = run;
-  }
+  __syncwarp();
+  if (plan.kind != PLAN_NONE) plan_pass(run, plan);
 }
 
 // ... and the exclusive prefix of the chunks' totals (u64), with the grand
@@ -1244,11 +1255,10 @@ static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const Pa
   const uint32_t* nt_dev = P.tiles ? P.ntiles_dev : nullptr;
   if (tail) {
   } else if (nchunk == 1) {
-    k_tile_scan_chunk<true><<<1, 32, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, 1, tchunk, plan);
+    k_tile_scan_one<<<1, 32, 0, st>>>(tcnt, nt_dev, P.ntiles, tchunk, plan);
     count_launch();
   } else {
-    k_tile_scan_chunk<false><<<(nchunk * TC_STRIDE + 255) / 256, 256, 0, st>>>(
-        tcnt, nt_dev, P.ntiles, Q.chsh, nchunk, tchunk, plan);
+    k_tile_scan_chunk<<<nchunk, 256, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk);
     k_tile_scan_top<<<1, 1024, 0, st>>>(tchunk, nchunk, plan);
     count_launch(2);
   }

@@ -33,3 +33,22 @@ def test_tiles_at_chunk_edges(tiles, short):
     ex = h.export()
     assert np.array_equal(ex.bits.reshape(ot.shape), ot) and np.array_equal(ex.zeros, oz)
     h.free()
+
+
+def test_chunks_of_more_than_64_tiles():
+    """More than 2^20 tiles of 2048 symbols against fewer of 8192 (the same
+    bits, whole numbers: equal)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1610_03524_gb300 as wt
+    n, sigma = (1 << 31) + 4097, 20
+    g = torch.Generator(device="cuda").manual_seed(1)
+    d = torch.randint(0, sigma, (n,), device="cuda", dtype=torch.uint8, generator=g)
+    got = []
+    for tile in (2048, 8192):
+        h = wt.wm_build(d, sigma, tile_symbols=tile)
+        ex = h.export()
+        got.append((ex.bits.copy(), ex.zeros.copy()))
+        h.free()
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
