@@ -185,8 +185,11 @@ def measured_peak_hbm():
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("k_pass.cuh", "wt_internal.cuh"):
-        with open(os.path.join(ROOT, "paper_1610_03524_gb300", "csrc", f), "rb") as fh:
+    for f in ("k_pass.cuh", "wt_internal.cuh", "bitplane.cuh"):
+        p = os.path.join(ROOT, "paper_1610_03524_gb300", "csrc", f)
+        if f == "bitplane.cuh" and not os.path.exists(p):
+            continue
+        with open(p, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
@@ -376,18 +379,17 @@ def run_native(args):
     value = ws * n * L / (ms_max * 1e-3) / 1e9
 
     # roofline of the partition-pass kernel: algorithmic bytes per launch
-    # (tau = 8: pass 0 reads 2 B, writes 1 B of the next sequence and 8 levels
-    # = 1 B; pass 1 reads 1 B and writes 1 B of levels)
+    # (four levels a pass: 4.5, 3.5, 2.5 and 1.5 B per symbol)
     alg_bytes = args.steps * sum(pass_bytes(n, L, 2, tau))
     achieved = alg_bytes / (pass_ms * 1e-3) / 1e9 if pass_ms > 0 else None
     peak, peak_kind = measured_peak_hbm()
     # (the committed figure is per launch at n = 2^30: scaled to this n, as
     # a tile's traffic is its own data and two table rows)
     traffic = profiled_traffic()
-    if traffic is not None and tau == 8:
+    if traffic is not None and tau == 4:
         traffic = traffic * n / float(1 << 30)
     elif traffic is not None:
-        traffic = None  # taken at tau = 8 only
+        traffic = None  # taken at four levels a pass only
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": traffic, "kernel": "k_pass (level-group partition pass)",
@@ -405,8 +407,8 @@ def run_native(args):
                                     "inst_per_cycle_per_sm": pf.get("inst_per_cycle_per_sm"),
                                     "peak_inst_per_cycle_per_sm": 4.0,
                                     "source": "ncu --set full, 2^26 symbols (profiles/)"}
-    # whole-step byte models: B(tau) (tau = 8: ~10.16 n = histogram 2n,
-    # passes 6n, directory 2.16n); B_min = n w + L n / 8 + directory writes
+    # whole-step byte models: B(tau) (tau = 4: ~16.16 n = check of the symbols
+    # 2n, passes 12n, directory 2.16n); B_min = n w + L n / 8 + directory writes
     # (L n / 128 + L n / 512 select samples) = 4.156 n, a single ideal pass
     roof["whole_step_frac_of_B_tau"] = (step_bytes(n, L, 2, tau) / (ms * 1e-3) / 1e9) / peak
     roof["whole_step_frac_of_Bmin"] = ((2 + 2 + 16 / 128 + 16 / 512) * n / (ms * 1e-3) / 1e9) / peak

@@ -6,10 +6,10 @@
 // decomposition across sequences: the tiles of every sequence form one work
 // list, each tile carries its sequence's parameters, and the per-tile class
 // counts are chained only between tiles of the same sequence.  So a batch of
-// m sequences costs one histogram launch, one planning launch, one partition
-// launch per pass index (two if some sequences need 32-bit working
-// elements), and one set of directory launches over all levels of all
-// sequences, instead of m times that.  Every device array of the batch sits
+// m sequences costs, per pass index and width of its elements, one launch of
+// tile counts, two of their scans, one of plans and one of the partition, and
+// one set of directory launches over all levels of all sequences, instead of
+// m times that.  Every device array of the batch sits
 // in one allocation (the arena) shared by the m handles.
 #include <algorithm>
 #include <cmath>

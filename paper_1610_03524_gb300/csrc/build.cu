@@ -2,15 +2,16 @@
 // 4-ary wavelet trees on one GPU.
 //
 // Pipeline of one build (all on one stream, no host synchronisation except
-// the Huffman code construction):
-//   1. histogram + validation pass over S (Section 4.1: counting for the
-//      integer sort; for the wavelet matrix one digit histogram per pass,
-//      since a histogram does not depend on the order of the elements);
-//   2. plan: node/class start offsets of every level by prefix sums
-//      (Section 4.2), zero counts z_l (Section 4.3), tile ticket reset;
-//   3. one partition pass per tau levels (k_pass.cuh), each after the
-//      per-tile digit counts and their prefix sums across the tiles;
-//   4. rank/select directories on every level (dirq.cu).
+// for a Huffman code's tables):
+//   1. Huffman-shaped trees: symbol counts, code (huffdev.cu, or huffman.cpp
+//      for small alphabets) and the symbols' codewords, which the passes read;
+//   2. per pass of up to four levels: every tile's digit counts (Section 4.1:
+//      counting for the integer sort), the first pass's with the check of the
+//      symbols; their prefix sums across the tiles (Section 4.2); from the
+//      totals the start offsets of the pass's nodes or classes and its zero
+//      counts z_l (Section 4.3): one launch up to SCAN_TILES tiles, else three;
+//      then the partition (k_pass.cuh);
+//   3. rank/select directories on every level (dirq.cu).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -1465,8 +1466,8 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   h->bpe = 1;
   set_uniform_levels(h, n);
   const uint64_t W = level_words(n);
-  // the level buffer is zeroed by the build's kernels (the histogram kernel
-  // the first pass's levels, each pass the next pass's), not by a memset
+  // the level buffer is zeroed by the build's kernels (the first pass's counts
+  // the levels of two passes, each later pass the next one's), not by a memset
   TRY(alloc_outputs(h, W * L, n == 0));
   Work wk{st};
   if (n == 0) return build_directories(h);

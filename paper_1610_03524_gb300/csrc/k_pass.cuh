@@ -26,8 +26,9 @@
 // domain decomposition of Section 4.2 with K = number of tiles and per-node
 // offsets by prefix sums across the K sub-problems.
 //
-// What bounds it: instructions, most of them on the integer logic pipe (65% of
-// it used, 2.45 instructions per cycle and SM; DRAM below 15%).  An earlier
+// What bounds it: instructions, most of them on the integer logic pipe (66% of
+// it used, 2.6 instructions per cycle and SM; DRAM below 20%), and the warps'
+// waits for each other three times a tile.  An earlier
 // form moved the elements once per level through shared memory (a ballot, a
 // rank and a store per 32 elements and level): 231 and 198 warp instructions
 // per 32 elements for its two passes of 8 levels, 14.3 ms for the 2^30 16-bit
@@ -39,7 +40,8 @@
 // 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).  One warp's lanes for both kinds of
 // runs, pieces masked in place and the splits' shared parities: 9.5 ms (2^28:
 // 2.37 ms; 32-bit 0.82).  The other warps take the work that warp 0, which
-// they wait for, had beside the runs' layout: 9.3 ms (2.32; 0.80).
+// they wait for, had beside the runs' layout: 60 to 62 instructions (42 the
+// last pass) and 9.2 ms (2.32; 0.80).
 #pragma once
 #include <type_traits>
 

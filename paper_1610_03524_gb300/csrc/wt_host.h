@@ -190,7 +190,7 @@ struct Work {
 
 // Host -> device copy of a small table through a kernel's parameters (no
 // copy engine: a small copy would otherwise queue behind large transfers of
-// other streams); larger tables by cudaMemcpyAsync.
+// other streams); larger tables through a pinned staging buffer.
 wt_status upload(void* d_dst, const void* h_src, size_t bytes, cudaStream_t st);
 
 // Launch accounting (all kernels of the library) and optional CUDA-event

@@ -22,7 +22,7 @@ enum : uint32_t { ERR_SYMBOL = 1u, ERR_INTERNAL = 4u };
 enum Shape : int { SHAPE_WM = 0, SHAPE_WT = 1, SHAPE_HUFF = 2 };
 
 // One tile of a pass: `count` consecutive elements of T_a starting at
-// `start`, all inside node `node` (bit 31 of `flags`: first tile of its node).
+// `start`, all inside node `node` (first: the first tile of its node).
 struct TileDesc {
   uint64_t start;
   uint32_t count;
