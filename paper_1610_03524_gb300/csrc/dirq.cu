@@ -170,37 +170,50 @@ __device__ uint32_t find_in_sb(const uint64_t* lbits, uint64_t rel, uint64_t s, 
   return (uint32_t)((8 * b + at) * 64) + sel64(word, r);
 }
 
-// Select samples of 32 consecutive superblocks of a level, one per lane (live;
-// superblock s0 + lane, zeros zb before it and zs in it, rel the second word
-// of its record): every 4096th zero and one.  About half of the superblocks of
-// a dense level hold a sample, so the warp's searches are dealt to its lanes
-// in one go instead of the zeros' and the ones' in turn with half of the lanes
-// idle.
-__device__ __forceinline__ void warp_samples(bool live, uint64_t s0, uint64_t zb, uint32_t zs,
-                                             uint64_t rel, const LevelMeta& m, const uint64_t* lb,
-                                             bool aligned, uint64_t* samp) {
+// Select samples of a group: every 4096th zero and one of the level's
+// superblocks s0 + 2 lane and the next (live; zeros zb before it and zs in it,
+// rel the second word of its record).  About half of the superblocks of a dense
+// level hold a sample, so a lane has about one search, and the warp's are dealt
+// to its lanes instead of the zeros' and the ones' in turn.
+__device__ __forceinline__ void warp_samples(const bool live[2], uint64_t s0, const uint64_t zb[2],
+                                             const uint32_t zs[2], const uint64_t rel[2],
+                                             const LevelMeta& m, const uint64_t* lb, bool aligned,
+                                             uint64_t* samp) {
   const int lane = threadIdx.x & 31;
-  const uint64_t s = s0 + lane;
-  const uint64_t nvalid = live ? std::min<uint64_t>(2048, m.n - 2048 * s) : 0;
-  const uint64_t ob = 2048 * s - zb;
-  const bool h0 = live && ((zb + 4095) & ~4095ull) < zb + zs;
-  const bool h1 = live && ((ob + 4095) & ~4095ull) < ob + (nvalid - zs);
-  const uint32_t m0 = __ballot_sync(FULL, h0), m1 = __ballot_sync(FULL, h1);
-  const uint32_t n0 = __popc(m0), total = n0 + __popc(m1);
-  for (uint32_t b = 0; b < total; b += 32) {
+  // lanes with a sample: zeros of the first, of the second superblock; ones
+  uint32_t has[4], first[5] = {0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const int e = c & 1;
+    const uint64_t s = s0 + 2 * lane + e;
+    bool h;
+    if (c < 2) {
+      h = live[e] && ((zb[e] + 4095) & ~4095ull) < zb[e] + zs[e];
+    } else {
+      const uint64_t nvalid = live[e] ? std::min<uint64_t>(2048, m.n - 2048 * s) : 0;
+      const uint64_t ob = 2048 * s - zb[e];
+      h = live[e] && ((ob + 4095) & ~4095ull) < ob + (nvalid - zs[e]);
+    }
+    has[c] = __ballot_sync(FULL, h);
+    first[c + 1] = first[c] + __popc(has[c]);
+  }
+  for (uint32_t b = 0; b < first[4]; b += 32) {
     const uint32_t task = b + lane;
-    const bool on = task < total;
-    const int bv = task >= n0 ? 1 : 0;
-    const int src = on ? nth_bit(bv ? m1 : m0, bv ? task - n0 : task) : 0;
-    const uint64_t szb = __shfl_sync(FULL, zb, src), srel = __shfl_sync(FULL, rel, src);
+    const bool on = task < first[4];
+    const int c = task >= first[3] ? 3 : (task >= first[2] ? 2 : (task >= first[1] ? 1 : 0));
+    const uint32_t mask = c == 3 ? has[3] : (c == 2 ? has[2] : (c == 1 ? has[1] : has[0]));
+    const uint32_t f = c == 3 ? first[3] : (c == 2 ? first[2] : (c == 1 ? first[1] : 0u));
+    const int src = on ? nth_bit(mask, task - f) : 0, e = c & 1, bv = c >> 1;
+    const uint64_t z0 = __shfl_sync(FULL, zb[0], src), z1 = __shfl_sync(FULL, zb[1], src);
+    const uint64_t r0 = __shfl_sync(FULL, rel[0], src), r1 = __shfl_sync(FULL, rel[1], src);
     if (on) {
-      const uint64_t ss = s0 + src;
-      const uint64_t before = bv ? 2048 * ss - szb : szb, k = (before + 4095) >> 12;
+      const uint64_t ss = s0 + 2 * src + e, z = e ? z1 : z0;
+      const uint64_t before = bv ? 2048 * ss - z : z, k = (before + 4095) >> 12;
       // a whole superblock's words can all be read; the last one's, and those
       // of a caller's bitvector off a 16-byte boundary, one by one up to the end
       const uint64_t nw = ss + 1 < m.nsb && aligned ? PADDED : (m.n + 63) / 64;
       samp[(bv ? m.s1_off : m.s0_off) + k] =
-          2048 * ss + find_in_sb(lb, srel, ss, bv, (uint32_t)(4096 * k - before), nw);
+          2048 * ss + find_in_sb(lb, e ? r1 : r0, ss, bv, (uint32_t)(4096 * k - before), nw);
     }
   }
 }
@@ -333,11 +346,11 @@ __global__ void __launch_bounds__(256) k_dir_count(const uint64_t* bits, const L
       if (zeros) zeros[blockIdx.x] = total;
     }
     __syncthreads();
-    if (warp < 2) {
-      const uint64_t i = 32 * warp + lane;
-      const uint32_t at = __shfl_sync(FULL, inc - a - b, 16 * warp + (lane >> 1));
-      const uint32_t pa = __shfl_sync(FULL, a, 16 * warp + (lane >> 1));
-      warp_samples(i < m.nsb, 32 * warp, at + ((lane & 1) ? pa : 0u), s_z[i], s_rel[i], m, lb, vec, samp);
+    if (warp == 0) {
+      const bool live[2] = {2 * (uint64_t)lane < m.nsb, 2 * (uint64_t)lane + 1 < m.nsb};
+      const uint64_t zb[2] = {inc - a - b, inc - b}, rl[2] = {s_rel[2 * lane], s_rel[2 * lane + 1]};
+      const uint32_t zs[2] = {a, b};
+      warp_samples(live, 0, zb, zs, rl, m, lb, vec, samp);
     }
   }
 }
@@ -433,20 +446,21 @@ __global__ void __launch_bounds__(32) k_dir_groups(const LevelMeta* meta, const 
   dir_groups<false>((int)blockIdx.x, 0, meta, blk_first, blk_tot, dir, zeros, dl);
 }
 
-// Absolute counts and select samples: 64 threads per group.  (Whole records
-// are stored: 2^33 bits in 83 us, against 93 with their changed half only,
-// every other 8 bytes.)
+// Absolute counts and select samples: a warp per group, two superblocks a lane.
+// (2^33 bits: 62 us; 83 with a superblock a lane, half of whose searches were
+// idle, and 93 with only the changed half of each record stored.)
 template <bool SMALL>
 __global__ void __launch_bounds__(256) k_dir_finish(const uint64_t* bits, const LevelMeta* meta,
                                                     int nlev, const uint64_t* blk_first,
                                                     uint64_t ngroups, const uint64_t* blk,
                                                     uint64_t* dir, uint64_t* samp,
                                                     const __grid_constant__ DirLevels dl) {
+  static_assert(DIR_GROUP == 64, "two superblocks a lane");
   const int lane = threadIdx.x & 31;
-  const uint64_t g = (uint64_t)blockIdx.x * (256 / DIR_GROUP) + threadIdx.x / DIR_GROUP;
-  const bool in = g < ngroups;
+  const uint64_t g = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (g >= ngroups) return;  // a whole warp
   LevelMeta m;
-  uint64_t s0;
+  uint64_t s0;  // the group's first superblock
   if (SMALL) {
     int l = 0;
     while (l + 1 < dl.nlev && dl.blk_first[l + 1] <= g) l++;
@@ -457,27 +471,27 @@ __global__ void __launch_bounds__(256) k_dir_finish(const uint64_t* bits, const 
     m = meta[l];
     s0 = (g - blk_first[l]) * DIR_GROUP;
   }
-  s0 += threadIdx.x % DIR_GROUP - lane;  // the warp's first superblock
-  const uint64_t s = s0 + lane;
-  const bool live = in && s < m.nsb;
+  const uint64_t s = s0 + 2 * lane;
+  const bool live[2] = {s < m.nsb, s + 1 < m.nsb};
   uint64_t* const ld = dir + m.dir_off;
-  ulonglong2 rec = make_ulonglong2(0, 0);
-  uint64_t end = 0;  // zeros before the next superblock
-  if (live) {
-    rec = *(const ulonglong2*)(ld + 2 * s);
-    rec.x += blk[g];
-    // the last superblock of the level, and of the group
-    if (s + 1 == m.nsb) end = ld[2 * m.nsb];
-    else if ((s + 1) % DIR_GROUP == 0) end = blk[g + 1];
-    else if (lane == 31) end = blk[g] + ld[2 * s + 2];
-  }
-  const uint64_t next = __shfl_down_sync(FULL, rec.x, 1);
-  if (live && lane < 31 && s + 1 < m.nsb && (s + 1) % DIR_GROUP) end = next;
-  // the middle of a group is read by one warp and written by the other
-  __syncthreads();
-  if (live) *(ulonglong2*)(ld + 2 * s) = rec;
+  const uint64_t base = blk[g];
+  ulonglong2 r0 = make_ulonglong2(0ull, 0ull), r1 = r0;
+  if (live[0]) r0 = *(const ulonglong2*)(ld + 2 * s);
+  if (live[1]) r1 = *(const ulonglong2*)(ld + 2 * s + 2);
+  r0.x += base;
+  r1.x += base;
+  // zeros before the next superblock: of the level's last one, its total; after
+  // the group's last one, the next group's
+  uint64_t end0 = r1.x, end1 = __shfl_down_sync(FULL, r0.x, 1);
+  if (live[0] && !live[1]) end0 = ld[2 * m.nsb];
+  if (live[1] && s + 2 == m.nsb) end1 = ld[2 * m.nsb];
+  else if (live[1] && lane == 31) end1 = blk[g + 1];
+  if (live[0]) *(ulonglong2*)(ld + 2 * s) = r0;
+  if (live[1]) *(ulonglong2*)(ld + 2 * s + 2) = r1;
   const uint64_t* lb = bits + m.bit_off;
-  warp_samples(live, s0, rec.x, (uint32_t)(end - rec.x), rec.y, m, lb, (((uintptr_t)lb) & 15) == 0, samp);
+  const uint64_t zb[2] = {r0.x, r1.x}, rel[2] = {r0.y, r1.y};
+  const uint32_t zs[2] = {(uint32_t)(end0 - r0.x), (uint32_t)(end1 - r1.x)};
+  warp_samples(live, s0, zb, zs, rel, m, lb, (((uintptr_t)lb) & 15) == 0, samp);
 }
 
 // ---------------------------------------------------------------------------
@@ -752,7 +766,7 @@ wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32
   Work wk{st};
   uint64_t *d_first = nullptr, *blk;
   TRY(wk.get(&blk, nblk + 1));
-  const unsigned fgrid = (unsigned)((nblk + 256 / DIR_GROUP - 1) / (256 / DIR_GROUP));
+  const unsigned fgrid = (unsigned)((nblk + 7) / 8);
   if (small) {
     k_dir_count<true, false><<<(unsigned)nblk, 256, 0, st>>>(bits, nullptr, (int)nlev, nullptr, dir,
                                                             blk, samp, nullptr, dl);
