@@ -14,6 +14,7 @@
 //   3. rank/select directories on every level (dirq.cu).
 #include <algorithm>
 #include <cmath>
+#include <cooperative_groups.h>
 #include <type_traits>
 #include <atomic>
 #include <cstdio>
@@ -1135,17 +1136,22 @@ __global__ void __launch_bounds__(32) k_tile_scan_one(uint32_t* tcnt, const uint
 }
 
 // ... and the exclusive prefix of the chunks' totals (u64), with the grand
-// total after the last chunk, and the pass's plan from it: one block, 64 runs
-// of chunks side by side whose sums are known before they are scanned.
-__global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32_t nchunk,
-                                                        const PassPlan plan) {
+// total after the last chunk, and the pass's plan from it: a cluster of blocks,
+// 64 runs of chunks side by side in each, whose sums are known before they are
+// scanned.  (4096 chunks 8 us, 16384 chunks 14; one block, whose loads in flight
+// bound it, 19 and 62.)
+constexpr int TOP_CLUSTER = 8;
+__global__ void __cluster_dims__(TOP_CLUSTER, 1, 1) __launch_bounds__(1024)
+    k_tile_scan_top(uint64_t* tchunk, uint32_t nchunk, const PassPlan plan) {
+  namespace cg = cooperative_groups;
   constexpr int S = TC_STRIDE, RUN = 1024 / S;
   __shared__ uint64_t sums[RUN][S];
-  __shared__ uint64_t total[S];
+  __shared__ uint64_t total[S];  // the block's
+  const uint32_t rank = cg::this_cluster().block_rank();
   const uint32_t r = threadIdx.x % S, w = threadIdx.x / S;
-  const uint32_t per = (nchunk + RUN - 1) / RUN;
-  const uint32_t c0 = min(w * per, nchunk), c1 = min(c0 + per, nchunk);
-  constexpr int B = 16;
+  const uint32_t per = (nchunk + RUN * TOP_CLUSTER - 1) / (RUN * TOP_CLUSTER);
+  const uint32_t c0 = min((rank * RUN + w) * per, nchunk), c1 = min(c0 + per, nchunk);
+  constexpr int B = 8;
   uint64_t sum = 0;
   for (uint32_t c = c0; c < c1; c += B) {
     uint64_t v[B];
@@ -1157,7 +1163,18 @@ __global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32
   sums[w][r] = sum;
   __syncthreads();
   uint64_t run = 0;
+#pragma unroll 8
   for (uint32_t k = 0; k < w; k++) run += sums[k][r];
+  if (w == RUN - 1) total[r] = run + sum;
+  cg::this_cluster().sync();
+  uint64_t all = 0;
+#pragma unroll
+  for (uint32_t q = 0; q < TOP_CLUSTER; q++) {
+    const uint64_t x = cg::this_cluster().map_shared_rank(total, q)[r];
+    all += x;
+    run += q < rank ? x : 0ull;
+  }
+  cg::this_cluster().sync();  // the totals are read before a block ends
   for (uint32_t c = c0; c < c1; c += B) {
     uint64_t v[B];
 #pragma unroll
@@ -1168,13 +1185,9 @@ __global__ void __launch_bounds__(1024) k_tile_scan_top(uint64_t* tchunk, uint32
       run += v[k];
     }
   }
-  if (w == RUN - 1) {
-    tchunk[(uint64_t)nchunk * S + r] = run;
-    total[r] = run;
-  }
-  __syncthreads();
-  if (threadIdx.x < 32 && plan.kind != PLAN_NONE)
-    plan_pass(threadIdx.x < S ? total[threadIdx.x] : 0ull, plan);
+  if (rank) return;
+  if (w == 0) tchunk[(uint64_t)nchunk * S + r] = all;
+  if (threadIdx.x < 32 && plan.kind != PLAN_NONE) plan_pass(threadIdx.x < S ? all : 0ull, plan);
 }
 
 template <int EW, bool DIG, bool BATCH, int NT>
@@ -1260,7 +1273,7 @@ static wt_status run_pass(const PassParams& P, uint64_t mt, uint32_t T, const Pa
     count_launch();
   } else {
     k_tile_scan_chunk<<<nchunk, 256, 0, st>>>(tcnt, nt_dev, P.ntiles, Q.chsh, tchunk);
-    k_tile_scan_top<<<1, 1024, 0, st>>>(tchunk, nchunk, plan);
+    k_tile_scan_top<<<TOP_CLUSTER, 1024, 0, st>>>(tchunk, nchunk, plan);
     count_launch(2);
   }
   if (BATCH) {
