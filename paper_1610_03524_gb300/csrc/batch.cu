@@ -104,6 +104,8 @@ struct SeqPlan {
   // arena offsets (u64 units inside each region)
   uint64_t bits_base, dir_base, samp_base, zeros_base, meta_base;
   // workspace offsets
+  int src_w;           // the caller's bytes per symbol (w: the first pass's)
+  uint64_t wide_off;   // the widened sequence, where they differ
   uint64_t cls_off, seq_off;  // seq_off: bytes in each ping-pong buffer
   uint64_t seq_bytes;
 };
@@ -112,6 +114,8 @@ void plan_seq(SeqPlan& p, const wt_build_opts* o) {
   p.L = (int)levels_of_b(p.sigma);
   p.tau = (o && o->tau) ? (int)std::min<uint32_t>(o->tau, TAU_MAX) : tuned_tau(p.L, p.n);
   if (p.tau < 1) p.tau = 1;
+  p.src_w = p.w;
+  p.w = pass_width(p.w, p.L);
   p.ps.clear();
   for (int a = 0; a < p.L; a += p.tau) {
     Pass1 q;
@@ -153,7 +157,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
                          cudaStream_t st, wt_struct** hs) {
   std::vector<SeqPlan> sp(m);
   uint64_t nbits = 0, ndir = 0, nsamp = 0, nzeros = 0, nmeta = 0;
-  uint64_t ncls = 0, nseq = 0;
+  uint64_t ncls = 0, nseq = 0, nwide = 0;
   uint64_t nlev_tot = 0;
   int Gmax = 0;
   for (uint32_t i = 0; i < m; i++) {
@@ -176,6 +180,8 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     for (const Pass1& q : p.ps) ncls += (2u << q.t) + q.t + 1;
     p.seq_off = nseq;
     nseq += p.G > 1 ? p.seq_bytes : 0;
+    p.wide_off = nwide;
+    nwide += p.w != p.src_w ? up(p.n * (uint64_t)p.w, 256) : 0;
     nlev_tot += p.L;
     Gmax = std::max(Gmax, p.n ? p.G : 0);
   }
@@ -245,7 +251,8 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   const uint64_t w_tab_end = up(w_sseg + sizeof(SegDesc) * std::max<uint64_t>(nsegs_tot, 1), 256);
   const uint64_t w_seq0 = w_tab_end;
   const uint64_t w_seq1 = up(w_seq0 + nseq, 256);
-  const uint64_t ws_bytes = up(w_seq1 + nseq, 256);
+  const uint64_t w_wide = up(w_seq1 + nseq, 256);
+  const uint64_t ws_bytes = up(w_wide + nwide, 256);
   void* wsv = nullptr;
   CK(dmalloc(&wsv, ws_bytes, st));
   uint8_t* Wd = (uint8_t*)wsv;
@@ -297,7 +304,8 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
           uint64_t coff = p.cls_off;
           for (int g2 = 0; g2 < g; g2++) coff += (2u << p.ps[g2].t) + p.ps[g2].t + 1;
           SegDesc& d = h_sseg[k++];
-          d.in = g == 0 ? items[i].d_seq : (const void*)(d_seq[(g - 1) & 1] + p.seq_off);
+          d.in = g == 0 ? (p.w != p.src_w ? (const void*)(Wd + w_wide + p.wide_off) : items[i].d_seq)
+                        : (const void*)(d_seq[(g - 1) & 1] + p.seq_off);
           d.out = (g + 1 < p.G) ? (void*)(d_seq[g & 1] + p.seq_off) : nullptr;
           d.bits = a_bits + p.bits_base;
           d.wm_cls = d_cls + coff;
@@ -326,6 +334,9 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   if (nzeros) CK(cudaMemsetAsync(a_zeros, 0, 8 * nzeros, st));  // empty sequences plan nothing
   wt_status s = nmeta ? upload(a_meta, h_meta_all.data(), sizeof(LevelMeta) * nmeta, st) : WT_OK;
   if (s == WT_OK) s = upload(Wd + w_gmeta, img.data(), img.size(), st);
+  for (uint32_t i = 0; i < m && nwide && s == WT_OK; i++)
+    if (sp[i].n && sp[i].w != sp[i].src_w)
+      s = widen(items[i].d_seq, sp[i].src_w, Wd + w_wide + sp[i].wide_off, sp[i].w, sp[i].n, st);
   for (size_t li = 0; li < launches.size() && s == WT_OK; li++) {
     const Launch& L0 = launches[li];
     PassParams P;

@@ -807,7 +807,7 @@ static wt_status launch_hist_full(const void* seq, int w, uint64_t n, uint32_t s
       CK(cudaMemsetAsync(dst, 0, (size_t)ncopy * sigma * 8, st));
     }
   }
-  if (!use_smem && n >= HIST_SLOTS_MIN) {
+  if (!use_smem && w > 1 && n >= HIST_SLOTS_MIN) {
     constexpr int bytes = 8 * (int)HIST_SLOTS;
     auto kern = w == 2 ? k_hist_slots<2> : k_hist_slots<4>;
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -1467,6 +1467,41 @@ wt_status upload(void* d_dst, const void* h_src, size_t bytes, cudaStream_t st) 
   return WT_OK;
 }
 
+// An alphabet can be larger than the sequence's elements can hold; the passes
+// read a digit's bits inside the element, so such a sequence is widened first
+// (reading zeros past the element's end in the pass itself cost every build 1%).
+__global__ void __launch_bounds__(256) k_widen(const void* in, int w, void* out, int ow, uint64_t n) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t x = load_elem(in, w, i);
+    if (ow == 2) ((uint16_t*)out)[i] = (uint16_t)x;
+    else ((uint32_t*)out)[i] = x;
+  }
+}
+
+// bytes per element the passes need for L levels
+int pass_width(int w, int L) { return L > 8 * w ? width_for_bits(L) : w; }
+
+wt_status widen(const void* d_in, int w, void* d_out, int ow, uint64_t n, cudaStream_t st) {
+  const unsigned grid = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms() * 16);
+  k_widen<<<grid, 256, 0, st>>>(d_in, w, d_out, ow, n);
+  count_launch();
+  CK(cudaGetLastError());
+  return WT_OK;
+}
+
+// the sequence as the passes read it
+static wt_status widened(const void** d_seq, int* w, int L, uint64_t n, Work& wk) {
+  const int ow = pass_width(*w, L);
+  if (ow == *w) return WT_OK;
+  uint8_t* wide;
+  TRY(wk.get(&wide, (size_t)n * ow));
+  TRY(widen(*d_seq, *w, wide, ow, n, wk.st));
+  *d_seq = wide;
+  *w = ow;
+  return WT_OK;
+}
+
 // ---------------------------------------------------------------------------
 // wavelet matrix
 // ---------------------------------------------------------------------------
@@ -1484,6 +1519,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   TRY(alloc_outputs(h, W * L, n == 0));
   Work wk{st};
   if (n == 0) return build_directories(h);
+  TRY(widened(&d_seq, &w, L, n, wk));
   // levels per pass, symbols per tile and CTAs per SM: the caller's, else
   // the autotuner's for (L, ceil(log2 n)), else 4 / 4096 / the occupancy limit
   const TuneConfig tc = tuned_config((uint32_t)L, n);
@@ -1557,13 +1593,14 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   h->bpe = multiary ? 2 : 1;
   set_uniform_levels(h, n);
   const int tau = pick_tau(o, L, multiary);
-  std::vector<PassGeom> ps = make_passes(L, tau, w);
+  std::vector<PassGeom> ps = make_passes(L, tau, pass_width(w, L));
   const int G = (int)ps.size();
   // a tree of one pass has its level buffer zeroed by the counting kernel
   const bool one = G == 1;
   TRY(alloc_outputs(h, h->level_off.back(), !one || n == 0));
   Work wk{st};
   if (n == 0) return build_directories(h);
+  TRY(widened(&d_seq, &w, L, n, wk));
   const uint32_t T = PT;
   const uint64_t ntiles0 = (n + T - 1) / T;
   uint64_t *scr = nullptr, *tcnt = nullptr, *toff = nullptr;

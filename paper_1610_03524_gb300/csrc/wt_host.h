@@ -188,6 +188,11 @@ struct Work {
     if (s_ != WT_OK) return s_;    \
   } while (0)
 
+// Bytes per element the passes need for L levels of w-byte symbols, and the
+// conversion to them (more than w only for alphabets that w bytes cannot hold).
+int pass_width(int w, int L);
+wt_status widen(const void* d_in, int w, void* d_out, int ow, uint64_t n, cudaStream_t st);
+
 // Host -> device copy of a small table through a kernel's parameters (no
 // copy engine: a small copy would otherwise queue behind large transfers of
 // other streams); larger tables through a pinned staging buffer.
