@@ -37,6 +37,12 @@
  *    of the k-th occurrence of c, k >= 1.  An invalid argument (i >= n,
  *    c >= sigma, k == 0, k > count of c) yields UINT64_MAX in that slot and
  *    does not fail the batch.
+ *  * wt_free, wt_batch_free and wt_server_release return a handle's arrays in
+ *    the order of the stream it was built on: queries on other streams, and the
+ *    caller's own work on exported arrays, must have finished or stand before
+ *    that point of the build stream.  Huffman-shaped trees, whose stream is the
+ *    library's, are released after every query queued on them by any stream
+ *    (captured queries excepted, which must have run).
  *  * Thread safety: distinct handles may be used from distinct threads;
  *    one handle must not be built/freed concurrently with its own use.
  */

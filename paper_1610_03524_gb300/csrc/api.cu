@@ -262,6 +262,24 @@ namespace wtk {
 wt_status join_build(wt_struct* h, cudaStream_t st, bool order) {
   return join_build_impl(h, st, order);
 }
+
+wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st, bool own) {
+  auto other = [&](const wt_struct* h) { return h->stream != st && (h->own_stream || !own); };
+  if (std::none_of(hs, hs + nh, other)) return WT_OK;
+  // queries being captured run when their graph does, which the caller orders
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+    return WT_OK;
+  cudaEvent_t ev = nullptr;
+  bool ok = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventRecord(ev, st) == cudaSuccess;
+  for (uint32_t i = 0; i < nh && ok; i++)
+    if (other(hs[i])) ok = cudaStreamWaitEvent(hs[i]->stream, ev, 0) == cudaSuccess;
+  if (ev) cudaEventDestroy(ev);
+  if (ok) return WT_OK;
+  cudaGetLastError();
+  return cudaStreamSynchronize(st) == cudaSuccess ? WT_OK : WT_ERR_CUDA;
+}
 }  // namespace wtk
 
 extern "C" {
@@ -393,7 +411,8 @@ wt_status wt_access(wt_handle h, const uint64_t* d_i, uint64_t q, uint64_t* d_ou
   if (!h || (q && (!d_i || !d_out))) return WT_ERR_INVALID_ARG;
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
-  return launch_query(h, 0, nullptr, d_i, q, d_out, (cudaStream_t)stream);
+  TRY(launch_query(h, 0, nullptr, d_i, q, d_out, (cudaStream_t)stream));
+  return release_after(&h, 1, (cudaStream_t)stream, true);
 }
 
 wt_status wt_rank(wt_handle h, const uint32_t* d_c, const uint64_t* d_i, uint64_t q,
@@ -401,7 +420,8 @@ wt_status wt_rank(wt_handle h, const uint32_t* d_c, const uint64_t* d_i, uint64_
   if (!h || (q && (!d_c || !d_i || !d_out))) return WT_ERR_INVALID_ARG;
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
-  return launch_query(h, 1, d_c, d_i, q, d_out, (cudaStream_t)stream);
+  TRY(launch_query(h, 1, d_c, d_i, q, d_out, (cudaStream_t)stream));
+  return release_after(&h, 1, (cudaStream_t)stream, true);
 }
 
 wt_status wt_select(wt_handle h, const uint32_t* d_c, const uint64_t* d_k, uint64_t q,
@@ -409,7 +429,8 @@ wt_status wt_select(wt_handle h, const uint32_t* d_c, const uint64_t* d_k, uint6
   if (!h || (q && (!d_c || !d_k || !d_out))) return WT_ERR_INVALID_ARG;
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
-  return launch_query(h, 2, d_c, d_k, q, d_out, (cudaStream_t)stream);
+  TRY(launch_query(h, 2, d_c, d_k, q, d_out, (cudaStream_t)stream));
+  return release_after(&h, 1, (cudaStream_t)stream, true);
 }
 
 wt_status wt_sync(wt_handle h) {

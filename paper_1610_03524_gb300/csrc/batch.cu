@@ -679,5 +679,6 @@ extern "C" wt_status wt_query_multi(const wt_handle* hs, uint32_t nh, const uint
     const wt_status s = join_build(hs[i], (cudaStream_t)stream, true);
     if (s != WT_OK) return s;
   }
-  return launch_query_multi(hs, nh, d_sid, d_op, d_c, d_x, q, d_out, (cudaStream_t)stream);
+  TRY(launch_query_multi(hs, nh, d_sid, d_op, d_c, d_x, q, d_out, (cudaStream_t)stream));
+  return release_after(hs, nh, (cudaStream_t)stream, true);
 }

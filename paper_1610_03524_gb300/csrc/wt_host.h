@@ -116,6 +116,11 @@ namespace wtk {
 // the handle's deferred status
 wt_status join_build(wt_struct* h, cudaStream_t st, bool order);
 
+// What has just been queued on st reads the arrays of the nh handles: make the
+// streams on which wt_free will release them wait for it.
+// own: only handles on a stream of their own, which no caller can order.
+wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st, bool own);
+
 // device memory helpers (stream-ordered pools)
 cudaError_t dmalloc(void** p, size_t bytes, cudaStream_t s);
 void dfree(void* p, cudaStream_t s);

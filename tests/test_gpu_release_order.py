@@ -1,0 +1,65 @@
+"""Arrays that other streams still read when a handle is freed are given back
+after those reads: Huffman-shaped trees, which live on a stream of the
+library's, under queries queued on the caller's streams."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from gpu_util import from_dev_u64, to_dev
+
+pytestmark = pytest.mark.gpu
+
+SPIN = 100_000_000  # clock cycles, about 50 ms
+
+
+@pytest.fixture(scope="module")
+def wt():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1610_03524_gb300 as m
+    m.load_library()
+    return m
+
+
+@pytest.mark.parametrize("sigma", [300, 1 << 16])
+@pytest.mark.parametrize("how", ["access", "rank", "select", "multi"])
+def test_huffman_tree_freed_behind_queued_queries(wt, sigma, how):
+    import torch
+    n, q = 200_003, 4096
+    S = synth.zipf(5, n, sigma, 1.1, 4)
+    rng = np.random.default_rng(6)
+    x = rng.integers(0, n, q).astype(np.uint64)
+    c = S[x].astype(np.uint32)
+    one = np.ones(q, np.uint64)
+    exp = {"access": c.astype(np.uint64), "rank": oracle.rank(S, sigma, c, x),
+           "select": oracle.select(S, sigma, c, one),
+           "multi": oracle.rank(S, sigma, c, x)}[how]
+    side, build = torch.cuda.Stream(), torch.cuda.Stream()
+    h = wt.huff_wt_build(to_dev(S), sigma)
+    h.sync()
+    dx, dc, dk = to_dev(x), to_dev(c), to_dev(one)
+    out = torch.zeros(q, dtype=torch.int64, device="cuda")
+    multi = (torch.zeros(q, dtype=torch.int32, device="cuda"),
+             torch.ones(q, dtype=torch.uint8, device="cuda"), dc, dx, out)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(SPIN)
+        if how == "access":
+            h.access(dx, out)
+        elif how == "rank":
+            h.rank(dc, dx, out)
+        elif how == "select":
+            h.select(dc, dk, out)
+        else:
+            wt.query_multi([h], *multi)
+    h.free()
+    assert side.query()  # the queries, queued behind the spin, are over
+    # memory given back is taken by the next build on another stream
+    with torch.cuda.stream(build):
+        T = synth.zipf(7, n, sigma, 1.1, 4)
+        h2 = wt.huff_wt_build(to_dev(T), sigma)
+        h2.sync()
+    assert np.array_equal(from_dev_u64(out), exp)
+    h2.free()
