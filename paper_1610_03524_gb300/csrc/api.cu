@@ -403,6 +403,7 @@ wt_status wt_dd_merge(const wt_handle* parts, uint32_t r, const wt_build_opts* o
   h->kind = p0->kind;
   h->L = h->levels = p0->L;
   s = dd_merge(parts, r, h);
+  if (s == WT_OK) s = release_after(parts, r, h->stream, false);
   return finish(h, s, out);
 }
 

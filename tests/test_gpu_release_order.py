@@ -1,6 +1,7 @@
 """Arrays that other streams still read when a handle is freed are given back
 after those reads: Huffman-shaped trees, which live on a stream of the
-library's, under queries queued on the caller's streams."""
+library's, under queries queued on the caller's streams, and the parts of a
+merge on another stream than theirs."""
 import numpy as np
 import pytest
 
@@ -63,3 +64,26 @@ def test_huffman_tree_freed_behind_queued_queries(wt, sigma, how):
         h2.sync()
     assert np.array_equal(from_dev_u64(out), exp)
     h2.free()
+
+
+def test_parts_freed_behind_a_queued_merge(wt):
+    import torch
+    n, sigma = 1 << 24, 256
+    S = synth.zipf(9, n, sigma, 1.1, 1)
+    ob, oz = oracle.wm_build(S, sigma)
+    build, merge = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(build):
+        parts = [wt.wm_build(to_dev(S[a:b].copy()), sigma) for a, b in ((0, n // 3), (n // 3, n))]
+        build.synchronize()
+    with torch.cuda.stream(merge):
+        h = wt.dd_merge(parts)
+    parts[0].free()  # waits for its stream, which waits for the merge
+    assert merge.query()
+    parts[1].free()
+    with torch.cuda.stream(build):
+        again = wt.wm_build(to_dev(S[::-1].copy()), sigma)
+        again.sync()
+    ex = h.export()
+    assert np.array_equal(ex.bits.reshape(ob.shape), ob) and np.array_equal(ex.zeros, oz)
+    h.free()
+    again.free()
