@@ -34,6 +34,7 @@ wt_status dir_build_levels(const uint64_t* bits, const LevelMeta* d_meta, uint32
     cudaError_t e_ = (x);                                       \
     if (e_ != cudaSuccess) {                                    \
       fprintf(stderr, "wavelet: %s -> %s\n", #x, cudaGetErrorString(e_)); \
+      cudaGetLastError(); /* reported here */                   \
       return e_ == cudaErrorMemoryAllocation ? WT_ERR_NO_MEMORY : WT_ERR_CUDA; \
     }                                                           \
   } while (0)

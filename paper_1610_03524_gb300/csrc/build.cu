@@ -34,6 +34,7 @@ namespace wtk {
     cudaError_t e_ = (x);                                       \
     if (e_ != cudaSuccess) {                                    \
       fprintf(stderr, "wavelet: %s -> %s\n", #x, cudaGetErrorString(e_)); \
+      cudaGetLastError(); /* reported here */                   \
       return e_ == cudaErrorMemoryAllocation ? WT_ERR_NO_MEMORY : WT_ERR_CUDA; \
     }                                                           \
   } while (0)
@@ -66,7 +67,10 @@ cudaError_t dmalloc(void** p, size_t bytes, cudaStream_t s) {
     }
   }
   if (bytes == 0) bytes = 16;
-  return cudaMallocAsync(p, bytes, s);
+  const cudaError_t e = cudaMallocAsync(p, bytes, s);
+  // the caller has the error: the thread's next call does not meet it again
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 void dfree(void* p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);

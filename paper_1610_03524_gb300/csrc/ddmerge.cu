@@ -39,6 +39,7 @@ uint64_t scan_scratch_pub(uint64_t n);
     cudaError_t e_ = (x);                                                       \
     if (e_ != cudaSuccess) {                                                    \
       fprintf(stderr, "wavelet: %s -> %s\n", #x, cudaGetErrorString(e_));      \
+      cudaGetLastError(); /* reported here */                                   \
       return e_ == cudaErrorMemoryAllocation ? WT_ERR_NO_MEMORY : WT_ERR_CUDA; \
     }                                                                           \
   } while (0)

@@ -30,6 +30,7 @@ constexpr uint64_t NONE = ~0ull;
     cudaError_t e_ = (x);                                       \
     if (e_ != cudaSuccess) {                                    \
       fprintf(stderr, "wavelet: %s -> %s\n", #x, cudaGetErrorString(e_)); \
+      cudaGetLastError(); /* reported here */                   \
       return e_ == cudaErrorMemoryAllocation ? WT_ERR_NO_MEMORY : WT_ERR_CUDA; \
     }                                                           \
   } while (0)

@@ -76,7 +76,10 @@ struct Pinned {
     p = nullptr;
     cap = 0;
     size_t c = std::max<size_t>(n, 1 << 20);
-    if (cudaHostAlloc(&p, c, cudaHostAllocDefault) != cudaSuccess) return false;
+    if (cudaHostAlloc(&p, c, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
     cap = c;
     return true;
   }
