@@ -107,8 +107,8 @@ struct SeqPlan {
   // workspace offsets
   int src_w;           // the caller's bytes per symbol (w: the first pass's)
   uint64_t wide_off;   // the widened sequence, where they differ
-  uint64_t cls_off, seq_off;  // seq_off: bytes in each ping-pong buffer
-  uint64_t seq_bytes;
+  uint64_t cls_off;
+  uint64_t seq_off[2], seq_bytes[2];  // in the buffers of the even and of the odd passes' outputs
 };
 
 void plan_seq(SeqPlan& p, const wt_build_opts* o) {
@@ -131,9 +131,11 @@ void plan_seq(SeqPlan& p, const wt_build_opts* o) {
   p.W = level_words_b(p.n);
   p.nsb = (p.n + 2047) / 2048;
   p.cap = p.n / 4096 + 1;
-  int ow = 0;
-  for (const Pass1& q : p.ps) ow = std::max(ow, q.out_w);
-  p.seq_bytes = up(p.n * (uint64_t)ow, 256);
+  for (int k = 0; k < 2; k++) {
+    int ow = 0;
+    for (int g = k; g < p.G; g += 2) ow = std::max(ow, p.ps[g].out_w);
+    p.seq_bytes[k] = up(p.n * (uint64_t)ow, 256);
+  }
 }
 
 // bytes of the arena regions of one sequence
@@ -158,7 +160,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
                          cudaStream_t st, wt_struct** hs) {
   std::vector<SeqPlan> sp(m);
   uint64_t nbits = 0, ndir = 0, nsamp = 0, nzeros = 0, nmeta = 0;
-  uint64_t ncls = 0, nseq = 0, nwide = 0;
+  uint64_t ncls = 0, nseq[2] = {0, 0}, nwide = 0;
   uint64_t nlev_tot = 0;
   int Gmax = 0;
   for (uint32_t i = 0; i < m; i++) {
@@ -179,8 +181,10 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     nmeta += p.L;
     p.cls_off = ncls;
     for (const Pass1& q : p.ps) ncls += (2u << q.t) + q.t + 1;
-    p.seq_off = nseq;
-    nseq += p.G > 1 ? p.seq_bytes : 0;
+    for (int k = 0; k < 2; k++) {
+      p.seq_off[k] = nseq[k];
+      nseq[k] += p.seq_bytes[k];
+    }
     p.wide_off = nwide;
     nwide += p.w != p.src_w ? up(p.n * (uint64_t)p.w, 256) : 0;
     nlev_tot += p.L;
@@ -251,8 +255,8 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   const uint64_t w_sseg = up(w_gmeta + sizeof(LevelMeta) * nlev_tot, 256);
   const uint64_t w_tab_end = up(w_sseg + sizeof(SegDesc) * std::max<uint64_t>(nsegs_tot, 1), 256);
   const uint64_t w_seq0 = w_tab_end;
-  const uint64_t w_seq1 = up(w_seq0 + nseq, 256);
-  const uint64_t w_wide = up(w_seq1 + nseq, 256);
+  const uint64_t w_seq1 = w_seq0 + nseq[0];
+  const uint64_t w_wide = w_seq1 + nseq[1];
   const uint64_t ws_bytes = up(w_wide + nwide, 256);
   void* wsv = nullptr;
   CK(dmalloc(&wsv, ws_bytes, st));
@@ -306,8 +310,8 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
           for (int g2 = 0; g2 < g; g2++) coff += (2u << p.ps[g2].t) + p.ps[g2].t + 1;
           SegDesc& d = h_sseg[k++];
           d.in = g == 0 ? (p.w != p.src_w ? (const void*)(Wd + w_wide + p.wide_off) : items[i].d_seq)
-                        : (const void*)(d_seq[(g - 1) & 1] + p.seq_off);
-          d.out = (g + 1 < p.G) ? (void*)(d_seq[g & 1] + p.seq_off) : nullptr;
+                        : (const void*)(d_seq[(g - 1) & 1] + p.seq_off[(g - 1) & 1]);
+          d.out = (g + 1 < p.G) ? (void*)(d_seq[g & 1] + p.seq_off[g & 1]) : nullptr;
           d.bits = a_bits + p.bits_base;
           d.wm_cls = d_cls + coff;
           d.zeros = a_zeros + p.zeros_base;

@@ -936,13 +936,6 @@ struct PassGeom {
   int a, t, rbits, in_w, out_w;
 };
 
-// bytes per element of the widest intermediate sequence
-static int max_out_w(const std::vector<PassGeom>& ps) {
-  int w = 1;
-  for (const PassGeom& p : ps) w = std::max(w, p.out_w);
-  return w;
-}
-
 static std::vector<PassGeom> make_passes(int L, int tau, int first_w) {
   std::vector<PassGeom> ps;
   for (int a = 0; a < L; a += tau) {
@@ -955,6 +948,19 @@ static std::vector<PassGeom> make_passes(int L, int tau, int first_w) {
     ps.push_back(p);
   }
   return ps;
+}
+
+// The sequences between the passes: pass g writes buffer g & 1, which holds the
+// largest of the outputs that it gets (count(g): elements that pass g writes).
+template <typename Count>
+static void want_seqbufs(Work& wk, uint8_t* buf[2], const std::vector<PassGeom>& ps, Count&& count) {
+  const int G = (int)ps.size();
+  for (int k = 0; k < std::min(G - 1, 2); k++) {
+    uint64_t bytes = 0;
+    for (int g = k; g + 1 < G; g += 2)
+      bytes = std::max<uint64_t>(bytes, count(g) * (uint64_t)ps[g].out_w);
+    wk.want(&buf[k], bytes);
+  }
 }
 
 // Batched builds, one warp per sequence of the launch: the plan of its pass
@@ -1544,7 +1550,7 @@ wt_status build_wm(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
   uint8_t* seqbuf[2] = {nullptr, nullptr};  // intermediate sequences
   wk.want(&cls, ncls);
   tb.want(wk, ntiles);
-  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  want_seqbufs(wk, seqbuf, ps, [&](int) { return n; });
   TRY(wk.take());
   const void* in = d_seq;
   int coff = 0;
@@ -1623,7 +1629,7 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     wk.want(&tiles, ntiles0 + max_nodes + 1);
     wk.want(&d_ntiles, 1);
   }
-  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  want_seqbufs(wk, seqbuf, ps, [&](int) { return n; });
   TRY(wk.take());
   // Every pass is planned from its own tiles' digit counts (no histogram of
   // the symbols): C holds the starts of the nodes of level a, and the totals
@@ -2067,7 +2073,7 @@ wt_status build_huff(void* d_seq, uint64_t n, uint32_t sigma, int w, const uint8
   wk.want(&d_ntiles, 1);
   tb.want(wk, most);
   if (w < 4) wk.want(&codes, n);
-  for (int g = 0; g < std::min(G - 1, 2); g++) wk.want(&seqbuf[g], (size_t)n * max_out_w(ps));
+  want_seqbufs(wk, seqbuf, ps, [&](int g) { return h->level_len[ps[g + 1].a]; });
   TRY(wk.take());
   TRY(upload(d_off, h->level_off.data(), (Lm + 1) * 8, st));
   TRY(upload(d_len, h->level_len.data(), Lm * 8, st));

@@ -138,3 +138,40 @@ def first_diff(a: np.ndarray, b: np.ndarray):
         return True, ""
     i = int(np.flatnonzero(a.reshape(-1) != b.reshape(-1))[0])
     return False, f"word {i}: {int(a.reshape(-1)[i]):#x} vs {int(b.reshape(-1)[i]):#x}"
+
+
+class PoolUse:
+    """Bytes that the device's memory pool, from which the library allocates,
+    hands out inside a with block: peak (the most at a time, above the start's)
+    and kept (at the end, above the start's)."""
+
+    USED_CURRENT, USED_HIGH = 7, 8  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+
+    def __init__(self):
+        import ctypes
+        import torch
+        self._c = ctypes
+        self._sync = torch.cuda.synchronize
+        self._sync()
+        self._cu = ctypes.CDLL("libcuda.so.1")
+        self._pool = ctypes.c_void_p()
+        assert self._cu.cuDeviceGetDefaultMemPool(ctypes.byref(self._pool),
+                                                  torch.cuda.current_device()) == 0
+
+    def _attr(self, attr, put=None):
+        v = self._c.c_uint64(0)
+        fn = self._cu.cuMemPoolGetAttribute if put is None else self._cu.cuMemPoolSetAttribute
+        assert fn(self._pool, attr, self._c.byref(v)) == 0
+        return v.value
+
+    def __enter__(self):
+        self._sync()
+        self._attr(self.USED_HIGH, put=0)  # the only value there is: the mark starts anew
+        self._base = self._attr(self.USED_CURRENT)
+        return self
+
+    def __exit__(self, *exc):
+        self._sync()
+        self.peak = self._attr(self.USED_HIGH) - self._base
+        self.kept = self._attr(self.USED_CURRENT) - self._base
+        return False
