@@ -103,7 +103,7 @@ struct SeqPlan {
   std::vector<Pass1> ps;
   uint64_t W, nsb, cap;      // words per level, superblocks per level, samples per value
   // arena offsets (u64 units inside each region)
-  uint64_t bits_base, dir_base, samp_base, zeros_base, meta_base;
+  uint64_t bits_base, dir_base, samp_base, zeros_base;
   // workspace offsets
   int src_w;           // the caller's bytes per symbol (w: the first pass's)
   uint64_t wide_off;   // the widened sequence, where they differ
@@ -151,15 +151,14 @@ uint64_t wm_resident_bytes(uint64_t n, uint32_t sigma) {
   p.sigma = sigma;
   p.w = 2;
   plan_seq(p, nullptr);
-  return 8 * (bits_u64(p) + dir_u64(p) + samp_u64(p) + (uint64_t)p.L) +
-         (uint64_t)p.L * sizeof(LevelMeta) + 8;
+  return 8 * (bits_u64(p) + dir_u64(p) + samp_u64(p) + (uint64_t)p.L) + 8;
 }
 
 // Builds m wavelet matrices with directories; outs[i] receives handle i.
 wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_opts* o,
                          cudaStream_t st, wt_struct** hs) {
   std::vector<SeqPlan> sp(m);
-  uint64_t nbits = 0, ndir = 0, nsamp = 0, nzeros = 0, nmeta = 0;
+  uint64_t nbits = 0, ndir = 0, nsamp = 0, nzeros = 0;
   uint64_t ncls = 0, nseq[2] = {0, 0}, nwide = 0;
   uint64_t nlev_tot = 0;
   int Gmax = 0;
@@ -173,12 +172,10 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     p.dir_base = ndir;
     p.samp_base = nsamp;
     p.zeros_base = nzeros;
-    p.meta_base = nmeta;
     nbits += bits_u64(p);
     ndir += dir_u64(p);
     nsamp += samp_u64(p);
     nzeros += p.L;
-    nmeta += p.L;
     p.cls_off = ncls;
     for (const Pass1& q : p.ps) ncls += (2u << q.t) + q.t + 1;
     for (int k = 0; k < 2; k++) {
@@ -190,12 +187,11 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     nlev_tot += p.L;
     Gmax = std::max(Gmax, p.n ? p.G : 0);
   }
-  // ---- arena: bits | dir | samp | zeros | meta | err[m] -----------------
+  // ---- arena: bits | dir | samp | zeros | err[m] ------------------------
   const uint64_t off_dir = 8 * nbits;
   const uint64_t off_samp = off_dir + 8 * ndir;
   const uint64_t off_zeros = off_samp + 8 * nsamp;
-  const uint64_t off_meta = up(off_zeros + 8 * nzeros, 256);
-  const uint64_t off_err = up(off_meta + sizeof(LevelMeta) * nmeta, 256);
+  const uint64_t off_err = up(off_zeros + 8 * nzeros, 256);
   const uint64_t arena_bytes = off_err + up(4 * (uint64_t)m, 256);
   Arena* ar = new Arena();
   ar->bytes = arena_bytes;
@@ -211,7 +207,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   uint64_t* a_dir = (uint64_t*)(A + off_dir);
   uint64_t* a_samp = (uint64_t*)(A + off_samp);
   uint64_t* a_zeros = (uint64_t*)(A + off_zeros);
-  LevelMeta* a_meta = (LevelMeta*)(A + off_meta);
   uint32_t* a_err = (uint32_t*)(A + off_err);
   // level l of a sequence inside its own arrays
   auto meta_of = [](const SeqPlan& p, int l) {
@@ -242,7 +237,6 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     h->d_dir = a_dir + p.dir_base;
     h->d_samp = a_samp + p.samp_base;
     h->d_zeros = a_zeros + p.zeros_base;
-    h->d_meta = a_meta + p.meta_base;
     h->d_err = a_err + i;
   }
   // ---- workspace ----------------------------------------------------------
@@ -272,14 +266,12 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   LevelMeta* h_gmeta = (LevelMeta*)at(w_gmeta);
   SegDesc* h_sseg = (SegDesc*)at(w_sseg);
   std::vector<uint64_t> sb_first(nlev_tot + 1, 0);
-  std::vector<LevelMeta> h_meta_all(nmeta);
   {
     uint64_t lev = 0;
     for (uint32_t i = 0; i < m; i++) {
       const SeqPlan& p = sp[i];
       for (int l = 0; l < p.L; l++, lev++) {
         LevelMeta mt = meta_of(p, l);
-        h_meta_all[p.meta_base + l] = mt;
         mt.bit_off += p.bits_base;
         mt.dir_off += p.dir_base;
         mt.s0_off += p.samp_base;
@@ -337,8 +329,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
   if (nbits) CK(cudaMemsetAsync(a_bits, 0, 8 * nbits, st));
   CK(cudaMemsetAsync(a_err, 0, 4 * (uint64_t)m, st));
   if (nzeros) CK(cudaMemsetAsync(a_zeros, 0, 8 * nzeros, st));  // empty sequences plan nothing
-  wt_status s = nmeta ? upload(a_meta, h_meta_all.data(), sizeof(LevelMeta) * nmeta, st) : WT_OK;
-  if (s == WT_OK) s = upload(Wd + w_gmeta, img.data(), img.size(), st);
+  wt_status s = upload(Wd + w_gmeta, img.data(), img.size(), st);
   for (uint32_t i = 0; i < m && nwide && s == WT_OK; i++)
     if (sp[i].n && sp[i].w != sp[i].src_w)
       s = widen(items[i].d_seq, sp[i].src_w, Wd + w_wide + sp[i].wide_off, sp[i].w, sp[i].n, st);
@@ -368,16 +359,12 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
     h->level_off.resize(p.L + 1);
     h->dir_off.resize(p.L + 1);
     h->samp_off.resize(2 * p.L + 1);
-    h->meta.resize(p.L);
     for (int l = 0; l <= p.L; l++) {
       const LevelMeta mt = meta_of(p, l);
       h->level_off[l] = mt.bit_off;
       h->dir_off[l] = mt.dir_off;
       h->samp_off[2 * l] = mt.s0_off;
-      if (l < p.L) {
-        h->samp_off[2 * l + 1] = mt.s1_off;
-        h->meta[l] = mt;
-      }
+      if (l < p.L) h->samp_off[2 * l + 1] = mt.s1_off;
     }
   }
   return WT_OK;

@@ -77,7 +77,7 @@ struct wt_struct {
   uint32_t* d_err = nullptr;     // device error word (8 bytes), zeroed with the handle,
   uint64_t* d_zeros = nullptr;   // and after it the levels' zero counts (batched: elsewhere)
   uint32_t* d_tick = nullptr;    // and tickets of the build's kernels, or null
-  wtk::LevelMeta* d_meta = nullptr;
+  wtk::LevelMeta* d_meta = nullptr;  // Huffman-shaped trees (other levels' offsets follow from n)
   // Huffman tables (device)
   uint32_t* d_code = nullptr;
   uint8_t* d_len = nullptr;
