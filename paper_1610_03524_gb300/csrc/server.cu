@@ -283,8 +283,9 @@ void wt_server_s::query_loop() {
     uint64_t q = 0;
     for (auto& r : take) q += r->q;
     // pack (sid, op, c, x) into one host staging buffer
-    const size_t b_sid = 0, b_op = b_sid + 4 * q, b_c = (b_op + q + 7) / 8 * 8, b_x = b_c + 4 * q,
-                 b_end = b_x + 8 * q, b_out = (b_end + 255) / 256 * 256, d_need = b_out + 8 * q;
+    const size_t b_sid = 0, b_op = b_sid + 4 * q, b_c = (b_op + q + 7) / 8 * 8,
+                 b_x = (b_c + 4 * q + 7) / 8 * 8, b_end = b_x + 8 * q,
+                 b_out = (b_end + 255) / 256 * 256, d_need = b_out + 8 * q;
     wt_status s = WT_OK;
     if (!pin_in.reserve(b_end) || !pin_out.reserve(8 * q)) s = WT_ERR_NO_MEMORY;
     if (s == WT_OK && d_cap < d_need) {
