@@ -142,16 +142,28 @@ void plan_seq(SeqPlan& p, const wt_build_opts* o) {
 uint64_t bits_u64(const SeqPlan& p) { return (uint64_t)p.L * p.W; }
 uint64_t dir_u64(const SeqPlan& p) { return up((uint64_t)p.L * 2 * (p.nsb + 1), 32); }
 uint64_t samp_u64(const SeqPlan& p) { return up((uint64_t)p.L * 2 * p.cap, 32); }
+// of the workspace: the sequence as the passes read it, where that is wider
+uint64_t wide_bytes(const SeqPlan& p) { return p.w != p.src_w ? up(p.n * (uint64_t)p.w, 256) : 0; }
 
 }  // namespace
 
-uint64_t wm_resident_bytes(uint64_t n, uint32_t sigma) {
+uint64_t wm_batch_bytes(uint64_t n, uint32_t sigma, uint32_t width) {
   SeqPlan p{};
   p.n = n;
   p.sigma = sigma;
-  p.w = 2;
+  p.w = (int)width;
   plan_seq(p, nullptr);
-  return 8 * (bits_u64(p) + dir_u64(p) + samp_u64(p) + (uint64_t)p.L) + 8;
+  const uint64_t L = (uint64_t)p.L;
+  const uint64_t kept = 8 * (bits_u64(p) + dir_u64(p) + samp_u64(p) + L) + 4;
+  uint64_t work = p.seq_bytes[0] + p.seq_bytes[1] + wide_bytes(p);
+  for (const Pass1& q : p.ps) work += 8 * ((2ull << q.t) + q.t + 1) + sizeof(SegDesc);
+  work += L * sizeof(LevelMeta);
+  // a pass's count tables (the tiles of the batch's sequences of the same width
+  // share a launch), and after the passes the directories' group totals
+  const uint64_t tiles = (n + PASS_T - 1) / PASS_T;
+  work += tiles * 4 * TC_STRIDE + (tiles / 64 + 1) * 8 * TC_STRIDE;
+  work += 8 * L * (p.nsb / 64 + 2);
+  return kept + work;
 }
 
 // Builds m wavelet matrices with directories; outs[i] receives handle i.
@@ -183,7 +195,7 @@ wt_status batch_build_wm(const wt_batch_item* items, uint32_t m, const wt_build_
       nseq[k] += p.seq_bytes[k];
     }
     p.wide_off = nwide;
-    nwide += p.w != p.src_w ? up(p.n * (uint64_t)p.w, 256) : 0;
+    nwide += wide_bytes(p);
     nlev_tot += p.L;
     Gmax = std::max(Gmax, p.n ? p.G : 0);
   }

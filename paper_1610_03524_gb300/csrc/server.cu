@@ -40,7 +40,7 @@ struct Request {
   std::vector<uint8_t> seq;
   uint64_t n = 0;
   uint32_t sigma = 0, width = 0;
-  uint64_t need = 0;  // bytes the build holds while it runs and after
+  uint64_t need = 0;  // bytes the build holds while it runs, set when it is admitted
   // queries
   uint64_t q = 0;
   std::vector<uint64_t> sid, x, out;
@@ -114,15 +114,14 @@ struct wt_server_s {
 
 namespace {
 
-// device bytes a build of (n, sigma, width) holds: the structure, plus while
-// it runs the device copy of the sequence, its intermediate sequences and its
-// tiles' digit counts (1 KB per 4096-symbol tile)
+// device bytes a build of (n, sigma, width) holds while it runs: the copy of
+// the sequence, the structure and the build's workspace
 uint64_t build_need(uint64_t n, uint32_t sigma, uint32_t width) {
-  return wtk::wm_resident_bytes(n, sigma) + n * (uint64_t)width + 2 * n * 2 + n / 4 + 8192;
+  return (n * (uint64_t)width + 255) / 256 * 256 + wtk::wm_batch_bytes(n, sigma, width);
 }
 
-// bytes a batched build holds besides its sequences' needs (tile counts,
-// tables, directory scratch)
+// bytes a batched build holds besides its sequences' needs (alignment and the
+// rounding of its allocations)
 constexpr uint64_t BATCH_OVERHEAD = 16ull << 20;
 
 }  // namespace
@@ -140,6 +139,8 @@ void wt_server_s::build_loop() {
       uint64_t add = BATCH_OVERHEAD;
       while (!pend_build.empty() && take.size() < opts.max_batch_builds) {
         auto& r = pend_build.front();
+        // (now, as the levels per pass may have been tuned since it was submitted)
+        r->need = build_need(r->n, r->sigma, r->width);
         if (r->need + BATCH_OVERHEAD > opts.budget_bytes) {
           finish(r, WT_ERR_NO_MEMORY);
           structs[r->id].failed = true;
@@ -381,7 +382,6 @@ wt_status wt_server_submit_build(wt_server s, const void* h_seq, uint64_t n, uin
   r->n = n;
   r->sigma = sigma;
   r->width = width_bytes;
-  r->need = build_need(n, sigma, width_bytes);
   r->seq.assign((const uint8_t*)h_seq, (const uint8_t*)h_seq + n * width_bytes);
   r->submit_ns = now_ns();
   {

@@ -241,8 +241,9 @@ struct TuneConfig {
 };
 TuneConfig tuned_config(uint32_t L, uint64_t n);
 int tuned_tau(uint32_t L, uint64_t n);
-// bytes a batched wavelet-matrix build keeps for one sequence
-uint64_t wm_resident_bytes(uint64_t n, uint32_t sigma);
+// bytes a batched wavelet-matrix build holds for one sequence while it runs,
+// besides the sequence: the structure that it keeps and its workspace
+uint64_t wm_batch_bytes(uint64_t n, uint32_t sigma, uint32_t width);
 // domain-decomposition merge of the structures of consecutive parts into
 // h (kind, L, levels, n, sigma, flags set)
 wt_status dd_merge(wt_struct* const* parts, uint32_t R, wt_struct* h);
