@@ -1077,7 +1077,6 @@ __global__ void k_tiles_write(const uint64_t* bnd, uint64_t nn, uint32_t T, uint
   d.start = s;
   d.count = (uint32_t)std::min<uint64_t>(T, e - s);
   d.node = (uint32_t)(node_base + p);
-  d.first = (k == 0);
   d.seg0 = (uint32_t)toff[p];
   tiles[i] = d;
 }
@@ -1346,11 +1345,8 @@ static int pick_tau(const wt_build_opts* o, int L, bool even, uint64_t n = 0) {
   if (tau < 1) tau = 1;
   if (tau > TAU_MAX) tau = TAU_MAX;
   if (even && (tau & 1)) tau = tau > 1 ? tau - 1 : 2;
-  (void)L;
   return tau;
 }
-
-// common workspace of a build
 
 // zero_bits: false when the build's own kernels zero the level buffer
 static wt_status alloc_outputs(wt_struct* h, uint64_t total_words, bool zero_bits = true) {
@@ -1671,7 +1667,6 @@ wt_status build_wt(const void* d_seq, uint64_t n, uint32_t sigma, int w, const w
     P.t = pg.t;
     P.rbits = pg.rbits;
     P.shape = SHAPE_WT;
-    P.digits = multiary ? 1 : 0;
     P.wt_C = Cn;
     P.ntiles = (uint32_t)ntiles0;
     P.n_in = n;

@@ -22,12 +22,11 @@ enum : uint32_t { ERR_SYMBOL = 1u, ERR_INTERNAL = 4u };
 enum Shape : int { SHAPE_WM = 0, SHAPE_WT = 1, SHAPE_HUFF = 2 };
 
 // One tile of a pass: `count` consecutive elements of T_a starting at
-// `start`, all inside node `node` (first: the first tile of its node).
+// `start`, all inside node `node`.
 struct TileDesc {
   uint64_t start;
   uint32_t count;
   uint32_t node;
-  uint32_t first;
   uint32_t seg0;  // index of the node's first tile
 };
 
@@ -88,7 +87,6 @@ struct PassParams {
   int a, t;                 // first level of the pass, levels in the pass
   int rbits;                // bits per input element that matter (L - a)
   int shape;
-  int digits;               // 1: emit 2-bit digit levels at even levels (multiary)
   // outputs
   uint64_t* bits;           // level bitmaps (or digit levels)
   const uint64_t* lvl_off;  // HUFF: word offset per level (the others' levels, of n_in
