@@ -21,6 +21,7 @@ from __future__ import annotations
 
 import argparse
 import ctypes
+import glob
 import hashlib
 import json
 import os
@@ -184,11 +185,10 @@ def measured_peak_hbm():
 
 
 def kernel_hash():
+    """Of the sources that the pass kernel is compiled from: its own file and
+    the headers beside it, every one that is there."""
     h = hashlib.sha256()
-    for f in ("k_pass.cuh", "wt_internal.cuh", "bitplane.cuh"):
-        p = os.path.join(ROOT, "paper_1610_03524_gb300", "csrc", f)
-        if f == "bitplane.cuh" and not os.path.exists(p):
-            continue
+    for p in sorted(glob.glob(os.path.join(ROOT, "paper_1610_03524_gb300", "csrc", "*.cuh"))):
         with open(p, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

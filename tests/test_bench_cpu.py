@@ -48,6 +48,32 @@ def test_kernel_hash_covers_the_pass_kernel_sources(tmp_path, monkeypatch):
         h0 = h1
 
 
+def test_kernel_hash_covers_every_header_of_the_pass_kernel(tmp_path, monkeypatch):
+    """Those that it includes, and one that is added beside them."""
+    import re
+    import shutil
+    src = os.path.join(ROOT, "paper_1610_03524_gb300", "csrc")
+    files, todo = set(), ["k_pass.cuh"]
+    while todo:
+        f = todo.pop()
+        files.add(f)
+        inc = re.findall(r'#include "([^"]+)"', open(os.path.join(src, f)).read())
+        todo += [g for g in inc if g not in files]
+    assert "bitplane.cuh" in files
+    dst = tmp_path / "paper_1610_03524_gb300" / "csrc"
+    dst.mkdir(parents=True)
+    for f in files:
+        shutil.copy(os.path.join(src, f), dst / f)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    seen = {bench.kernel_hash()}
+    for f in sorted(files) + ["another.cuh"]:
+        with open(dst / f, "a") as fh:
+            fh.write("\n")
+        h = bench.kernel_hash()
+        assert h not in seen, f
+        seen.add(h)
+
+
 def test_reference_arm_line():
     r = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference",
                         "--steps", "1", "--warmup", "0", "--cpu-log2n", "16"],
