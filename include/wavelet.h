@@ -16,11 +16,11 @@
  *    there); results are final once the stream is synchronised.  Calls that
  *    hand results to the host
  *    (wt_sync, wt_export, wt_export_select, wt_dd_merge for its parts,
- *    wt_free, wm_autotune, wm_autotune_config) synchronise the handle's stream themselves.  Device-side errors found during
- *    a build (a symbol >= sigma: WT_ERR_SYMBOL_GE_SIGMA; an internal table
- *    that disagrees with the data, which leaves the affected bits unwritten:
- *    WT_ERR_CUDA) are
- *    reported by wt_sync() or by the next call on the handle.
+ *    wt_free, wm_autotune, wm_autotune_config) synchronise the handle's stream
+ *    themselves.  Device-side errors found during a build (a symbol >= sigma:
+ *    WT_ERR_SYMBOL_GE_SIGMA; an internal table that disagrees with the data,
+ *    which leaves the affected bits unwritten: WT_ERR_CUDA) are reported by
+ *    wt_sync() or by the next call on the handle.
  *  * Symbol sequences are contiguous arrays of width_bytes = 1, 2 or 4
  *    (little-endian unsigned), read-only, borrowed for the duration of the
  *    call and never retained.  n must be below 2^40; longer sequences return
@@ -162,11 +162,13 @@ wt_status wm_build_host(const void* h_seq, uint64_t n, uint32_t sigma, uint32_t 
  * derive Huffman lengths from the sequence's histogram, limited to 32 bits.
  * Codes are canonical.  Level l holds the elements with code length > l,
  * ordered by their l-bit code prefix; its bit is code bit l.  sigma in
- * [1, 2^24].  The code is built on the host from the sequence's histogram,
- * so this build is asynchronous in a different way from the others: the call
- * enqueues a copy of d_seq on `stream` (d_seq may be released once the
- * stream has passed that point) and returns; a library thread then builds the
- * histogram, the code and the tree on the handle's own stream, which starts
+ * [1, 2^24].  The code is built from the sequence's histogram, on the device
+ * for alphabets of at least 2^16 symbols (without caller lengths, n below 2^32),
+ * else, and where a code would be longer than 32 bits, on the host.  Its level
+ * sizes decide what is launched, so this build is asynchronous in a different
+ * way from the others: the call enqueues a copy of d_seq on `stream` (d_seq may be released once the
+ * stream has passed that point) and returns; a library thread then has the
+ * histogram, the code and the tree built on the handle's own stream, which starts
  * after the copy.  Every later call on the handle (queries, wt_sync,
  * wt_export, wt_export_select, wt_query_multi, wt_free, wt_symbol_levels)
  * first waits for that thread and orders its own stream after the build.
@@ -260,7 +262,8 @@ wt_status wt_batch_free(wt_batch b);
 /* Autotuner for the levels per pass tau (Section 4.2: fewer, wider passes
  * against more work per pass).  Times wavelet-matrix builds of d_seq
  * (without directories; one untimed and the best of two timed builds) for
- * tau = 1 .. min(8, L), writes the fastest (at most 4) to *best_tau and the times to
+ * tau = 1 .. min(8, L) (above 4 as a build with that option runs, in passes of
+ * 4), writes the fastest (at most 4) to *best_tau and the times to
  * ms_out[tau-1] (ms_out may be NULL; 0 where not tried), and records it (with
  * the default tile and occupancy) for every later wm_build / wm_batch_build
  * with opts->tau == 0 of a sequence with the same L and ceil(log2 n).

@@ -147,10 +147,12 @@ __global__ void k_copy_bytes(uint8_t* dst, const uint8_t* src, uint64_t bytes) {
 
 // Huffman-shaped tree, asynchronous: the call enqueues a copy of the input on
 // the caller's stream (the input is borrowed only until that stream reaches
-// the copy) and returns; a library thread builds the code on the host from
-// the histogram and enqueues the build on the handle's own stream, which
-// starts after the copy.  Every later call on the handle first waits for
-// that thread and orders its own stream after the build (join_build).
+// the copy) and returns; a library thread enqueues the histogram, the code's
+// construction (on the device from HUFF_DEVICE_MIN symbols on, else on the host)
+// and the tree on the handle's own stream, which starts after the copy; either
+// way it waits for the code's level sizes.  Every later call on the handle first
+// waits for that thread and orders its own stream after the build (join_build);
+// the handle's stream waits for the queries in turn (release_after).
 wt_status huff_async(const void* d_seq, uint64_t n, uint32_t sigma, uint32_t width,
                      const uint8_t* h_len, const wt_build_opts* opts, wt_stream stream,
                      wt_handle* out) {

@@ -449,8 +449,9 @@ __global__ void __launch_bounds__(256) k_tile_counts(const __grid_constant__ Pas
 // and the lanes' sums by four warp reductions a tile.  No atomics, shared
 // memory or barriers: about 3 instructions per 32 symbols, so that DRAM is
 // the bound (2^32 symbols over 5 values with the zeroing of three levels:
-// 1.0 ms, 5.9 TB/s; shared-memory atomics per symbol took 1.8 ms).  A symbol >= SIG is flagged and counted as a zero (a single
-// pass scatters nothing by these counts).
+// 1.0 ms, 5.9 TB/s; shared-memory atomics per symbol took 1.8 ms).  A symbol >=
+// SIG is flagged; by which value it is counted does not matter (a single pass
+// scatters nothing by these counts).
 template <int SIG>
 __global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, uint64_t n,
                                                            uint32_t* err, uint32_t* tcnt,
@@ -519,7 +520,6 @@ __global__ void __launch_bounds__(256) k_count_tiles_bytes(const uint8_t* seq, u
   if (__any_sync(FULL, bad != 0u) && lane == 0) atomicOr(err, ERR_SYMBOL);
 }
 
-// Launch of a pass's tile counts into tcnt (mt tiles at most).
 // counts by k_count_tiles_bytes
 static bool byte_counts(const PassParams& P) {
   return P.in_w == 1 && !P.tiles && P.sigma >= 2 && P.sigma <= 8 && P.t == P.L;
@@ -533,7 +533,8 @@ static void launch_tile_counts(const PassParams& P, uint32_t T, unsigned grid, u
   else k_tile_counts<4, BATCH, SCAN><<<grid, 256, 0, st>>>(P, tcnt, T, sc);
 }
 
-// sc: the scans and the plan too (at most SCAN_TILES tiles)
+// Launch of a pass's tile counts into tcnt (mt tiles at most); sc: the scans and
+// the plan too (at most SCAN_TILES tiles).
 template <bool BATCH>
 static wt_status launch_counts(const PassParams& P, uint32_t T, uint64_t mt, uint32_t* tcnt,
                                const TileScan* sc, cudaStream_t st) {
@@ -1981,9 +1982,11 @@ static wt_status huff_tables_host(const uint64_t* hist, uint32_t sigma, const ui
 wt_status huff_tables_device(const uint64_t* hist, uint64_t n, uint32_t sigma, wt_struct* h,
                              uint32_t* d_left, std::vector<uint64_t>& node_lvl, bool* done);
 
-// Alphabets from which the code is built on the device: its launches take
-// about 0.6 ms whatever the alphabet, the host about 1 ms for 2^16 symbols and
-// 16 ms for 2^20 (and no time of the device's, if another build has it).
+// Alphabets from which the code is built on the device.  Whole trees over 2^16
+// symbols, with the code built here and on the host: 2^16 elements 0.92 and 1.53
+// ms, 2^22 1.13 and 3.55, 2^28 4.9 and 7.5.  Below some tens of thousands of
+// symbols the device's launches outweigh the host's work (2^16 elements over
+// 4000: 0.57 ms with the host's code).
 constexpr uint32_t HUFF_DEVICE_MIN = 1u << 16;
 
 // Copies of h->d_len and h->d_code into the handle's host vectors, ordered after

@@ -97,8 +97,9 @@ constexpr int DIR_SB_PER_WARP = WT_DIR_SB_PER_WARP;
 constexpr int DIR_SB_PER_BLOCK = 8 * DIR_SB_PER_WARP;  // 256 threads
 constexpr int DIR_GROUP = DIR_SB_PER_BLOCK;
 
-// Up to DIR_SMALL levels: their first groups and metadata ride in the kernel parameters, so a block finds its level without
-// a dependent load (else the tables are searched in global memory).
+// Up to DIR_SMALL levels: their first groups and metadata ride in the kernel
+// parameters, so a block finds its level without a dependent load (else the
+// tables are searched in global memory).
 constexpr int DIR_SMALL = 32;
 struct DirLevels {
   int nlev;

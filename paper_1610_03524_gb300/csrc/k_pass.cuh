@@ -27,21 +27,18 @@
 // offsets by prefix sums across the K sub-problems.
 //
 // What bounds it: instructions, most of them on the integer logic pipe (66% of
-// it used, 2.6 instructions per cycle and SM; DRAM below 20%), and the warps'
-// waits for each other three times a tile.  An earlier
-// form moved the elements once per level through shared memory (a ballot, a
-// rank and a store per 32 elements and level): 231 and 198 warp instructions
-// per 32 elements for its two passes of 8 levels, 14.3 ms for the 2^30 16-bit
-// symbols of 16 levels.  The four passes here took 69 (46 the last) and 10.8 ms
-// with the first element in a plane's low bit; with it in the top bit, where
-// half of a split's moves are multiplications, 10.1 ms (2^28 symbols: 2.74 and
-// 2.53 ms; 2^26 32-bit ones 0.93 and 0.86), and with the runs taken out by bulk
-// copies instead of a search for the run and a store for every word 64 (43) and
-// 9.8 ms (2^28: 2.44 ms; 32-bit 0.83).  One warp's lanes for both kinds of
-// runs, pieces masked in place and the splits' shared parities: 9.5 ms (2^28:
-// 2.37 ms; 32-bit 0.82).  The other warps take the work that warp 0, which
-// they wait for, had beside the runs' layout: 60 to 62 instructions (42 the
-// last pass) and 9.2 ms (2.32; 0.80).
+// its rate, 2.6 instructions per cycle and SM; DRAM at 10-20%), and the warps'
+// waits for each other three times a tile.  Per 32 elements a pass takes 60 to
+// 62 warp instructions, 42 the last one: the splits 13, the pieces 10, the move
+// 11, loading, planes and prefix sums 15, the runs and their way out the rest.
+// 2^30 16-bit symbols of 16 levels: 9.2 ms in four passes.  Moving every element
+// through shared memory once per level (a ballot, a rank and a store per 32
+// elements) in two passes of eight levels takes 231 and 198 instructions and
+// 14.3 ms.  Three choices carry the difference: planes, which move 32 elements'
+// bits at once; the first element in a plane's top bit, where half of a split's
+// moves are multiplications on an idle pipe (2^28 symbols: 2.53 ms of passes
+// against 2.74); and one bulk copy per run instead of a search and a store per
+// word (2.44 against 2.53).
 #pragma once
 #include <type_traits>
 

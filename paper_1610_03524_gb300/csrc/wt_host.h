@@ -102,8 +102,8 @@ struct wt_struct {
   // batched builds: the shared allocation holding every device array above
   wtk::Arena* arena = nullptr;
   // asynchronous builds (huff_wt_build): the library thread that builds the
-  // code on the host and enqueues the rest of the build on `stream` (then
-  // the handle's own stream), and the event recorded after its last work
+  // code or has it built, and enqueues the build on `stream` (then the
+  // handle's own), and the event recorded after its last work
   std::thread* worker = nullptr;
   cudaEvent_t built = nullptr;
   bool own_stream = false;

@@ -37,8 +37,8 @@ struct TileDesc {
 // (u64), the totals after the last chunk.
 constexpr int TC_STRIDE = 1 << TAU_MAX;  // row stride of both tables
 // Tiles per chunk: 64, which a block of 256 threads holds in one round of
-// loads, and more from 2^20 tiles on, so that the one block that scans the
-// chunks walks at most 16384.
+// loads, and more from 2^20 tiles on, so that the cluster that scans the chunks
+// walks at most 16384.
 constexpr uint64_t MAX_CHUNKS = 16384;
 inline int chunk_shift(uint64_t tiles) {
   int s = 6;
