@@ -151,11 +151,14 @@ struct Work {
     *p = (T*)q;
     return WT_OK;
   }
-  // several buffers: want() each, then take() them all; the small ones by one
-  // allocation (an allocation and its release cost the host about as much as a
-  // launch), the large ones each by its own, so that the pool finds blocks of
-  // their sizes again in the next build (one 4 GB block for all of them was
-  // split by the next build's levels and mapped anew: 0.3 ms)
+  // several buffers: want() each, then take() them all; the large ones each by
+  // its own allocation, so that the pool finds blocks of their sizes again in the
+  // next build (one 4 GB block for all of them was split by the next build's
+  // levels and mapped anew: 0.3 ms); then the small ones by one (an allocation and
+  // its release cost the host about as much as a launch).  The large ones first:
+  // the pool otherwise cuts the small ones out of a block that one of them needs,
+  // and maps memory anew (builds of 2^30 16-bit symbols, each result kept until
+  // the next is there: 11.1 ms; 12.1 with the small ones first).
   static constexpr size_t LARGE = 32u << 20;
   struct Want {
     void** p;
@@ -168,19 +171,20 @@ struct Work {
   }
   wt_status take() {
     size_t small = 0, at = 0;
-    for (const Want& w : wants) small += w.bytes < LARGE ? w.bytes : 0;
-    uint8_t* b = nullptr;
-    wt_status s = get(&b, small);
+    wt_status s = WT_OK;
     for (const Want& w : wants) {
-      if (s != WT_OK) return s;
-      if (w.bytes >= LARGE) {
-        uint8_t* q = nullptr;
-        s = get(&q, w.bytes);
-        *w.p = q;
-      } else {
-        *w.p = b + at;
-        at += w.bytes;
-      }
+      small += w.bytes < LARGE ? w.bytes : 0;
+      if (w.bytes < LARGE || s != WT_OK) continue;
+      uint8_t* q = nullptr;
+      s = get(&q, w.bytes);
+      *w.p = q;
+    }
+    uint8_t* b = nullptr;
+    if (s == WT_OK) s = get(&b, small);
+    for (const Want& w : wants) {
+      if (w.bytes >= LARGE || s != WT_OK) continue;
+      *w.p = b + at;
+      at += w.bytes;
     }
     wants.clear();
     return s;
