@@ -152,7 +152,7 @@ __global__ void k_copy_bytes(uint8_t* dst, const uint8_t* src, uint64_t bytes) {
 // and the tree on the handle's own stream, which starts after the copy; either
 // way it waits for the code's level sizes.  Every later call on the handle first
 // waits for that thread and orders its own stream after the build (join_build);
-// the handle's stream waits for the queries in turn (release_after).
+// wt_free makes the handle's stream wait for the queries in turn (queries_queued).
 wt_status huff_async(const void* d_seq, uint64_t n, uint32_t sigma, uint32_t width,
                      const uint8_t* h_len, const wt_build_opts* opts, wt_stream stream,
                      wt_handle* out) {
@@ -265,19 +265,59 @@ wt_status join_build(wt_struct* h, cudaStream_t st, bool order) {
   return join_build_impl(h, st, order);
 }
 
-wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st, bool own) {
-  auto other = [&](const wt_struct* h) { return h->stream != st && (h->own_stream || !own); };
-  if (std::none_of(hs, hs + nh, other)) return WT_OK;
+// One event for all of the handles, each of which keeps the last one of every
+// stream; recorded and stored under one lock, so that what is stored last covers
+// the queries of other threads on the same stream.
+static bool note_queries(wt_struct* const* hs, uint32_t nh, cudaStream_t st) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> g(mu);
+  unsigned long long id = 0;
+  if (cudaStreamGetId(st, &id) != cudaSuccess) return false;
+  std::shared_ptr<Event> ev;
+  for (uint32_t i = 0; i < nh; i++) {
+    wt_struct* const h = hs[i];
+    if (!h->own_stream || h->stream == st) continue;
+    std::vector<wt_struct::Used>& v = h->used;
+    auto u = std::find_if(v.begin(), v.end(), [&](const wt_struct::Used& x) { return x.stream == id; });
+    if (u == v.end()) {
+      // a new stream: those of streams that are done with the handle go
+      v.erase(std::remove_if(v.begin(), v.end(), [](const wt_struct::Used& x) {
+                return !x.ev || cudaEventQuery(x.ev->e) == cudaSuccess;
+              }), v.end());
+      if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();
+      u = v.insert(v.end(), wt_struct::Used{id, nullptr});
+    }
+    if (!ev) {
+      ev = u->ev && u->ev.use_count() == 1 ? u->ev : std::make_shared<Event>();
+      if (!ev->e && cudaEventCreateWithFlags(&ev->e, cudaEventDisableTiming) != cudaSuccess) return false;
+      if (cudaEventRecord(ev->e, st) != cudaSuccess) return false;
+    }
+    u->ev = ev;
+  }
+  return true;
+}
+
+wt_status queries_queued(wt_struct* const* hs, uint32_t nh, cudaStream_t st) {
+  if (std::none_of(hs, hs + nh, [&](wt_struct* h) { return h->own_stream && h->stream != st; }))
+    return WT_OK;
   // queries being captured run when their graph does, which the caller orders
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
     return WT_OK;
-  cudaEvent_t ev = nullptr;
-  bool ok = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventRecord(ev, st) == cudaSuccess;
+  try {
+    if (note_queries(hs, nh, st)) return WT_OK;
+  } catch (const std::bad_alloc&) {
+  }
+  cudaGetLastError();
+  return cudaStreamSynchronize(st) == cudaSuccess ? WT_OK : WT_ERR_CUDA;
+}
+
+wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st) {
+  Event ev;
+  bool ok = cudaEventCreateWithFlags(&ev.e, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventRecord(ev.e, st) == cudaSuccess;
   for (uint32_t i = 0; i < nh && ok; i++)
-    if (other(hs[i])) ok = cudaStreamWaitEvent(hs[i]->stream, ev, 0) == cudaSuccess;
-  if (ev) cudaEventDestroy(ev);
+    if (hs[i]->stream != st) ok = cudaStreamWaitEvent(hs[i]->stream, ev.e, 0) == cudaSuccess;
   if (ok) return WT_OK;
   cudaGetLastError();
   return cudaStreamSynchronize(st) == cudaSuccess ? WT_OK : WT_ERR_CUDA;
@@ -405,7 +445,7 @@ wt_status wt_dd_merge(const wt_handle* parts, uint32_t r, const wt_build_opts* o
   h->kind = p0->kind;
   h->L = h->levels = p0->L;
   s = dd_merge(parts, r, h);
-  if (s == WT_OK) s = release_after(parts, r, h->stream, false);
+  if (s == WT_OK) s = release_after(parts, r, h->stream);
   return finish(h, s, out);
 }
 
@@ -415,7 +455,7 @@ wt_status wt_access(wt_handle h, const uint64_t* d_i, uint64_t q, uint64_t* d_ou
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
   TRY(launch_query(h, 0, nullptr, d_i, q, d_out, (cudaStream_t)stream));
-  return release_after(&h, 1, (cudaStream_t)stream, true);
+  return queries_queued(&h, 1, (cudaStream_t)stream);
 }
 
 wt_status wt_rank(wt_handle h, const uint32_t* d_c, const uint64_t* d_i, uint64_t q,
@@ -424,7 +464,7 @@ wt_status wt_rank(wt_handle h, const uint32_t* d_c, const uint64_t* d_i, uint64_
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
   TRY(launch_query(h, 1, d_c, d_i, q, d_out, (cudaStream_t)stream));
-  return release_after(&h, 1, (cudaStream_t)stream, true);
+  return queries_queued(&h, 1, (cudaStream_t)stream);
 }
 
 wt_status wt_select(wt_handle h, const uint32_t* d_c, const uint64_t* d_k, uint64_t q,
@@ -433,7 +473,7 @@ wt_status wt_select(wt_handle h, const uint32_t* d_c, const uint64_t* d_k, uint6
   const wt_status s = join_build(h, (cudaStream_t)stream, true);
   if (s != WT_OK) return s;
   TRY(launch_query(h, 2, d_c, d_k, q, d_out, (cudaStream_t)stream));
-  return release_after(&h, 1, (cudaStream_t)stream, true);
+  return queries_queued(&h, 1, (cudaStream_t)stream);
 }
 
 wt_status wt_sync(wt_handle h) {
@@ -474,6 +514,8 @@ wt_status wt_free(wt_handle h) {
   // handle of a batch that is not the last one frees nothing and waits for
   // nothing
   join_build(h, h->stream, false);
+  for (const wt_struct::Used& u : h->used)
+    if (u.ev && cudaStreamWaitEvent(h->stream, u.ev->e, 0) != cudaSuccess) cudaEventSynchronize(u.ev->e);
   const bool owner = !h->arena;
   free_arrays(h, true);
   // the memory is back in the pool, for allocations on any stream

@@ -684,5 +684,5 @@ extern "C" wt_status wt_query_multi(const wt_handle* hs, uint32_t nh, const uint
     if (s != WT_OK) return s;
   }
   TRY(launch_query_multi(hs, nh, d_sid, d_op, d_c, d_x, q, d_out, (cudaStream_t)stream));
-  return release_after(hs, nh, (cudaStream_t)stream, true);
+  return queries_queued(hs, nh, (cudaStream_t)stream);
 }

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -21,6 +22,13 @@ struct Arena {
   void* base = nullptr;
   std::atomic<int> refs{0};
   uint64_t bytes = 0;
+};
+
+struct Event {
+  cudaEvent_t e = nullptr;
+  ~Event() {
+    if (e) cudaEventDestroy(e);
+  }
 };
 
 // Per-level metadata used by the query kernels (device copy in the handle).
@@ -107,6 +115,13 @@ struct wt_struct {
   std::thread* worker = nullptr;
   cudaEvent_t built = nullptr;
   bool own_stream = false;
+  // with own_stream: an event after the last query of every stream that had any,
+  // which wt_free waits for
+  struct Used {
+    unsigned long long stream;  // its id (a destroyed stream's pointer comes back)
+    std::shared_ptr<wtk::Event> ev;
+  };
+  std::vector<Used> used;
 };
 
 namespace wtk {
@@ -116,10 +131,12 @@ namespace wtk {
 // the handle's deferred status
 wt_status join_build(wt_struct* h, cudaStream_t st, bool order);
 
-// What has just been queued on st reads the arrays of the nh handles: make the
-// streams on which wt_free will release them wait for it.
-// own: only handles on a stream of their own, which no caller can order.
-wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st, bool own);
+// What has just been queued on st reads the arrays of the nh handles.
+// queries_queued: wt_free of the handles on a stream of their own, which no
+// caller can order, waits for it.  release_after: the streams of all of them,
+// on which wt_free releases them, wait for it.
+wt_status queries_queued(wt_struct* const* hs, uint32_t nh, cudaStream_t st);
+wt_status release_after(wt_struct* const* hs, uint32_t nh, cudaStream_t st);
 
 // device memory helpers (stream-ordered pools)
 cudaError_t dmalloc(void** p, size_t bytes, cudaStream_t s);

@@ -87,3 +87,35 @@ def test_parts_freed_behind_a_queued_merge(wt):
     assert np.array_equal(ex.bits.reshape(ob.shape), ob) and np.array_equal(ex.zeros, oz)
     h.free()
     again.free()
+
+
+def test_queries_of_several_streams(wt):
+    """Every stream's queries are waited for, by the release only: a stream's
+    last ones after earlier ones on it and on others, and trees that share a
+    launch."""
+    import torch
+    n, sigma, q = 150_001, 500, 1000
+    S = synth.zipf(15, n, sigma, 1.1, 2)
+    x = np.random.default_rng(16).integers(0, n, q).astype(np.uint64)
+    dx = to_dev(x)
+    hs = [wt.huff_wt_build(to_dev(S), sigma) for _ in range(2)]
+    for h in hs:
+        h.sync()
+    zero = torch.zeros(q, dtype=torch.int32, device="cuda")
+    ops = torch.zeros(q, dtype=torch.uint8, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = [torch.zeros(q, dtype=torch.int64, device="cuda") for _ in range(6)]
+    torch.cuda.synchronize()
+    for k, s in enumerate(streams):
+        with torch.cuda.stream(s):
+            hs[0].access(dx, outs[k])
+            torch.cuda._sleep((k + 1) * SPIN // 2)
+            wt.query_multi(hs, zero + (k & 1), ops, zero, dx, outs[3 + k])
+    for h in hs:
+        h.sync()  # of the build alone
+    assert not streams[2].query()
+    hs[0].free()
+    assert all(s.query() for s in streams)
+    hs[1].free()
+    for o in outs:
+        assert np.array_equal(from_dev_u64(o), S[x].astype(np.uint64))
